@@ -423,6 +423,7 @@ static cudaError_t bp_dispatch_vol(const BpArgs &a, const Images &img)
 cudaError_t launch_backproject(const BpArgs &a)
 {
     const Grid &G = *a.grid;
+    if (a.column) return launch_backproject_column(a);
     if (a.atlas) return bp_dispatch_vol(a, AtlasImages{*a.atlas});
     if (a.r_dtype == CTREX_F32)
         return bp_dispatch_vol(a, LinearImages<float>{static_cast<const float *>(a.r), G.nu, G.nv});

@@ -1,0 +1,387 @@
+// bp_column.cu -- the weighted backprojection of backproject.cu for scans
+// whose detector columns run along z: a warp takes 32 voxels of a z column,
+// whose projections run along one detector column, and the correction images
+// are in column layout (column.cuh), (value v, value v + 1) per element.
+#include "column.cuh"
+#include "cylinder.cuh"
+
+#include <type_traits>
+
+namespace ctrex {
+
+constexpr int BPC_WX = 8, BPC_WY = 1;  // z columns of a CTA (one per warp)
+constexpr int BPC_COLS = BPC_WX * BPC_WY;
+constexpr int BPC_THREADS = 32 * BPC_COLS;
+constexpr int BPC_CHUNK = 128;  // views staged at a time
+constexpr int BPC_MIN_BLOCKS = 5;  // 48 registers (4 and 6: 22.1 and 21.8 ms where 5 takes 19.2)
+constexpr int BPC_SUBV_MIN_BLOCKS = 4;
+
+// The correction images [n][nu][nv] in column layout: pair (u, v) of image k,
+// padded indices (u + 1, v + 1), at k view + (v >> 4) sv + (u << 4) + v.
+struct ColImages {
+    const float2 *p;
+    size_t view;    // pairs per image
+    unsigned sv;    // pairs from chunk to chunk, less the 16 that v itself counts
+    unsigned bias;  // -index(bits of 2^23, bits of 2^23): see bp_load
+};
+
+// One view of the staged chunk.
+struct ColView {
+    float4 p0, p1, p2;                   // rows of P; p2 = 0: skipped
+    const float2 *img;
+    // -1: every voxel of the CTA projects outside the window; 1: every one
+    // inside it; 2: and at one depth along z, to FP32 rounding; 0: neither
+    int inside;
+    int pad;
+};
+
+__device__ __forceinline__ float col_recip(float x)
+{
+    float r0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x));
+    return r0 * fmaf(-x, r0, 2.0f);
+}
+
+// The loads of a bilinear sample at (u, v), each in [-1, n), and its
+// fractions: floor + 1 comes out of adding 2^23 + 1 rounded down (the low
+// mantissa bits), without a conversion.
+struct BpTaps {
+    float2 q0, q1;
+    float au, av;
+};
+__device__ __forceinline__ BpTaps bp_load(const ColImages &I, const float2 *img, float u, float v)
+{
+    constexpr float M = 8388609.0f;
+    BpTaps t;
+    const float mu = __fadd_rd(u, M), mv = __fadd_rd(v, M);
+    t.au = u - (mu - M);
+    t.av = v - (mv - M);
+    const unsigned bu = __float_as_uint(mu), bv = __float_as_uint(mv);
+    const unsigned i = (bv >> COL_LOG) * I.sv + ((bu << COL_LOG) + (bv + I.bias));
+    const float2 *q = img + i;
+    t.q0 = __ldg(q);
+    t.q1 = __ldg(q + (1 << COL_LOG));
+    return t;
+}
+__device__ __forceinline__ float bp_interp(const BpTaps &t)
+{
+    const float2 c = lerp2(t.q0, t.q1, two(t.au));
+    return fmaf(t.av, c.y - c.x, c.x);
+}
+
+// One voxel-view term in general position, as bp_term in backproject.cu.
+__device__ __forceinline__ void bp_edge(const ColImages &I, const float2 *img, float h1, float h2,
+                                        float h3, float4 win, float &b, float &c)
+{
+    if (!(h3 > 0.0f)) return;
+    const float inv = col_recip(h3);
+    const float u = h1 * inv, v = h2 * inv;
+    if (!(u > win.x - 1.0f && u < win.y + 1.0f && v > win.z - 1.0f && v < win.w + 1.0f)) return;
+    const BpTaps t = bp_load(I, img, u, v);
+    const float2 q0 = t.q0, q1 = t.q1;
+    const float au = t.au, av = t.av;
+    const float fu = u - au, fv = v - av;
+    const float wu0 = fu >= win.x ? 1.0f - au : 0.0f, wu1 = fu + 1.0f <= win.y ? au : 0.0f;
+    const float wv0 = fv >= win.z ? 1.0f - av : 0.0f, wv1 = fv + 1.0f <= win.w ? av : 0.0f;
+    b += fmaf(wv0, fmaf(wu0, q0.x, wu1 * q1.x), wv1 * fmaf(wu0, q0.y, wu1 * q1.y));
+    c += (wu0 + wu1) * (wv0 + wv1);
+}
+
+// ColView::inside of the points of a box: its corners decide (the image of a
+// box in front of the source is the hull of its corners' images), by a margin
+// that covers the rounding of u and v, bounded from the size of the terms
+// they are summed from.
+__device__ __forceinline__ int box_inside(float4 p0, float4 p1, float4 p2, const float lo[3], const float hi[3],
+                                          float4 win)
+{
+    const float e = 0.02f;
+    float m[3], h3min = INFINITY, u0 = INFINITY, u1 = -INFINITY, v0 = INFINITY, v1 = -INFINITY;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m[a] = fmaxf(fabsf(lo[a]), fabsf(hi[a]));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float x = i & 1 ? hi[0] : lo[0], y = i & 2 ? hi[1] : lo[1], z = i & 4 ? hi[2] : lo[2];
+        const float h3 = fmaf(p2.x, x, fmaf(p2.y, y, fmaf(p2.z, z, p2.w)));
+        const float u = fmaf(p0.x, x, fmaf(p0.y, y, fmaf(p0.z, z, p0.w))) / h3;
+        const float v = fmaf(p1.x, x, fmaf(p1.y, y, fmaf(p1.z, z, p1.w))) / h3;
+        h3min = fminf(h3min, h3);
+        u0 = fminf(u0, u);
+        u1 = fmaxf(u1, u);
+        v0 = fminf(v0, v);
+        v1 = fmaxf(v1, v);
+    }
+    const float s1 = fabsf(p0.x) * m[0] + fabsf(p0.y) * m[1] + fabsf(p0.z) * m[2] + fabsf(p0.w);
+    const float s2 = fabsf(p1.x) * m[0] + fabsf(p1.y) * m[1] + fabsf(p1.z) * m[2] + fabsf(p1.w);
+    const float s3 = fabsf(p2.x) * m[0] + fabsf(p2.y) * m[1] + fabsf(p2.z) * m[2] + fabsf(p2.w);
+    const float umax = fmaxf(fabsf(u0), fabsf(u1)), vmax = fmaxf(fabsf(v0), fabsf(v1));
+    if (!(h3min > 0.0f && fmaxf(s1 + umax * s3, s2 + vmax * s3) * 1e-6f < e * h3min)) return 0;
+    if (u1 < win.x - 1.0f - e || u0 > win.y + 1.0f + e || v1 < win.z - 1.0f - e || v0 > win.w + 1.0f + e) return -1;
+    if (!(u0 >= win.x + e && u1 <= win.y - e && v0 >= win.z + e && v1 <= win.w - e)) return 0;
+    // depth changes by less than half a unit in the last place along z
+    return fabsf(p2.z) * (hi[2] - lo[2]) < h3min * 0x1p-25f ? 2 : 1;
+}
+
+// VZ: voxels per thread, 32 slices apart.  SUBV, CYL: as bp_kernel in backproject.cu; DYR: as bp_dyrect_kernel.
+template <typename TV, int VZ, bool WINDOW, bool SUBV, bool CYL, bool DYR>
+__global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR ? 4 : BPC_MIN_BLOCKS))
+    bp_column_kernel(Grid G, const ViewGPU *__restrict__ views, const int *__restrict__ view_idx, int n_idx,
+                     const ColImages I, const int4 *__restrict__ window, TV *__restrict__ vol,
+                     const float *__restrict__ w, float alpha, int normalize, int accumulate, int sv, const CylGPU cyl,
+                     const float *__restrict__ tau, const float *__restrict__ t_view)
+{
+    constexpr int NP = DYR ? 2 : 1;  // value fields
+    __shared__ ColView sV[BPC_CHUNK];
+    __shared__ float4 sWin[WINDOW ? BPC_CHUNK : 1];
+    __shared__ float sT[DYR ? BPC_CHUNK : 1];
+    __shared__ int sAll;  // the least `inside` of the chunk's views
+    __shared__ float2 sOut[32 * VZ][BPC_COLS + 1];
+    __shared__ float sXY[2][BPC_COLS];
+    const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+    // (warps past the volume's edge repeat its last column and write nothing)
+    const int ix = min(blockIdx.x * BPC_WX + warp % BPC_WX, G.nx - 1);
+    const int iy = min(blockIdx.y * BPC_WY + warp / BPC_WX, G.ny - 1);
+    // the last block of a column starts early enough to be full and writes
+    // only the slices that the block before it did not take
+    const int zfirst = blockIdx.z * (32 * VZ), z0 = max(min(zfirst, G.nz - 32 * VZ), 0), iz = z0 + lane;
+    const float4 det = make_float4(0.0f, (float)(G.nu - 1), 0.0f, (float)(G.nv - 1));
+    // the frame point of the first voxel, and the step to the next one
+    float x = (float)ix, y = (float)iy, z = (float)iz, dz = 32.0f;
+    float zlo = (float)z0, zhi = zlo + 32.0f * VZ - 1.0f;
+    if (CYL && !SUBV) {
+        cyl_point(cyl, x, y, (float)iz, x, y, z);
+        dz = 32.0f * cyl.dz;
+        zlo = (zlo - cyl.zc) * cyl.dz;
+        zhi = (zhi - cyl.zc) * cyl.dz;
+    }
+    if (lane == 0) {
+        sXY[0][warp] = x;
+        sXY[1][warp] = y;
+    }
+    __syncthreads();
+    // box of the CTA's points
+    float lo[3] = {sXY[0][0], sXY[1][0], zlo}, hi[3] = {sXY[0][0], sXY[1][0], zhi};
+#pragma unroll
+    for (int i = 1; i < BPC_COLS; ++i)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            lo[a] = fminf(lo[a], sXY[a][i]);
+            hi[a] = fmaxf(hi[a], sXY[a][i]);
+        }
+    if (SUBV)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] -= 0.5f;
+            hi[a] += 0.5f;
+        }
+    float ta[VZ];
+    if (DYR)
+#pragma unroll
+        for (int q = 0; q < VZ; ++q)
+            ta[q] = iz + 32 * q < G.nz ? __ldg(tau + ((size_t)(iz + 32 * q) * G.ny + iy) * G.nx + ix) : 0.0f;
+    float b[NP][VZ], c[NP][VZ];
+#pragma unroll
+    for (int f = 0; f < NP; ++f)
+#pragma unroll
+        for (int q = 0; q < VZ; ++q) b[f][q] = c[f][q] = 0.0f;
+    const int total = n_idx * G.n_sub;
+    for (int base = 0; base < total; base += BPC_CHUNK) {
+        const int cnt = min(BPC_CHUNK, total - base);
+        __syncthreads();
+        if (tid == 0) sAll = SUBV ? 0 : 2;
+        __syncthreads();
+        for (int t = tid; t < cnt; t += BPC_THREADS) {
+            const int k = (base + t) / G.n_sub, s = base + t - k * G.n_sub;
+            int view = view_idx ? view_idx[k] : k;
+            const bool ok = view >= 0 && view < G.n_views;
+            if (!ok) view = 0;
+            const float *P = views[view * G.n_sub + s].P;
+            ColView V;
+            V.p0 = make_float4(P[0], P[1], P[2], P[3]);
+            V.p1 = make_float4(P[4], P[5], P[6], P[7]);
+            // an invalid view index gets a zero depth row: it is skipped
+            V.p2 = ok ? make_float4(P[8], P[9], P[10], P[11]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            V.img = I.p + (size_t)k * I.view;
+            float4 win = det;
+            if (WINDOW) {
+                const int4 wd = window[view];
+                win = make_float4((float)wd.x, (float)wd.y, (float)wd.z, (float)wd.w);
+                sWin[t] = win;
+            }
+            V.inside = SUBV && CYL ? 0 : box_inside(V.p0, V.p1, V.p2, lo, hi, win);
+            sV[t] = V;
+            if (V.inside < 2) atomicMin(&sAll, V.inside);
+            if (DYR) sT[t] = __ldg(t_view + view);
+        }
+        __syncthreads();
+        // ALL: what is known of every view of the chunk
+        auto term = [&](int m, auto all) {
+            constexpr int ALL = decltype(all)::value;
+            const float4 p0 = sV[m].p0, p1 = sV[m].p1, p2 = sV[m].p2;
+            const float2 *img = sV[m].img;
+            const bool inside = sV[m].inside > 0;
+            if (ALL == 0 && sV[m].inside < 0) return;
+            const float4 win = WINDOW ? sWin[m] : det;
+            const float tv = DYR ? sT[m] : 0.0f;
+            auto add = [&](int q, float tb, float tc) {
+                if (DYR) {
+                    const bool early = tv < ta[q];
+                    b[0][q] += early ? tb : 0.0f;
+                    c[0][q] += early ? tc : 0.0f;
+                    b[NP - 1][q] += early ? 0.0f : tb;
+                    c[NP - 1][q] += early ? 0.0f : tc;
+                } else {
+                    b[0][q] += tb;
+                    c[0][q] += tc;
+                }
+            };
+            // the VZ points h + q (d0, d1, d2); inside: all their loads first
+            auto points = [&](float h1, float h2, float h3, float d0, float d1, float d2) {
+                if (ALL || inside) {
+                    BpTaps t[VZ];
+                    const float inv0 = ALL == 2 ? col_recip(h3) : 0.0f;
+#pragma unroll
+                    for (int q = 0; q < VZ; ++q) {
+                        const float inv = ALL == 2 ? inv0 : col_recip(fmaf((float)q, d2, h3));
+                        t[q] = bp_load(I, img, fmaf((float)q, d0, h1) * inv, fmaf((float)q, d1, h2) * inv);
+                    }
+#pragma unroll
+                    for (int q = 0; q < VZ; ++q) add(q, bp_interp(t[q]), ALL > 0 && !DYR ? 0.0f : 1.0f);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < VZ; ++q) {
+                        float tb = 0.0f, tc = 0.0f;
+                        bp_edge(I, img, fmaf((float)q, d0, h1), fmaf((float)q, d1, h2), fmaf((float)q, d2, h3), win, tb,
+                                tc);
+                        add(q, tb, tc);
+                    }
+                }
+            };
+            if (SUBV) {
+                const float d = 1.0f / (float)sv, o = 0.5f * d - 0.5f;
+                for (int az = 0; az < sv; ++az)
+                    for (int ay = 0; ay < sv; ++ay) {
+                        const float gy = (float)iy + fmaf((float)ay, d, o);
+                        float sn = 0.0f, cs = 0.0f;
+                        if (CYL) sincosf((gy + 0.5f) * cyl.dphi, &sn, &cs);
+                        for (int ax = 0; ax < sv; ++ax) {
+                            const float gx = (float)ix + fmaf((float)ax, d, o);
+                            float X = gx, Y = gy, Z = (float)iz + fmaf((float)az, d, o), D = 32.0f;
+                            if (CYL) {
+                                const float r = (gx + 0.5f) * cyl.dr;
+                                X = r * cs;
+                                Y = r * sn;
+                                Z = (Z - cyl.zc) * cyl.dz;
+                                D = 32.0f * cyl.dz;
+                            }
+                            const float h1 = fmaf(p0.x, X, fmaf(p0.y, Y, fmaf(p0.z, Z, p0.w)));
+                            const float h2 = fmaf(p1.x, X, fmaf(p1.y, Y, fmaf(p1.z, Z, p1.w)));
+                            const float h3 = fmaf(p2.x, X, fmaf(p2.y, Y, fmaf(p2.z, Z, p2.w)));
+                            points(h1, h2, h3, D * p0.z, D * p1.z, D * p2.z);
+                        }
+                    }
+                return;
+            }
+            const float h1 = fmaf(p0.x, x, fmaf(p0.y, y, fmaf(p0.z, z, p0.w)));
+            const float h2 = fmaf(p1.x, x, fmaf(p1.y, y, fmaf(p1.z, z, p1.w)));
+            const float h3 = fmaf(p2.x, x, fmaf(p2.y, y, fmaf(p2.z, z, p2.w)));
+            points(h1, h2, h3, dz * p0.z, dz * p1.z, dz * p2.z);
+        };
+        const int all = sAll;
+        if (all == 2)
+            for (int m = 0; m < cnt; ++m) term(m, std::integral_constant<int, 2>());
+        else if (all == 1)
+            for (int m = 0; m < cnt; ++m) term(m, std::integral_constant<int, 1>());
+        else
+            for (int m = 0; m < cnt; ++m) term(m, std::integral_constant<int, 0>());
+        if (!DYR && all > 0)  // each view weighed 1
+#pragma unroll
+            for (int q = 0; q < VZ; ++q) c[0][q] += (float)cnt;
+    }
+    // The sums go to shared memory, and from there to the volume with the
+    // threads along x: a z column's own order would touch a line per voxel.
+    const float mean = SUBV ? G.inv_sub / (float)(sv * sv * sv) : G.inv_sub;
+    const size_t nvox = (size_t)G.nx * G.ny * G.nz;
+    const int oc = tid % BPC_COLS, ox = blockIdx.x * BPC_WX + oc % BPC_WX, oy = blockIdx.y * BPC_WY + oc / BPC_WX;
+#pragma unroll
+    for (int f = 0; f < NP; ++f) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < VZ; ++q) {
+            const float cc = c[f][q] * mean;
+            sOut[lane + 32 * q][warp] =
+                make_float2(b[f][q] * mean, normalize ? alpha * (cc > 1e-6f ? 1.0f / cc : 0.0f) : alpha);
+        }
+        __syncthreads();
+        if (ox >= G.nx || oy >= G.ny) continue;
+        for (int r = tid / BPC_COLS; r < 32 * VZ; r += BPC_THREADS / BPC_COLS) {
+            const int oz = z0 + r;
+            if (oz < zfirst || oz >= G.nz) continue;
+            const size_t j = ((size_t)oz * G.ny + oy) * G.nx + ox + (size_t)f * nvox;
+            const float2 o = sOut[r][oc];
+            const float upd = (w ? o.y * __ldg(w + j) : o.y) * o.x;
+            Storage<TV>::store(vol + j, accumulate ? Storage<TV>::load(vol + j) + upd : upd);
+        }
+    }
+}
+
+template <typename TV, int VZ, bool SUBV, bool CYL, bool DYR>
+static cudaError_t bpc_launch(const BpArgs &a)
+{
+    const Grid &G = *a.grid;
+    const ColStore &s = *a.column;
+    ColImages I;
+    I.p = s.buf;
+    I.view = s.view;
+    I.sv = s.sy;
+    const unsigned m = 0x4B000000u;  // the bits of 2^23
+    I.bias = 0u - ((m >> COL_LOG) * I.sv + (m << COL_LOG) + m);
+    const dim3 grid((G.nx + BPC_WX - 1) / BPC_WX, (G.ny + BPC_WY - 1) / BPC_WY, (G.nz + 32 * VZ - 1) / (32 * VZ));
+    const CylGPU cyl = a.cyl ? *a.cyl : CylGPU{};
+    const float *tau = a.dyr ? a.dyr->tau : nullptr, *tv = a.dyr ? a.dyr->t_view : nullptr;
+    if (a.window)
+        bp_column_kernel<TV, VZ, true, SUBV, CYL, DYR><<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
+            G, a.views, a.view_idx, a.n_idx, I, a.window, static_cast<TV *>(a.vol), a.w, a.alpha, a.normalize,
+            a.accumulate, a.subvox, cyl, tau, tv);
+    else
+        bp_column_kernel<TV, VZ, false, SUBV, CYL, DYR><<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
+            G, a.views, a.view_idx, a.n_idx, I, nullptr, static_cast<TV *>(a.vol), a.w, a.alpha, a.normalize,
+            a.accumulate, a.subvox, cyl, tau, tv);
+    return cudaGetLastError();
+}
+
+// Voxels per thread: 4 where 128-slice blocks fit the volume to within 14 %
+// of 64-slice ones (144 views at 512^3: 21.7 ms with 4, 24.7 with 2, 27 with 8).
+static bool four_voxels(int nz)
+{
+    const int n4 = (nz + 127) / 128 * 128, n2 = (nz + 63) / 64 * 64;
+    return 100 * n4 < 114 * n2;
+}
+
+template <typename TV, bool CYL> static cudaError_t bpc_plain(const BpArgs &a)
+{
+    return four_voxels(a.grid->nz) ? bpc_launch<TV, 4, false, CYL, false>(a)
+                                   : bpc_launch<TV, 2, false, CYL, false>(a);
+}
+
+template <typename TV> static cudaError_t bpc_dispatch(const BpArgs &a)
+{
+    if (a.dyr) {
+        if (a.cyl || a.subvox > 1) return cudaErrorInvalidValue;
+        return bpc_launch<TV, 2, false, false, true>(a);
+    }
+    if (a.subvox > 1)
+        return a.cyl ? bpc_launch<TV, 2, true, true, false>(a) : bpc_launch<TV, 2, true, false, false>(a);
+    return a.cyl ? bpc_plain<TV, true>(a) : bpc_plain<TV, false>(a);
+}
+
+cudaError_t launch_backproject_column(const BpArgs &a)
+{
+    return a.vol_dtype == CTREX_F32 ? bpc_dispatch<float>(a) : bpc_dispatch<__nv_bfloat16>(a);
+}
+
+bool backproject_column_fits(const Grid &G)
+{
+    return (G.ny + BPC_WY - 1) / BPC_WY <= 65535 && (G.nz + 63) / 64 <= 65535;
+}
+
+}  // namespace ctrex

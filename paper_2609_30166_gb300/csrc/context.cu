@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "atlas.cuh"
+#include "column.cuh"
 #include "ctrex_internal.cuh"
 
 using namespace ctrex;
@@ -46,6 +47,10 @@ struct ctrex_ctx {
     // texture atlas of the volume read by the forward projector
     AtlasStore vol_atlas;
     Atlas vol_atlas_view;
+    // the volume in column layout, where the scan's detector columns run along z
+    double col_lean = 10.0, col_step = 1.0;  // detector_column_step
+    ColStore vol_col;
+    ColStore img_col;  // the correction images
     // texture atlas of the correction images read by the backprojector
     AtlasStore img_atlas;
     Atlas img_atlas_view;
@@ -222,6 +227,39 @@ void dyr_release(ctrex_ctx *c)
     atlas_release(c->tau_atlas);
 }
 
+// Which scans take the column kernels (fwd_column.cu, bp_column.cu) and which
+// stay with texture gathers, by measurement on a 512^3 volume:
+// - the detector rotated in its plane (768^2 pixels, 72 views; ms column /
+//   texture at 0, 20, 30, 45, 90 degrees): forward 30 / 73, 53 / 81, 65 / 92,
+//   81 / 113, 231 / 183; backprojection 9.4 / 17.8, 12.9 / 17.8, 16.9 / 17.8,
+//   24.2 / 17.8, 64 / 17.7;
+// - coarse pixels spread a warp's rays (pixel steps of 2, 4, 8 voxels):
+//   forward FP32 13.6 / 27.0, 11.7 / 22.3, 19.4 / 15.9 ms, BF16 13.6 / 14.4,
+//   11.7 / 10.9, 19.4 / 7.8 ms;
+// - fine pixels spread a warp's voxels (768^2 pixels, 90 views, voxel steps
+//   of 2 and 4 pixels): backprojection 2.0 / 3.0 ms, 0.66 / 0.62 ms.
+constexpr double COL_LEAN_FWD = 1.0, COL_LEAN_BP = 0.55, COL_STEP_FP32 = 6.0, COL_STEP_BF16 = 3.0;
+constexpr double COL_STEP_BP_MIN = 0.3;
+
+// The forward projector: also the lanes that each kernel's tiles (4 x 32
+// columns x rows here, 32 x 4 there) waste on a ragged detector, against the
+// kernels' speeds (2.4 : 1 with FP32 volumes, whose gathers carry one slice,
+// and 1.27 : 1 with BF16 ones).
+bool column_forward(const ctrex_ctx *c, int vdt)
+{
+    if (!(c->col_lean <= COL_LEAN_FWD && column_grid_fits(c->grid))) return false;
+    if (c->col_step > (vdt == CTREX_F32 ? COL_STEP_FP32 : COL_STEP_BF16)) return false;
+    const double u4 = (c->grid.nu + 3) / 4 * 4.0, u32 = (c->grid.nu + 31) / 32 * 32.0;
+    const double v4 = (c->grid.nv + 3) / 4 * 4.0, v32 = (c->grid.nv + 31) / 32 * 32.0;
+    return u4 * v32 <= u32 * v4 * (vdt == CTREX_F32 ? 2.2 : 1.2);
+}
+
+bool column_backproject(const ctrex_ctx *c)
+{
+    return c->col_lean <= COL_LEAN_BP && c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(c->grid) &&
+           (!c->roi || backproject_column_fits(c->roi_grid));
+}
+
 // Uploads vol into the context's texture atlas and points a.atlas at it; if
 // the volume does not fit the 2D texture limits the row-major path is used.
 int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
@@ -301,6 +339,16 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
         c->vol_atlas_view = atlas_view(c->vol_atlas);
         a.atlas = &c->vol_atlas_view;
         return CTREX_OK;
+    }
+    if (!c->has_motion && column_forward(c, vdt)) {
+        cudaError_t e = col_ensure(c->vol_col, c->grid.nx, c->grid.ny, c->grid.nz, c->stream);
+        if (e == cudaSuccess) {
+            e = col_upload(c->vol_col, vol, vdt, c->stream);
+            if (e != cudaSuccess) return cuda_fail(c, e, "volume column upload");
+            a.column = &c->vol_col;
+            return CTREX_OK;
+        }
+        if (e != cudaErrorInvalidValue) return cuda_fail(c, e, "volume column layout");
     }
     if (c->atlas_unfit) return CTREX_OK;
     // BF16 volumes: slice pairs packed in 32-bit texels, one gather per sample
@@ -417,6 +465,8 @@ int ctrex_destroy(ctrex_ctx *c)
         dfree(c->d_window);
         dfree(c->d_subset_sums);
         atlas_release(c->vol_atlas);
+        col_release(c->vol_col);
+        col_release(c->img_col);
         atlas_release(c->img_atlas);
         atlas_release(c->jos_atlas);
         atlas_release(c->roi_atlas);
@@ -506,6 +556,21 @@ static int compute_views(ctrex_ctx *c, const double *P, int nvs, int n_sub, cons
     return CTREX_OK;
 }
 
+// A pixel step along a detector column, in index coordinates at the volume's
+// depth: its sideways part over its part along z, and the latter (means over
+// the views).
+static void detector_column_step(const std::vector<ViewGPU> &hv, double &lean, double &step)
+{
+    lean = step = 0.0;
+    for (const ViewGPU &V : hv) {
+        const double xy = sqrt((double)V.qv[0] * V.qv[0] + (double)V.qv[1] * V.qv[1]), z = fabs((double)V.qv[2]);
+        lean += xy <= 10.0 * z ? xy / z : 10.0;
+        step += z;
+    }
+    lean /= (double)hv.size();
+    step /= (double)hv.size();
+}
+
 static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub, const int n[3], const double vox[3],
                           const double origin[3], const double ctr[3], double min_pitch, const ctrex_det_grid *det,
                           double step_vox)
@@ -564,6 +629,7 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
     c->has_geom = true;
     c->atlas_unfit = false;
     c->img_atlas_unfit = false;
+    detector_column_step(hv, c->col_lean, c->col_step);
     set_clip_box(c);
     return CTREX_OK;
 }
@@ -965,7 +1031,17 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
     a.subvox = c->bp_subvoxel;
     a.cyl = c->cyl ? &c->cylg : nullptr;
     a.dyr = c->dyr ? &c->dyra : nullptr;
-    if (n_idx > 0 && !c->img_atlas_unfit) {
+    if (n_idx > 0 && column_backproject(c)) {
+        cudaError_t ae = col_ensure_images(c->img_col, c->grid.nu, c->grid.nv, n_idx, c->stream);
+        if (ae == cudaSuccess) {
+            ae = col_upload_images(c->img_col, r, rdt, n_idx, c->stream);
+            if (ae != cudaSuccess) return cuda_fail(c, ae, "image column upload");
+            a.column = &c->img_col;
+        } else if (ae != cudaErrorInvalidValue) {
+            return cuda_fail(c, ae, "image column layout");
+        }
+    }
+    if (n_idx > 0 && !a.column && !c->img_atlas_unfit) {
         cudaError_t ae = atlas_ensure(c->img_atlas, c->grid.nu, c->grid.nv, n_idx, rdt == CTREX_BF16, c->device);
         if (ae == cudaErrorInvalidValue) {
             cudaGetLastError();

@@ -97,6 +97,7 @@ enum : unsigned { DEVCHECK_OOB = 1u };
 // ---- host-side launchers (defined in project.cu / backproject.cu / ...) ----
 
 struct Atlas;
+struct ColStore;
 
 // Event-based 4D model (Sec. 3.3): with these set, volume buffers hold mu0
 // followed by mu1 (2 nx ny nz elements) and view v sees mu0 at the voxels
@@ -126,6 +127,7 @@ cudaError_t launch_tau_bricks(const float *tau, int nx, int ny, int nz, float2 *
 struct FwdArgs {
     const Grid *grid;           // host copy
     const Atlas *atlas = nullptr;  // volume uploaded into a texture atlas, or nullptr
+    const ColStore *column = nullptr;  // volume in column layout (static trilinear projector), or nullptr
     const ViewGPU *views;       // device [n_views * n_sub]
     const MotionGPU *motion;    // device [n_views] or nullptr
     const float *coef_idx;      // device [8][8][8][3] voxels, or nullptr
@@ -148,11 +150,17 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
                                    int r_dtype, float *partials, int n_partials_cap,
                                    double *sums);
 int forward_partials_needed(const Grid &g, int n_idx);
+// The static trilinear projector on a.column (fwd_column.cu).
+cudaError_t launch_forward_column(const FwdArgs &a, bool correct, int pdt, void *out, float *rowsum, const void *p,
+                                  float *partials);
+int column_partials_needed(const Grid &g, int n_idx);
+bool column_grid_fits(const Grid &g);  // its launch shape stays within the grid limits
 cudaError_t launch_count_samples(const FwdArgs &a, unsigned long long *out);
 
 struct BpArgs {
     const Grid *grid;
     const Atlas *atlas = nullptr;  // correction images uploaded into a texture atlas, or nullptr
+    const ColStore *column = nullptr;  // correction images in column layout, or nullptr
     const int4 *window = nullptr;  // per-view detector window of the backprojector, or nullptr
     const ViewGPU *views;
     const int *view_idx;
@@ -171,6 +179,9 @@ struct BpArgs {
     cudaStream_t stream;
 };
 cudaError_t launch_backproject(const BpArgs &a);
+// The same on a.column (bp_column.cu).
+cudaError_t launch_backproject_column(const BpArgs &a);
+bool backproject_column_fits(const Grid &g);  // its launch shape stays within the grid limits
 
 cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol);
 cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *grad_M, double *grad_b,

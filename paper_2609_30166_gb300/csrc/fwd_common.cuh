@@ -14,14 +14,14 @@ constexpr int FWD_TY = 4;   // pixels per CTA along v
 enum FwdMode { MODE_PROJECT = 0, MODE_CORRECT = 1 };
 
 // Pixel (iu, iv) of list entry k (view `view`; ok = the view index was
-// valid).  s_red: shared scratch of 2 x (warps per CTA) floats.  Every
+// valid).  s_red: shared scratch of 2 x NW floats, NW warps per CTA.  Every
 // thread of the CTA must call it (the correction mode synchronises).
-template <typename TP, int MODE>
+template <typename TP, int MODE, int NW = FWD_TX * FWD_TY / 32>
 __device__ __forceinline__ void fwd_epilogue(const Grid &G, int k, int view, bool ok, bool in_pix, int iu, int iv,
                                              float val, float rs, TP *__restrict__ out,
                                              float *__restrict__ rowsum_out, const TP *__restrict__ p,
                                              float *__restrict__ partials, int p_by_view,
-                                             float (*s_red)[FWD_TX * FWD_TY / 32])
+                                             float (*s_red)[NW])
 {
     const bool inside = ok && in_pix;
     const size_t pix = ((size_t)k * G.nv + iv) * G.nu + iu;
@@ -58,7 +58,7 @@ __device__ __forceinline__ void fwd_epilogue(const Grid &G, int k, int view, boo
         if (threadIdx.x == 0 && threadIdx.y == 0) {
             float a = 0.0f, b = 0.0f;
 #pragma unroll
-            for (int w = 0; w < FWD_TX * FWD_TY / 32; ++w) {
+            for (int w = 0; w < NW; ++w) {
                 a += s_red[0][w];
                 b += s_red[1][w];
             }

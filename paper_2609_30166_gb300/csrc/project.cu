@@ -259,7 +259,8 @@ static dim3 fwd_grid(const Grid &G, int n_idx)
 int forward_partials_needed(const Grid &G, int n_idx)
 {
     const dim3 g = fwd_grid(G, n_idx);
-    return (int)(g.x * g.y * g.z);
+    const int col = column_partials_needed(G, n_idx), n = (int)(g.x * g.y * g.z);
+    return n > col ? n : col;  // either launch shape
 }
 
 template <typename Sampler, typename TP, int MODE>
@@ -328,6 +329,7 @@ template <int MODE>
 static cudaError_t fwd_dispatch(const FwdArgs &a, int pdt, void *out, float *rowsum, const void *p,
                                 float *partials)
 {
+    if (a.column) return launch_forward_column(a, MODE == MODE_CORRECT, pdt, out, rowsum, p, partials);
     if (pdt == CTREX_F32)
         return fwd_dispatch_sampler<float, MODE>(a, (float *)out, rowsum, (const float *)p, partials);
     return fwd_dispatch_sampler<__nv_bfloat16, MODE>(a, (__nv_bfloat16 *)out, rowsum, (const __nv_bfloat16 *)p,
@@ -348,7 +350,8 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
         if (sums) return cudaMemsetAsync(sums, 0, 2 * sizeof(double), a.stream);
         return cudaSuccess;
     }
-    const int n = forward_partials_needed(*a.grid, a.n_idx);
+    const dim3 fg = fwd_grid(*a.grid, a.n_idx);
+    const int n = a.column ? column_partials_needed(*a.grid, a.n_idx) : (int)(fg.x * fg.y * fg.z);
     if (n > n_partials_cap) return cudaErrorInvalidValue;
     cudaError_t e = fwd_dispatch<MODE_CORRECT>(a, p_dtype, r, nullptr, p, partials);
     if (e != cudaSuccess || sums == nullptr) return e;

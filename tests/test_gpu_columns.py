@@ -1,0 +1,101 @@
+"""The column kernels (fwd_column.cu, bp_column.cu) at the edges of their tiles
+and of the rules that choose them, against the FP64 oracle.
+
+Both choices compute the same operator, so every case holds to the projector's
+contract, 1e-5 relative L2 (FP32 storage): detectors of 31, 32 and 33 rows and
+of widths beside a multiple of 4, volumes of 1 to 130 slices (a thread's 2 or 4
+voxels, 64- and 128-slice blocks that overlap), detectors turned to either side
+of the rules' limits, a detector smaller than the object's shadow (blocks of
+voxels inside, across and outside its edge), and a source inside the volume.
+"""
+
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_30166_gb300 import inputs
+from tests.helpers import rel_l2
+
+pytestmark = pytest.mark.gpu
+
+TOL32 = 1e-5
+
+# (nx, ny, nz), (nu, nv), views, sub-angles, in-plane turn of the detector (deg), detector width (mm), SOD (mm)
+CASES = [
+    ((33, 20, 64), (45, 31), 7, 1, 0.4, 96.0, 200.0),
+    ((32, 33, 65), (48, 32), 6, 2, 0.0, 96.0, 200.0),
+    ((19, 37, 130), (31, 33), 5, 1, -0.3, 96.0, 200.0),
+    ((40, 8, 127), (130, 96), 3, 1, 1.0, 96.0, 200.0),
+    ((41, 29, 1), (50, 64), 5, 1, 0.2, 96.0, 200.0),
+    ((1, 40, 40), (50, 40), 5, 1, 0.2, 96.0, 200.0),
+    ((24, 24, 66), (36, 64), 5, 1, 28.0, 96.0, 200.0),   # below both limits
+    ((24, 24, 40), (36, 64), 5, 1, 40.0, 96.0, 200.0),   # forward by columns, backprojection by gathers
+    ((24, 24, 40), (36, 64), 5, 1, 55.0, 96.0, 200.0),   # both by gathers
+    ((48, 40, 90), (33, 40), 9, 1, 0.5, 40.0, 200.0),    # truncated: part of the object off the detector
+    ((24, 24, 40), (48, 48), 6, 1, 0.0, 96.0, 10.0),     # source inside the volume
+    ((96, 90, 70), (24, 32), 6, 1, 0.0, 96.0, 200.0),    # pixel steps of several voxels
+    ((16, 16, 40), (96, 160), 6, 1, 0.0, 96.0, 200.0),   # voxel steps of several pixels
+]
+
+
+def _matrices(views, sub, turn, nu, nv, width, sod):
+    rng = np.random.default_rng(5)
+    t, pitch = math.radians(turn), width / nu
+    P = np.zeros((views, sub, 3, 4))
+    for v in range(views):
+        du, dv = rng.uniform(-1.5, 1.5, 2)
+        for s in range(sub):
+            R = inputs.rot_z(0.3 + 2 * math.pi * (v + 0.2 * s) / views)
+            u, w = R @ np.array([0.0, pitch, 0.0]), np.array([0.0, 0.0, pitch])
+            ctr = R @ np.array([200.0, 0.0, 0.0]) + du * u + dv * w
+            P[v, s] = inputs.cone_matrix(R @ np.array([-sod, 0.0, 0.0]), ctr, math.cos(t) * u + math.sin(t) * w,
+                                         math.cos(t) * w - math.sin(t) * u, nu, nv)
+    return P
+
+
+def _t(a, dtype=torch.float32):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64).to(dtype).cuda().contiguous()
+
+
+def _np(t):
+    return t.detach().double().cpu().numpy()
+
+
+@pytest.mark.parametrize("n,det,views,sub,turn,width,sod", CASES)
+def test_columns_match_oracle(n, det, views, sub, turn, width, sod):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    (nx, ny, nz), (nu, nv) = n, det
+    P = _matrices(views, sub, turn, nu, nv, width, sod)
+    pitch = 32.0 / max(nx, ny, 1.3 * nz)
+    vox = (pitch, pitch, 1.3 * pitch)
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(9)
+    x = rng.uniform(0.2, 1.0, size=(nz, ny, nx))
+    pb = oracle.Problem(P, (nz, ny, nx), vox, org, det, 0.5)
+    c = ctrex.Context()
+    c.set_geometry(P, (nz, ny, nx), vox, org, det)
+    ref, rs = oracle.forward(pb, _np(_t(x)))
+    rows = torch.empty(ref.shape, device="cuda")
+    assert rel_l2(_np(c.fwd_project(_t(x), rowsum=rows)), ref) <= TOL32
+    assert rel_l2(_np(rows), rs) <= TOL32
+    # BF16 volume, FP32 result; a second pass over the kept store
+    x16 = _t(x, torch.bfloat16)
+    assert rel_l2(_np(c.fwd_project(x16, out_dtype=torch.float32)), oracle.forward(pb, _np(x16))[0]) <= TOL32
+    # smooth images: an FP32 detector coordinate resolves noise to ~1e-4 only
+    iu, iv = np.meshgrid(np.arange(nu), np.arange(nv))
+    r = np.stack([np.cos(0.11 * iu + k) + np.sin(0.07 * iv * (k + 1)) + 2.5 for k in range(views)])
+    w = rng.uniform(0.5, 1.0, size=x.shape)
+    want, b, _ = oracle.backproject(pb, _np(_t(r)), w=_np(_t(w)), alpha=0.7, x=_np(_t(x)))
+    got = c.back_project(_t(r), vol=_t(x), w=_t(w), alpha=0.7)
+    assert rel_l2(_np(got), want) <= TOL32
+    assert rel_l2(_np(c.back_project(_t(r), normalize=False, accumulate=False)), b) <= TOL32
+    # a view list: out of order, fewer images than the kept store holds
+    vi = np.arange(views)[::-2].astype(np.int32).copy()
+    _, b, _ = oracle.backproject(pb, _np(_t(r[vi])), views=vi)
+    assert rel_l2(_np(c.back_project(_t(r[vi]), normalize=False, accumulate=False, view_idx=vi)), b) <= TOL32
+    c.close()
