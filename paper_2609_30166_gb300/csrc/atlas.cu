@@ -34,14 +34,10 @@ void atlas_release(AtlasStore &s)
     s = AtlasStore();
 }
 
-cudaError_t atlas_ensure(AtlasStore &s, int w, int h, int n, bool bf16, int device, bool packed, bool wrap)
+// Tiling of n slices of w x h in one array of W x H texels, 1 << tshift tiles
+// per row; false if the device's 2D limits cannot hold it.
+static bool atlas_shape(int w, int h, int n, int device, int &tshift, long long &W, long long &H)
 {
-    packed = packed && bf16;
-    if (wrap) h += 1;
-    if (s.array && s.w == w && s.h == h && s.n == n && s.bf16 == (bf16 ? 1 : 0) && s.packed == (packed ? 1 : 0) &&
-        s.wrap == (wrap ? 1 : 0))
-        return cudaSuccess;
-    atlas_release(s);
     int maxw = 0, maxh = 0;
     cudaDeviceGetAttribute(&maxw, cudaDevAttrMaxSurface2DWidth, device);
     cudaDeviceGetAttribute(&maxh, cudaDevAttrMaxSurface2DHeight, device);
@@ -51,17 +47,37 @@ cudaError_t atlas_ensure(AtlasStore &s, int w, int h, int n, bool bf16, int devi
     maxw = min(maxw, tw);
     maxh = min(maxh, th);
     // tiles per row: a power of two giving a roughly square atlas
-    int tshift = 0;
+    tshift = 0;
     while ((1LL << tshift) * (long long)w * (1LL << tshift) * (long long)w < (long long)n * w * h) ++tshift;
-    long long W = (1LL << tshift) * (long long)w;
+    W = (1LL << tshift) * (long long)w;
     long long rows = (n + (1 << tshift) - 1) >> tshift;
     while (W > maxw && tshift > 0) {
         --tshift;
         W = (1LL << tshift) * (long long)w;
         rows = (n + (1 << tshift) - 1) >> tshift;
     }
-    const long long H = rows * h;
-    if (W > maxw || H > maxh || W < 1 || H < 1) return cudaErrorInvalidValue;
+    H = rows * h;
+    return W <= maxw && H <= maxh && W >= 1 && H >= 1;
+}
+
+bool atlas_fits(int w, int h, int n, int device)
+{
+    int tshift;
+    long long W, H;
+    return atlas_shape(w, h, n, device, tshift, W, H);
+}
+
+cudaError_t atlas_ensure(AtlasStore &s, int w, int h, int n, bool bf16, int device, bool packed, bool wrap)
+{
+    packed = packed && bf16;
+    if (wrap) h += 1;
+    if (s.array && s.w == w && s.h == h && s.n == n && s.bf16 == (bf16 ? 1 : 0) && s.packed == (packed ? 1 : 0) &&
+        s.wrap == (wrap ? 1 : 0))
+        return cudaSuccess;
+    atlas_release(s);
+    int tshift;
+    long long W, H;
+    if (!atlas_shape(w, h, n, device, tshift, W, H)) return cudaErrorInvalidValue;
     cudaChannelFormatDesc desc = packed ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
                                  : bf16 ? cudaCreateChannelDesc(16, 0, 0, 0, cudaChannelFormatKindUnsigned)
                                         : cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindFloat);

@@ -216,6 +216,8 @@ struct AtlasStore {
 // Returns cudaErrorInvalidValue if it cannot fit the device's 2D texture limits.
 cudaError_t atlas_ensure(AtlasStore &s, int w, int h, int n, bool bf16, int device, bool packed = false,
                          bool wrap = false);
+// Whether an atlas of that shape fits the device's 2D texture limits.
+bool atlas_fits(int w, int h, int n, int device);
 void atlas_release(AtlasStore &s);
 Atlas atlas_view(const AtlasStore &s);
 // Copies a [nz][ny][nx] volume into a three-stack atlas of nx + ny + nz tiles

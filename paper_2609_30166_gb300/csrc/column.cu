@@ -30,9 +30,9 @@ static cudaError_t col_alloc(ColStore &s, size_t n, cudaStream_t stream)
     return cudaMemsetAsync(s.buf, 0, bytes, stream);
 }
 
-cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream)
+cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream, bool wrap)
 {
-    if (s.buf && s.nx == nx && s.ny == ny && s.nz == nz) return cudaSuccess;
+    if (s.buf && s.nx == nx && s.ny == ny && s.nz == nz && s.wrap == (wrap ? 1 : 0)) return cudaSuccess;
     const size_t sy = ((size_t)nx + 2) << COL_LOG, sz = sy * ((size_t)ny + 2);
     const size_t n = sz * ((((size_t)nz + 1) >> COL_LOG) + 1);
     if (n >= (1ull << 32)) return cudaErrorInvalidValue;
@@ -41,6 +41,7 @@ cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream)
     s.nx = nx;
     s.ny = ny;
     s.nz = nz;
+    s.wrap = wrap ? 1 : 0;
     s.sy = (unsigned)sy;
     s.sz = (unsigned)(sz - (1u << COL_LOG));
     return cudaSuccess;
@@ -98,7 +99,11 @@ static cudaError_t upload(const void *src, int dtype, float2 *dst, int nu, int n
 
 cudaError_t col_upload(const ColStore &s, const void *src, int dtype, cudaStream_t stream)
 {
-    return upload(src, dtype, s.buf + s.sy, s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, s.ny, stream);
+    cudaError_t e = upload(src, dtype, s.buf + s.sy, s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, s.ny, stream);
+    if (e == cudaSuccess && s.wrap)
+        e = upload(src, dtype, s.buf + (size_t)s.sy * (s.ny + 1), s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, 1,
+                   stream);
+    return e;
 }
 
 cudaError_t col_ensure_images(ColStore &s, int nu, int nv, int n, cudaStream_t stream)

@@ -46,6 +46,7 @@ struct ColStore {
     size_t bytes = 0;
     int nx = 0, ny = 0, nz = 0;  // what it was laid out for (0: nothing)
     unsigned sy = 0, sz = 0;
+    int wrap = 0;     // the row past the last repeats row 0 (periodic axis)
     size_t view = 0;  // image stacks: pairs per image (nz: images; sy: chunk to chunk)
 };
 void col_release(ColStore &s);
@@ -53,7 +54,7 @@ void col_release(ColStore &s);
 // that fits is kept.  cudaErrorInvalidValue: the layout's 32-bit indices
 // cannot hold it, or it would take more than half of the free device memory
 // (the caller keeps its other path).
-cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream);
+cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream, bool wrap = false);
 // Transposes a [nz][ny][nx] volume into the store.
 cudaError_t col_upload(const ColStore &s, const void *src, int dtype, cudaStream_t stream);
 

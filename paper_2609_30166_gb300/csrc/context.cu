@@ -50,6 +50,9 @@ struct ctrex_ctx {
     // the volume in column layout, where the scan's detector columns run along z
     double col_lean = 10.0, col_step = 1.0;  // detector_column_step
     ColStore vol_col;
+    ColStore col1;     // the ROI grid, or the event model's final values
+    ColStore tau_col;  // the event model's transition times
+    bool tau_col_set = false;
     ColStore img_col;  // the correction images
     // texture atlas of the correction images read by the backprojector
     AtlasStore img_atlas;
@@ -84,6 +87,8 @@ struct ctrex_ctx {
     float *d_tau = nullptr;     // [nz][ny][nx] transition times
     float *d_tview = nullptr;   // [n_views] acquisition times
     float2 *d_tau_brick = nullptr;  // (min, max) transition time per 8^3 brick
+    float2 *d_tau_block = nullptr;  // the same around each brick (launch_tau_bricks)
+    float2 *d_tau_cell = nullptr;   // its scratch
     AtlasStore dyr_atlas1;      // the final values (the volume atlas holds the initial ones)
     AtlasStore tau_atlas;
     Atlas dyr_atlas1_view, tau_atlas_view;
@@ -223,6 +228,11 @@ void dyr_release(ctrex_ctx *c)
     if (c->d_tau_brick) cudaFree(c->d_tau_brick);
     c->d_tau = c->d_tview = nullptr;
     c->d_tau_brick = nullptr;
+    dfree(c->d_tau_block);
+    dfree(c->d_tau_cell);
+    col_release(c->tau_col);
+    col_release(c->col1);
+    c->tau_col_set = false;
     atlas_release(c->dyr_atlas1);
     atlas_release(c->tau_atlas);
 }
@@ -248,7 +258,8 @@ constexpr double COL_STEP_BP_MIN = 0.3;
 bool column_forward(const ctrex_ctx *c, int vdt)
 {
     if (!(c->col_lean <= COL_LEAN_FWD && column_grid_fits(c->grid))) return false;
-    if (c->col_step > (vdt == CTREX_F32 ? COL_STEP_FP32 : COL_STEP_BF16)) return false;
+    const double step = c->col_step * (c->roi ? fmax(1.0, c->roig.sc[2]) : 1.0);
+    if (step > (vdt == CTREX_F32 ? COL_STEP_FP32 : COL_STEP_BF16)) return false;
     const double u4 = (c->grid.nu + 3) / 4 * 4.0, u32 = (c->grid.nu + 31) / 32 * 32.0;
     const double v4 = (c->grid.nv + 3) / 4 * 4.0, v32 = (c->grid.nv + 31) / 32 * 32.0;
     return u4 * v32 <= u32 * v4 * (vdt == CTREX_F32 ? 2.2 : 1.2);
@@ -260,10 +271,46 @@ bool column_backproject(const ctrex_ctx *c)
            (!c->roi || backproject_column_fits(c->roi_grid));
 }
 
+// Uploads vol into the context's column stores and points a.column at them; a
+// shape that the model's texture atlases refuse, and a store that does not
+// fit, are left to the atlas path (a.column stays null).
+int prepare_columns(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
+{
+    const int nx = c->grid.nx, ny = c->grid.ny, nz = c->grid.nz, d = c->device;
+    const int rx = c->roi_grid.nx, ry = c->roi_grid.ny, rz = c->roi_grid.nz;
+    if (c->projector == CTREX_PROJ_JOSEPH && !atlas_fits(nx > ny ? nx : ny, ny > nz ? ny : nz, nx + ny + nz, d))
+        return CTREX_OK;
+    if ((c->cyl && !atlas_fits(nx, ny + 1, nz, d)) || (c->dyr && !atlas_fits(nx, ny, nz, d)) ||
+        (c->roi && !(atlas_fits(nx, ny, nz, d) && atlas_fits(rx, ry, rz, d))))
+        return CTREX_OK;
+    cudaError_t e = col_ensure(c->vol_col, nx, ny, nz, c->stream, c->cyl);
+    if (e == cudaSuccess && c->dyr) e = col_ensure(c->col1, nx, ny, nz, c->stream);
+    if (e == cudaSuccess && c->roi) e = col_ensure(c->col1, rx, ry, rz, c->stream);
+    if (e == cudaSuccess && c->dyr && !c->tau_col_set) {
+        e = col_ensure(c->tau_col, nx, ny, nz, c->stream);
+        if (e == cudaSuccess) e = col_upload(c->tau_col, c->d_tau, CTREX_F32, c->stream);
+        c->tau_col_set = e == cudaSuccess;
+    }
+    if (e == cudaErrorInvalidValue) return CTREX_OK;
+    if (e == cudaSuccess) e = col_upload(c->vol_col, vol, vdt, c->stream);
+    if (e == cudaSuccess && (c->dyr || c->roi))
+        e = col_upload(c->col1, static_cast<const char *>(vol) + grid_voxels(c->grid) * dtype_size(vdt), vdt,
+                       c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "volume column layout");
+    a.column = &c->vol_col;
+    a.column1 = &c->col1;
+    a.column_tau = &c->tau_col;
+    return CTREX_OK;
+}
+
 // Uploads vol into the context's texture atlas and points a.atlas at it; if
 // the volume does not fit the 2D texture limits the row-major path is used.
 int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
 {
+    if (!c->has_motion && column_forward(c, vdt)) {
+        const int e = prepare_columns(c, a, vol, vdt);
+        if (e != CTREX_OK || a.column) return e;
+    }
     if (c->projector == CTREX_PROJ_JOSEPH) {
         // x-, y- and z-slice stacks in one atlas; no row-major fallback
         const int nx = c->grid.nx, ny = c->grid.ny, nz = c->grid.nz;
@@ -339,16 +386,6 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
         c->vol_atlas_view = atlas_view(c->vol_atlas);
         a.atlas = &c->vol_atlas_view;
         return CTREX_OK;
-    }
-    if (!c->has_motion && column_forward(c, vdt)) {
-        cudaError_t e = col_ensure(c->vol_col, c->grid.nx, c->grid.ny, c->grid.nz, c->stream);
-        if (e == cudaSuccess) {
-            e = col_upload(c->vol_col, vol, vdt, c->stream);
-            if (e != cudaSuccess) return cuda_fail(c, e, "volume column upload");
-            a.column = &c->vol_col;
-            return CTREX_OK;
-        }
-        if (e != cudaErrorInvalidValue) return cuda_fail(c, e, "volume column layout");
     }
     if (c->atlas_unfit) return CTREX_OK;
     // BF16 volumes: slice pairs packed in 32-bit texels, one gather per sample
@@ -471,7 +508,7 @@ int ctrex_destroy(ctrex_ctx *c)
         atlas_release(c->jos_atlas);
         atlas_release(c->roi_atlas);
         dfree(c->d_views_roi);
-        dyr_release(c);
+        dyr_release(c);  // col1 with it
     }
     delete c;
     return CTREX_OK;
@@ -738,6 +775,7 @@ int ctrex_set_geometry_cylinder(ctrex_ctx *c, const double *P, int n_views, int 
     c->grid.lo[2] = -C.Z;
     c->grid.hi[2] = C.Z;
     c->cyl = true;
+    c->col_step /= cyl->dz;  // frame mm to slices
     c->projector = CTREX_PROJ_TRILINEAR;
     return CTREX_OK;
 }
@@ -827,6 +865,7 @@ int ctrex_set_roi(ctrex_ctx *c, const ctrex_vol_grid *roi)
         c->roi = false;
         dfree(c->d_views_roi);
         atlas_release(c->roi_atlas);
+        col_release(c->col1);
         return CTREX_OK;
     }
     if (c->cyl || c->has_motion || c->dyr || c->projector != CTREX_PROJ_TRILINEAR)
@@ -937,9 +976,17 @@ int ctrex_set_dyrect(ctrex_ctx *c, const float *tau, const float *t_view)
     const int bnx = (c->grid.nx + 7) / 8, bny = (c->grid.ny + 7) / 8, bnz = (c->grid.nz + 7) / 8;
     if (!c->d_tau_brick)
         CT_CUDA(c, cudaMalloc((void **)&c->d_tau_brick, sizeof(float2) * (size_t)bnx * bny * bnz));
-    e = launch_tau_bricks(c->d_tau, c->grid.nx, c->grid.ny, c->grid.nz, c->d_tau_brick, c->stream);
+    if (!c->d_tau_block)
+        CT_CUDA(c, cudaMalloc((void **)&c->d_tau_block, sizeof(float2) * (size_t)bnx * bny * bnz));
+    const int cnx = (c->grid.nx + 3) / 4, cny = (c->grid.ny + 3) / 4, cnz = (c->grid.nz + 3) / 4;
+    if (!c->d_tau_cell)
+        CT_CUDA(c, cudaMalloc((void **)&c->d_tau_cell, sizeof(float2) * (size_t)cnx * cny * cnz));
+    e = launch_tau_bricks(c->d_tau, c->grid.nx, c->grid.ny, c->grid.nz, c->d_tau_cell, c->d_tau_brick, c->d_tau_block,
+                          c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "transition-time bricks");
+    c->tau_col_set = false;
     c->dyra.tau_brick = c->d_tau_brick;
+    c->dyra.tau_block = c->d_tau_block;
     c->dyra.bnx = bnx;
     c->dyra.bny = bny;
     c->dyra.tau = c->d_tau;

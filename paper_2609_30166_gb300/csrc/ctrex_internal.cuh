@@ -108,6 +108,7 @@ struct DyrArgs {
     const float *tau = nullptr;     // device [nz][ny][nx]
     const float *t_view = nullptr;  // device [n_views]
     const float2 *tau_brick = nullptr;  // device: (min, max) of tau per 8^3 brick and its upper neighbours
+    const float2 *tau_block = nullptr;  // device: the same of voxels 8 b - 4 .. 8 b + 15
     int bnx = 0, bny = 0;               // bricks along x and y
 };
 
@@ -119,15 +120,18 @@ long long correct_scratch_pairs(long long n);
 cudaError_t launch_correct(const void *p, const void *q, const float *rowsum, void *r, int dtype, long long n,
                            float eps_R, double *sums, double *scratch, cudaStream_t stream);
 
-// (min, max) transition time of each 8^3 brick of tau [nz][ny][nx], taken
-// over the brick and the voxel past each of its upper faces (within the
-// grid).
-cudaError_t launch_tau_bricks(const float *tau, int nx, int ny, int nz, float2 *out, cudaStream_t stream);
+// (min, max) transition times of tau [nz][ny][nx]: of each 8^3 brick and the
+// voxel past each of its upper faces (brick), and of voxels 8 b - 4 .. 8 b + 15
+// around brick b (block); cell: scratch, one pair per 4^3 cell.
+cudaError_t launch_tau_bricks(const float *tau, int nx, int ny, int nz, float2 *cell, float2 *brick, float2 *block,
+                              cudaStream_t stream);
 
 struct FwdArgs {
     const Grid *grid;           // host copy
     const Atlas *atlas = nullptr;  // volume uploaded into a texture atlas, or nullptr
-    const ColStore *column = nullptr;  // volume in column layout (static trilinear projector), or nullptr
+    const ColStore *column = nullptr;  // volume in column layout, or nullptr (texture atlas, row-major loads)
+    const ColStore *column1 = nullptr;     // with it: the ROI grid, or the event model's final values
+    const ColStore *column_tau = nullptr;  // with it: the event model's transition times
     const ViewGPU *views;       // device [n_views * n_sub]
     const MotionGPU *motion;    // device [n_views] or nullptr
     const float *coef_idx;      // device [8][8][8][3] voxels, or nullptr
@@ -150,9 +154,11 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
                                    int r_dtype, float *partials, int n_partials_cap,
                                    double *sums);
 int forward_partials_needed(const Grid &g, int n_idx);
-// The static trilinear projector on a.column (fwd_column.cu).
+// The projectors on a.column (fwd_column.cu, fwd_column_models.cu).
 cudaError_t launch_forward_column(const FwdArgs &a, bool correct, int pdt, void *out, float *rowsum, const void *p,
                                   float *partials);
+cudaError_t launch_forward_column_models(const FwdArgs &a, bool correct, int pdt, void *out, float *rowsum,
+                                         const void *p, float *partials);
 int column_partials_needed(const Grid &g, int n_idx);
 bool column_grid_fits(const Grid &g);  // its launch shape stays within the grid limits
 cudaError_t launch_count_samples(const FwdArgs &a, unsigned long long *out);

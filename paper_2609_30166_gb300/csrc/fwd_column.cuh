@@ -1,0 +1,129 @@
+// fwd_column.cuh -- what the column projectors share (fwd_column.cu: the
+// static model; fwd_column_models.cu: event model, multi-resolution ROI,
+// cylindrical domain, classical Joseph): launch shape, fixed-point runs of
+// interior samples, edge samples.
+#pragma once
+
+#include "column.cuh"
+#include "fwd_common.cuh"
+#include "ray.cuh"
+
+namespace ctrex {
+
+// A CTA is 32 pixels along v by 4 columns (8 columns: the same within 1 %).
+constexpr int COL_TU = 4;
+constexpr int COL_MIN_BLOCKS = 8;  // CTAs per SM of the models' kernels (7 and 10: within 3 %)
+constexpr int COL_UNROLL = 2;  // samples per step of the interior loop (1: +3 %, 4: +11 %, out of registers)
+// CTAs are ordered in strips of 32 tiles (128 columns), then views, then
+// strips and bands of 32 rows: the views resident together then cross one
+// strip of the volume instead of all of it, and what they share stays in L2
+// (DRAM reads of 16 views of the 512^3 scan: 2.0 GB, 10.3 GB with whole rows
+// of tiles; strips of 8 to 64 tiles measured alike).
+constexpr int COL_STRIP = 32;
+
+// Whether an axis's fixed-point samples p, p + d, .., p + (n - 1) d lie in
+// padded indices 1 .. h + 1 (the grid): they run evenly from end to end (sg
+// is the step as a float: its bound keeps the products below 2^63).
+__device__ __forceinline__ bool axis_inside(long long p, long long d, float sg, int n, float h)
+{
+    if (n < 1 || !(fabsf(sg) * (float)n < 1.0e9f)) return false;
+    const long long q = p + (long long)(n - 1) * d, top = ((long long)h + 1) << 32;
+    return p >= (1ll << 32) && p <= top && q >= (1ll << 32) && q <= top;
+}
+
+// Samples ka .. kb - 1 of a ray, g0 + k sg, in 32.32 fixed point and padded
+// index coordinates: a 64-bit add per axis and step, whose high word is the
+// cell and whose low word the fraction; exact, where a float position rounds
+// at the coordinate's magnitude.
+struct ColRun {
+    long long px, py, pz, dx, dy, dz;
+
+    // False if a sample is not inside the grid (a ray with non-finite
+    // parameters): such a range is left to the clamped path.
+    __device__ __forceinline__ bool start(const ColVolume &V, const float g0[3], const float sg[3], int ka, int n)
+    {
+        const float F = 4294967296.0f;
+        dx = __float2ll_rn(sg[0] * F);
+        dy = __float2ll_rn(sg[1] * F);
+        dz = __float2ll_rn(sg[2] * F);
+        px = __float2ll_rn(g0[0] * F) + (1ll << 32) + ka * dx;
+        py = __float2ll_rn(g0[1] * F) + (1ll << 32) + ka * dy;
+        pz = __float2ll_rn(g0[2] * F) + (1ll << 32) + ka * dz;
+        return axis_inside(px, dx, sg[0], n, V.hx) && axis_inside(py, dy, sg[1], n, V.hy) &&
+               axis_inside(pz, dz, sg[2], n, V.hz);
+    }
+    __device__ __forceinline__ unsigned index(const ColVolume &V) const
+    {
+        return V.index((unsigned)(px >> 32), (unsigned)(py >> 32), (unsigned)(pz >> 32));
+    }
+    __device__ __forceinline__ float interp(const ColTaps &t) const
+    {
+        return col_interp(t, fixed_fraction((unsigned)px), fixed_fraction((unsigned)py), fixed_fraction((unsigned)pz));
+    }
+    __device__ __forceinline__ void next()
+    {
+        px += dx;
+        py += dy;
+        pz += dz;
+    }
+    // a plus the next n samples
+    __device__ __forceinline__ float sum(const ColVolume &V, int n, float a)
+    {
+#pragma unroll COL_UNROLL
+        for (int left = n; left > 0; --left) {
+            a += interp(col_load(V, index(V)));
+            next();
+        }
+        return a;
+    }
+};
+
+// A sample beside the interior range: inside the border by the clip box, and
+// clamped for any input; ws: its summed weight of the taps inside the grid.
+template <typename Taps>
+__device__ __forceinline__ float col_edge(const ColVolume &V, float gx, float gy, float gz, float &ws, Taps taps)
+{
+    gx = fminf(fmaxf(gx, -1.0f), V.hx + 0.75f);
+    gy = fminf(fmaxf(gy, -1.0f), V.hy + 0.75f);
+    gz = fminf(fmaxf(gz, -1.0f), V.hz + 0.75f);
+    const float fx = floorf(gx), fy = floorf(gy), fz = floorf(gz);
+    const float ax = gx - fx, ay = gy - fy, az = gz - fz;
+    ws = col_inside(gx, ax, V.hx) * col_inside(gy, ay, V.hy) * col_inside(gz, az, V.hz);
+    return col_interp(taps(V.index((int)fx + 1, (int)fy + 1, (int)fz + 1)), ax, ay, az);
+}
+
+// The kernel's frame: the CTA's pixels, one integral per thread by `pixel`
+// (view, u, v, value, row sum), and the epilogue.
+template <typename TP, int MODE, typename Pixel>
+__device__ __forceinline__ void col_body(const Grid &G, const int *__restrict__ view_idx, TP *__restrict__ out,
+                                         float *__restrict__ rowsum_out, const TP *__restrict__ p,
+                                         float *__restrict__ partials, unsigned *devcheck, int p_by_view, int n_strips,
+                                         Pixel pixel)
+{
+    __shared__ float s_red[2][COL_TU];
+    const int k = blockIdx.y;
+    int view = view_idx ? view_idx[k] : k;
+    bool ok = true;
+    if (view < 0 || view >= G.n_views) {
+        if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(devcheck, (unsigned)DEVCHECK_OOB);
+        ok = false;
+        view = 0;
+    }
+    const int strip = blockIdx.z % n_strips, band = blockIdx.z / n_strips;
+    const int iu = (strip * gridDim.x + blockIdx.x) * COL_TU + threadIdx.y, iv = band * 32 + threadIdx.x;
+    const bool in_pix = iu < G.nu && iv < G.nv;
+    float val = 0.0f, rs = 0.0f;
+    if (ok && in_pix) pixel(view, (float)iu, (float)iv, val, rs);
+    fwd_epilogue<TP, MODE, COL_TU>(G, k, view, ok, in_pix, iu, iv, val, rs, out, rowsum_out, p, partials, p_by_view,
+                                   s_red);
+}
+
+// grid: tiles of a strip, views, strips x bands
+inline dim3 col_grid(const Grid &G, int n_idx, int &n_strips)
+{
+    const int tiles = (G.nu + COL_TU - 1) / COL_TU, per = tiles < COL_STRIP ? tiles : COL_STRIP;
+    n_strips = (tiles + per - 1) / per;
+    return dim3(per, n_idx, n_strips * ((G.nv + 31) / 32));
+}
+
+}  // namespace ctrex

@@ -377,37 +377,95 @@ cudaError_t launch_count_samples(const FwdArgs &a, unsigned long long *out)
     return cudaGetLastError();
 }
 
-// (min, max) of tau over each 8^3 brick and the voxel past each of its
-// upper faces: one thread per brick (run once, by ctrex_set_dyrect).
-__global__ void tau_brick_kernel(const float *__restrict__ tau, int nx, int ny, int nz, int bnx, int bny, int bnz,
-                                 float2 *__restrict__ out)
+// (min, max) transition times of parts of the volume, computed once by
+// ctrex_set_dyrect.  A NaN transition time sends its tap to mu1 (t < NaN is
+// false): a part with one never takes the mu0 shortcut, and the mu1 one only
+// for t = +inf.
+//
+// Cells of 4^3 voxels: a warp takes 8 of them along x, a lane 4 x 4 values.
+__global__ void __launch_bounds__(128) tau_cell_kernel(const float *__restrict__ tau, int nx, int ny, int nz, int cnx,
+                                                       int cny, int cnz, float2 *__restrict__ cell)
 {
-    const long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= (long long)bnx * bny * bnz) return;
-    const int bx = (int)(b % bnx), by = (int)((b / bnx) % bny), bz = (int)(b / ((long long)bnx * bny));
-    const int x1 = min(8 * bx + 8, nx - 1), y1 = min(8 * by + 8, ny - 1), z1 = min(8 * bz + 8, nz - 1);
+    const int per = (cnx + 7) / 8, lane = threadIdx.x & 31;
+    const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= (long long)per * cny * cnz) return;
+    const int gx = (int)(w % per), cy = (int)((w / per) % cny), cz = (int)(w / ((long long)per * cny));
+    const int x = gx * 32 + lane;
     float lo = INFINITY, hi = -INFINITY;
     bool nan = false;
-    for (int z = 8 * bz; z <= z1; ++z)
-        for (int y = 8 * by; y <= y1; ++y) {
-            const float *row = tau + ((size_t)z * ny + y) * nx;
-            for (int x = 8 * bx; x <= x1; ++x) {
-                const float v = __ldg(row + x);
-                nan |= v != v;
-                lo = fminf(lo, v);
-                hi = fmaxf(hi, v);
-            }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int y = 4 * cy + (i & 3), z = 4 * cz + (i >> 2);
+        if (x < nx && y < ny && z < nz) {
+            const float v = __ldg(tau + ((size_t)z * ny + y) * nx + x);
+            nan |= v != v;
+            lo = fminf(lo, v);
+            hi = fmaxf(hi, v);
         }
-    // a NaN transition time sends its tap to mu1 (t < NaN is false): such a
-    // brick never takes the mu0 shortcut, and the mu1 one only for t = +inf
-    out[b] = nan ? make_float2(-INFINITY, INFINITY) : make_float2(lo, hi);
+    }
+    if (nan) {
+        lo = -INFINITY;
+        hi = INFINITY;
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+    }
+    const int cx = gx * 8 + lane / 4;
+    if ((lane & 3) == 0 && cx < cnx) cell[((size_t)cz * cny + cy) * cnx + cx] = make_float2(lo, hi);
 }
 
-cudaError_t launch_tau_bricks(const float *tau, int nx, int ny, int nz, float2 *out, cudaStream_t stream)
+// brick: the 8^3 brick b and the voxel past each of its upper faces; block:
+// voxels 8 b - 4 .. 8 b + 15.  One warp per brick.
+__global__ void __launch_bounds__(128) tau_brick_kernel(const float *__restrict__ tau, const float2 *__restrict__ cell,
+                                                        int nx, int ny, int nz, int bnx, int bny, int bnz, int cnx,
+                                                        int cny, int cnz, float2 *__restrict__ brick,
+                                                        float2 *__restrict__ block)
+{
+    const long long b = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (b >= (long long)bnx * bny * bnz) return;
+    const int lane = threadIdx.x & 31;
+    const int bx = (int)(b % bnx), by = (int)((b / bnx) % bny), bz = (int)(b / ((long long)bnx * bny));
+    float lo = INFINITY, hi = -INFINITY, blo = INFINITY, bhi = -INFINITY;
+    bool nan = false;
+    for (int i = lane; i < 729; i += 32) {
+        const int x = min(8 * bx + i % 9, nx - 1), y = min(8 * by + i / 9 % 9, ny - 1), z = min(8 * bz + i / 81, nz - 1);
+        const float v = __ldg(tau + ((size_t)z * ny + y) * nx + x);
+        nan |= v != v;
+        lo = fminf(lo, v);
+        hi = fmaxf(hi, v);
+    }
+    for (int i = lane; i < 125; i += 32) {
+        const int x = min(max(2 * bx - 1 + i % 5, 0), cnx - 1), y = min(max(2 * by - 1 + i / 5 % 5, 0), cny - 1),
+                  z = min(max(2 * bz - 1 + i / 25, 0), cnz - 1);
+        const float2 c = __ldg(cell + ((size_t)z * cny + y) * cnx + x);
+        blo = fminf(blo, c.x);
+        bhi = fmaxf(bhi, c.y);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+        blo = fminf(blo, __shfl_xor_sync(0xffffffffu, blo, off));
+        bhi = fmaxf(bhi, __shfl_xor_sync(0xffffffffu, bhi, off));
+    }
+    nan = __any_sync(0xffffffffu, nan);
+    if (lane == 0) {
+        brick[b] = nan ? make_float2(-INFINITY, INFINITY) : make_float2(lo, hi);
+        block[b] = make_float2(blo, bhi);
+    }
+}
+
+cudaError_t launch_tau_bricks(const float *tau, int nx, int ny, int nz, float2 *cell, float2 *brick, float2 *block,
+                              cudaStream_t stream)
 {
     const int bnx = (nx + 7) / 8, bny = (ny + 7) / 8, bnz = (nz + 7) / 8;
-    const long long n = (long long)bnx * bny * bnz;
-    tau_brick_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(tau, nx, ny, nz, bnx, bny, bnz, out);
+    const int cnx = (nx + 3) / 4, cny = (ny + 3) / 4, cnz = (nz + 3) / 4;
+    const long long nb = (long long)bnx * bny * bnz, nw = (long long)((cnx + 7) / 8) * cny * cnz;
+    tau_cell_kernel<<<(unsigned)((nw + 3) / 4), 128, 0, stream>>>(tau, nx, ny, nz, cnx, cny, cnz, cell);
+    tau_brick_kernel<<<(unsigned)((nb + 3) / 4), 128, 0, stream>>>(tau, cell, nx, ny, nz, bnx, bny, bnz, cnx, cny, cnz,
+                                                                  brick, block);
     return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-"""The column kernels (fwd_column.cu, bp_column.cu) at the edges of their tiles
+"""The column kernels (fwd_column*.cu, bp_column.cu) at the edges of their tiles
 and of the rules that choose them, against the FP64 oracle.
 
 Both choices compute the same operator, so every case holds to the projector's
@@ -6,7 +6,9 @@ contract, 1e-5 relative L2 (FP32 storage): detectors of 31, 32 and 33 rows and
 of widths beside a multiple of 4, volumes of 1 to 130 slices (a thread's 2 or 4
 voxels, 64- and 128-slice blocks that overlap), detectors turned to either side
 of the rules' limits, a detector smaller than the object's shadow (blocks of
-voxels inside, across and outside its edge), and a source inside the volume.
+voxels inside, across and outside its edge), and a source inside the volume;
+and each other forward model on both sides of the rule, by columns and by
+texture gathers.
 """
 
 import math
@@ -98,4 +100,55 @@ def test_columns_match_oracle(n, det, views, sub, turn, width, sod):
     vi = np.arange(views)[::-2].astype(np.int32).copy()
     _, b, _ = oracle.backproject(pb, _np(_t(r[vi])), views=vi)
     assert rel_l2(_np(c.back_project(_t(r[vi]), normalize=False, accumulate=False, view_idx=vi)), b) <= TOL32
+    c.close()
+
+
+@pytest.mark.parametrize("model", ["event", "joseph", "roi", "cylinder"])
+@pytest.mark.parametrize("turn,tall", [(0.4, False), (44.0, True), (60.0, False)])
+def test_models_match_oracle(model, turn, tall):
+    """turn: columns, columns near the limit, gathers.  tall: steep rays over a
+    short detector distance, so that the Joseph projector's principal axis is
+    z on some of them and x or y on others."""
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    n, det, views = (22, 27, 41), (37, 66), 6
+    P = _matrices(views, 1, turn, det[0], det[1], 250.0 if tall else 80.0, 60.0 if tall else 200.0)
+    vox = (1.0, 0.9, 0.8)
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(4)
+    shape = n[::-1]
+    c = ctrex.Context()
+    if model == "cylinder":
+        shape = (41, 30, 17)  # slices, sectors, rings
+        args = dict(n_r=17, n_phi=30, n_z=41, dr=0.8, dz=0.8)
+        c.set_geometry_cylinder(P, det=det, **args)
+        pb = oracle.cylinder_problem(P, det=det, **args)
+    else:
+        c.set_geometry(P, shape, vox, org, det)
+        pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    if model == "event":
+        # regions that change early, late, never and (NaN) at once, and a gradual front
+        tau = np.full(shape, 2.0)
+        tau[:, :13] = 0.1 + 0.8 * np.linspace(0, 1, shape[0])[:, None, None]
+        tau[5:9, 20:23, 3:9] = np.nan
+        tv = np.linspace(0, 1, views)
+        c.set_dyrect(_t(tau), _t(tv))
+        pb = pb.with_dyrect(_np(_t(tau)), _np(_t(tv)))
+        shape = (2,) + shape
+    elif model == "joseph":
+        c.set_projector("joseph")
+        pb = pb.with_joseph()
+    elif model == "roi":
+        roi = ((19, 21, 23), (0.3, 0.3, 0.35), (-2.5, -1.0, 0.7))
+        c.set_roi(*roi)
+        pb = pb.with_roi(*roi)
+        shape = (c.vol_shape[0],)
+    x = rng.uniform(0.2, 1.0, size=shape)
+    rows = torch.empty((views, det[1], det[0]), device="cuda")
+    for dt in (torch.float32, torch.bfloat16):
+        ref, rs = oracle.forward(pb, _np(_t(x, dt)))
+        got = c.fwd_project(_t(x, dt), rowsum=rows, out_dtype=torch.float32)
+        assert rel_l2(_np(got), ref) <= TOL32
+        assert rel_l2(_np(rows), rs) <= TOL32
     c.close()
