@@ -165,11 +165,10 @@ __device__ __forceinline__ void scatter_trilinear(float *__restrict__ vol, int n
 template <bool MOTION, bool DYR>
 __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
     adjoint_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
-                   const float *__restrict__ coef_g, const int *__restrict__ view_idx,
+                   const float4 *spline, const int *__restrict__ view_idx,
                    const float *__restrict__ proj, float *__restrict__ vol, unsigned *devcheck,
                    const float *__restrict__ tau, const float *__restrict__ t_view)
 {
-    __shared__ float4 s_coef[MOTION ? NCOEF_PAD : 1];  // zero-padded 9^3 float4 copy of the coefficients
     const int k = blockIdx.y;
     const int view = view_idx ? view_idx[k] : k;
     if (view < 0 || view >= G.n_views) {
@@ -177,12 +176,12 @@ __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
         return;
     }
     MotionGPU mo;
-    const float4 *coef = nullptr;
+    __shared__ float4 s_spline[MOTION ? SPLINE_TABLE : 1];
     if (MOTION) {
         mo = motion[view];
-        if (coef_g) {
-            load_coef_padded(s_coef, coef_g, threadIdx.y * ADJ_TX + threadIdx.x, ADJ_TX * ADJ_TY);
-            coef = s_coef;
+        if (spline != nullptr) {
+            load_spline(s_spline, spline, threadIdx.y * ADJ_TX + threadIdx.x, ADJ_TX * ADJ_TY);
+            spline = s_spline;
         }
         __syncthreads();
     }
@@ -200,33 +199,18 @@ __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
     for (int s = 0; s < G.n_sub; ++s) {
         Ray R;  // sample positions relative to the grid centre
         if (!setup_ray(G, views[view * G.n_sub + s], (float)iu, (float)iv, R, cen)) continue;
-        const float ys = y * G.step_mm;
-        for (int kk = 0; kk < R.K; ++kk) {
-            float g[3];
-            float val = ys;
-            if (kk < R.K - 1) {
-                g[0] = fmaf((float)kk, R.sg[0], R.g0[0]);
-                g[1] = fmaf((float)kk, R.sg[1], R.g0[1]);
-                g[2] = fmaf((float)kk, R.sg[2], R.g0[2]);
-            } else {
-                if (!(R.w_last > 0.0f)) break;
-                g[0] = R.g_last[0];
-                g[1] = R.g_last[1];
-                g[2] = R.g_last[2];
-                val = y * R.w_last;
+        for (int kk = 0; kk < R.K; kk += 2) {
+            float g[2][3], w[2], gc[2][3];
+            sample_pair(G, R, kk, g, w);
+            if (MOTION)
+                warp_pair_c(G, mo, spline, g, gc);
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const float *q = MOTION ? gc[n] : g[n];
+                if (w[n] > 0.0f && q[0] >= -1.0f - cen[0] && q[0] < (float)G.nx - cen[0] && q[1] >= -1.0f - cen[1] &&
+                    q[1] < (float)G.ny - cen[1] && q[2] >= -1.0f - cen[2] && q[2] < (float)G.nz - cen[2])
+                    scatter_trilinear<DYR>(vol, G.nx, G.ny, G.nz, cen, q, y * w[n], vec, nvox, F, tau, t);
             }
-            float gc[3];
-            if (MOTION) {
-                warp_sample_c(G, mo, coef, g, gc);
-            } else {
-                gc[0] = g[0];
-                gc[1] = g[1];
-                gc[2] = g[2];
-            }
-            if (!(gc[0] >= -1.0f - cen[0] && gc[0] < (float)G.nx - cen[0] && gc[1] >= -1.0f - cen[1] &&
-                  gc[1] < (float)G.ny - cen[1] && gc[2] >= -1.0f - cen[2] && gc[2] < (float)G.nz - cen[2]))
-                continue;
-            scatter_trilinear<DYR>(vol, G.nx, G.ny, G.nz, cen, gc, val, vec, nvox, F, tau, t);
         }
     }
     if (F.live) {
@@ -245,7 +229,7 @@ cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol)
     const dim3 block(ADJ_TX, ADJ_TY);
     if (a.dyr && a.motion) return cudaErrorInvalidValue;  // the event model is defined without motion
     if (a.motion)
-        adjoint_kernel<true, false><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.coef_idx, a.view_idx,
+        adjoint_kernel<true, false><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx,
                                                                  proj, vol, a.devcheck, nullptr, nullptr);
     else if (a.dyr)
         adjoint_kernel<false, true><<<grid, block, 0, a.stream>>>(G, a.views, nullptr, nullptr, a.view_idx, proj,
@@ -301,59 +285,64 @@ __device__ __forceinline__ void trilinear_grad_c(const TV *__restrict__ vol, int
 }
 
 // Displacement u and its derivatives with respect to the three spline
-// coordinates, by sum factorisation over the separable 4 x 4 x 4 support:
-// the x sums first (value and x-derivative weights), then y, then z --
-// 576 FMAs instead of 64 taps x 12 accumulators with per-tap weight products.
-__device__ __forceinline__ void spline_value_jacobian(const float4 *coef, const int i0[3], const float wx[4],
-                                                      const float wy[4], const float wz[4], const float dx[4],
-                                                      const float dy[4], const float dz[4], float u[3],
-                                                      float Jx[3], float Jy[3], float Jz[3])
+// coordinates at fractions f of the cell at `c`: the x polynomials and their
+// derivatives, then the weighted sums over y and z.
+__device__ __forceinline__ void spline_value_jacobian(const float4 *c, const float f[3], float u[3], float Jx[3],
+                                                      float Jy[3], float Jz[3])
 {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) u[c] = Jx[c] = Jy[c] = Jz[c] = 0.0f;
-    const float4 *plane = coef_cell(coef, i0);
-    // the z loop's two weights are picked by selects, which keeps the
-    // arrays in registers when the loop stays rolled (CTREX_MGRAD_UNROLL_Z
-    // 0); the y loop is unrolled: 16 independent float4 loads per plane.
+    float wy[4], wz[4], ey[4], ez[4];
+    bspline_weights(f[1], wy);
+    bspline_weights(f[2], wz);
+    bspline_dweights(f[1], ey);
+    bspline_dweights(f[2], ez);
+    // the x and y components packed, z beside them
+    float2 U = two(0.f), X = two(0.f), Y = two(0.f), Z = two(0.f);
+    float uz = 0.f, xz = 0.f, yz = 0.f, zz = 0.f;
+    const float2 fx = two(f[0]);
+    // a rolled z loop (CTREX_MGRAD_UNROLL_Z 0) picks its weights by selects,
+    // which keeps the arrays in registers
 #if CTREX_MGRAD_UNROLL_Z
 #pragma unroll
 #else
 #pragma unroll 1
 #endif
-    for (int k = 0; k < 4; ++k, plane += CPAD * CPAD) {
-        const float wzk = k == 0 ? wz[0] : (k == 1 ? wz[1] : (k == 2 ? wz[2] : wz[3]));
-        const float dzk = k == 0 ? dz[0] : (k == 1 ? dz[1] : (k == 2 ? dz[2] : dz[3]));
-        float a[3] = {0.f, 0.f, 0.f}, bx[3] = {0.f, 0.f, 0.f}, by[3] = {0.f, 0.f, 0.f};
-        const float4 *row = plane;
+    for (int k = 0; k < 4; ++k) {
+        const float wk = k == 0 ? wz[0] : (k == 1 ? wz[1] : (k == 2 ? wz[2] : wz[3]));
+        const float ek = k == 0 ? ez[0] : (k == 1 ? ez[1] : (k == 2 ? ez[2] : ez[3]));
+        float2 v = two(0.f), dx = two(0.f), dy = two(0.f);
+        float vz = 0.f, dxz = 0.f, dyz = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j, row += CPAD) {
-            const float wyj = wy[j], dyj = dy[j];
-            float sx[3] = {0.f, 0.f, 0.f}, tx[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 cf = row[i];
-                sx[0] = fmaf(wx[i], cf.x, sx[0]);
-                sx[1] = fmaf(wx[i], cf.y, sx[1]);
-                sx[2] = fmaf(wx[i], cf.z, sx[2]);
-                tx[0] = fmaf(dx[i], cf.x, tx[0]);
-                tx[1] = fmaf(dx[i], cf.y, tx[1]);
-                tx[2] = fmaf(dx[i], cf.z, tx[2]);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                a[c] = fmaf(wyj, sx[c], a[c]);
-                bx[c] = fmaf(wyj, tx[c], bx[c]);
-                by[c] = fmaf(dyj, sx[c], by[c]);
-            }
+        for (int j = 0; j < 4; ++j) {
+            const float4 *row = c + k * SPL_PLANE + j * SPL_ROW;
+            const float4 c3 = row[3], c2 = row[2], c1 = row[1], c0 = row[0];
+            // q0: the polynomial, d: its derivative
+            const float2 p3 = make_float2(c3.x, c3.y);
+            const float2 q2 = __ffma2_rn(fx, p3, make_float2(c2.x, c2.y));
+            const float2 q1 = __ffma2_rn(fx, q2, make_float2(c1.x, c1.y));
+            const float2 q0 = __ffma2_rn(fx, q1, make_float2(c0.x, c0.y));
+            const float2 d = __ffma2_rn(fx, __ffma2_rn(fx, p3, q2), q1);
+            v = __ffma2_rn(two(wy[j]), q0, v);
+            dx = __ffma2_rn(two(wy[j]), d, dx);
+            dy = __ffma2_rn(two(ey[j]), q0, dy);
+            const float z2 = fmaf(f[0], c3.z, c2.z), z1 = fmaf(f[0], z2, c1.z), z0 = fmaf(f[0], z1, c0.z);
+            const float dz = fmaf(f[0], fmaf(f[0], c3.z, z2), z1);
+            vz = fmaf(wy[j], z0, vz);
+            dxz = fmaf(wy[j], dz, dxz);
+            dyz = fmaf(ey[j], z0, dyz);
         }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            u[c] = fmaf(wzk, a[c], u[c]);
-            Jx[c] = fmaf(wzk, bx[c], Jx[c]);
-            Jy[c] = fmaf(wzk, by[c], Jy[c]);
-            Jz[c] = fmaf(dzk, a[c], Jz[c]);
-        }
+        U = __ffma2_rn(two(wk), v, U);
+        X = __ffma2_rn(two(wk), dx, X);
+        Y = __ffma2_rn(two(wk), dy, Y);
+        Z = __ffma2_rn(two(ek), v, Z);
+        uz = fmaf(wk, vz, uz);
+        xz = fmaf(wk, dxz, xz);
+        yz = fmaf(wk, dyz, yz);
+        zz = fmaf(ek, vz, zz);
     }
+    u[0] = U.x, u[1] = U.y, u[2] = uz;
+    Jx[0] = X.x, Jx[1] = X.y, Jx[2] = xz;
+    Jy[0] = Y.x, Jy[1] = Y.y, Jy[2] = yz;
+    Jz[0] = Z.x, Jz[1] = Z.y, Jz[2] = zz;
 }
 
 // --- coefficient gradient on the tensor cores --------------------------------
@@ -403,16 +392,6 @@ __device__ __forceinline__ void mma_tf32_16x8x8(float d[4], const unsigned a[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Power-basis coefficients (f^0 .. f^3) of the uniform cubic B-spline piece m
-// (m = 0..3: weight of control point i0 - 1 + m at fraction f).
-__device__ __forceinline__ float4 bspline_piece(int m)
-{
-    return m == 0 ? make_float4(1.0f / 6.0f, -0.5f, 0.5f, -1.0f / 6.0f)
-                  : (m == 1 ? make_float4(2.0f / 3.0f, 0.0f, -1.0f, 0.5f)
-                            : (m == 2 ? make_float4(1.0f / 6.0f, 0.5f, 0.5f, -0.5f)
-                                      : make_float4(0.0f, 0.0f, 0.0f, 1.0f / 6.0f)));
-}
-
 __device__ __forceinline__ float horner(const float4 p, float f)
 {
     return fmaf(fmaf(fmaf(p.w, f, p.z), f, p.y), f, p.x);
@@ -426,8 +405,6 @@ struct CoefAcc {
 };
 
 // Adds the sums of acc's cell to the CTA's FP64 partials and clears them.
-// Entries whose control point index passes 7 carry an exactly zero weight
-// (cubic piece 3 at fraction 0) and are skipped.
 __device__ __forceinline__ void coef_flush(CoefAcc &A, double *s_g64, int lane)
 {
     if (A.cell >= 0) {
@@ -442,8 +419,7 @@ __device__ __forceinline__ void coef_flush(CoefAcc &A, double *s_g64, int lane)
                 A.acc[h][q] = 0.0f;
                 if (row >= 12 || v == 0.0f) continue;
                 const int comp = row >> 2, kz = row & 3, j = col >> 2, i = col & 3;
-                const int cx = i0x - 1 + i, cy = i0y - 1 + j, cz = i0z - 1 + kz;
-                if (cx > 7 || cy > 7 || cz > 7) continue;
+                const int cx = i0x + i, cy = i0y + j, cz = i0z + kz;
                 atomicAdd(s_g64 + 3 * ((cz * 8 + cy) * 8 + cx) + comp, (double)v);
             }
     }
@@ -465,6 +441,7 @@ __device__ __forceinline__ void coef_step(CoefAcc &A, double *s_g64, int cell, c
         const int leader = __ffs(pending) - 1;
         const int lcell = __shfl_sync(full, cell, leader);
         const bool mine = ((pending >> lane) & 1u) && cell == lcell;
+        const unsigned who = __ballot_sync(full, mine);
         if (lcell != A.cell) {
             coef_flush(A, s_g64, lane);
             A.cell = lcell;
@@ -474,6 +451,7 @@ __device__ __forceinline__ void coef_step(CoefAcc &A, double *s_g64, int cell, c
         float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
+            if (!((who >> (8 * q)) & 0xffu)) continue;  // warp-uniform: no sample of this chunk
             float a[4], b[2][2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -505,19 +483,19 @@ __device__ __forceinline__ void coef_step(CoefAcc &A, double *s_g64, int cell, c
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int e = 0; e < 4; ++e) A.acc[h][e] += d[h][e];
-        pending &= ~__ballot_sync(full, mine);
+        pending &= ~who;
     }
 }
 
 template <typename TV>
 __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
     motion_grad_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
-                       const float *__restrict__ coef_g, const int *__restrict__ view_idx,
+                       const float4 *table, const int *__restrict__ view_idx,
                        const TV *__restrict__ vol, const float *__restrict__ gproj,
                        double *__restrict__ grad_M, double *__restrict__ grad_b,
                        double *__restrict__ grad_coef, unsigned *devcheck)
 {
-    __shared__ float4 s_coef[NCOEF_PAD];  // zero-padded 9^3 float4 copy of the coefficients
+    __shared__ float4 s_spline[SPLINE_TABLE];
     __shared__ double s_g64[NCOEF];       // the CTA's coefficient-gradient partials
     __shared__ double s_red[12][MG_WARPS];
     __shared__ float4 s_piece[4];
@@ -530,9 +508,9 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
         return;  // uniform over the CTA
     }
     const MotionGPU mo = motion[view];
-    const bool spline = coef_g != nullptr && mo.s != 0.0f;
+    const bool spline = table != nullptr && mo.s != 0.0f;
     const bool want_coef = spline && grad_coef != nullptr;
-    if (spline) load_coef_padded(s_coef, coef_g, tid, MG_THREADS);
+    if (spline) load_spline(s_spline, table, tid, MG_THREADS);
     if (want_coef)
         for (int i = tid; i < NCOEF; i += MG_THREADS) s_g64[i] = 0.0;
     if (tid < 4) s_piece[tid] = bspline_piece(tid);
@@ -580,7 +558,7 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
 #pragma unroll
             for (int r = 0; r < 3; ++r)
                 d[r] = fmaf(mo.D[3 * r], gc[0], fmaf(mo.D[3 * r + 1], gc[1], fmaf(mo.D[3 * r + 2], gc[2], mo.bc[r])));
-            int i0[3] = {1, 1, 1};
+            int i0[3] = {0, 0, 0};
             float f[3] = {0.f, 0.f, 0.f};
             float u[3] = {0.f, 0.f, 0.f}, Jx[3] = {0.f, 0.f, 0.f}, Jy[3] = {0.f, 0.f, 0.f},
                   Jz[3] = {0.f, 0.f, 0.f};
@@ -588,14 +566,7 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
                 bool on[3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) spline_coord(gc[a] + d[a] + cen[a], G.spl_scale[a], i0[a], f[a], on[a]);
-                float wx[4], wy[4], wz[4], dx[4], dy[4], dz[4];
-                bspline_weights(f[0], wx);
-                bspline_weights(f[1], wy);
-                bspline_weights(f[2], wz);
-                bspline_dweights(f[0], dx);
-                bspline_dweights(f[1], dy);
-                bspline_dweights(f[2], dz);
-                spline_value_jacobian(s_coef, i0, wx, wy, wz, dx, dy, dz, u, Jx, Jy, Jz);
+                spline_value_jacobian(spline_cell(s_spline, i0), f, u, Jx, Jy, Jz);
                 const float sx = on[0] ? G.spl_scale[0] : 0.f, sy = on[1] ? G.spl_scale[1] : 0.f,
                             sz = on[2] ? G.spl_scale[2] : 0.f;
 #pragma unroll
@@ -671,12 +642,12 @@ cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *gra
     const dim3 grid((G.nu + 8 * MG_WARPS - 1) / (8 * MG_WARPS), a.n_idx, (G.nv + 3) / 4);
     const dim3 block(32, MG_WARPS);
     if (a.vol_dtype == CTREX_F32)
-        motion_grad_kernel<float><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.coef_idx, a.view_idx,
+        motion_grad_kernel<float><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx,
                                                                (const float *)a.vol, gproj, grad_M, grad_b,
                                                                grad_coef_idx, a.devcheck);
     else
         motion_grad_kernel<__nv_bfloat16><<<grid, block, 0, a.stream>>>(
-            G, a.views, a.motion, a.coef_idx, a.view_idx, (const __nv_bfloat16 *)a.vol, gproj, grad_M, grad_b,
+            G, a.views, a.motion, a.spline, a.view_idx, (const __nv_bfloat16 *)a.vol, gproj, grad_M, grad_b,
             grad_coef_idx, a.devcheck);
     return cudaGetLastError();
 }
@@ -777,15 +748,23 @@ __global__ void motion_setup_kernel(const float *__restrict__ theta, const float
     for (int q = 0; q < 27; ++q) dRdw[27 * v + q] = (float)dR[q];
 }
 
-__global__ void coef_to_index_kernel(const float *__restrict__ coef, Frame F, float *__restrict__ coef_idx)
+// The spline's table (ray.cuh), FP64: thread = (z, y, cell, power).
+__global__ void __launch_bounds__(SPL_PLANE) spline_table_kernel(const float *__restrict__ coef, Frame F,
+                                                                 float4 *__restrict__ table)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NCOEF) coef_idx[i] = (float)(coef[i] / F.vox[i % 3]);
+    // f^p coefficients of piece m (B-spline matrix times 6)
+    const double B[4][4] = {{1, -3, 3, -1}, {4, 0, -6, 3}, {1, 3, 3, -3}, {0, 0, 0, 1}};
+    const int p = threadIdx.x & 3, cell = threadIdx.x / 4 % 5, y = threadIdx.x / SPL_ROW, z = blockIdx.x;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int m = 0; m < 4; ++m)
+        for (int a = 0; a < 3; ++a) s[a] += B[m][p] / 6.0 * (double)coef[3 * ((z * 8 + y) * 8 + cell + m) + a];
+    table[z * SPL_PLANE + threadIdx.x] =
+        make_float4((float)(s[0] / F.vox[0]), (float)(s[1] / F.vox[1]), (float)(s[2] / F.vox[2]), 0.f);
 }
 
 cudaError_t launch_motion_setup(const float *theta, const float *coef, const float *s_view, int n_views,
                                 const Grid &G, const double vox[3], const double origin[3], MotionGPU *motion,
-                                float *coef_idx, float *dRdw, cudaStream_t stream)
+                                float4 *spline, float *dRdw, cudaStream_t stream)
 {
     Frame F;
     const int n[3] = {G.nx, G.ny, G.nz};
@@ -798,7 +777,7 @@ cudaError_t launch_motion_setup(const float *theta, const float *coef, const flo
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (coef) {
-        coef_to_index_kernel<<<(NCOEF + 255) / 256, 256, 0, stream>>>(coef, F, coef_idx);
+        spline_table_kernel<<<8, SPL_PLANE, 0, stream>>>(coef, F, spline);
         e = cudaGetLastError();
     }
     return e;

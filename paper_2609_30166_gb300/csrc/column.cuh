@@ -86,7 +86,6 @@ __device__ __forceinline__ ColTaps col_load(const ColVolume &V, unsigned i)
     const float2 *a = V.p + i, *b = V.p + V.sy + i;
     return {__ldg(a), __ldg(a + (1 << COL_LOG)), __ldg(b), __ldg(b + (1 << COL_LOG))};
 }
-__device__ __forceinline__ float2 two(float x) { return make_float2(x, x); }
 // a + f (b - a) for both z neighbours
 __device__ __forceinline__ float2 lerp2(float2 a, float2 b, float2 f)
 {

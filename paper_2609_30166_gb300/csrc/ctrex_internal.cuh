@@ -91,6 +91,11 @@ template <> struct Storage<__nv_bfloat16> {
     static __device__ __forceinline__ void store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
+#ifdef __CUDACC__
+// operand of packed FP32 arithmetic
+__device__ __forceinline__ float2 two(float x) { return make_float2(x, x); }
+#endif
+
 // Status word written by kernels whose own bounds checks fire (never trap).
 enum : unsigned { DEVCHECK_OOB = 1u };
 
@@ -134,7 +139,7 @@ struct FwdArgs {
     const ColStore *column_tau = nullptr;  // with it: the event model's transition times
     const ViewGPU *views;       // device [n_views * n_sub]
     const MotionGPU *motion;    // device [n_views] or nullptr
-    const float *coef_idx;      // device [8][8][8][3] voxels, or nullptr
+    const float4 *spline;       // device: the deformation's table (ray.cuh), or nullptr
     const void *vol;
     int vol_dtype;
     const int *view_idx;        // device or nullptr
@@ -190,11 +195,17 @@ cudaError_t launch_backproject_column(const BpArgs &a);
 bool backproject_column_fits(const Grid &g);  // its launch shape stays within the grid limits
 
 cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol);
+// The same through a scatter volume of adjoint_column_elems(G) floats
+// (adjoint_column.cu); 0: not for this grid.  along_z: detector columns run
+// nearly along z.
+cudaError_t launch_adjoint_column(const FwdArgs &a, bool along_z, const float *proj, float *vol, float *scratch);
+size_t adjoint_column_elems(const Grid &g);
 cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *grad_M, double *grad_b,
                                double *grad_coef_idx);
+constexpr int SPLINE_TABLE = 8 * 8 * 5 * 4;  // float4 elements of the deformation's table (ray.cuh)
 cudaError_t launch_motion_setup(const float *theta, const float *coef, const float *s_view,
                                 int n_views, const Grid &g, const double vox[3],
-                                const double origin[3], MotionGPU *motion, float *coef_idx,
+                                const double origin[3], MotionGPU *motion, float4 *spline,
                                 float *dRdw, cudaStream_t stream);
 cudaError_t launch_motion_grad_finish(const float *theta, const float *dRdw, const double *grad_M,
                                       const double *grad_b, const double *grad_coef_idx, int n_views,

@@ -39,7 +39,7 @@ __device__ __forceinline__ float LinearSampler<TV>::interior(float gx, float gy,
 // every sample is mapped to (r, phi, z) by the sampler; the rest is shared.
 template <typename Sampler, bool MOTION>
 __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__restrict__ views,
-                                               const MotionGPU &mo, const float4 *coef,
+                                               const MotionGPU &mo, const float4 *spline,
                                                const Sampler &vol, int view, float u,
                                                float v, float &val, float &rs)
 {
@@ -70,44 +70,39 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
         const int Km1 = R.K - 1;
         int ka = Km1, kb = Km1;
         if (!MOTION && !Sampler::CYLINDER) interior_range(G, R, ka, kb);
-        auto general = [&](int k) {
-            float g[3];
-            g[0] = fmaf((float)k, R.sg[0], R.g0[0]);
-            g[1] = fmaf((float)k, R.sg[1], R.g0[1]);
-            g[2] = fmaf((float)k, R.sg[2], R.g0[2]);
-            if (MOTION) {
-                float y[3];
-                warp_sample(G, mo, coef, g, y);
-                g[0] = y[0];
-                g[1] = y[1];
-                g[2] = y[2];
+        if constexpr (MOTION) {
+            for (int k = 0; k < R.K; k += 2) {
+                float g[2][3], w[2], y[2][3];
+                sample_pair(G, R, k, g, w);
+                warp_pair(G, mo, spline, g, y);
+#pragma unroll
+                for (int n = 0; n < 2; ++n) {
+                    float ws;
+                    a = fmaf(w[n], vol(y[n][0], y[n][1], y[n][2], ws), a);
+                    ars = fmaf(w[n], ws, ars);
+                }
             }
+            acc += a;
+            acc_rs += ars;
+            continue;
+        }
+        auto general = [&](int k) {
             float ws;
-            a += vol(g[0], g[1], g[2], ws);
+            a += vol(fmaf((float)k, R.sg[0], R.g0[0]), fmaf((float)k, R.sg[1], R.g0[1]),
+                     fmaf((float)k, R.sg[2], R.g0[2]), ws);
             ars += ws;
         };
-        const int kstop = MOTION ? Km1 : ka;
-        for (int k = 0; k < kstop; ++k) general(k);
-        if (!MOTION) {
-            for (int k = ka; k < kb; ++k)
-                a += vol.interior(fmaf((float)k, R.sg[0], R.g0[0]), fmaf((float)k, R.sg[1], R.g0[1]),
-                                  fmaf((float)k, R.sg[2], R.g0[2]));
-            ars += (float)(kb - ka);
-            for (int k = kb; k < Km1; ++k) general(k);
-        }
+        for (int k = 0; k < ka; ++k) general(k);
+        for (int k = ka; k < kb; ++k)
+            a += vol.interior(fmaf((float)k, R.sg[0], R.g0[0]), fmaf((float)k, R.sg[1], R.g0[1]),
+                              fmaf((float)k, R.sg[2], R.g0[2]));
+        ars += (float)(kb - ka);
+        for (int k = kb; k < Km1; ++k) general(k);
         a *= G.step_mm;
         ars *= G.step_mm;
         if (R.w_last > 0.0f) {
-            float g[3] = {R.g_last[0], R.g_last[1], R.g_last[2]};
-            if (MOTION) {
-                float y[3];
-                warp_sample(G, mo, coef, g, y);
-                g[0] = y[0];
-                g[1] = y[1];
-                g[2] = y[2];
-            }
             float ws;
-            a = fmaf(R.w_last, vol(g[0], g[1], g[2], ws), a);
+            a = fmaf(R.w_last, vol(R.g_last[0], R.g_last[1], R.g_last[2], ws), a);
             ars = fmaf(R.w_last, ws, ars);
         }
         acc += a;
@@ -119,13 +114,12 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
 
 template <typename Sampler, typename TP, int MODE, bool MOTION>
 __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ views,
-                                         const MotionGPU *__restrict__ motion, const float *__restrict__ coef_g,
+                                         const MotionGPU *__restrict__ motion, const float4 *spline,
                                          const Sampler &vol_in, const int *__restrict__ view_idx,
                                          TP *__restrict__ out, float *__restrict__ rowsum_out,
                                          const TP *__restrict__ p, float *__restrict__ partials, unsigned *devcheck,
                                          int p_by_view)
 {
-    __shared__ float4 s_coef[MOTION ? NCOEF_PAD : 1];  // zero-padded 9^3 float4 copy of the coefficients
     __shared__ float s_red[2][FWD_TX * FWD_TY / 32];
     __shared__ float2 s_tile[Sampler::TILE_TABLE];
     Sampler vol = vol_in;
@@ -140,12 +134,12 @@ __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ vie
     }
     if constexpr (Sampler::DYRECT) vol.set_view(view);  // the view's acquisition time
     MotionGPU mo;
-    const float4 *coef = nullptr;
+    __shared__ float4 s_spline[MOTION ? SPLINE_TABLE : 1];
     if (MOTION) {
         mo = motion[view];
-        if (coef_g != nullptr) {
-            load_coef_padded(s_coef, coef_g, threadIdx.y * FWD_TX + threadIdx.x, FWD_TX * FWD_TY);
-            coef = s_coef;
+        if (spline != nullptr) {
+            load_spline(s_spline, spline, threadIdx.y * FWD_TX + threadIdx.x, FWD_TX * FWD_TY);
+            spline = s_spline;
         }
         __syncthreads();
     }
@@ -154,7 +148,7 @@ __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ vie
     const bool in_pix = iu < G.nu && iv < G.nv;
     const bool inside = ok && in_pix;
     float val = 0.0f, rs = 0.0f;
-    if (inside) pixel_integral<Sampler, MOTION>(G, views, mo, coef, vol, view, (float)iu, (float)iv, val, rs);
+    if (inside) pixel_integral<Sampler, MOTION>(G, views, mo, spline, vol, view, (float)iu, (float)iv, val, rs);
     fwd_epilogue<TP, MODE>(G, k, view, ok, in_pix, iu, iv, val, rs, out, rowsum_out, p, partials, p_by_view,
                            s_red);
 }
@@ -162,11 +156,11 @@ __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ vie
 template <typename Sampler, typename TP, int MODE, bool MOTION>
 __global__ void __launch_bounds__(FWD_TX *FWD_TY)
     fwd_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
-               const float *__restrict__ coef_g, const Sampler vol_in, const int *__restrict__ view_idx,
+               const float4 *spline, const Sampler vol_in, const int *__restrict__ view_idx,
                TP *__restrict__ out, float *__restrict__ rowsum_out, const TP *__restrict__ p,
                float *__restrict__ partials, unsigned *devcheck, int p_by_view)
 {
-    fwd_body<Sampler, TP, MODE, MOTION>(G, views, motion, coef_g, vol_in, view_idx, out, rowsum_out, p, partials,
+    fwd_body<Sampler, TP, MODE, MOTION>(G, views, motion, spline, vol_in, view_idx, out, rowsum_out, p, partials,
                                         devcheck, p_by_view);
 }
 
@@ -272,7 +266,7 @@ static cudaError_t fwd_launch(const FwdArgs &a, const Sampler &smp, TP *out, flo
     if constexpr (!Sampler::CYLINDER && !Sampler::JOSEPH && !Sampler::ROI && !Sampler::DYRECT) {
         if (a.motion) {
             fwd_kernel<Sampler, TP, MODE, true><<<grid, block, 0, a.stream>>>(
-                G, a.views, a.motion, a.coef_idx, smp, a.view_idx, out, rowsum, p, partials, a.devcheck,
+                G, a.views, a.motion, a.spline, smp, a.view_idx, out, rowsum, p, partials, a.devcheck,
                 a.p_by_view);
             return cudaGetLastError();
         }

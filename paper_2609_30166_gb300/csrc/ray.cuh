@@ -153,8 +153,28 @@ __device__ __forceinline__ float trilinear(const TV *__restrict__ vol, int nx, i
     return fmaf(wz0, c0, wz1 * c1);
 }
 
-// Uniform cubic B-spline weights of control points i0-1 .. i0+2 at fractional
-// offset f in [0, 1) (i0 = floor of the spline coordinate), and derivatives.
+// The deformation.  Along x the uniform cubic B-spline is held as one cubic
+// polynomial per cell (between two control planes), along y and z by its
+// basis functions: x by Horner's scheme (3 multiply-adds a row and component
+// instead of 4, and no x weights), then weighted sums over y and z.  One pass
+// over a cell's 64 coefficients serves two samples of a ray (their loads are
+// what bounds it: a vector load fills a register of every lane, shared
+// address or not).  Table: [z 8][y 8][cell 5][power of f 4] float4 (x, y, z
+// components in voxels), 20 KB, copied to shared memory by each CTA.
+//
+// 45 views of the 256^3 motion workload, basis functions on three axes and a
+// pass per sample / this: projector 29.7 / 23.8 ms, gradient 118.7 / 104.3 ms
+// (all 64 monomials per cell from a 125 KB table in global memory: 39.5 ms).
+constexpr int SPL_ROW = 5 * 4, SPL_PLANE = 8 * SPL_ROW;
+static_assert(SPLINE_TABLE == 8 * SPL_PLANE, "spline table size");
+
+__device__ __forceinline__ void load_spline(float4 *s, const float4 *__restrict__ table, int tid, int nthreads)
+{
+    for (int i = tid; i < SPLINE_TABLE; i += nthreads) s[i] = __ldg(table + i);
+}
+
+// Uniform cubic B-spline weights of the cell's control points at fraction f,
+// and their derivatives.
 __device__ __forceinline__ void bspline_weights(float f, float w[4])
 {
     const float f2 = f * f, f3 = f2 * f, g = 1.0f - f;
@@ -173,16 +193,105 @@ __device__ __forceinline__ void bspline_dweights(float f, float d[4])
     d[3] = 0.5f * f2;
 }
 
-// Spline coordinate of index coordinate gp along one axis (clamped to [1, 6]);
-// i0 in [1, 6], f in [0, 1); `active` is false where the clamp holds.
-__device__ __forceinline__ void spline_coord(float gp, float scale, int &i0, float &f, bool &active)
+// Power-basis coefficients (f^0 .. f^3) of the uniform cubic B-spline piece m
+// (m = 0..3: weight of control point i0 - 1 + m at fraction f).
+__host__ __device__ __forceinline__ float4 bspline_piece(int m)
+{
+    return m == 0 ? make_float4(1.0f / 6.0f, -0.5f, 0.5f, -1.0f / 6.0f)
+                  : (m == 1 ? make_float4(2.0f / 3.0f, 0.0f, -1.0f, 0.5f)
+                            : (m == 2 ? make_float4(1.0f / 6.0f, 0.5f, 0.5f, -0.5f)
+                                      : make_float4(0.0f, 0.0f, 0.0f, 1.0f / 6.0f)));
+}
+
+// Spline coordinate of index coordinate gp along one axis (clamped to [1,
+// 6]): cell i in [0, 4] and fraction f in [0, 1]; `active` is false where the
+// clamp holds.
+__device__ __forceinline__ void spline_coord(float gp, float scale, int &i, float &f, bool &active)
 {
     float xi = fmaf(gp + 0.5f, scale, 1.0f);
     active = (xi > 1.0f) && (xi < 6.0f);
     xi = fminf(fmaxf(xi, 1.0f), 6.0f);
-    const float fl = floorf(xi);
-    i0 = (int)fl;
+    const float fl = fminf(floorf(xi), 5.0f);
+    i = (int)fl - 1;
     f = xi - fl;
+}
+
+__device__ __forceinline__ const float4 *spline_cell(const float4 *table, const int i[3])
+{
+    return table + i[2] * SPL_PLANE + i[1] * SPL_ROW + i[0] * 4;
+}
+
+// Displacement u (voxels) of N samples in the cell at `c`, fractions f.
+template <int N>
+__device__ __forceinline__ void spline_value(const float4 *c, const float (&f)[N][3], float (&u)[N][3])
+{
+    float wy[N][4], wz[N][4];
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        bspline_weights(f[n][1], wy[n]);
+        bspline_weights(f[n][2], wz[n]);
+    }
+    float2 uxy[N];
+    float uz[N];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float2 yxy[N];
+        float yz[N];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 *row = c + k * SPL_PLANE + j * SPL_ROW;
+            const float4 c3 = row[3], c2 = row[2], c1 = row[1], c0 = row[0];
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                const float2 fx = make_float2(f[n][0], f[n][0]), w = make_float2(wy[n][j], wy[n][j]);
+                float2 r = __ffma2_rn(fx, make_float2(c3.x, c3.y), make_float2(c2.x, c2.y));
+                r = __ffma2_rn(fx, r, make_float2(c1.x, c1.y));
+                r = __ffma2_rn(fx, r, make_float2(c0.x, c0.y));
+                const float z = fmaf(f[n][0], fmaf(f[n][0], fmaf(f[n][0], c3.z, c2.z), c1.z), c0.z);
+                yxy[n] = j == 0 ? __fmul2_rn(w, r) : __ffma2_rn(w, r, yxy[n]);
+                yz[n] = j == 0 ? w.x * z : fmaf(w.x, z, yz[n]);
+            }
+        }
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const float2 w = make_float2(wz[n][k], wz[n][k]);
+            uxy[n] = k == 0 ? __fmul2_rn(w, yxy[n]) : __ffma2_rn(w, yxy[n], uxy[n]);
+            uz[n] = k == 0 ? w.x * yz[n] : fmaf(w.x, yz[n], uz[n]);
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        u[n][0] = uxy[n].x;
+        u[n][1] = uxy[n].y;
+        u[n][2] = uz[n];
+    }
+}
+
+// Displacements of two samples at index coordinates g: one pass over the
+// first one's cell serves both, and a second sample beyond its face (a step
+// is a small part of a cell) takes a pass of its own.
+__device__ __forceinline__ void spline_pair(const Grid &G, const float4 *table, const float g[2][3], float u[2][3])
+{
+    float f[2][3];
+    int i[2][3];
+    bool on;
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) spline_coord(g[n][a], G.spl_scale[a], i[n][a], f[n][a], on);
+    float v[2][3];
+    spline_value<2>(spline_cell(table, i[0]), f, v);
+    if (i[0][0] != i[1][0] || i[0][1] != i[1][1] || i[0][2] != i[1][2]) {
+        const float f1[1][3] = {{f[1][0], f[1][1], f[1][2]}};
+        float w[1][3];
+        spline_value<1>(spline_cell(table, i[1]), f1, w);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[1][a] = w[0][a];
+    }
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[n][a] = v[n][a];
 }
 
 // Pixel of this thread in a 32 x 4 pixel CTA tile.  Row layout: warp w is
@@ -204,35 +313,6 @@ __device__ __forceinline__ void tile_pixel(int tile_u0, int tile_v0, int &iu, in
     }
 }
 
-// Shared-memory copy of the [8][8][8][3] B-spline coefficients as float4
-// (one vector load each), zero-padded to 9 x 9 x 9: the 4 x 4 x 4 support of
-// spline cell i0 (i0 in [1, 6] per axis) spans control points i0 - 1 ..
-// i0 + 2, at most 8, so no index needs clamping; a point 8 is reached only
-// at spline coordinate 6 exactly, where its weight (cubic piece 3 at
-// fraction 0) is zero.  Tap (i, j, k) of the cell is base[k * 81 + j * 9 + i]
-// with base = coef_cell(coef, i0): constant offsets from one address.
-constexpr int CPAD = 9;
-constexpr int NCOEF_PAD = CPAD * CPAD * CPAD;
-
-__device__ __forceinline__ void load_coef_padded(float4 *__restrict__ s, const float *__restrict__ coef_g, int tid,
-                                                 int nthreads)
-{
-    for (int i = tid; i < NCOEF_PAD; i += nthreads) {
-        const int cx = i % CPAD, cy = (i / CPAD) % CPAD, cz = i / (CPAD * CPAD);
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (cx < 8 && cy < 8 && cz < 8) {
-            const float *c = coef_g + 3 * ((cz * 8 + cy) * 8 + cx);
-            v = make_float4(c[0], c[1], c[2], 0.0f);
-        }
-        s[i] = v;
-    }
-}
-
-__device__ __forceinline__ const float4 *coef_cell(const float4 *coef, const int i0[3])
-{
-    return coef + ((i0[2] - 1) * CPAD + (i0[1] - 1)) * CPAD + (i0[0] - 1);
-}
-
 // Integer grid centre c = floor((n - 1) / 2) per axis (index coordinates).
 __device__ __forceinline__ void grid_centre(const Grid &G, float c[3])
 {
@@ -241,96 +321,68 @@ __device__ __forceinline__ void grid_centre(const Grid &G, float c[3])
     c[2] = (float)((G.nz - 1) >> 1);
 }
 
-// Warp of one sample (Sec. 2.2.2 pose, then Sec. 3.1 displacement), in
+// Warp of two samples (Sec. 2.2.2 pose, then Sec. 3.1 displacement), in
 // coordinates centred on the integer grid centre c: gc = g - c in (g index
 // coordinates), yc = y - c out, with y = M g + b + s u(M g + b).  It runs as
 // yc = gc + (D gc + bc + s u) with gc = g - c, D = M - I, bc = M c + b - c:
 // the bracket is a displacement of a few voxels for a near-identity pose,
 // so its roundings are small, and only the last addition rounds at the
 // magnitude of the coordinate (up to n / 2).  Since c is an integer, floor
-// and fraction of y follow exactly from yc.  coef: the padded shared-memory
-// copy of the coefficients in voxels (load_coef_padded), or nullptr.
-__device__ __forceinline__ void warp_sample_c(const Grid &G, const MotionGPU &m, const float4 *coef, const float gc[3],
-                                              float yc[3])
+// and fraction of y follow exactly from yc.  table: the spline's table in shared
+// memory, or nullptr.
+__device__ __forceinline__ void warp_pair_c(const Grid &G, const MotionGPU &m, const float4 *table,
+                                            const float gc[2][3], float yc[2][3])
 {
     float c[3];
     grid_centre(G, c);
-    float d[3];  // displacement D gc + bc (+ s u below)
+    float d[2][3], g[2][3], u[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};  // d: displacement D gc + bc
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
-        d[r] = fmaf(m.D[3 * r], gc[0], fmaf(m.D[3 * r + 1], gc[1], fmaf(m.D[3 * r + 2], gc[2], m.bc[r])));
-    float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
-    if (coef != nullptr && m.s != 0.0f) {
-        int i0[3];
-        float f[3], wx[4], wy[4], wz[4];
-        bool act[3];
+    for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) spline_coord(gc[a] + d[a] + c[a], G.spl_scale[a], i0[a], f[a], act[a]);
-        bspline_weights(f[0], wx);
-        bspline_weights(f[1], wy);
-        bspline_weights(f[2], wz);
-        const float4 *base = coef_cell(coef, i0);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float wyz = wz[k] * wy[j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float wt = wyz * wx[i];
-                    const float4 cf = base[k * CPAD * CPAD + j * CPAD + i];
-                    u0 = fmaf(wt, cf.x, u0);
-                    u1 = fmaf(wt, cf.y, u1);
-                    u2 = fmaf(wt, cf.z, u2);
-                }
-            }
+        for (int r = 0; r < 3; ++r) {
+            d[n][r] = fmaf(m.D[3 * r], gc[n][0],
+                           fmaf(m.D[3 * r + 1], gc[n][1], fmaf(m.D[3 * r + 2], gc[n][2], m.bc[r])));
+            g[n][r] = gc[n][r] + d[n][r] + c[r];
         }
-    }
-    yc[0] = gc[0] + fmaf(m.s, u0, d[0]);
-    yc[1] = gc[1] + fmaf(m.s, u1, d[1]);
-    yc[2] = gc[2] + fmaf(m.s, u2, d[2]);
+    if (table != nullptr && m.s != 0.0f) spline_pair(G, table, g, u);
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) yc[n][r] = gc[n][r] + fmaf(m.s, u[n][r], d[n][r]);
 }
 
 // The same warp in plain index coordinates, as the forward projector uses it:
 // y = M g + b + s u(M g + b) formed directly (fewer operations; the forward
 // averages the position rounding out along the ray, so it needs no centring).
-__device__ __forceinline__ void warp_sample(const Grid &G, const MotionGPU &m, const float4 *coef, const float g[3],
-                                            float y[3])
+__device__ __forceinline__ void warp_pair(const Grid &G, const MotionGPU &m, const float4 *table, const float g[2][3],
+                                          float y[2][3])
 {
-    float gp[3];
+    float gp[2][3], u[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
-        gp[r] = fmaf(m.M[3 * r], g[0], fmaf(m.M[3 * r + 1], g[1], fmaf(m.M[3 * r + 2], g[2], m.b[r])));
-    float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
-    if (coef != nullptr && m.s != 0.0f) {
-        int i0[3];
-        float f[3], wx[4], wy[4], wz[4];
-        bool act[3];
+    for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) spline_coord(gp[a], G.spl_scale[a], i0[a], f[a], act[a]);
-        bspline_weights(f[0], wx);
-        bspline_weights(f[1], wy);
-        bspline_weights(f[2], wz);
-        const float4 *base = coef_cell(coef, i0);
+        for (int r = 0; r < 3; ++r)
+            gp[n][r] = fmaf(m.M[3 * r], g[n][0],
+                            fmaf(m.M[3 * r + 1], g[n][1], fmaf(m.M[3 * r + 2], g[n][2], m.b[r])));
+    if (table != nullptr && m.s != 0.0f) spline_pair(G, table, gp, u);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+    for (int n = 0; n < 2; ++n)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float wyz = wz[k] * wy[j];
+        for (int r = 0; r < 3; ++r) y[n][r] = fmaf(m.s, u[n][r], gp[n][r]);
+}
+
+// Samples kk and kk + 1 of a ray and their weights (mm): the last one is the
+// clipped segment's remainder, one past it weighs nothing (and repeats it).
+__device__ __forceinline__ void sample_pair(const Grid &G, const Ray &R, int kk, float g[2][3], float w[2])
+{
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float wt = wyz * wx[i];
-                    const float4 cf = base[k * CPAD * CPAD + j * CPAD + i];
-                    u0 = fmaf(wt, cf.x, u0);
-                    u1 = fmaf(wt, cf.y, u1);
-                    u2 = fmaf(wt, cf.z, u2);
-                }
-            }
-        }
+    for (int n = 0; n < 2; ++n) {
+        const bool last = kk + n >= R.K - 1;
+        const float kf = (float)(kk + n);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) g[n][a] = last ? R.g_last[a] : fmaf(kf, R.sg[a], R.g0[a]);
+        w[n] = last ? (kk + n == R.K - 1 ? fmaxf(R.w_last, 0.0f) : 0.0f) : G.step_mm;
     }
-    y[0] = fmaf(m.s, u0, gp[0]);
-    y[1] = fmaf(m.s, u1, gp[1]);
-    y[2] = fmaf(m.s, u2, gp[2]);
 }
 
 }  // namespace ctrex

@@ -1,4 +1,4 @@
-"""The column kernels (fwd_column*.cu, bp_column.cu) at the edges of their tiles
+"""The column kernels (*_column*.cu) at the edges of their tiles
 and of the rules that choose them, against the FP64 oracle.
 
 Both choices compute the same operator, so every case holds to the projector's
@@ -151,4 +151,47 @@ def test_models_match_oracle(model, turn, tall):
         got = c.fwd_project(_t(x, dt), rowsum=rows, out_dtype=torch.float32)
         assert rel_l2(_np(got), ref) <= TOL32
         assert rel_l2(_np(rows), rs) <= TOL32
+    c.close()
+
+
+@pytest.mark.parametrize("n,det,views,sub,turn", [
+    ((37, 22, 65), (45, 33), 5, 1, 0.4),    # rows of a detector column
+    ((32, 64, 31), (130, 40), 3, 2, 2.0),
+    ((20, 31, 96), (33, 64), 5, 1, 30.0),   # patches
+    ((41, 24, 30), (31, 50), 5, 1, 70.0),
+    ((1, 40, 33), (40, 40), 5, 1, 0.0),
+    ((64, 64, 64), (12, 5), 1, 1, 0.0),     # few rays: in place
+])
+@pytest.mark.parametrize("motion", [False, True])
+def test_adjoint_matches_oracle(n, det, views, sub, turn, motion):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    P = _matrices(views, sub, turn, det[0], det[1], 96.0, 200.0)
+    pitch = 30.0 / max(n)
+    vox, shape = (pitch, 0.9 * pitch, 1.1 * pitch), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det)
+    rng = np.random.default_rng(21)
+    if motion:
+        theta = np.zeros((views, 15))
+        theta[:, :6] = rng.uniform(-0.02, 0.02, (views, 6))
+        theta[:, 6:] = np.eye(3).ravel() + rng.uniform(-0.01, 0.01, (views, 9))
+        coef, sv = rng.uniform(-1, 1, (8, 8, 8, 3)) * 1.5 * pitch, np.linspace(0.2, 1.0, views)
+        theta, coef, sv = (_np(_t(a)) for a in (theta, coef, sv))  # as the GPU sees them
+        pb = pb.with_motion(theta, coef, sv, margin=0.5)
+        c.set_motion(_t(theta), _t(coef), _t(sv), 0.5)
+    y = rng.uniform(0.5, 1.5, size=(views, det[1], det[0]))
+    x0 = rng.uniform(size=shape)
+    want = oracle.adjoint(pb, _np(_t(y)))
+    got = _np(c.adjoint_project(_t(y), vol=_t(x0))) - _np(_t(x0))  # accumulates
+    assert rel_l2(got, want) <= TOL32
+    vi = np.arange(views)[::-2].astype(np.int32).copy()
+    want = oracle.adjoint(pb, _np(_t(y[vi])), views=vi)
+    assert rel_l2(_np(c.adjoint_project(_t(y[vi]), view_idx=vi)), want) <= TOL32
+    if motion:
+        x = rng.uniform(0.2, 1.0, size=shape)
+        assert rel_l2(_np(c.fwd_project(_t(x))), oracle.forward(pb, _np(_t(x)))[0]) <= TOL32
     c.close()
