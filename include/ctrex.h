@@ -465,6 +465,37 @@ int ctrex_conv3d_wgrad(const void *x, const void *dy, float *dw, int nb, int d, 
                        int cout, int *status, void *cuda_stream);
 
 /*
+ * Backward pass of a convolution layer's activation and bias: with y (the
+ * layer's output after its ReLU) g = dy * (y > 0), without y (NULL) the ReLU
+ * mask is skipped and g is not written; db[c] = sum over the voxels of g (of
+ * dy without y), overwritten.  dy, y, g: DEVICE bf16 [voxels][channels],
+ * 16-byte aligned; db: DEVICE float [channels]; scratch: DEVICE float
+ * [1216][channels].  channels / 8 must be a power of two up to 256
+ * (CTREX_E_SHAPE otherwise).  Deterministic.
+ */
+int ctrex_conv3d_bias_grad(const void *dy, const void *y, void *g, float *db, float *scratch, long long voxels,
+                           int channels, void *cuda_stream);
+
+/*
+ * The warm-start network's forward pass, y = x + correction(x): four levels
+ * of base, 2, 4, 8 x base channels, two 3x3x3 convolutions with ReLU per
+ * level, max pooling down, nearest upsampling with skip concatenation up, a
+ * per-voxel linear head.  x, y: DEVICE float [nb][d][h][w] (d, h, w multiples
+ * of 8; base a multiple of 8; x and y must not overlap).  weights, bias: HOST
+ * arrays of 14 DEVICE pointers, float [cout][27][cin] (cast to BF16 on each
+ * call) and float [cout], in the order encoder level 0 .. 3, decoder level 2
+ * .. 0, two layers each (the first with 16 input channels, of which x is
+ * channel 0 and the others zero; decoder inputs are [upsampled | skip]).
+ * head_w: DEVICE float [base]; head_b: DEVICE float [1].  workspace: DEVICE,
+ * 256-byte aligned, ctrex_unet_workspace bytes (negative: an error code), free
+ * for reuse once the call's work is done.  status: as ctrex_conv3d_fwd.
+ */
+long long ctrex_unet_workspace(int nb, int d, int h, int w, int base);
+int ctrex_unet_forward(const float *x, float *y, const float *const *weights, const float *const *bias,
+                       const float *head_w, const float *head_b, int nb, int d, int h, int w, int base,
+                       void *workspace, int *status, void *cuda_stream);
+
+/*
  * Measured ceiling of the texture path: tex2Dgather calls per second on the
  * current device, on a 64 KiB texture that stays in L1 (each call returns a
  * 2x2 footprint, four 32-bit values, per thread).  Allocates and frees a

@@ -35,7 +35,7 @@ EXPORTS = (
     "ctrex_sirt_iterate", "ctrex_sirt_host", "ctrex_count_samples", "ctrex_correct_static",
     "ctrex_conv3d_fwd", "ctrex_conv3d_wgrad", "ctrex_os_sirt_iterate", "ctrex_set_bp_window",
     "ctrex_probe_gather_rate", "ctrex_probe_l2_read_bandwidth", "ctrex_set_dyrect", "ctrex_set_bp_subvoxel", "ctrex_set_geometry_cylinder", "ctrex_set_projector",
-    "ctrex_set_roi",
+    "ctrex_set_roi", "ctrex_conv3d_bias_grad", "ctrex_unet_workspace", "ctrex_unet_forward",
 )
 
 PROJ_TRILINEAR, PROJ_JOSEPH = 0, 1
@@ -109,6 +109,9 @@ def load_library(path: str = LIB_PATH):
         "ctrex_probe_gather_rate": ([vp, ctypes.POINTER(d)], i),
         "ctrex_probe_l2_read_bandwidth": ([vp, ctypes.POINTER(d)], i),
         "ctrex_set_dyrect": ([vp, vp, vp], i),
+        "ctrex_conv3d_bias_grad": ([vp, vp, vp, vp, vp, ctypes.c_longlong, i, vp], i),
+        "ctrex_unet_workspace": ([i, i, i, i, i], ctypes.c_longlong),
+        "ctrex_unet_forward": ([vp, vp, ctypes.POINTER(vp), ctypes.POINTER(vp), vp, vp, i, i, i, i, i, vp, vp, vp], i),
     }
     for name, (args, res) in sig.items():
         fn = getattr(lib, name)
@@ -537,6 +540,52 @@ def conv3d_wgrad(x, dy, dw=None):
     if rc != OK:
         raise CtrexError(rc, "ctrex_conv3d_wgrad failed")
     return dw
+
+
+def conv3d_bias_grad(dy, y=None):
+    """(g, db) of a layer's activation and bias for the output gradient dy
+    (bf16, channels last): g = dy * (y > 0) with the layer's output y (its
+    ReLU's), dy itself without; db [channels] float32 = g summed over the
+    voxels.  None if the layer's channel count is not one the kernel takes."""
+    c = dy.shape[-1]
+    if c % 8 or (c // 8) & (c // 8 - 1) or c // 8 > 256 or dy.numel() == 0 or dy.data_ptr() % 16:
+        return None
+    if y is not None and (y.shape != dy.shape or y.dtype != dy.dtype or not y.is_contiguous() or y.data_ptr() % 16):
+        return None
+    lib = load_library()
+    g = dy if y is None else torch.empty_like(dy)
+    db = torch.empty(c, dtype=torch.float32, device=dy.device)
+    scratch = torch.empty((1216, c), dtype=torch.float32, device=dy.device)
+    stream = torch.cuda.current_stream(dy.device).cuda_stream
+    with torch.cuda.device(dy.device):
+        rc = lib.ctrex_conv3d_bias_grad(_ptr(dy), _ptr(y), None if y is None else _ptr(g), _ptr(db), _ptr(scratch),
+                                        dy.numel() // c, c, ctypes.c_void_p(stream))
+    if rc != OK:
+        raise CtrexError(rc, f"ctrex_conv3d_bias_grad failed for dy {tuple(dy.shape)}")
+    return g, db
+
+
+def unet_forward(x, weights, bias, head_w, head_b):
+    """The warm-start network's forward pass in one call (see
+    ``ctrex_unet_forward``): x float32 [N, D, H, W]; weights and bias: the 14
+    layers' float32 parameters.  None for a size that the call does not take."""
+    lib = load_library()
+    nb, d, h, w = x.shape
+    base = head_w.numel()
+    n = lib.ctrex_unet_workspace(nb, d, h, w, base)
+    if n < 0:
+        return None
+    ws = torch.empty(n, dtype=torch.uint8, device=x.device)
+    y = torch.empty_like(x)
+    arr = ctypes.c_void_p * len(weights)
+    stream = torch.cuda.current_stream(x.device).cuda_stream
+    with torch.cuda.device(x.device):
+        rc = lib.ctrex_unet_forward(_ptr(x), _ptr(y), arr(*[t.data_ptr() for t in weights]),
+                                    arr(*[t.data_ptr() for t in bias]), _ptr(head_w), _ptr(head_b), nb, d, h, w, base,
+                                    _ptr(ws), _ptr(_status(x.device)), ctypes.c_void_p(stream))
+    if rc != OK:
+        raise CtrexError(rc, f"ctrex_unet_forward failed for x {tuple(x.shape)}, base {base}")
+    return y
 
 
 def flip_weights(wt):

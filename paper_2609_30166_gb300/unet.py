@@ -36,14 +36,18 @@ class _Conv3(torch.autograd.Function):
     @staticmethod
     def backward(actx, dy):
         x, wb, y = actx.saved_tensors
-        dy = dy.to(torch.bfloat16)
-        if actx.relu:
-            dy = dy * (y > 0).to(dy.dtype)
-        dy = dy.contiguous()
+        dy = dy.to(torch.bfloat16).contiguous()
+        # ReLU mask and bias gradient in one pass
+        both = ctrex.conv3d_bias_grad(dy, y if actx.relu else None) if actx.needs_input_grad[2] else None
+        if both is not None:
+            dy, db = both
+        else:
+            if actx.relu:
+                dy = (dy * (y > 0).to(dy.dtype)).contiguous()
+            db = dy.float().sum(dim=(0, 1, 2, 3)) if actx.needs_input_grad[2] else None
         dx = ctrex.conv3d(dy, ctrex.flip_weights(wb), None, relu=False, out_dtype=torch.bfloat16) \
             if actx.needs_input_grad[0] else None
         dw = ctrex.conv3d_wgrad(x, dy) if actx.needs_input_grad[1] else None
-        db = dy.float().sum(dim=(0, 1, 2, 3)) if actx.needs_input_grad[2] else None
         return dx, dw, db, None
 
 
@@ -104,8 +108,52 @@ class UNet3D(torch.nn.Module):
             x = c(x)
         return x
 
+    def _layers(self):
+        return [c for block in (self.e1, self.e2, self.e3, self.e4, self.d3, self.d2, self.d1) for c in block]
+
+    def _one_call(self, x):
+        """The layers' parameters if the whole pass can run as one native call:
+        plain inference of an unmodified network (no gradients, hooks, tracing
+        or tensor subclasses that would have to see the single operations)."""
+        layers = self._layers()
+        params = list(self.parameters())
+        tensors = [x] + params
+        if torch.is_grad_enabled() and any(t.requires_grad for t in tensors):
+            return None
+        if any(type(t) not in (torch.Tensor, torch.nn.Parameter) or t.dtype != torch.float32 or t.device != x.device
+               or not t.is_contiguous() for t in tensors) or x.device.type != "cuda" or x.dim() != 4:
+            return None
+        if len(layers) != 14 or len(params) != 30 or any(type(c) is not Conv3 or not c.relu for c in layers):
+            return None
+        m = torch.nn.modules.module
+        if m._global_forward_hooks or m._global_forward_pre_hooks or any(
+                s._forward_hooks or s._forward_pre_hooks for s in self.modules() if s is not self):
+            return None
+        if torch.is_autocast_enabled() or torch.jit.is_tracing() or torch.compiler.is_compiling():
+            return None
+        if torch._C._functorch.peek_interpreter_stack() is not None or torch._C._len_torch_dispatch_stack() \
+                or torch._C._len_torch_function_stack():
+            return None
+        nb, d, h, w = x.shape
+        c1 = self.head_w.numel()
+        want, cin = [], 16
+        for c in (c1, 2 * c1, 4 * c1, 8 * c1):
+            want += [(cin, c), (c, c)]
+            cin = c
+        for c in (4 * c1, 2 * c1, c1):
+            want += [(3 * c, c), (c, c)]
+        if any(tuple(c.w.shape) != (co, 27, ci) or c.b.numel() != co for c, (ci, co) in zip(layers, want)):
+            return None
+        if c1 % 8 or nb < 1 or min(d, h, w) < 8 or d % 8 or h % 8 or w % 8 or self.head_b.numel() != 1:
+            return None
+        return [c.w for c in layers], [c.b for c in layers]
+
     def forward(self, x):
         """x: [N, D, H, W] float32 (D, H, W divisible by 8); returns the same shape."""
+        native = self._one_call(x)
+        y = ctrex.unet_forward(x, *native, self.head_w, self.head_b) if native is not None else None
+        if y is not None:
+            return y
         xin = torch.nn.functional.pad(x.to(torch.bfloat16).unsqueeze(-1), (0, 15)).contiguous()
         s1 = self._block(self.e1, xin)
         s2 = self._block(self.e2, _pool(s1))

@@ -1,0 +1,72 @@
+"""The warm-start network's passes around its convolutions: the fused ReLU mask
+and bias gradient, and the one-call forward pass, against the single torch
+operations of the same layers.
+
+Tolerances: masked gradients and pooled or copied activations are exact; a bias
+gradient is a sum of n BF16 values held in FP32 on both sides, so it may differ
+from the FP64 sum by a few units of 2^-24 of sum |g|; the forward pass differs
+from the layer-by-layer one in the order of the head's 16-term FP32 sum only.
+"""
+
+import copy
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mods():
+    from paper_2609_30166_gb300 import _build, ctrex, unet
+
+    _build.build_library()
+    return ctrex, unet
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1, 8), (1, 3, 5, 7, 16), (2, 9, 8, 33, 32), (1, 4, 4, 4, 128),
+                                   (1, 1, 1, 2, 2048), (2, 64, 64, 40, 16)])
+@pytest.mark.parametrize("relu", [True, False])
+def test_bias_grad(mods, shape, relu):
+    ctrex, _ = mods
+    g = torch.Generator(device="cuda").manual_seed(1)
+    dy = torch.randn(shape, generator=g, device="cuda").to(torch.bfloat16)
+    y = torch.randn(shape, generator=g, device="cuda").relu().to(torch.bfloat16) if relu else None
+    want = dy * (y > 0).to(dy.dtype) if relu else dy
+    got, db = ctrex.conv3d_bias_grad(dy, y)
+    assert torch.equal(got, want)
+    ref = want.double().reshape(-1, shape[-1])
+    assert bool(((db.double() - ref.sum(0)).abs() <= 8 * 2.0 ** -24 * ref.abs().sum(0) + 1e-30).all())
+
+
+def test_bias_grad_of_other_channel_counts_is_left_alone(mods):
+    ctrex, _ = mods
+    for c in (4, 24, 40):
+        assert ctrex.conv3d_bias_grad(torch.zeros((1, 2, 2, 2, c), dtype=torch.bfloat16, device="cuda")) is None
+
+
+@pytest.mark.parametrize("shape,base", [((1, 8, 8, 8), 16), ((2, 16, 24, 8), 16), ((1, 40, 32, 48), 16),
+                                        ((1, 16, 16, 16), 8), ((1, 16, 8, 16), 32)])
+def test_one_call_forward(mods, shape, base):
+    ctrex, unet = mods
+    net = unet.UNet3D(base=base, seed=3)
+    with torch.no_grad():
+        net.head_w.normal_()
+        net.head_b.fill_(0.3)
+        for layer in net._layers():
+            layer.b.normal_(std=0.1)
+    net = net.cuda()
+    x = torch.rand(shape, generator=torch.Generator(device="cuda").manual_seed(2), device="cuda")
+    want = net(x).detach()  # parameters require gradients: layer by layer
+    with torch.no_grad():
+        assert net._one_call(x) is not None
+        got = net(x)
+        assert torch.allclose(got, want, rtol=0, atol=1e-5 * float((want - x).abs().max()) + 1e-6)
+        # whatever has to see single operations keeps the layers
+        hooked = copy.deepcopy(net)
+        seen = []
+        hooked.d1[1].register_forward_hook(lambda *a: seen.append(1))
+        assert torch.equal(hooked(x), want) and seen
+        assert net._one_call(x.transpose(1, 2)) is None and net._one_call(x.double()) is None
+    assert net._one_call(x) is None
+    ctrex.conv_status_check()
