@@ -4,13 +4,16 @@
 // layout (column.cuh).
 //
 // What bounds it: L1's data path (82 % busy, 12.6 wavefronts per 32 samples,
-// of which 8 are the taps themselves) and next to it issue (68 %, 39
-// instructions per sample); the texture kernel's bound was the gathers'
-// return path.  On 144 views of the 512^3 x 768^2 scan, FP32 / BF16 volume:
-// 146.5 / 75.8 ms with texture gathers, 59.6 / 65.8 ms here.  What each part
-// gave there (FP32): columns with floor by conversion-free adds 70.5 ms; the
-// CTA order below 62.6; fixed-point positions, the x neighbour at an
-// immediate offset and packed lerps 59.6.
+// of which 8 are the taps themselves; 16-byte loads of x pairs too need as
+// many) and next to it issue (68 %, 39 instructions per sample); the texture
+// kernel's bound was the gathers' return path.  On 144 views of the 512^3 x
+// 768^2 scan, FP32 / BF16 volume: 146.5 / 75.8 ms with texture gathers, 55.5 /
+// 55.5 ms here.  What each part gave there (FP32): columns with floor by
+// conversion-free adds 70.5 ms; the CTA order below 62.6; fixed-point
+// positions, the x neighbour at an immediate offset and packed lerps 59.4;
+// every sample in the fast loop, with only the weights of those beside the
+// interior on the side, 55.5 (64^3 x 90 views: 0.164 -> 0.141 ms, sparse 128^3:
+// 0.549 -> 0.490).
 #include "fwd_column.cuh"
 
 namespace ctrex {
@@ -26,26 +29,36 @@ __device__ __forceinline__ void col_pixel(const Grid &G, const ViewGPU *__restri
         Ray R;
         if (!setup_ray(G, views[view * G.n_sub + s], u, v, R)) continue;
         const int Km1 = R.K - 1;
-        int ka, kb;
-        interior_range(G, R, ka, kb);
+        // The border makes every sample's value the fast loop's; the row sum
+        // takes the weights of the few samples beside the interior range.
         ColRun run;
-        if (!run.start(vol, R.g0, R.sg, ka, kb - ka)) kb = ka;
-        // the few samples beside the interior range first: the long loop then
-        // holds little more than the ray itself in registers
+        int n = Km1;
         float a = 0.0f, ars = 0.0f, ws;
-        for (int k = ka > 0 ? 0 : kb; k < Km1; k = k + 1 == ka ? kb : k + 1) {
-            const float kf = (float)k;
-            a += col_edge(vol, fmaf(kf, R.sg[0], R.g0[0]), fmaf(kf, R.sg[1], R.g0[1]), fmaf(kf, R.sg[2], R.g0[2]), ws,
-                          taps);
-            ars += ws;
+        if (run.start_all(vol, R.g0, R.sg, n)) {
+            int ka, kb;
+            col_interior(vol, R.g0, R.sg, n, ka, kb);
+            for (int k = ka > 0 ? 0 : kb; k < Km1; k = k + 1 == ka ? kb : k + 1) {
+                const float kf = (float)k;
+                ars += col_weight(vol, fmaf(kf, R.sg[0], R.g0[0]), fmaf(kf, R.sg[1], R.g0[1]),
+                                  fmaf(kf, R.sg[2], R.g0[2]));
+            }
+            ars += (float)(kb - ka);
+        } else {
+            n = 0;
+            for (int k = 0; k < Km1; ++k) {
+                const float kf = (float)k;
+                a += col_edge(vol, fmaf(kf, R.sg[0], R.g0[0]), fmaf(kf, R.sg[1], R.g0[1]),
+                              fmaf(kf, R.sg[2], R.g0[2]), ws, taps);
+                ars += ws;
+            }
         }
-        ars = (ars + (float)(kb - ka)) * G.step_mm;
+        ars *= G.step_mm;
         if (R.w_last > 0.0f) {
             acc = fmaf(R.w_last, col_edge(vol, R.g_last[0], R.g_last[1], R.g_last[2], ws, taps), acc);
             ars = fmaf(R.w_last, ws, ars);
         }
         acc_rs += ars;
-        acc = fmaf(run.sum(vol, kb - ka, a), G.step_mm, acc);
+        acc = fmaf(run.sum(vol, n, a), G.step_mm, acc);
     }
     val = acc * G.inv_sub;
     rs = acc_rs * G.inv_sub;

@@ -31,26 +31,50 @@ __device__ __forceinline__ bool axis_inside(long long p, long long d, float sg, 
     return p >= (1ll << 32) && p <= top && q >= (1ll << 32) && q <= top;
 }
 
-// Samples ka .. kb - 1 of a ray, g0 + k sg, in 32.32 fixed point and padded
+// Samples ka, ka + 1, .. of a ray, g0 + k sg, in 32.32 fixed point and padded
 // index coordinates: a 64-bit add per axis and step, whose high word is the
 // cell and whose low word the fraction; exact, where a float position rounds
 // at the coordinate's magnitude.
 struct ColRun {
     long long px, py, pz, dx, dy, dz;
 
-    // False if a sample is not inside the grid (a ray with non-finite
-    // parameters): such a range is left to the clamped path.
-    __device__ __forceinline__ bool start(const ColVolume &V, const float g0[3], const float sg[3], int ka, int n)
+    __device__ __forceinline__ void set(const float g0[3], const float sg[3])
     {
         const float F = 4294967296.0f;
         dx = __float2ll_rn(sg[0] * F);
         dy = __float2ll_rn(sg[1] * F);
         dz = __float2ll_rn(sg[2] * F);
-        px = __float2ll_rn(g0[0] * F) + (1ll << 32) + ka * dx;
-        py = __float2ll_rn(g0[1] * F) + (1ll << 32) + ka * dy;
-        pz = __float2ll_rn(g0[2] * F) + (1ll << 32) + ka * dz;
+        px = __float2ll_rn(g0[0] * F) + (1ll << 32);
+        py = __float2ll_rn(g0[1] * F) + (1ll << 32);
+        pz = __float2ll_rn(g0[2] * F) + (1ll << 32);
+    }
+    // From sample ka on.  False if one of the n samples is not inside the
+    // grid (a ray with non-finite parameters): such a range is left to the
+    // clamped path.
+    __device__ __forceinline__ bool start(const ColVolume &V, const float g0[3], const float sg[3], int ka, int n)
+    {
+        set(g0, sg);
+        px += ka * dx;
+        py += ka * dy;
+        pz += ka * dz;
         return axis_inside(px, dx, sg[0], n, V.hx) && axis_inside(py, dy, sg[1], n, V.hy) &&
                axis_inside(pz, dz, sg[2], n, V.hz);
+    }
+    // From sample 0 on.  False if one of the n samples comes within a quarter
+    // of a voxel of the border's outer edge (the clip box ends half a voxel
+    // inside it, so this too takes a ray with non-finite parameters): the two
+    // end positions decide, in FP32, whose rounding is far smaller.
+    __device__ __forceinline__ bool start_all(const ColVolume &V, const float g0[3], const float sg[3], int n)
+    {
+        const float h[3] = {V.hx, V.hy, V.hz}, k = (float)(n - 1);
+        bool ok = n > 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float e = fmaf(k, sg[a], g0[a]);
+            ok = ok && fminf(g0[a], e) >= -0.75f && fmaxf(g0[a], e) <= h[a] + 0.75f && h[a] < 4.0e6f;
+        }
+        set(g0, sg);
+        return ok;
     }
     __device__ __forceinline__ unsigned index(const ColVolume &V) const
     {
@@ -90,6 +114,34 @@ __device__ __forceinline__ float col_edge(const ColVolume &V, float gx, float gy
     const float ax = gx - fx, ay = gy - fy, az = gz - fz;
     ws = col_inside(gx, ax, V.hx) * col_inside(gy, ay, V.hy) * col_inside(gz, az, V.hz);
     return col_interp(taps(V.index((int)fx + 1, (int)fy + 1, (int)fz + 1)), ax, ay, az);
+}
+
+// Samples ka .. kb - 1 of the n ones at g0 + k sg, all taps of which lie in the
+// grid by a margin of 0.01 voxel (or a few less: the weights of the others
+// come from col_weight, which is 1 there too).
+__device__ __forceinline__ void col_interior(const ColVolume &V, const float g0[3], const float sg[3], int n, int &ka,
+                                             int &kb)
+{
+    const float h[3] = {V.hx, V.hy, V.hz};
+    float lo = 0.0f, hi = (float)(n - 1);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float inv = __frcp_rn(sg[a]), l = 0.01f - g0[a], u = h[a] - 0.01f - g0[a];
+        const bool moves = fabsf(sg[a]) > 1.0e-9f;
+        const float t0 = moves ? l * inv : (l <= 0.0f ? -1.0f : 1.0e9f), t1 = moves ? u * inv : (u >= 0.0f ? 1.0e9f : -1.0f);
+        lo = fmaxf(lo, fminf(t0, t1));
+        hi = fminf(hi, fmaxf(t0, t1));
+        if (!(u >= l)) hi = -1.0f;  // one voxel along this axis
+    }
+    ka = min(max((int)ceilf(lo), 0), n);
+    kb = max(min((int)floorf(hi) + 1, n), ka);
+}
+
+// Summed weight of a sample's taps inside the grid, from its position alone.
+__device__ __forceinline__ float col_weight(const ColVolume &V, float gx, float gy, float gz)
+{
+    return __saturatef(fminf(gx + 1.0f, V.hx + 1.0f - gx)) * __saturatef(fminf(gy + 1.0f, V.hy + 1.0f - gy)) *
+           __saturatef(fminf(gz + 1.0f, V.hz + 1.0f - gz));
 }
 
 // The kernel's frame: the CTA's pixels, one integral per thread by `pixel`

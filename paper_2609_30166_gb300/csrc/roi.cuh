@@ -62,7 +62,9 @@ __device__ __forceinline__ void piece_interior(const float X[3], const float dg[
     for (int ax = 0; ax < 3; ++ax) {
         const float g0 = fmaf(a + 0.5f * h, dg[ax], X[ax]), sg = h * dg[ax];
         const float l = eps, u = (float)(n[ax] - 1) - eps;
-        if (sg != 0.0f) {
+        if (!(u >= l)) {  // one voxel along this axis: nothing is interior
+            hi = -1.0f;
+        } else if (sg != 0.0f) {
             const float inv = 1.0f / sg;
             const float t0 = (l - g0) * inv, t1 = (u - g0) * inv;
             lo = fmaxf(lo, fminf(t0, t1));
