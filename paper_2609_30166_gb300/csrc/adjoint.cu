@@ -5,30 +5,24 @@
 // The paper motivates geometry refinement and learned components (Sec. 5)
 // but prints no such operator; both are the transpose / derivative of its
 // Sec. 4.1 projector with the Sec. 2.2.2 / 3.1 warp.
+#include "column.cuh"
 #include "ray.cuh"
 
-// Motion gradient CTA: CTREX_MGRAD_WARPS warps, each on an 8 x 4 pixel
-// patch (the CTA covers 8 * warps detector columns x 4 rows), with
-// CTREX_MGRAD_MIN_BLOCKS resident CTAs per SM (two warps and six CTAs cap
-// the registers at 168; 5 or 4 CTAs with more registers, or 4-warp CTAs,
-// were no faster).  The spline's y and z loops are unrolled
-// (CTREX_MGRAD_UNROLL_Z): 616 -> 564 ms on the motion workload, with 4
-// bytes of spills.  Few warps per CTA shorten the wait of warps with short
-// rays for the CTA's final reduction.
-#ifndef CTREX_MGRAD_WARPS
-#define CTREX_MGRAD_WARPS 2
-#endif
-#ifndef CTREX_MGRAD_MIN_BLOCKS
-#define CTREX_MGRAD_MIN_BLOCKS (12 / CTREX_MGRAD_WARPS)
-#endif
-#ifndef CTREX_MGRAD_UNROLL_Z
-#define CTREX_MGRAD_UNROLL_Z 1
-#endif
+#include <type_traits>
 
 namespace ctrex {
 
 constexpr int ADJ_TX = 32, ADJ_TY = 4;
-constexpr int MG_WARPS = CTREX_MGRAD_WARPS, MG_THREADS = 32 * MG_WARPS;
+// Motion gradient CTA: four warps on 8 x 4 pixel patches side by side, which
+// share the spline table and the CTA's partial sums; three CTAs per SM (168
+// registers), by runs and sample by sample (45 views of the 256^3 motion
+// workload: 40.4 and 94.7 ms; two warps, six CTAs: 50.5 and 106 ms).
+constexpr int MG_WARPS = 4, MG_THREADS = 32 * MG_WARPS, MG_MIN_BLOCKS = 3;
+// Samples per spline cell from which the gradient goes by runs.  60 views at
+// 64^3 / 80^3 / 96^3 / 128^3 (26 / 32 / 38 / 51 samples), by samples: 4.6 /
+// 7.4 / 10.9 / 21.9 ms, by runs: 4.8 / 6.7 / 8.7 / 14.1 ms; pose only: 1.37 /
+// 2.40 / 3.79 / 8.14 and 1.80 / 2.73 / 3.82 / 6.89 ms.
+constexpr float MG_RUN_MIN = 30.0f, MG_RUN_MIN_POSE = 40.0f;
 constexpr int NCOEF = 8 * 8 * 8 * 3;
 
 // ---------------------------------------------------------------------------
@@ -299,16 +293,9 @@ __device__ __forceinline__ void spline_value_jacobian(const float4 *c, const flo
     float2 U = two(0.f), X = two(0.f), Y = two(0.f), Z = two(0.f);
     float uz = 0.f, xz = 0.f, yz = 0.f, zz = 0.f;
     const float2 fx = two(f[0]);
-    // a rolled z loop (CTREX_MGRAD_UNROLL_Z 0) picks its weights by selects,
-    // which keeps the arrays in registers
-#if CTREX_MGRAD_UNROLL_Z
 #pragma unroll
-#else
-#pragma unroll 1
-#endif
     for (int k = 0; k < 4; ++k) {
-        const float wk = k == 0 ? wz[0] : (k == 1 ? wz[1] : (k == 2 ? wz[2] : wz[3]));
-        const float ek = k == 0 ? ez[0] : (k == 1 ? ez[1] : (k == 2 ? ez[2] : ez[3]));
+        const float wk = wz[k], ek = ez[k];
         float2 v = two(0.f), dx = two(0.f), dy = two(0.f);
         float vz = 0.f, dxz = 0.f, dyz = 0.f;
 #pragma unroll
@@ -487,18 +474,58 @@ __device__ __forceinline__ void coef_step(CoefAcc &A, double *s_g64, int cell, c
     }
 }
 
-template <typename TV>
-__global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
+// The volume's trilinear gradient at centred index coordinates yc (zero
+// outside the grid), from row-major memory or from a column store.
+template <typename TV> struct RowVolume {
+    const TV *p;
+    __device__ __forceinline__ void gradient(const Grid &G, const float c[3], const float yc[3], float g[3]) const
+    {
+        trilinear_grad_c(p, G.nx, G.ny, G.nz, c, yc, g);
+    }
+};
+struct ColumnVolume {
+    ColVolume V;
+    __device__ __forceinline__ void gradient(const Grid &, const float c[3], const float yc[3], float g[3]) const
+    {
+        const float fx = floorf(yc[0]), fy = floorf(yc[1]), fz = floorf(yc[2]);
+        const ColTaps t = col_load(V, V.index((int)fx + (int)c[0] + 1, (int)fy + (int)c[1] + 1, (int)fz + (int)c[2] + 1));
+        const float2 ax = two(yc[0] - fx), ay = two(yc[1] - fy);
+        const float az = yc[2] - fz;
+        // x differences and values of both rows, then of both z neighbours
+        const float2 d0 = __ffma2_rn(t.q00, two(-1.0f), t.q10), d1 = __ffma2_rn(t.q01, two(-1.0f), t.q11);
+        const float2 v0 = __ffma2_rn(ax, d0, t.q00), v1 = __ffma2_rn(ax, d1, t.q01);
+        const float2 gx = lerp2(d0, d1, ay), gy = __ffma2_rn(v0, two(-1.0f), v1), v = __ffma2_rn(ay, gy, v0);
+        g[0] = fmaf(az, gx.y - gx.x, gx.x);
+        g[1] = fmaf(az, gy.y - gy.x, gy.x);
+        g[2] = v.y - v.x;
+    }
+};
+
+// Per ray, the samples of each run in one spline cell are reduced to 10: the
+// coefficient gradient sums v(t) times polynomials of degree 9 over the run's
+// samples, and so do the pose sums (J^T v times a linear position), so the
+// Chebyshev moments C_j = sum v(t) T_j(t) of the samples' v = dL/dy determine
+// them, and the run's samples may be replaced by the 10 nodes with
+//   V_n = 1/10 (C_0 + 2 sum_{j > 0} T_j(tau_n) C_j).
+// Only the displacement (by its Chebyshev form), the volume's gradient and
+// the moments are left per sample; the spline's Jacobian and the tensor-core
+// step run per node.  45 views of the 256^3 motion workload: sample by sample
+// with the volume row-major 104.3 ms (spline loads and the tensor-core step's
+// shuffles), from the columns 94.7, by runs 40.4 (pose only 60.3, 42.6, 25.1).
+// RUNS: as above; without, sample by sample (short runs, MG_RUN_MIN).
+template <typename Volume, bool RUNS>
+__global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
     motion_grad_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
-                       const float4 *table, const int *__restrict__ view_idx,
-                       const TV *__restrict__ vol, const float *__restrict__ gproj,
-                       double *__restrict__ grad_M, double *__restrict__ grad_b,
+                       const float4 *table, const int *__restrict__ view_idx, const Volume vol,
+                       const float *__restrict__ gproj, double *__restrict__ grad_M, double *__restrict__ grad_b,
                        double *__restrict__ grad_coef, unsigned *devcheck)
 {
     __shared__ float4 s_spline[SPLINE_TABLE];
     __shared__ double s_g64[NCOEF];       // the CTA's coefficient-gradient partials
     __shared__ double s_red[12][MG_WARPS];
     __shared__ float4 s_piece[4];
+    __shared__ float s_pose[12][MG_THREADS];
+    extern __shared__ float s_V[][MG_THREADS];  // RUNS: the nodes' dL/dy of each thread's run, 3 CHEB_N
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const int lane = tid & 31;
     const int k = blockIdx.y;
@@ -507,8 +534,8 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
         if (tid == 0) atomicOr(devcheck, (unsigned)DEVCHECK_OOB);
         return;  // uniform over the CTA
     }
-    const MotionGPU mo = motion[view];
-    const bool spline = table != nullptr && mo.s != 0.0f;
+    const float mos = motion[view].s;
+    const bool spline = table != nullptr && mos != 0.0f;
     const bool want_coef = spline && grad_coef != nullptr;
     if (spline) load_spline(s_spline, table, tid, MG_THREADS);
     if (want_coef)
@@ -523,7 +550,10 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
 #pragma unroll
         for (int e = 0; e < 4; ++e) CA.acc[h][e] = 0.0f;
     CA.cell = -1;
-    float G1[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gb[3] = {0.f, 0.f, 0.f};
+    // this thread's 12 pose sums (9 of dL/dM, 3 of dL/db): in shared memory,
+    // for want of registers
+#pragma unroll
+    for (int q = 0; q < 12; ++q) s_pose[q][tid] = 0.0f;
     int iu, iv;
     tile_pixel<true>(blockIdx.x * 8 * MG_WARPS, blockIdx.z * 4, iu, iv);
     const bool pix_ok = iu < G.nu && iv < G.nv;
@@ -532,88 +562,178 @@ __global__ void __launch_bounds__(MG_THREADS, CTREX_MGRAD_MIN_BLOCKS)
         Ray R;  // sample positions relative to the grid centre
         const bool hit = pix_ok && setup_ray(G, views[view * G.n_sub + s], (float)(pix_ok ? iu : 0),
                                              (float)(pix_ok ? iv : 0), R, cen);
-        // the warp-collective coefficient step needs every lane: lanes without
-        // work run the loop with zero weight up to the warp's longest ray
-        const int K = hit ? R.K : 0;
-        int Kmax = K;
+        const int K = hit && y != 0.0f ? R.K : 0;
+        // displacement by the pose at sample index kappa: d = D g + bc, linear
+        float d0[3], ds[3];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) Kmax = max(Kmax, __shfl_xor_sync(0xffffffffu, Kmax, off));
-        for (int kk = 0; kk < Kmax; ++kk) {
-            float gc[3] = {0.f, 0.f, 0.f};
-            float sc = 0.0f;
-            if (hit && kk < K - 1) {
-                gc[0] = fmaf((float)kk, R.sg[0], R.g0[0]);
-                gc[1] = fmaf((float)kk, R.sg[1], R.g0[1]);
-                gc[2] = fmaf((float)kk, R.sg[2], R.g0[2]);
-                sc = y * G.step_mm;
-            } else if (hit && kk == K - 1) {
-                gc[0] = R.g_last[0];
-                gc[1] = R.g_last[1];
-                gc[2] = R.g_last[2];
-                sc = R.w_last > 0.0f ? y * R.w_last : 0.0f;
-            }
-            const bool act = hit && kk < K && sc != 0.0f;
-            // warp: d = D gc + bc (+ s u), g' - c = gc + d
-            float d[3];
+        for (int r = 0; r < 3; ++r) {
+            const float *D = motion[view].D + 3 * r;
+            d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], motion[view].bc[r])));
+            ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
+        }
+        const float kl = last_kappa(G, R);
+        // dL/dy of one sample with spline displacement u (voxels)
+        auto sample = [&](int kk, const float u[3], float g[3]) {
+            const bool last = kk == K - 1;
+            const float kap = last ? kl : (float)kk, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
+            float yc[3];
 #pragma unroll
             for (int r = 0; r < 3; ++r)
-                d[r] = fmaf(mo.D[3 * r], gc[0], fmaf(mo.D[3 * r + 1], gc[1], fmaf(mo.D[3 * r + 2], gc[2], mo.bc[r])));
-            int i0[3] = {0, 0, 0};
-            float f[3] = {0.f, 0.f, 0.f};
-            float u[3] = {0.f, 0.f, 0.f}, Jx[3] = {0.f, 0.f, 0.f}, Jy[3] = {0.f, 0.f, 0.f},
-                  Jz[3] = {0.f, 0.f, 0.f};
-            if (spline) {
-                bool on[3];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) spline_coord(gc[a] + d[a] + cen[a], G.spl_scale[a], i0[a], f[a], on[a]);
-                spline_value_jacobian(spline_cell(s_spline, i0), f, u, Jx, Jy, Jz);
-                const float sx = on[0] ? G.spl_scale[0] : 0.f, sy = on[1] ? G.spl_scale[1] : 0.f,
-                            sz = on[2] ? G.spl_scale[2] : 0.f;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    Jx[c] *= sx;
-                    Jy[c] *= sy;
-                    Jz[c] *= sz;
-                }
-            }
-            const float yc[3] = {gc[0] + fmaf(mo.s, u[0], d[0]), gc[1] + fmaf(mo.s, u[1], d[1]),
-                                 gc[2] + fmaf(mo.s, u[2], d[2])};
-            float gy[3] = {0.f, 0.f, 0.f};
-            if (act && yc[0] >= -1.0f - cen[0] && yc[0] < (float)G.nx - cen[0] && yc[1] >= -1.0f - cen[1] &&
+                yc[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(mos, u[r], fmaf(kap, ds[r], d0[r]));
+            g[0] = g[1] = g[2] = 0.0f;
+            if (w > 0.0f && yc[0] >= -1.0f - cen[0] && yc[0] < (float)G.nx - cen[0] && yc[1] >= -1.0f - cen[1] &&
                 yc[1] < (float)G.ny - cen[1] && yc[2] >= -1.0f - cen[2] && yc[2] < (float)G.nz - cen[2])
-                trilinear_grad_c(vol, G.nx, G.ny, G.nz, cen, yc, gy);
+                vol.gradient(G, cen, yc, g);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) gy[c] *= sc;  // dL/dy (index units)
-            // dL/dg' = dL/dy (I + s J), J[c][a] = du_c / dg'_a
-            const float gg[3] = {gy[0] + mo.s * (gy[0] * Jx[0] + gy[1] * Jx[1] + gy[2] * Jx[2]),
-                                 gy[1] + mo.s * (gy[0] * Jy[0] + gy[1] * Jy[1] + gy[2] * Jy[2]),
-                                 gy[2] + mo.s * (gy[0] * Jz[0] + gy[1] * Jz[1] + gy[2] * Jz[2])};
+            for (int c = 0; c < 3; ++c) g[c] *= y * w;
+        };
+        auto pose = [&](float kap, const float gg[3]) {
+            float gc[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) gc[r] = fmaf(kap, R.sg[r], R.g0[r]);
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
-                gb[r] += gg[r];
-                G1[3 * r + 0] = fmaf(gg[r], gc[0], G1[3 * r + 0]);
-                G1[3 * r + 1] = fmaf(gg[r], gc[1], G1[3 * r + 1]);
-                G1[3 * r + 2] = fmaf(gg[r], gc[2], G1[3 * r + 2]);
+                s_pose[9 + r][tid] += gg[r];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) s_pose[3 * r + c][tid] = fmaf(gg[r], gc[c], s_pose[3 * r + c][tid]);
             }
-            if (want_coef) {  // CTA-uniform
-                const float v[3] = {mo.s * gy[0], mo.s * gy[1], mo.s * gy[2]};
-                const bool live = act && (v[0] != 0.0f || v[1] != 0.0f || v[2] != 0.0f);
-                const int cell = (i0[2] * 8 + i0[1]) * 8 + i0[0];
-                coef_step(CA, s_g64, cell, f, v, live, s_piece);
+        };
+        // pose sums of dL/dy = gy at kappa: dL/dg' = dL/dy (I + s J), J[c][a] =
+        // du_c / dg'_a
+        auto point = [&](float kap, const float gy[3], const bool on[3], const float Jx[3], const float Jy[3],
+                         const float Jz[3]) {
+            const float sx = on[0] ? mos * G.spl_scale[0] : 0.f, sy = on[1] ? mos * G.spl_scale[1] : 0.f,
+                        sz = on[2] ? mos * G.spl_scale[2] : 0.f;
+            const float gg[3] = {fmaf(sx, gy[0] * Jx[0] + gy[1] * Jx[1] + gy[2] * Jx[2], gy[0]),
+                                 fmaf(sy, gy[0] * Jy[0] + gy[1] * Jy[1] + gy[2] * Jy[2], gy[1]),
+                                 fmaf(sz, gy[0] * Jz[0] + gy[1] * Jz[1] + gy[2] * Jz[2], gy[2])};
+            pose(kap, gg);
+        };
+        if (!spline) {  // CTA-uniform: the pose alone
+            const float u[3] = {0.f, 0.f, 0.f};
+            for (int kk = 0; kk < K; ++kk) {
+                float g[3];
+                sample(kk, u, g);
+                pose(kk == K - 1 ? kl : (float)kk, g);
+            }
+            continue;
+        }
+        SplineLine L;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            L.x0[a] = fmaf(R.g0[a] + d0[a] + cen[a] + 0.5f, G.spl_scale[a], 1.0f);
+            L.xs[a] = (R.sg[a] + ds[a]) * G.spl_scale[a];
+        }
+        if constexpr (!RUNS) {
+            // the coefficient step is collective: lanes without work run the
+            // loop with zero weight up to the warp's longest ray
+            int Kmax = K;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) Kmax = max(Kmax, __shfl_xor_sync(0xffffffffu, Kmax, off));
+            for (int kk = 0; kk < Kmax; ++kk) {
+                const float kap = kk == K - 1 ? kl : (float)kk;
+                int i0[3];
+                float f[3], u[3], Jx[3], Jy[3], Jz[3], gy[3] = {0.f, 0.f, 0.f};
+                bool on[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) spline_cell_of(fmaf(kap, L.xs[a], L.x0[a]), i0[a], f[a], on[a]);
+                spline_value_jacobian(spline_cell(s_spline, i0), f, u, Jx, Jy, Jz);
+                if (kk < K) {
+                    sample(kk, u, gy);
+                    point(kap, gy, on, Jx, Jy, Jz);
+                }
+                if (want_coef) {  // CTA-uniform
+                    const float v[3] = {mos * gy[0], mos * gy[1], mos * gy[2]};
+                    coef_step(CA, s_g64, (i0[2] * 8 + i0[1]) * 8 + i0[0], f, v,
+                              kk < K && (v[0] != 0.0f || v[1] != 0.0f || v[2] != 0.0f), s_piece);
+                }
+            }
+            continue;
+        }
+        // run after run, the warp together (the coefficient step is collective)
+        int k = 0;
+        while (__any_sync(0xffffffffu, k < K)) {
+            SplineRun run;
+            const bool act = k < K;
+            const int end = run.find(L, act ? k : 0, act ? K : 1, kl);
+            if (act) {
+                float2 Cxy[CHEB_N], axy[CHEB_N];
+                float Cz[CHEB_N], az[CHEB_N];
+                run.fit(s_spline, L, axy, az);
+#pragma unroll
+                for (int j = 0; j < CHEB_N; ++j) {
+                    Cxy[j] = two(0.0f);
+                    Cz[j] = 0.0f;
+                }
+                const float ih = 1.0f / run.half;
+                for (int kk = k; kk < end; ++kk) {
+                    float T[CHEB_N], u[3], g[3];
+                    cheb_values(((kk == K - 1 ? kl : (float)kk) - run.mid) * ih, T);
+                    SplineRun::value(axy, az, T, u);
+                    sample(kk, u, g);
+                    const float2 gxy = make_float2(g[0], g[1]);
+#pragma unroll
+                    for (int j = 0; j < CHEB_N; ++j) {
+                        Cxy[j] = __ffma2_rn(two(T[j]), gxy, Cxy[j]);
+                        Cz[j] = fmaf(T[j], g[2], Cz[j]);
+                    }
+                }
+                k = end;
+                // the nodes' V: even moments count alike at +-tau, odd ones
+                // with opposite signs
+#pragma unroll
+                for (int n = 0; n < CHEB_N / 2; ++n) {
+                    float2 e = two(0.0f), o = two(0.0f);
+                    float ez = 0.0f, oz = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < CHEB_N; ++j) {
+                        const float w = cheb_cos20(j * (2 * n + 1)) * (j == 0 ? 0.1f : 0.2f);
+                        if (j & 1) {
+                            o = __ffma2_rn(two(w), Cxy[j], o);
+                            oz = fmaf(w, Cz[j], oz);
+                        } else {
+                            e = __ffma2_rn(two(w), Cxy[j], e);
+                            ez = fmaf(w, Cz[j], ez);
+                        }
+                    }
+                    s_V[3 * n][tid] = e.x + o.x;
+                    s_V[3 * n + 1][tid] = e.y + o.y;
+                    s_V[3 * n + 2][tid] = ez + oz;
+                    s_V[3 * (CHEB_N - 1 - n)][tid] = e.x - o.x;
+                    s_V[3 * (CHEB_N - 1 - n) + 1][tid] = e.y - o.y;
+                    s_V[3 * (CHEB_N - 1 - n) + 2][tid] = ez - oz;
+                }
+            }
+            const int cell = (run.cell[2] * 8 + run.cell[1]) * 8 + run.cell[0];
+            const float4 *cc = spline_cell(s_spline, run.cell);
+#pragma unroll 1
+            for (int n = 0; n < CHEB_N; ++n) {
+                const int m = n < CHEB_N / 2 ? n : CHEB_N - 1 - n;
+                const float sign = n < CHEB_N / 2 ? 1.0f : -1.0f;
+                float gy[3] = {0.f, 0.f, 0.f};
+                if (act) {
+                    gy[0] = s_V[3 * n][tid];
+                    gy[1] = s_V[3 * n + 1][tid];
+                    gy[2] = s_V[3 * n + 2][tid];
+                }
+                const float kap = fmaf(sign * c_cheb.t[m][1], run.half, run.mid);
+                float f[3], u[3], Jx[3], Jy[3], Jz[3];
+                run.fraction(L, kap, f);
+                spline_value_jacobian(cc, f, u, Jx, Jy, Jz);
+                if (act) point(kap, gy, run.on, Jx, Jy, Jz);
+                if (want_coef) {  // CTA-uniform
+                    const float v[3] = {mos * gy[0], mos * gy[1], mos * gy[2]};
+                    coef_step(CA, s_g64, cell, f, v, act && (v[0] != 0.0f || v[1] != 0.0f || v[2] != 0.0f), s_piece);
+                }
             }
         }
     }
     if (want_coef) coef_flush(CA, s_g64, lane);
     // CTA reduction of the 12 pose-gradient entries: FP32 warp sums, FP64 over
     // the warps and across CTAs
-    float vals[12];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) vals[q] = G1[q];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) vals[9 + q] = gb[q];
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-        float v = vals[q];
+        float v = s_pose[q][tid];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
         if (lane == 0) s_red[q][tid >> 5] = (double)v;
@@ -641,15 +761,25 @@ cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *gra
     const Grid &G = *a.grid;
     const dim3 grid((G.nu + 8 * MG_WARPS - 1) / (8 * MG_WARPS), a.n_idx, (G.nv + 3) / 4);
     const dim3 block(32, MG_WARPS);
-    if (a.vol_dtype == CTREX_F32)
-        motion_grad_kernel<float><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx,
-                                                               (const float *)a.vol, gproj, grad_M, grad_b,
-                                                               grad_coef_idx, a.devcheck);
+    cudaError_t err = cudaSuccess;
+    const bool runs = spline_runs(G, a.spline && grad_coef_idx ? MG_RUN_MIN : MG_RUN_MIN_POSE);
+    auto launch = [&](const auto &vol) {
+        typedef std::decay_t<decltype(vol)> V;
+        auto *kernel = runs ? motion_grad_kernel<V, true> : motion_grad_kernel<V, false>;
+        const int nodes = runs ? 3 * CHEB_N * MG_THREADS * (int)sizeof(float) : 0;  // 53 KB with the static part
+        if (runs) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nodes);
+        if (err != cudaSuccess) return;
+        kernel<<<grid, block, nodes, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx, vol, gproj, grad_M,
+                                                 grad_b, grad_coef_idx, a.devcheck);
+        err = cudaGetLastError();
+    };
+    if (a.column)
+        launch(ColumnVolume{col_view(*a.column)});
+    else if (a.vol_dtype == CTREX_F32)
+        launch(RowVolume<float>{static_cast<const float *>(a.vol)});
     else
-        motion_grad_kernel<__nv_bfloat16><<<grid, block, 0, a.stream>>>(
-            G, a.views, a.motion, a.spline, a.view_idx, (const __nv_bfloat16 *)a.vol, gproj, grad_M, grad_b,
-            grad_coef_idx, a.devcheck);
-    return cudaGetLastError();
+        launch(RowVolume<__nv_bfloat16>{static_cast<const __nv_bfloat16 *>(a.vol)});
+    return err;
 }
 
 // ---------------------------------------------------------------------------

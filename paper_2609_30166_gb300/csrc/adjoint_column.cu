@@ -7,7 +7,8 @@
 //
 // 45 views of the 256^3 motion geometry, scattered in place / here: 16.6 /
 // 5.7 ms without motion (bound there by the reductions' path through L1), 39.0
-// / 23.5 ms with motion (bound by the spline: issue 65 %, L1 75 %).
+// / 23.5 ms with motion (bound by the spline: issue 65 %, L1 75 %), 15.2 ms
+// with the deformation run by run (ray.cuh).
 #include "fwd_column.cuh"
 
 namespace ctrex {
@@ -19,6 +20,10 @@ constexpr int ADJ_LV = 32, ADJ_LV_PATCH = 8;
 // CTAs per SM: the spline needs 168 registers to keep out of local memory (4
 // CTAs at 128: 30.3 ms, 2: 26.6).
 constexpr int ADJ_MIN_BLOCKS = 8, ADJ_MIN_BLOCKS_MOTION = 3;
+// Samples per spline cell from which the deformation goes by runs.  60 views
+// at 64^3 / 80^3 / 96^3 (26 / 32 / 38 samples), by pairs: 0.76 / 1.36 / 2.14
+// ms, by runs: 0.82 / 1.30 / 1.90 ms.
+constexpr float ADJ_RUN_MIN = 30.0f;
 
 // The scatter volume: padded index (i, j, k) (one border element on every
 // side, never added back) at ((k >> 5) chunks + j rows + i) * 32 + (k & 31).
@@ -81,7 +86,8 @@ struct AdjFoot {
 
 // LV: lanes of a warp along v; the other 32 / LV and the four warps of the
 // CTA run along u.
-template <bool MOTION, int LV>
+// RUNS (motion): the deformation run by run (SplineRun), else pair by pair.
+template <bool MOTION, int LV, bool RUNS>
 __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_BLOCKS)
     adjoint_column_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                           const float4 *spline, const int *__restrict__ view_idx, const float *__restrict__ proj,
@@ -113,19 +119,59 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
     grid_centre(G, cen);
     const float n[3] = {(float)G.nx, (float)G.ny, (float)G.nz};
     AdjFoot F;
-    // val at centred index coordinates q, if a tap lies inside the grid
-    auto point = [&](const float *q, float val) {
-        if (!(val != 0.0f && q[0] >= -1.0f - cen[0] && q[0] < n[0] - cen[0] && q[1] >= -1.0f - cen[1] &&
-              q[1] < n[1] - cen[1] && q[2] >= -1.0f - cen[2] && q[2] < n[2] - cen[2]))
-            return;
+    // val at index coordinates base (whole numbers) + q, if a tap lies inside the grid
+    auto point = [&](const float *base, const float *q, float val) {
         const float fx = floorf(q[0]), fy = floorf(q[1]), fz = floorf(q[2]);
-        F.add(V, (int)fx + (int)cen[0] + 1, (int)fy + (int)cen[1] + 1, (int)fz + (int)cen[2] + 1, q[0] - fx, q[1] - fy,
-              q[2] - fz, val);
+        const float x = fx + base[0], y = fy + base[1], z = fz + base[2];
+        if (!(val != 0.0f && x >= -1.0f && x < n[0] && y >= -1.0f && y < n[1] && z >= -1.0f && z < n[2])) return;
+        F.add(V, (int)x + 1, (int)y + 1, (int)z + 1, q[0] - fx, q[1] - fy, q[2] - fz, val);
     };
     for (int s = 0; s < G.n_sub; ++s) {
         Ray R;  // sample positions relative to the grid centre
         if (!setup_ray(G, views[view * G.n_sub + s], (float)iu, (float)iv, R, cen)) continue;
-        if (MOTION) {
+        if (RUNS) {
+            // displacement by the pose at sample index kappa, linear
+            float d0[3], ds[3];
+            SplineLine L;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float *D = mo.D + 3 * r;
+                d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], mo.bc[r])));
+                ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
+                L.x0[r] = fmaf(R.g0[r] + d0[r] + cen[r] + 0.5f, G.spl_scale[r], 1.0f);
+                L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
+            }
+            const float kl = last_kappa(G, R);
+            for (int k = 0; k < R.K;) {
+                SplineRun run;
+                const int end = run.find(L, k, R.K, kl);
+                float2 axy[CHEB_N];
+                float az[CHEB_N];
+                run.fit(spline, L, axy, az);
+                const float ih = 1.0f / run.half;
+                // positions from the run's middle, less its whole number (which
+                // keeps their rounding below that of the pairs' positions)
+                float m[3], base[3];
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const float whole = rintf(fmaf(run.mid, R.sg[r], R.g0[r]));
+                    m[r] = fmaf(run.mid, R.sg[r], R.g0[r] - whole);
+                    base[r] = whole + cen[r];
+                }
+#pragma unroll 1
+                for (; k < end; ++k) {
+                    const bool last = k == R.K - 1;
+                    const float kap = last ? kl : (float)k, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
+                    float T[CHEB_N], u[3], q[3];
+                    cheb_values((kap - run.mid) * ih, T);
+                    SplineRun::value(axy, az, T, u);
+#pragma unroll
+                    for (int r = 0; r < 3; ++r)
+                        q[r] = fmaf(kap - run.mid, R.sg[r], m[r]) + fmaf(mo.s, u[r], fmaf(kap, ds[r], d0[r]));
+                    point(base, q, y * w);
+                }
+            }
+        } else if (MOTION) {
             for (int kk = 0; kk < R.K; kk += 2) {
                 float g[2][3], w[2], gc[2][3];
                 sample_pair(G, R, kk, g, w);
@@ -133,7 +179,7 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
 #pragma unroll 1
                 for (int m = 0; m < 2; ++m) {
                     const float q[3] = {m ? gc[1][0] : gc[0][0], m ? gc[1][1] : gc[0][1], m ? gc[1][2] : gc[0][2]};
-                    point(q, y * (m ? w[1] : w[0]));
+                    point(cen, q, y * (m ? w[1] : w[0]));
                 }
             }
         } else {
@@ -141,9 +187,9 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
             for (int kk = 0; kk < R.K - 1; ++kk) {
                 const float kf = (float)kk;
                 const float q[3] = {fmaf(kf, R.sg[0], R.g0[0]), fmaf(kf, R.sg[1], R.g0[1]), fmaf(kf, R.sg[2], R.g0[2])};
-                point(q, ys);
+                point(cen, q, ys);
             }
-            if (R.w_last > 0.0f) point(R.g_last, y * R.w_last);
+            if (R.w_last > 0.0f) point(cen, R.g_last, y * R.w_last);
         }
     }
     if (F.live) F.flush(V);
@@ -185,7 +231,8 @@ size_t adjoint_column_elems(const Grid &G)
     return n < (1ull << 32) && (G.nz + 31) / 32 <= 65535 ? n : 0;
 }
 
-template <bool MOTION, int LV> static cudaError_t adj_launch(const FwdArgs &a, const float *proj, const AdjVolume &V)
+template <bool MOTION, int LV, bool RUNS = false>
+static cudaError_t adj_launch(const FwdArgs &a, const float *proj, const AdjVolume &V)
 {
     const Grid &G = *a.grid;
     constexpr int TU = 4 * (32 / LV);  // columns per CTA
@@ -193,7 +240,7 @@ template <bool MOTION, int LV> static cudaError_t adj_launch(const FwdArgs &a, c
     const int n_strips = (tiles + per - 1) / per;
     const dim3 grid(per, a.n_idx, n_strips * ((G.nv + LV - 1) / LV));
     if (grid.z > 65535) return cudaErrorNotSupported;
-    adjoint_column_kernel<MOTION, LV><<<grid, 128, 0, a.stream>>>(
+    adjoint_column_kernel<MOTION, LV, RUNS><<<grid, 128, 0, a.stream>>>(
         G, a.views, MOTION ? a.motion : nullptr, MOTION ? a.spline : nullptr, a.view_idx, proj, V, a.devcheck, n_strips);
     return cudaGetLastError();
 }
@@ -206,7 +253,8 @@ cudaError_t launch_adjoint_column(const FwdArgs &a, bool along_z, const float *p
     cudaError_t e = cudaMemsetAsync(scratch, 0, n * sizeof(float), a.stream);
     if (e != cudaSuccess) return e;
     if (a.motion)
-        e = adj_launch<true, ADJ_LV_PATCH>(a, proj, V);
+        e = a.spline && spline_runs(G, ADJ_RUN_MIN) ? adj_launch<true, ADJ_LV_PATCH, true>(a, proj, V)
+                                       : adj_launch<true, ADJ_LV_PATCH>(a, proj, V);
     else
         e = along_z ? adj_launch<false, ADJ_LV>(a, proj, V) : adj_launch<false, ADJ_LV_PATCH>(a, proj, V);
     if (e != cudaSuccess) return e;

@@ -1189,8 +1189,13 @@ int ctrex_motion_grad(ctrex_ctx *c, const void *vol, int vdt, const float *gproj
     CT_CUDA(c, cudaMemsetAsync(c->d_gM, 0, sizeof(double) * 9 * (size_t)V, c->stream));
     CT_CUDA(c, cudaMemsetAsync(c->d_gb, 0, sizeof(double) * 3 * (size_t)V, c->stream));
     CT_CUDA(c, cudaMemsetAsync(c->d_gcoef, 0, sizeof(double) * 1536, c->stream));
-    cudaError_t ce = launch_motion_grad(fwd_args(c, vol, vdt, view_idx, n_idx), gproj, c->d_gM, c->d_gb,
-                                        grad_coef ? c->d_gcoef : nullptr);
+    FwdArgs a = fwd_args(c, vol, vdt, view_idx, n_idx);
+    // the volume from its column store if that can be had, row-major otherwise
+    if (col_ensure(c->vol_col, c->grid.nx, c->grid.ny, c->grid.nz, c->stream) == cudaSuccess) {
+        CT_CUDA(c, col_upload(c->vol_col, vol, vdt, c->stream));
+        a.column = &c->vol_col;
+    }
+    cudaError_t ce = launch_motion_grad(a, gproj, c->d_gM, c->d_gb, grad_coef ? c->d_gcoef : nullptr);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "motion_grad launch");
     ce = launch_motion_grad_finish(c->theta_valid ? c->d_theta : nullptr, c->d_dRdw, c->d_gM, c->d_gb, c->d_gcoef, V,
                                    c->grid, c->vox, c->origin, grad_theta, grad_coef, c->stream);

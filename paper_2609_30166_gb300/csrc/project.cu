@@ -20,6 +20,10 @@
 
 namespace ctrex {
 
+// Samples per spline cell from which the deformation goes by runs (ray.cuh).
+// 60 views at 80^3 / 96^3 / 112^3 / 128^3 (32 / 38 / 45 / 51 samples), by
+// pairs: 1.30 / 2.07 / 3.14 / 4.52 ms, by runs: 1.49 / 2.20 / 3.15 / 4.31 ms.
+constexpr float FWD_RUN_MIN = 45.0f;
 
 template <typename TV>
 __device__ __forceinline__ float LinearSampler<TV>::operator()(float gx, float gy, float gz, float &wsum) const
@@ -34,10 +38,62 @@ __device__ __forceinline__ float LinearSampler<TV>::interior(float gx, float gy,
     return trilinear(vol, nx, ny, nz, gx, gy, gz, ws);
 }
 
+// One ray's integral and row sum under motion, run by run (SplineRun).
+template <typename Sampler>
+__device__ __forceinline__ void motion_runs_integral(const Grid &G, const ViewGPU &V, const MotionGPU &mo,
+                                                     const float4 *spline, const Sampler &vol, float u, float v,
+                                                     float &a, float &ars)
+{
+    a = 0.0f;
+    ars = 0.0f;
+    float cen[3];
+    grid_centre(G, cen);
+    Ray R;
+    if (!setup_ray(G, V, u, v, R, cen)) return;
+    // displacement by the pose at sample index kappa, linear; positions
+    // relative to the grid centre (R's), see MotionGPU
+    float d0[3], ds[3];
+    SplineLine L;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const float *D = mo.D + 3 * r;
+        d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], mo.bc[r])));
+        ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
+        L.x0[r] = fmaf(R.g0[r] + d0[r] + cen[r] + 0.5f, G.spl_scale[r], 1.0f);
+        L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
+    }
+    const float kl = last_kappa(G, R);
+    for (int k = 0; k < R.K;) {
+        SplineRun run;
+        const int end = run.find(L, k, R.K, kl);
+        float2 axy[CHEB_N];
+        float az[CHEB_N];
+        run.fit(spline, L, axy, az);
+        const float ih = 1.0f / run.half;
+        float b = 0.0f, brs = 0.0f;  // the run's sums
+#pragma unroll 1
+        for (; k < end; ++k) {
+            const bool last = k == R.K - 1;
+            const float kap = last ? kl : (float)k, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
+            float T[CHEB_N], u[3], q[3], ws;
+            cheb_values((kap - run.mid) * ih, T);
+            SplineRun::value(axy, az, T, u);
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+                q[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(mo.s, u[r], fmaf(kap, ds[r], d0[r])) + cen[r];
+            b = fmaf(w, vol(q[0], q[1], q[2], ws), b);
+            brs = fmaf(w, ws, brs);
+        }
+        a += b;
+        ars += brs;
+    }
+}
+
 // Integral of one pixel (mean over its sub-angle rays): value and row sum.
 // On the cylindrical domain the ray is clipped to the bounding cylinder and
 // every sample is mapped to (r, phi, z) by the sampler; the rest is shared.
-template <typename Sampler, bool MOTION>
+// RUNS (motion): the deformation run by run (SplineRun), else pair by pair.
+template <typename Sampler, bool MOTION, bool RUNS>
 __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__restrict__ views,
                                                const MotionGPU &mo, const float4 *spline,
                                                const Sampler &vol, int view, float u,
@@ -56,6 +112,13 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
         if constexpr (Sampler::JOSEPH) {
             float a, ars;
             joseph_integral(G, vol, V, u, v, a, ars);
+            acc += a;
+            acc_rs += ars;
+            continue;
+        }
+        if constexpr (RUNS) {
+            float a, ars;
+            motion_runs_integral(G, V, mo, spline, vol, u, v, a, ars);
             acc += a;
             acc_rs += ars;
             continue;
@@ -112,7 +175,7 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
     rs = acc_rs * G.inv_sub;
 }
 
-template <typename Sampler, typename TP, int MODE, bool MOTION>
+template <typename Sampler, typename TP, int MODE, bool MOTION, bool RUNS = false>
 __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ views,
                                          const MotionGPU *__restrict__ motion, const float4 *spline,
                                          const Sampler &vol_in, const int *__restrict__ view_idx,
@@ -148,7 +211,7 @@ __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ vie
     const bool in_pix = iu < G.nu && iv < G.nv;
     const bool inside = ok && in_pix;
     float val = 0.0f, rs = 0.0f;
-    if (inside) pixel_integral<Sampler, MOTION>(G, views, mo, spline, vol, view, (float)iu, (float)iv, val, rs);
+    if (inside) pixel_integral<Sampler, MOTION, RUNS>(G, views, mo, spline, vol, view, (float)iu, (float)iv, val, rs);
     fwd_epilogue<TP, MODE>(G, k, view, ok, in_pix, iu, iv, val, rs, out, rowsum_out, p, partials, p_by_view,
                            s_red);
 }
@@ -162,6 +225,21 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY)
 {
     fwd_body<Sampler, TP, MODE, MOTION>(G, views, motion, spline, vol_in, view_idx, out, rowsum_out, p, partials,
                                         devcheck, p_by_view);
+}
+
+// The motion projector with the deformation run by run (ray.cuh): 45 views of
+// the 256^3 motion workload 18.4 ms (by pairs 23.8), and half the error of the
+// pairs against 64 bits (positions relative to the grid centre, a sum per
+// run).  Four CTAs per SM (128^3, 60 views: 4.31 ms; 3: 4.55, 5: 4.74).
+template <typename Sampler, typename TP, int MODE>
+__global__ void __launch_bounds__(FWD_TX *FWD_TY, 4)
+    fwd_run_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
+                   const float4 *spline, const Sampler vol_in, const int *__restrict__ view_idx,
+                   TP *__restrict__ out, float *__restrict__ rowsum_out, const TP *__restrict__ p,
+                   float *__restrict__ partials, unsigned *devcheck, int p_by_view)
+{
+    fwd_body<Sampler, TP, MODE, true, true>(G, views, motion, spline, vol_in, view_idx, out, rowsum_out, p, partials,
+                                            devcheck, p_by_view);
 }
 
 // Projectors whose sampler declares MIN_BLOCKS > 0 (the event model and
@@ -295,6 +373,11 @@ static cudaError_t fwd_launch(const FwdArgs &a, const Sampler &smp, TP *out, flo
     const Grid &G = *a.grid;
     const dim3 grid = fwd_grid(G, a.n_idx), block(FWD_TX, FWD_TY);
     if constexpr (!Sampler::CYLINDER && !Sampler::JOSEPH && !Sampler::ROI && !Sampler::DYRECT) {
+        if (a.motion && a.spline && spline_runs(G, FWD_RUN_MIN)) {
+            fwd_run_kernel<Sampler, TP, MODE><<<grid, block, 0, a.stream>>>(
+                G, a.views, a.motion, a.spline, smp, a.view_idx, out, rowsum, p, partials, a.devcheck, a.p_by_view);
+            return cudaGetLastError();
+        }
         if (a.motion) {
             fwd_kernel<Sampler, TP, MODE, true><<<grid, block, 0, a.stream>>>(
                 G, a.views, a.motion, a.spline, smp, a.view_idx, out, rowsum, p, partials, a.devcheck,

@@ -172,6 +172,7 @@ static_assert(SPLINE_TABLE == 8 * SPL_PLANE, "spline table size");
 
 __device__ __forceinline__ void load_spline(float4 *s, const float4 *__restrict__ table, int tid, int nthreads)
 {
+#pragma unroll 5
     for (int i = tid; i < SPLINE_TABLE; i += nthreads) s[i] = __ldg(table + i);
 }
 
@@ -205,17 +206,21 @@ __host__ __device__ __forceinline__ float4 bspline_piece(int m)
                                       : make_float4(0.0f, 0.0f, 0.0f, 1.0f / 6.0f)));
 }
 
-// Spline coordinate of index coordinate gp along one axis (clamped to [1,
-// 6]): cell i in [0, 4] and fraction f in [0, 1]; `active` is false where the
-// clamp holds.
-__device__ __forceinline__ void spline_coord(float gp, float scale, int &i, float &f, bool &active)
+// Cell i in [0, 4] and fraction f in [0, 1] of a spline coordinate (clamped
+// to [1, 6]); `active` is false where the clamp holds.
+__device__ __forceinline__ void spline_cell_of(float xi, int &i, float &f, bool &active)
 {
-    float xi = fmaf(gp + 0.5f, scale, 1.0f);
     active = (xi > 1.0f) && (xi < 6.0f);
     xi = fminf(fmaxf(xi, 1.0f), 6.0f);
     const float fl = fminf(floorf(xi), 5.0f);
     i = (int)fl - 1;
     f = xi - fl;
+}
+
+// The same of index coordinate gp along one axis.
+__device__ __forceinline__ void spline_coord(float gp, float scale, int &i, float &f, bool &active)
+{
+    spline_cell_of(fmaf(gp + 0.5f, scale, 1.0f), i, f, active);
 }
 
 __device__ __forceinline__ const float4 *spline_cell(const float4 *table, const int i[3])
@@ -224,7 +229,9 @@ __device__ __forceinline__ const float4 *spline_cell(const float4 *table, const 
 }
 
 // Displacement u (voxels) of N samples in the cell at `c`, fractions f.
-template <int N>
+// ROLLED: the z loop stays a loop (its weights picked by selects), where the
+// registers of the unrolled one's loads are not to be had.
+template <int N, bool ROLLED = false>
 __device__ __forceinline__ void spline_value(const float4 *c, const float (&f)[N][3], float (&u)[N][3])
 {
     float wy[N][4], wz[N][4];
@@ -236,6 +243,11 @@ __device__ __forceinline__ void spline_value(const float4 *c, const float (&f)[N
     float2 uxy[N];
     float uz[N];
 #pragma unroll
+    for (int n = 0; n < N; ++n) {
+        uxy[n] = two(0.0f);
+        uz[n] = 0.0f;
+    }
+#pragma unroll(ROLLED ? 1 : 4)
     for (int k = 0; k < 4; ++k) {
         float2 yxy[N];
         float yz[N];
@@ -256,9 +268,9 @@ __device__ __forceinline__ void spline_value(const float4 *c, const float (&f)[N
         }
 #pragma unroll
         for (int n = 0; n < N; ++n) {
-            const float2 w = make_float2(wz[n][k], wz[n][k]);
-            uxy[n] = k == 0 ? __fmul2_rn(w, yxy[n]) : __ffma2_rn(w, yxy[n], uxy[n]);
-            uz[n] = k == 0 ? w.x * yz[n] : fmaf(w.x, yz[n], uz[n]);
+            const float w = k == 0 ? wz[n][0] : (k == 1 ? wz[n][1] : (k == 2 ? wz[n][2] : wz[n][3]));
+            uxy[n] = __ffma2_rn(two(w), yxy[n], uxy[n]);
+            uz[n] = fmaf(w, yz[n], uz[n]);
         }
     }
 #pragma unroll
@@ -268,6 +280,148 @@ __device__ __forceinline__ void spline_value(const float4 *c, const float (&f)[N
         u[n][2] = uz[n];
     }
 }
+
+// Runs of a ray inside one spline cell.  The position is linear in the sample
+// index, so within a cell the displacement is a polynomial of degree 9 in it
+// (three cubics' products), and its values at 10 Chebyshev nodes determine it
+// exactly: u(t) = sum_j a_j T_j(t), t in [-1, 1] over the run, with
+//   a_j = (2 - [j = 0]) / 10 sum_n u(tau_n) T_j(tau_n),  tau_n = cos((2 n + 1) pi / 20).
+// A cell is 1/5 of the volume wide: at 128^3 a run has about 51 samples, so
+// 10 passes over the cell's 64 coefficients replace 26 (of two samples each).
+// (The Chebyshev form keeps the coefficients' rounding at that of u; powers of
+// t would not.)
+constexpr int CHEB_N = 10;
+__host__ __device__ constexpr float cheb_cos20(int m)  // cos(m pi / 20)
+{
+    const float c[11] = {1.0f,          0.98768834059513773f, 0.95105651629515357f, 0.89100652418836786f,
+                         0.80901699437494742f, 0.70710678118654752f, 0.58778525229247313f, 0.45399049973954675f,
+                         0.30901699437494742f, 0.15643446504023086f, 0.0f};
+    m %= 40;
+    if (m > 20) m = 40 - m;
+    return m <= 10 ? c[m] : -c[20 - m];
+}
+struct ChebTable {
+    float t[CHEB_N / 2][CHEB_N];  // T_j(tau_n) of the nodes tau_n > 0; T_j(-tau) = (-1)^j T_j(tau)
+    constexpr ChebTable() : t()
+    {
+        for (int n = 0; n < CHEB_N / 2; ++n)
+            for (int j = 0; j < CHEB_N; ++j) t[n][j] = cheb_cos20(j * (2 * n + 1));
+    }
+};
+static __constant__ ChebTable c_cheb = ChebTable();
+
+// T_0 .. T_9 at t.
+__device__ __forceinline__ void cheb_values(float t, float T[CHEB_N])
+{
+    const float t2 = t + t;
+    T[0] = 1.0f;
+    T[1] = t;
+#pragma unroll
+    for (int j = 2; j < CHEB_N; ++j) T[j] = fmaf(t2, T[j - 1], -T[j - 2]);
+}
+
+// Whether a cell holds at least `least` samples along its shortest axis, so
+// that the runs pay (51 at 128^3, 38 at 96^3, 26 at 64^3).
+inline bool spline_runs(const Grid &G, float least)
+{
+    float cell = 1.0f / 0.0f;
+    for (int a = 0; a < 3; ++a) cell = fminf(cell, G.vox[a] / (G.spl_scale[a] * G.step_mm));
+    return cell >= least;
+}
+
+// A ray's spline coordinates, linear in the sample index kappa.
+struct SplineLine {
+    float x0[3], xs[3];
+};
+
+// The run of samples k, k + 1, .. in the cell of sample k.
+struct SplineRun {
+    int cell[3];
+    float base[3];  // fraction along axis a: kappa xs + base where it moves, base (0 or 1) where the clamp holds
+    bool on[3];
+    float mid, half;  // t = (kappa - mid) / half
+
+    // kappa of the ray's samples: their index, except kl for the last one.
+    // Returns the first sample after the run.
+    __device__ __forceinline__ int find(const SplineLine &L, int k, int K, float kl)
+    {
+        const float kap = k == K - 1 ? kl : (float)k;
+        int end = K;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float xi = fmaf(kap, L.xs[a], L.x0[a]);
+            float face;  // the spline coordinate at which the ray leaves
+            bool leaves = L.xs[a] != 0.0f;
+            on[a] = xi > 1.0f && xi < 6.0f;
+            if (on[a]) {
+                const float fl = floorf(xi);
+                cell[a] = (int)fl - 1;
+                base[a] = L.x0[a] - fl;
+                face = L.xs[a] > 0.0f ? fl + 1.0f : fl;
+            } else {
+                const bool above = xi >= 6.0f;
+                cell[a] = above ? 4 : 0;
+                base[a] = above ? 1.0f : 0.0f;
+                face = above ? 6.0f : 1.0f;
+                leaves = above ? L.xs[a] < 0.0f : L.xs[a] > 0.0f;
+            }
+            const float e = (face - L.x0[a]) / L.xs[a];
+            if (leaves && e < (float)K) end = min(end, max((int)ceilf(e), k + 1));
+        }
+        const float last = end == K ? kl : (float)(end - 1);
+        mid = 0.5f * (kap + last);
+        half = fmaxf(0.5f * (last - kap), 0.5f);
+        return end;
+    }
+    __device__ __forceinline__ void fraction(const SplineLine &L, float kap, float f[3]) const
+    {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f[a] = on[a] ? fmaf(kap, L.xs[a], base[a]) : base[a];
+    }
+    // Chebyshev coefficients of the displacement (voxels): x and y packed, z.
+    __device__ __forceinline__ void fit(const float4 *table, const SplineLine &L, float2 axy[CHEB_N],
+                                        float az[CHEB_N]) const
+    {
+        const float4 *c = spline_cell(table, cell);
+#pragma unroll
+        for (int j = 0; j < CHEB_N; ++j) {
+            axy[j] = two(0.0f);
+            az[j] = 0.0f;
+        }
+#pragma unroll 1
+        for (int n = 0; n < CHEB_N / 2; ++n) {
+            const float tau = half * c_cheb.t[n][1];
+            float f[2][3], u[2][3];
+            fraction(L, mid + tau, f[0]);
+            fraction(L, mid - tau, f[1]);
+            spline_value<2, true>(c, f, u);
+            // even j take the sum of the two nodes' values, odd j the difference
+            const float2 e = make_float2(u[0][0] + u[1][0], u[0][1] + u[1][1]);
+            const float2 o = make_float2(u[0][0] - u[1][0], u[0][1] - u[1][1]);
+            const float ez = u[0][2] + u[1][2], oz = u[0][2] - u[1][2];
+#pragma unroll
+            for (int j = 0; j < CHEB_N; ++j) {
+                const float w = c_cheb.t[n][j] * (j == 0 ? 0.1f : 0.2f);
+                axy[j] = __ffma2_rn(two(w), j & 1 ? o : e, axy[j]);
+                az[j] = fmaf(w, j & 1 ? oz : ez, az[j]);
+            }
+        }
+    }
+    static __device__ __forceinline__ void value(const float2 axy[CHEB_N], const float az[CHEB_N],
+                                                 const float T[CHEB_N], float u[3])
+    {
+        float2 s = two(0.0f);  // the small terms first
+        float z = 0.0f;
+#pragma unroll
+        for (int j = CHEB_N - 1; j >= 0; --j) {
+            s = __ffma2_rn(two(T[j]), axy[j], s);
+            z = fmaf(T[j], az[j], z);
+        }
+        u[0] = s.x;
+        u[1] = s.y;
+        u[2] = z;
+    }
+};
 
 // Displacements of two samples at index coordinates g: one pass over the
 // first one's cell serves both, and a second sample beyond its face (a step
@@ -371,6 +525,13 @@ __device__ __forceinline__ void warp_pair(const Grid &G, const MotionGPU &m, con
     for (int n = 0; n < 2; ++n)
 #pragma unroll
         for (int r = 0; r < 3; ++r) y[n][r] = fmaf(m.s, u[n][r], gp[n][r]);
+}
+
+// The last sample of a ray sits at the middle of the clipped segment's rest:
+// its place in units of the sample index.
+__device__ __forceinline__ float last_kappa(const Grid &G, const Ray &R)
+{
+    return (float)(R.K - 1) + 0.5f * (R.w_last / G.step_mm - 1.0f);
 }
 
 // Samples kk and kk + 1 of a ray and their weights (mm): the last one is the

@@ -195,3 +195,60 @@ def test_adjoint_matches_oracle(n, det, views, sub, turn, motion):
         x = rng.uniform(0.2, 1.0, size=shape)
         assert rel_l2(_np(c.fwd_project(_t(x))), oracle.forward(pb, _np(_t(x)))[0]) <= TOL32
     c.close()
+
+
+# Motion by runs of samples in one spline cell: a step short enough for runs in
+# every operator, in the adjoint and the gradient only, and in the full gradient
+# but not in the pose's.  Poses that carry rays beyond the spline's domain (its
+# coordinate is clamped there), steps along a cell's faces, sub-angles.
+# Projector and adjoint: the contract.  Gradient: positions hold about 2e-6
+# voxels, so some 1e-5 of the samples lie on the other side of a voxel face,
+# where this volume's gradient turns by a few percent, in a sum that cancels to
+# about 1 % of its terms: 1e-4.
+@pytest.mark.parametrize("n,det,views,sub,turn,step,shift", [
+    ((30, 41, 35), (37, 22), 4, 1, 0.4, 0.1, 0.0),
+    ((33, 32, 30), (21, 33), 3, 2, 30.0, 0.08, 6.0),   # beyond the clamp on one side
+    ((30, 30, 50), (9, 40), 5, 1, 0.0, 0.17, -3.0),    # 35 samples a cell: not in the projector
+    ((5, 40, 40), (20, 12), 4, 1, 2.0, 0.02, 1.0),     # cells of one voxel
+    ((30, 30, 30), (31, 5), 3, 1, 0.0, 0.1, 0.0),
+])
+def test_motion_runs_match_oracle(n, det, views, sub, turn, step, shift):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    P = _matrices(views, sub, turn, det[0], det[1], 60.0, 200.0)
+    pitch = 30.0 / max(n)
+    vox, shape = (pitch, 0.95 * pitch, 1.05 * pitch), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(33)
+    theta = np.zeros((views, 15))
+    theta[:, :6] = rng.uniform(-0.03, 0.03, (views, 6))
+    theta[:, 3] += shift * pitch
+    theta[:, 6:] = np.eye(3).ravel() + rng.uniform(-0.01, 0.01, (views, 9))
+    coef, sv = rng.uniform(-1, 1, (8, 8, 8, 3)) * 0.05 * max(n) * pitch, np.linspace(0.2, 1.0, views)
+    theta, coef, sv = (_np(_t(a)) for a in (theta, coef, sv))  # as the GPU sees them
+    pb = oracle.Problem(P, shape, vox, org, det, step).with_motion(theta, coef, sv, margin=0.5)
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det, step_vox=step)
+    c.set_motion(_t(theta), _t(coef), _t(sv), 0.5)
+    axes = [(np.arange(m) + 1.0) * (m - np.arange(m)) / (m + 1.0) ** 2 for m in shape]
+    x = 64.0 * axes[0][:, None, None] * axes[1][:, None] * axes[2]
+    y = rng.uniform(0.5, 1.5, size=(views, det[1], det[0]))
+    y[:, ::3, 1::2] = 0.0  # rays without weight
+    x, y = _np(_t(x)), _np(_t(y))
+    rows = torch.empty((views, det[1], det[0]), device="cuda")
+    ref, rs = oracle.forward(pb, x)
+    assert rel_l2(_np(c.fwd_project(_t(x), rowsum=rows)), ref) <= TOL32
+    assert rel_l2(_np(rows), rs) <= TOL32
+    assert rel_l2(_np(c.adjoint_project(_t(y))), oracle.adjoint(pb, y)) <= TOL32
+    gt, gc = oracle.motion_grad(pb, x, y)
+    got_t, got_c = c.motion_grad(_t(x), _t(y))
+    assert rel_l2(_np(got_t), gt) <= 1e-4 and rel_l2(_np(got_c), gc) <= 1e-4
+    assert rel_l2(_np(c.motion_grad(_t(x), _t(y), want_coef=False)[0]), gt) <= 1e-4
+    vi = np.arange(views)[::-2].astype(np.int32).copy()
+    ref, _ = oracle.forward(pb, x, views=vi)
+    assert rel_l2(_np(c.fwd_project(_t(x), view_idx=vi)), ref) <= TOL32
+    gt, gc = oracle.motion_grad(pb, x, y[vi], views=vi)
+    got_t, got_c = c.motion_grad(_t(x), _t(y[vi]), view_idx=vi)
+    assert rel_l2(_np(got_t), gt) <= 1e-4 and rel_l2(_np(got_c), gc) <= 1e-4
+    c.close()
