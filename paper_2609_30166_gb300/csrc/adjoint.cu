@@ -489,15 +489,13 @@ struct ColumnVolume {
     {
         const float fx = floorf(yc[0]), fy = floorf(yc[1]), fz = floorf(yc[2]);
         const ColTaps t = col_load(V, V.index((int)fx + (int)c[0] + 1, (int)fy + (int)c[1] + 1, (int)fz + (int)c[2] + 1));
-        const float2 ax = two(yc[0] - fx), ay = two(yc[1] - fy);
-        const float az = yc[2] - fz;
-        // x differences and values of both rows, then of both z neighbours
-        const float2 d0 = __ffma2_rn(t.q00, two(-1.0f), t.q10), d1 = __ffma2_rn(t.q01, two(-1.0f), t.q11);
-        const float2 v0 = __ffma2_rn(ax, d0, t.q00), v1 = __ffma2_rn(ax, d1, t.q01);
-        const float2 gx = lerp2(d0, d1, ay), gy = __ffma2_rn(v0, two(-1.0f), v1), v = __ffma2_rn(ay, gy, v0);
-        g[0] = fmaf(az, gx.y - gx.x, gx.x);
-        g[1] = fmaf(az, gy.y - gy.x, gy.x);
-        g[2] = v.y - v.x;
+        const float ax = yc[0] - fx, ay = yc[1] - fy, az = yc[2] - fz;
+        const float a = col_value(t.q00, az), b = col_value(t.q10, az), d = col_value(t.q01, az),
+                    e = col_value(t.q11, az);
+        const float dx0 = b - a, dx1 = e - d;
+        g[0] = lerp(dx0, dx1, ay);
+        g[1] = fmaf(ax, dx1, d) - fmaf(ax, dx0, a);
+        g[2] = lerp(lerp(t.q00.y, t.q10.y, ax), lerp(t.q01.y, t.q11.y, ax), ay);
     }
 };
 

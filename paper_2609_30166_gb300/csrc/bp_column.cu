@@ -1,7 +1,7 @@
 // bp_column.cu -- the weighted backprojection of backproject.cu for scans
 // whose detector columns run along z: a warp takes 32 voxels of a z column,
 // whose projections run along one detector column, and the correction images
-// are in column layout (column.cuh), (value v, value v + 1) per element.
+// are in column layout (column.cuh).
 #include "column.cuh"
 #include "cylinder.cuh"
 
@@ -13,7 +13,7 @@ constexpr int BPC_WX = 8, BPC_WY = 1;  // z columns of a CTA (one per warp)
 constexpr int BPC_COLS = BPC_WX * BPC_WY;
 constexpr int BPC_THREADS = 32 * BPC_COLS;
 constexpr int BPC_CHUNK = 128;  // views staged at a time
-constexpr int BPC_MIN_BLOCKS = 5;  // 48 registers (4 and 6: 22.1 and 21.8 ms where 5 takes 19.2)
+constexpr int BPC_MIN_BLOCKS = 5;  // 48 registers (4 and 6: 21.1 and 21.8 ms where 5 takes 18.8)
 constexpr int BPC_SUBV_MIN_BLOCKS = 4;
 
 // The correction images [n][nu][nv] in column layout: pair (u, v) of image k,
@@ -65,8 +65,7 @@ __device__ __forceinline__ BpTaps bp_load(const ColImages &I, const float2 *img,
 }
 __device__ __forceinline__ float bp_interp(const BpTaps &t)
 {
-    const float2 c = lerp2(t.q0, t.q1, two(t.au));
-    return fmaf(t.av, c.y - c.x, c.x);
+    return lerp(col_value(t.q0, t.av), col_value(t.q1, t.av), t.au);
 }
 
 // One voxel-view term in general position, as bp_term in backproject.cu.
@@ -77,10 +76,13 @@ __device__ __forceinline__ void bp_edge(const ColImages &I, const float2 *img, f
     const float inv = col_recip(h3);
     const float u = h1 * inv, v = h2 * inv;
     if (!(u > win.x - 1.0f && u < win.y + 1.0f && v > win.z - 1.0f && v < win.w + 1.0f)) return;
-    const BpTaps t = bp_load(I, img, u, v);
-    const float2 q0 = t.q0, q1 = t.q1;
-    const float au = t.au, av = t.av;
-    const float fu = u - au, fv = v - av;
+    const float fu = floorf(u), fv = floorf(v), au = u - fu, av = v - fv;
+    // each value by itself: a difference would bring in one beyond the window
+    const unsigned bu = (unsigned)((int)fu + 1) << COL_LOG, bv = (unsigned)((int)fv + 1);
+    const float2 *r0 = img + ((bv >> COL_LOG) * I.sv + (bu + bv)),
+                 *r1 = img + (((bv + 1) >> COL_LOG) * I.sv + (bu + bv + 1));
+    const float2 q0 = make_float2(__ldg(&r0->x), __ldg(&r1->x)),
+                 q1 = make_float2(__ldg(&r0[1 << COL_LOG].x), __ldg(&r1[1 << COL_LOG].x));
     const float wu0 = fu >= win.x ? 1.0f - au : 0.0f, wu1 = fu + 1.0f <= win.y ? au : 0.0f;
     const float wv0 = fv >= win.z ? 1.0f - av : 0.0f, wv1 = fv + 1.0f <= win.w ? av : 0.0f;
     b += fmaf(wv0, fmaf(wu0, q0.x, wu1 * q1.x), wv1 * fmaf(wu0, q0.y, wu1 * q1.y));

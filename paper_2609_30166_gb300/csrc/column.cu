@@ -54,7 +54,7 @@ cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream,
 // along v two pairs to a thread (HBM-bound; with 32 x 32 tiles and single
 // pairs 90 images of 768^2 took 0.45 ms).  Pair j (padded) holds values j - 1
 // and j, zero outside the slice.
-template <typename T>
+template <typename T, bool PAIRS>
 __global__ void __launch_bounds__(256) col_upload_kernel(const T *__restrict__ src, float2 *__restrict__ dst, int nu,
                                                          int nv, size_t vs, size_t ss, size_t ds, unsigned chunk,
                                                          int tiles_u, int n)
@@ -74,32 +74,38 @@ __global__ void __launch_bounds__(256) col_upload_kernel(const T *__restrict__ s
         for (int i = 0; i < 4; ++i) {
             const int c = warp + 8 * i, r = 2 * lane;
             const unsigned j = j0 + r;
-            if (u0 + c < nu && (int)j <= nv)
+            if (u0 + c < nu && (int)j <= nv) {
+                const float a = tile[r][c], b = tile[r + 1][c], e = tile[r + 2][c];
                 *reinterpret_cast<float4 *>(dst + (size_t)k * ds + (size_t)(j >> COL_LOG) * chunk +
                                             ((size_t)(u0 + c + 1) << COL_LOG) + j) =
-                    make_float4(tile[r][c], tile[r + 1][c], tile[r + 1][c], tile[r + 2][c]);
+                    PAIRS ? make_float4(a, b, b, e) : make_float4(a, b - a, b, e - b);
+            }
         }
         __syncthreads();
     }
 }
 
 static cudaError_t upload(const void *src, int dtype, float2 *dst, int nu, int nv, size_t vs, size_t ss, size_t ds,
-                          unsigned chunk, int n, cudaStream_t stream)
+                          unsigned chunk, int n, cudaStream_t stream, bool pairs = false)
 {
     const int tu = (nu + 31) / 32;
     const dim3 grid(tu * ((nv + 1 + 63) / 64), n < 65535 ? n : 65535);
-    if (dtype == CTREX_BF16)
-        col_upload_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16 *>(src), dst, nu, nv, vs, ss, ds,
-                                                    chunk, tu, n);
-    else
-        col_upload_kernel<<<grid, 256, 0, stream>>>(static_cast<const float *>(src), dst, nu, nv, vs, ss, ds, chunk, tu,
-                                                    n);
+    auto go = [&](auto *kernel, auto *s) {
+        kernel<<<grid, 256, 0, stream>>>(s, dst, nu, nv, vs, ss, ds, chunk, tu, n);
+    };
+    if (dtype == CTREX_BF16) {
+        typedef __nv_bfloat16 T;
+        go(pairs ? col_upload_kernel<T, true> : col_upload_kernel<T, false>, static_cast<const T *>(src));
+    } else {
+        go(pairs ? col_upload_kernel<float, true> : col_upload_kernel<float, false>, static_cast<const float *>(src));
+    }
     return cudaGetLastError();
 }
 
-cudaError_t col_upload(const ColStore &s, const void *src, int dtype, cudaStream_t stream)
+cudaError_t col_upload(const ColStore &s, const void *src, int dtype, cudaStream_t stream, bool pairs)
 {
-    cudaError_t e = upload(src, dtype, s.buf + s.sy, s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, s.ny, stream);
+    cudaError_t e =
+        upload(src, dtype, s.buf + s.sy, s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, s.ny, stream, pairs);
     if (e == cudaSuccess && s.wrap)
         e = upload(src, dtype, s.buf + (size_t)s.sy * (s.ny + 1), s.nx, s.nz, (size_t)s.nx * s.ny, s.nx, s.sy, s.sz, 1,
                    stream);

@@ -320,14 +320,14 @@ int prepare_columns(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     if (e == cudaSuccess && c->roi) e = col_ensure(c->col1, rx, ry, rz, c->stream);
     if (e == cudaSuccess && c->dyr && !c->tau_col_set) {
         e = col_ensure(c->tau_col, nx, ny, nz, c->stream);
-        if (e == cudaSuccess) e = col_upload(c->tau_col, c->d_tau, CTREX_F32, c->stream);
+        if (e == cudaSuccess) e = col_upload(c->tau_col, c->d_tau, CTREX_F32, c->stream, true);
         c->tau_col_set = e == cudaSuccess;
     }
     if (e == cudaErrorInvalidValue) return CTREX_OK;
-    if (e == cudaSuccess) e = col_upload(c->vol_col, vol, vdt, c->stream);
+    if (e == cudaSuccess) e = col_upload(c->vol_col, vol, vdt, c->stream, c->dyr);
     if (e == cudaSuccess && (c->dyr || c->roi))
         e = col_upload(c->col1, static_cast<const char *>(vol) + grid_voxels(c->grid) * dtype_size(vdt), vdt,
-                       c->stream);
+                       c->stream, c->dyr);
     if (e != cudaSuccess) return cuda_fail(c, e, "volume column layout");
     a.column = &c->vol_col;
     a.column1 = &c->col1;

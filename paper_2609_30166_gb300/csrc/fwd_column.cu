@@ -3,17 +3,19 @@
 // pixel, a warp on 32 pixels of a detector column, the volume in column
 // layout (column.cuh).
 //
-// What bounds it: L1's data path (82 % busy, 12.6 wavefronts per 32 samples,
-// of which 8 are the taps themselves; 16-byte loads of x pairs too need as
-// many) and next to it issue (68 %, 39 instructions per sample); the texture
+// What bounds it: L1's data path (12.6 wavefronts per 32 samples, of which 8
+// are the taps themselves; 16-byte loads of x pairs too need as many; 89 % busy
+// at 512^3, 51 to 68 % at 64^3 and 128^3) and next to it the issue ports (68 %
+// busy at every size, and held longer by packed multiply-adds); the texture
 // kernel's bound was the gathers' return path.  On 144 views of the 512^3 x
-// 768^2 scan, FP32 / BF16 volume: 146.5 / 75.8 ms with texture gathers, 55.5 /
-// 55.5 ms here.  What each part gave there (FP32): columns with floor by
+// 768^2 scan, FP32 / BF16 volume: 146.5 / 75.8 ms with texture gathers, 52.5 /
+// 52.5 ms here.  What each part gave there (FP32): columns with floor by
 // conversion-free adds 70.5 ms; the CTA order below 62.6; fixed-point
 // positions, the x neighbour at an immediate offset and packed lerps 59.4;
 // every sample in the fast loop, with only the weights of those beside the
 // interior on the side, 55.5 (64^3 x 90 views: 0.164 -> 0.141 ms, sparse 128^3:
-// 0.549 -> 0.490).
+// 0.549 -> 0.490); differences instead of second values in the store 52.5 (0.137,
+// 0.466).
 #include "fwd_column.cuh"
 
 namespace ctrex {
@@ -24,7 +26,7 @@ __device__ __forceinline__ void col_pixel(const Grid &G, const ViewGPU *__restri
                                           float u, float v, float &val, float &rs)
 {
     float acc = 0.0f, acc_rs = 0.0f;
-    auto taps = [&](unsigned i) { return col_load(vol, i); };
+    auto taps = [&](unsigned i, unsigned j, unsigned k) { return col_load(vol, vol.index(i, j, k)); };
     for (int s = 0; s < G.n_sub; ++s) {
         Ray R;
         if (!setup_ray(G, views[view * G.n_sub + s], u, v, R)) continue;
@@ -65,7 +67,7 @@ __device__ __forceinline__ void col_pixel(const Grid &G, const ViewGPU *__restri
 }
 
 template <typename TP, int MODE>
-__global__ void __launch_bounds__(32 * COL_TU, 9)  // 56 registers (8 CTAs: 60.9 ms, 9: 59.4, 10: 59.7)
+__global__ void __launch_bounds__(32 * COL_TU, 9)  // 56 registers (8 CTAs: 53.8 ms, 9: 52.5, 10: 53.9)
     fwd_column_kernel(Grid G, const ViewGPU *__restrict__ views, const ColVolume vol,
                       const int *__restrict__ view_idx, TP *__restrict__ out, float *__restrict__ rowsum_out,
                       const TP *__restrict__ p, float *__restrict__ partials, unsigned *devcheck, int p_by_view,

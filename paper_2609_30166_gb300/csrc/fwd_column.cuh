@@ -13,7 +13,7 @@ namespace ctrex {
 // A CTA is 32 pixels along v by 4 columns (8 columns: the same within 1 %).
 constexpr int COL_TU = 4;
 constexpr int COL_MIN_BLOCKS = 8;  // CTAs per SM of the models' kernels (7 and 10: within 3 %)
-constexpr int COL_UNROLL = 2;  // samples per step of the interior loop (1: +3 %, 4: +11 %, out of registers)
+constexpr int COL_UNROLL = 2;  // samples per step of the interior loop (1: +3 %; 3, 4: +1 %)
 // CTAs are ordered in strips of 32 tiles (128 columns), then views, then
 // strips and bands of 32 rows: the views resident together then cross one
 // strip of the volume instead of all of it, and what they share stays in L2
@@ -80,7 +80,7 @@ struct ColRun {
     {
         return V.index((unsigned)(px >> 32), (unsigned)(py >> 32), (unsigned)(pz >> 32));
     }
-    __device__ __forceinline__ float interp(const ColTaps &t) const
+    template <typename Taps> __device__ __forceinline__ float interp(const Taps &t) const
     {
         return col_interp(t, fixed_fraction((unsigned)px), fixed_fraction((unsigned)py), fixed_fraction((unsigned)pz));
     }
@@ -91,11 +91,11 @@ struct ColRun {
         pz += dz;
     }
     // a plus the next n samples
-    __device__ __forceinline__ float sum(const ColVolume &V, int n, float a)
+    template <bool PAIRS = false> __device__ __forceinline__ float sum(const ColVolume &V, int n, float a)
     {
 #pragma unroll COL_UNROLL
         for (int left = n; left > 0; --left) {
-            a += interp(col_load(V, index(V)));
+            a += PAIRS ? interp(col_load_pairs(V, index(V))) : interp(col_load(V, index(V)));
             next();
         }
         return a;
@@ -113,7 +113,7 @@ __device__ __forceinline__ float col_edge(const ColVolume &V, float gx, float gy
     const float fx = floorf(gx), fy = floorf(gy), fz = floorf(gz);
     const float ax = gx - fx, ay = gy - fy, az = gz - fz;
     ws = col_inside(gx, ax, V.hx) * col_inside(gy, ay, V.hy) * col_inside(gz, az, V.hz);
-    return col_interp(taps(V.index((int)fx + 1, (int)fy + 1, (int)fz + 1)), ax, ay, az);
+    return col_interp(taps((int)fx + 1, (int)fy + 1, (int)fz + 1), ax, ay, az);
 }
 
 // Samples ka .. kb - 1 of the n ones at g0 + k sg, all taps of which lie in the

@@ -6,9 +6,9 @@
 //
 // Forward + correction of 90 views of 768^2 (event: 384^2), texture gathers /
 // columns: event model 256^3 with the 8-region scene 18.0 / 6.8 ms; ROI 256^3
-// in 256^3 48.9 / 21.3 ms; cylinder 256 x 1024 x 512 73.5 / 51.3 ms (bound by
+// in 256^3 48.9 / 19.4 ms; cylinder 256 x 1024 x 512 73.5 / 51.3 ms (bound by
 // issue: the square root and arctangent of each sample); Joseph 512^3 22.3 /
-// 12.5 ms.
+// 11.7 ms.
 #include "cylinder.cuh"
 #include "fwd_column.cuh"
 #include "joseph.cuh"
@@ -18,7 +18,8 @@ namespace ctrex {
 
 // ---- event model -------------------------------------------------------------
 //
-// mu0, mu1 and tau in column stores of one shape.  A run of DYR_BLOCK samples
+// mu0, mu1 and tau in column stores of one shape, of pairs (a footprint may
+// take its two z neighbours from different fields).  A run of DYR_BLOCK samples
 // first looks up the (min, max) transition time of the voxels within 4 of its
 // first sample's 8^3 brick: where the view's time lies outside it, the whole
 // run reads one field like the static model.  Elsewhere each sample looks at
@@ -38,7 +39,7 @@ struct PixelEvent {
     const ViewGPU *views;
     const Grid &G;
 
-    __device__ __forceinline__ ColTaps pick(unsigned i, float t) const
+    __device__ __forceinline__ ColPairs pick(unsigned i, float t) const
     {
         ColVolume v1 = E.v0, vt = E.v0;
         v1.p = E.p1;
@@ -59,7 +60,7 @@ struct PixelEvent {
     __device__ __forceinline__ void operator()(int view, float u, float v, float &val, float &rs) const
     {
         const float t = __ldg(E.t_view + view);
-        auto taps = [&](unsigned i) { return pick(i, t); };
+        auto taps = [&](unsigned i, unsigned j, unsigned k) { return pick(E.v0.index(i, j, k), t); };
         float acc = 0.0f, acc_rs = 0.0f;
         for (int s = 0; s < G.n_sub; ++s) {
             Ray R;
@@ -91,16 +92,16 @@ struct PixelEvent {
                 if (t < lh.x || t >= lh.y) {
                     ColVolume V = E.v0;
                     V.p = t < lh.x ? E.v0.p : E.p1;
-                    a = run.sum(V, n, a);
+                    a = run.sum<true>(V, n, a);
                 } else {
                     for (int i = 0; i < n; ++i) {
                         const float2 b = look(E.brick, run);
                         const unsigned j = run.index(E.v0);
-                        ColTaps q;
+                        ColPairs q;
                         if (t < b.x || t >= b.y) {
                             ColVolume V = E.v0;
                             V.p = t < b.x ? E.v0.p : E.p1;
-                            q = col_load(V, j);
+                            q = col_load_pairs(V, j);
                         } else {
                             q = pick(j, t);
                         }
@@ -132,7 +133,7 @@ __device__ __forceinline__ void col_piece(const ColVolume &V, const int n[3], co
     if (K < 1) K = 1;
     int ka, kb;
     piece_interior(X, dg, a, h, K, n, ka, kb);
-    auto taps = [&](unsigned i) { return col_load(V, i); };
+    auto taps = [&](unsigned i, unsigned j, unsigned k) { return col_load(V, V.index(i, j, k)); };
     float g0[3], sg[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -310,8 +311,7 @@ struct PixelJoseph {
                 const float e0 = fmaf(ap, c10 - c00, c00), e1 = fmaf(ap, c11 - c01, c01);
                 return fmaf(aq, e1 - e0, e0);
             }
-            const float2 c = lerp2(__ldg(vol.p + i), __ldg(vol.p + s1 + i), two(ap));
-            return fmaf(aq, c.y - c.x, c.x);
+            return lerp(col_value(__ldg(vol.p + i), aq), col_value(__ldg(vol.p + s1 + i), aq), ap);
         };
         float acc = 0.0f, wacc = 0.0f;
         for (int k = ka > k0 ? k0 : kb; k <= k1; k = k + 1 == ka ? kb : k + 1) {
@@ -335,8 +335,9 @@ struct PixelJoseph {
             for (int left = kb - ka; left > 0; --left) {
                 const unsigned iq = (unsigned)(q >> 32);
                 const unsigned i = (unsigned)(p >> 32) * s1 + (base + ((iq >> COL_LOG) * vol.sz + iq));
-                const float2 c = lerp2(__ldg(vol.p + i), __ldg(vol.p + s1 + i), two(fixed_fraction((unsigned)p)));
-                acc += fmaf(fixed_fraction((unsigned)q), c.y - c.x, c.x);
+                const float aq = fixed_fraction((unsigned)q);
+                acc += lerp(col_value(__ldg(vol.p + i), aq), col_value(__ldg(vol.p + s1 + i), aq),
+                            fixed_fraction((unsigned)p));
                 p += dp;
                 q += dq;
                 base += sm;
