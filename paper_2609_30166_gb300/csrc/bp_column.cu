@@ -93,7 +93,7 @@ __device__ __forceinline__ void bp_edge(const ColImages &I, const float2 *img, f
 // box in front of the source is the hull of its corners' images), by a margin
 // that covers the rounding of u and v, bounded from the size of the terms
 // they are summed from.
-__device__ __forceinline__ int box_inside(float4 p0, float4 p1, float4 p2, const float lo[3], const float hi[3],
+__host__ __device__ __forceinline__ int box_inside(float4 p0, float4 p1, float4 p2, const float lo[3], const float hi[3],
                                           float4 win)
 {
     const float e = 0.02f;
@@ -121,6 +121,34 @@ __device__ __forceinline__ int box_inside(float4 p0, float4 p1, float4 p2, const
     if (!(u0 >= win.x + e && u1 <= win.y - e && v0 >= win.z + e && v1 <= win.w - e)) return 0;
     // depth changes by less than half a unit in the last place along z
     return fabsf(p2.z) * (hi[2] - lo[2]) < h3min * 0x1p-25f ? 2 : 1;
+}
+
+// The sums of a CTA (b / c of field f, c already times `mean`) into the volume,
+// by way of shared memory, so that the threads run along x: a z column's own
+// order would touch a line per voxel.
+template <typename TV, int VZ>
+__device__ __forceinline__ void bp_store(const Grid &G, float2 (*out)[BPC_COLS + 1], TV *__restrict__ vol,
+                                         const float *__restrict__ w, const float b[VZ], const float c[VZ], float mean,
+                                         float alpha, int normalize, int accumulate, int z0, int zfirst, int f)
+{
+    const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+    const size_t nvox = (size_t)G.nx * G.ny * G.nz;
+    const int oc = tid % BPC_COLS, ox = blockIdx.x * BPC_WX + oc % BPC_WX, oy = blockIdx.y * BPC_WY + oc / BPC_WX;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < VZ; ++q)
+        out[lane + 32 * q][warp] =
+            make_float2(b[q] * mean, normalize ? alpha * (c[q] > 1e-6f ? 1.0f / c[q] : 0.0f) : alpha);
+    __syncthreads();
+    if (ox >= G.nx || oy >= G.ny) return;
+    for (int r = tid / BPC_COLS; r < 32 * VZ; r += BPC_THREADS / BPC_COLS) {
+        const int oz = z0 + r;
+        if (oz < zfirst || oz >= G.nz) continue;
+        const size_t j = ((size_t)oz * G.ny + oy) * G.nx + ox + (size_t)f * nvox;
+        const float2 o = out[r][oc];
+        const float upd = (w ? o.y * __ldg(w + j) : o.y) * o.x;
+        Storage<TV>::store(vol + j, accumulate ? Storage<TV>::load(vol + j) + upd : upd);
+    }
 }
 
 // VZ: voxels per thread, 32 slices apart.  SUBV, CYL: as bp_kernel in backproject.cu; DYR: as bp_dyrect_kernel.
@@ -299,31 +327,86 @@ __global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR
 #pragma unroll
             for (int q = 0; q < VZ; ++q) c[0][q] += (float)cnt;
     }
-    // The sums go to shared memory, and from there to the volume with the
-    // threads along x: a z column's own order would touch a line per voxel.
     const float mean = SUBV ? G.inv_sub / (float)(sv * sv * sv) : G.inv_sub;
-    const size_t nvox = (size_t)G.nx * G.ny * G.nz;
-    const int oc = tid % BPC_COLS, ox = blockIdx.x * BPC_WX + oc % BPC_WX, oy = blockIdx.y * BPC_WY + oc / BPC_WX;
 #pragma unroll
     for (int f = 0; f < NP; ++f) {
-        __syncthreads();
 #pragma unroll
-        for (int q = 0; q < VZ; ++q) {
-            const float cc = c[f][q] * mean;
-            sOut[lane + 32 * q][warp] =
-                make_float2(b[f][q] * mean, normalize ? alpha * (cc > 1e-6f ? 1.0f / cc : 0.0f) : alpha);
+        for (int q = 0; q < VZ; ++q) c[f][q] *= mean;
+        bp_store<TV, VZ>(G, sOut, vol, w, b[f], c[f], mean, alpha, normalize, accumulate, z0, zfirst, f);
+    }
+}
+
+// The same where every view has every voxel inside the detector and at one
+// depth along z (backproject_flat): u and v are linear in z.  A warp takes 32
+// views at a time: a lane forms one view's (u, v) at the column's first voxel
+// and their steps, and a term is a broadcast of these and two multiply-adds a
+// voxel.  In bp_column_kernel the view's rows took 3/10 of L1's data path (16
+// wavefronts of broadcasts beside the taps' 37) and a quarter of the
+// instructions.  144 views of the 512^3 scan 18.8 -> 17.5 ms, sparse 128^3
+// 0.142 -> 0.129, 64^3 0.048 -> 0.044; with the event model's sums it was
+// slower (256^3, 90 views: 2.57 ms for 2.31), which stays there.  u and v
+// count from a whole column and a chunk of rows below them (the image pointer
+// takes the rest), so that they round less.
+template <typename TV, int VZ>
+__global__ void __launch_bounds__(BPC_THREADS, BPC_MIN_BLOCKS)
+    bp_flat_kernel(Grid G, const ViewGPU *__restrict__ views, const int *__restrict__ view_idx, int n_idx,
+                   const ColImages I, TV *__restrict__ vol, const float *__restrict__ w, float alpha, int normalize,
+                   int accumulate)
+{
+    __shared__ union {
+        struct {
+            float4 f[BPC_COLS][32];  // u, u's step along z, v, v's step
+            const float2 *img[BPC_COLS][32];
+        } term;
+        float2 out[32 * VZ][BPC_COLS + 1];
+    } sh;
+    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int ix = min(blockIdx.x * BPC_WX + warp % BPC_WX, G.nx - 1);
+    const int iy = min(blockIdx.y * BPC_WY + warp / BPC_WX, G.ny - 1);
+    const int zfirst = blockIdx.z * (32 * VZ), z0 = max(min(zfirst, G.nz - 32 * VZ), 0);
+    float b[VZ], c[VZ];
+#pragma unroll
+    for (int q = 0; q < VZ; ++q) b[q] = 0.0f;
+    int count = 0;
+    const int total = n_idx * G.n_sub;
+    for (int base = 0; base < total; base += 32) {
+        const int m = base + lane, k = m / G.n_sub;
+        const int view = m < total ? (view_idx ? view_idx[k] : k) : -1;
+        const bool ok = view >= 0 && view < G.n_views;  // an invalid view index is skipped
+        const unsigned mask = __ballot_sync(0xffffffffu, ok);
+        const int n = __popc(mask), at = __popc(mask & ((1u << lane) - 1u));
+        __syncwarp();
+        if (ok) {
+            const float x = (float)ix, y = (float)iy, z = (float)z0;
+            const float *P = views[view * G.n_sub + (m - k * G.n_sub)].P;
+            auto row = [&](const float *p) { return fmaf(p[0], x, fmaf(p[1], y, fmaf(p[2], z, p[3]))); };
+            const float h1 = row(P), h2 = row(P + 4), h3 = row(P + 8), span = 32.0f * VZ;
+            const float du = __fdiv_rn(P[2], h3), dv = __fdiv_rn(P[6], h3), u = __fdiv_rn(h1, h3), v = __fdiv_rn(h2, h3);
+            const float bu = fmaxf(floorf(fminf(u, fmaf(span, du, u))), 0.0f),
+                        bv = 16.0f * fmaxf(floorf(fminf(v, fmaf(span, dv, v)) * 0.0625f), 0.0f);
+            sh.term.f[warp][at] = make_float4(__fdiv_rn(fmaf(-bu, h3, h1), h3), du, __fdiv_rn(fmaf(-bv, h3, h2), h3), dv);
+            const unsigned iv = (unsigned)bv;
+            sh.term.img[warp][at] =
+                I.p + (size_t)k * I.view + ((size_t)(iv >> COL_LOG) * I.sv + ((unsigned)bu << COL_LOG) + iv);
         }
-        __syncthreads();
-        if (ox >= G.nx || oy >= G.ny) continue;
-        for (int r = tid / BPC_COLS; r < 32 * VZ; r += BPC_THREADS / BPC_COLS) {
-            const int oz = z0 + r;
-            if (oz < zfirst || oz >= G.nz) continue;
-            const size_t j = ((size_t)oz * G.ny + oy) * G.nx + ox + (size_t)f * nvox;
-            const float2 o = sOut[r][oc];
-            const float upd = (w ? o.y * __ldg(w + j) : o.y) * o.x;
-            Storage<TV>::store(vol + j, accumulate ? Storage<TV>::load(vol + j) + upd : upd);
+        __syncwarp();
+        count += n;
+#pragma unroll 1  // (2: 18.8 ms, out of registers)
+        for (int i = 0; i < n; ++i) {
+            const float4 f = sh.term.f[warp][i];
+            const float2 *img = sh.term.img[warp][i];
+            const float u = fmaf((float)lane, f.y, f.x), v = fmaf((float)lane, f.w, f.z);
+            BpTaps t[VZ];
+#pragma unroll
+            for (int q = 0; q < VZ; ++q) t[q] = bp_load(I, img, fmaf(32.0f * q, f.y, u), fmaf(32.0f * q, f.w, v));
+#pragma unroll
+            for (int q = 0; q < VZ; ++q) b[q] += bp_interp(t[q]);
         }
     }
+    const float mean = G.inv_sub;
+#pragma unroll
+    for (int q = 0; q < VZ; ++q) c[q] = (float)count * mean;
+    bp_store<TV, VZ>(G, sh.out, vol, w, b, c, mean, alpha, normalize, accumulate, z0, zfirst, 0);
 }
 
 template <typename TV, int VZ, bool SUBV, bool CYL, bool DYR>
@@ -340,6 +423,12 @@ static cudaError_t bpc_launch(const BpArgs &a)
     const dim3 grid((G.nx + BPC_WX - 1) / BPC_WX, (G.ny + BPC_WY - 1) / BPC_WY, (G.nz + 32 * VZ - 1) / (32 * VZ));
     const CylGPU cyl = a.cyl ? *a.cyl : CylGPU{};
     const float *tau = a.dyr ? a.dyr->tau : nullptr, *tv = a.dyr ? a.dyr->t_view : nullptr;
+    if constexpr (!SUBV && !CYL && !DYR)
+        if (a.flat && !a.window) {
+            bp_flat_kernel<TV, VZ><<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
+                G, a.views, a.view_idx, a.n_idx, I, static_cast<TV *>(a.vol), a.w, a.alpha, a.normalize, a.accumulate);
+            return cudaGetLastError();
+        }
     if (a.window)
         bp_column_kernel<TV, VZ, true, SUBV, CYL, DYR><<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
             G, a.views, a.view_idx, a.n_idx, I, a.window, static_cast<TV *>(a.vol), a.w, a.alpha, a.normalize,
@@ -384,6 +473,22 @@ cudaError_t launch_backproject_column(const BpArgs &a)
 bool backproject_column_fits(const Grid &G)
 {
     return (G.ny + BPC_WY - 1) / BPC_WY <= 65535 && (G.nz + 63) / 64 <= 65535;
+}
+
+bool backproject_flat(const Grid &G, const ViewGPU *views, int n)
+{
+    // (a block of slices may reach beyond a thin volume)
+    const int block = four_voxels(G.nz) ? 128 : 64;
+    const float lo[3] = {0.0f, 0.0f, 0.0f},
+                hi[3] = {G.nx - 1.0f, G.ny - 1.0f, (G.nz > block ? G.nz : block) - 1.0f};
+    const float4 det = make_float4(0.0f, (float)(G.nu - 1), 0.0f, (float)(G.nv - 1));
+    for (int i = 0; i < n; ++i) {
+        const float *P = views[i].P;
+        if (box_inside(make_float4(P[0], P[1], P[2], P[3]), make_float4(P[4], P[5], P[6], P[7]),
+                       make_float4(P[8], P[9], P[10], P[11]), lo, hi, det) != 2)
+            return false;
+    }
+    return true;
 }
 
 }  // namespace ctrex

@@ -49,6 +49,7 @@ struct ctrex_ctx {
     Atlas vol_atlas_view;
     // the volume in column layout, where the scan's detector columns run along z
     double col_lean = 10.0, col_step = 1.0;  // detector_column_step
+    bool bp_flat = false, bp_flat_roi = false;  // backproject_flat (Cartesian grids)
     ColStore vol_col;
     ColStore col1;     // the ROI grid, or the event model's final values
     ColStore tau_col;  // the event model's transition times
@@ -700,6 +701,7 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
     c->atlas_unfit = false;
     c->img_atlas_unfit = false;
     detector_column_step(hv, c->col_lean, c->col_step);
+    c->bp_flat = backproject_flat(G, hv.data(), nvs);
     set_clip_box(c);
     return CTREX_OK;
 }
@@ -940,6 +942,7 @@ int ctrex_set_roi(ctrex_ctx *c, const ctrex_vol_grid *roi)
         F.lo[a] = -0.5f;
         F.hi[a] = (float)(n[a] - 0.5);
     }
+    c->bp_flat_roi = backproject_flat(F, hv.data(), nvs);
     F.step_mm = (float)(c->step_vox * minf);
     RoiGPU &R = c->roig;
     for (int a = 0; a < 3; ++a) {
@@ -1111,6 +1114,7 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
     a.subvox = c->bp_subvoxel;
     a.cyl = c->cyl ? &c->cylg : nullptr;
     a.dyr = c->dyr ? &c->dyra : nullptr;
+    a.flat = c->bp_flat && !c->cyl;
     if (n_idx > 0 && column_backproject(c)) {
         cudaError_t ae = col_ensure_images(c->img_col, c->grid.nu, c->grid.nv, n_idx, c->stream);
         if (ae == cudaSuccess) {
@@ -1141,6 +1145,7 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
         const size_t nc = grid_voxels(c->grid);
         a.grid = &c->roi_grid;
         a.views = c->d_views_roi;
+        a.flat = c->bp_flat_roi;
         a.vol = static_cast<char *>(vol) + nc * dtype_size(vdt);
         a.w = w ? w + nc : nullptr;
         ce = launch_backproject(a);

@@ -173,6 +173,7 @@ struct BpArgs {
     const Atlas *atlas = nullptr;  // correction images uploaded into a texture atlas, or nullptr
     const ColStore *column = nullptr;  // correction images in column layout, or nullptr
     const int4 *window = nullptr;  // per-view detector window of the backprojector, or nullptr
+    bool flat = false;             // backproject_flat() of the views
     const ViewGPU *views;
     const int *view_idx;
     int n_idx;
@@ -193,6 +194,9 @@ cudaError_t launch_backproject(const BpArgs &a);
 // The same on a.column (bp_column.cu).
 cudaError_t launch_backproject_column(const BpArgs &a);
 bool backproject_column_fits(const Grid &g);  // its launch shape stays within the grid limits
+// Whether every one of n views (on the host) has the whole volume inside the
+// detector and every z column at one depth, to FP32 rounding.
+bool backproject_flat(const Grid &g, const ViewGPU *views, int n);
 
 cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol);
 // The same through a scatter volume of adjoint_column_elems(G) floats

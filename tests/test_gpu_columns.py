@@ -252,3 +252,44 @@ def test_motion_runs_match_oracle(n, det, views, sub, turn, step, shift):
     got_t, got_c = c.motion_grad(_t(x), _t(y[vi]), view_idx=vi)
     assert rel_l2(_np(got_t), gt) <= 1e-4 and rel_l2(_np(got_c), gc) <= 1e-4
     c.close()
+
+
+# Backprojection where every view holds the whole volume, in lists of 32 terms:
+# one term, lists with a remainder, sub-angles, an image repeated; thin volumes
+# (blocks of slices beyond the last one) and a detector that the volume nearly
+# fills, or is just too large for.
+@pytest.mark.parametrize("n,det,views,sub,turn,width", [
+    ((9, 11, 130), (48, 90), 33, 1, 0.4, 96.0),
+    ((17, 8, 64), (40, 44), 35, 2, 0.0, 96.0),
+    ((8, 8, 5), (33, 31), 1, 1, -2.0, 96.0),
+    ((30, 30, 128), (41, 61), 32, 1, 1.0, 83.0),
+    ((30, 30, 30), (64, 64), 20, 4, 0.0, 74.0),
+    ((1, 31, 70), (50, 60), 7, 1, 0.3, 96.0),
+])
+def test_flat_backprojection_matches_oracle(n, det, views, sub, turn, width):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    P = _matrices(views, sub, turn, det[0], det[1], width, 200.0)
+    pitch = 30.0 / max(n)
+    vox, shape = (pitch, 0.9 * pitch, pitch), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det)
+    pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    rng = np.random.default_rng(17)
+    x, w = rng.uniform(0.2, 1.0, size=shape), rng.uniform(0.5, 1.0, size=shape)
+    iu, iv = np.meshgrid(np.arange(det[0]), np.arange(det[1]))
+    r = np.stack([np.cos(0.11 * iu + k) + np.sin(0.07 * iv * (k % 5 + 1)) + 2.5 for k in range(views)])
+    want, b, _ = oracle.backproject(pb, _np(_t(r)), w=_np(_t(w)), alpha=0.7, x=_np(_t(x)))
+    assert rel_l2(_np(c.back_project(_t(r), vol=_t(x), w=_t(w), alpha=0.7)), want) <= TOL32
+    assert rel_l2(_np(c.back_project(_t(r), normalize=False, accumulate=False)), b) <= TOL32
+    vi = np.concatenate([np.arange(views)[::-3], [0, 0]]).astype(np.int32)
+    _, b, _ = oracle.backproject(pb, _np(_t(r[vi])), views=vi)
+    assert rel_l2(_np(c.back_project(_t(r[vi]), normalize=False, accumulate=False, view_idx=vi)), b) <= TOL32
+    # 16-bit images and volume: one rounding of the result (2^-9)
+    r16 = _t(r, torch.bfloat16)
+    want, _, _ = oracle.backproject(pb, _np(r16), alpha=0.7)
+    got = c.back_project(r16, alpha=0.7, vol_dtype=torch.bfloat16)
+    assert rel_l2(_np(got), want) <= 2.0 ** -8
+    c.close()
