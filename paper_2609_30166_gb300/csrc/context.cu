@@ -1079,6 +1079,7 @@ int ctrex_fwd_correct(ctrex_ctx *c, const void *vol, int vdt, const void *p, int
     e = ensure_partials(c, n_idx);
     if (e) return e;
     FwdArgs a = fwd_args(c, vol, vdt, view_idx, n_idx);
+    a.norm_tiles = true;
     e = prepare_atlas(c, a, vol, vdt);
     if (e) return e;
     cudaError_t ce = launch_forward_correct(a, p, pdt, r, rdt, c->d_partials, c->partials_cap, sums);

@@ -147,6 +147,7 @@ struct FwdArgs {
     cudaStream_t stream;
     unsigned *devcheck;         // device status word
     int p_by_view = 0;          // correction: measured images indexed by view, not by list position
+    bool norm_tiles = false;      // correction: see norm_tiles_kernel (project.cu)
     const CylGPU *cyl = nullptr;  // cylindrical domain, or nullptr (Cartesian grid)
     int joseph = 0;               // classical Joseph projector; atlas = the three-stack atlas
     const RoiGPU *roi = nullptr;  // multi-resolution ROI: atlas = context grid, roi_atlas = ROI grid

@@ -4,8 +4,8 @@
 // layout (column.cuh).
 //
 // What bounds it: L1's data path (12.6 wavefronts per 32 samples, of which 8
-// are the taps themselves; 16-byte loads of x pairs too need as many; 89 % busy
-// at 512^3, 51 to 68 % at 64^3 and 128^3) and next to it the issue ports (68 %
+// are the taps themselves; 16-byte loads of x pairs too need as many; 86 % busy
+// at 512^3, 49 to 67 % at 64^3 and 128^3) and next to it the issue ports (68 %
 // busy at every size, and held longer by packed multiply-adds); the texture
 // kernel's bound was the gathers' return path.  On 144 views of the 512^3 x
 // 768^2 scan, FP32 / BF16 volume: 146.5 / 75.8 ms with texture gathers, 52.5 /

@@ -280,7 +280,8 @@ template <typename T> struct SumPart { typedef SumDouble type; };
 template <> struct SumPart<float> { typedef SumFloat type; };
 
 template <typename T>
-__global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ pairs, size_t n, double *__restrict__ out)
+__global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ pairs, size_t n, double *__restrict__ out,
+                                                          size_t second = 0, size_t n2 = 0)
 {
     __shared__ double s[2][16];
     const size_t per = (n + gridDim.x - 1) / gridDim.x, i0 = per * blockIdx.x, i1 = min(i0 + per, n);
@@ -291,8 +292,13 @@ __global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ 
 #pragma unroll 4
     for (size_t i = i0 + threadIdx.x; i < i1; i += 512) {
         sa.add(pairs[2 * i]);
-        sb.add(pairs[2 * i + 1]);
+        if (n2 == 0) sb.add(pairs[2 * i + 1]);
     }
+    // n2: the second sum is that of the n2 pairs from `second` on
+    const size_t per2 = (n2 + gridDim.x - 1) / gridDim.x, j0 = second + per2 * blockIdx.x,
+                 j1 = min(j0 + per2, second + n2);
+#pragma unroll 4
+    for (size_t i = j0 + threadIdx.x; i < j1; i += 512) sb.add(pairs[2 * i + 1]);
     double a = sa.value(), b = sb.value();
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -309,6 +315,37 @@ __global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ 
         for (int w = 0; w < 16; ++w) t += s[threadIdx.x][w];
         out[2 * blockIdx.x + threadIdx.x] = t;
     }
+}
+
+// |p|^2 in the texture kernel's tiles of 32 x 4 pixels and its order of
+// additions (a warp per tile), for ctrex_fwd_correct from the column kernels,
+// whose CTAs hold other pixels: the norm that it reports in FP64 is then the
+// same number whichever kernel projects (their FP32 partials differ by up to
+// 4e-9 of it).  One read of p: 0.1 ms for 360 images of 384^2, beside a Joseph
+// projection of 7.1.
+template <typename TP>
+__global__ void __launch_bounds__(256) norm_tiles_kernel(Grid G, const int *__restrict__ view_idx, dim3 tiles,
+                                                         const TP *__restrict__ p, float *__restrict__ partials)
+{
+    const size_t bid = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (bid >= (size_t)tiles.x * tiles.y * tiles.z) return;
+    const int tu = (int)(bid % tiles.x), k = (int)(bid / tiles.x % tiles.y), tv = (int)(bid / ((size_t)tiles.x * tiles.y));
+    const int view = view_idx ? view_idx[k] : k, lane = threadIdx.x & 31, iu = tu * FWD_TX + lane;
+    const bool ok = view >= 0 && view < G.n_views && iu < G.nu;
+    float p2[FWD_TY], b = 0.0f;
+#pragma unroll
+    for (int r = 0; r < FWD_TY; ++r) {
+        const int iv = tv * FWD_TY + r;
+        const float pm = ok && iv < G.nv ? Storage<TP>::load(p + ((size_t)k * G.nv + iv) * G.nu + iu) : 0.0f;
+        p2[r] = pm * pm;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int r = 0; r < FWD_TY; ++r) p2[r] += __shfl_xor_sync(0xffffffffu, p2[r], off);
+#pragma unroll
+    for (int r = 0; r < FWD_TY; ++r) b += p2[r];
+    if (lane == 0) partials[2 * bid + 1] = b;
 }
 
 // Exact sample count (same set-up arithmetic as the projector): ray
@@ -363,7 +400,7 @@ int forward_partials_needed(const Grid &G, int n_idx)
     const dim3 g = fwd_grid(G, n_idx);
     const int col = column_partials_needed(G, n_idx), n = (int)(g.x * g.y * g.z);
     // either launch shape, and room for the second pass
-    return (n > col ? n : col) + 2 * FINISH_CTAS;
+    return n + col + 2 * FINISH_CTAS;
 }
 
 template <typename Sampler, typename TP, int MODE>
@@ -460,14 +497,25 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
     }
     const dim3 fg = fwd_grid(*a.grid, a.n_idx);
     const int n = a.column ? column_partials_needed(*a.grid, a.n_idx) : (int)(fg.x * fg.y * fg.z);
-    if (n + 2 * FINISH_CTAS > n_partials_cap) return cudaErrorInvalidValue;
+    const bool norm = a.column && a.norm_tiles && sums;
+    const size_t nt = norm ? (size_t)fg.x * fg.y * fg.z : 0;
+    if (n + nt + 2 * FINISH_CTAS > (size_t)n_partials_cap) return cudaErrorInvalidValue;
     cudaError_t e = fwd_dispatch<MODE_CORRECT>(a, p_dtype, r, nullptr, p, partials);
     if (e != cudaSuccess || sums == nullptr) return e;
+    if (norm) {
+        const unsigned ctas = (unsigned)((nt + 7) / 8);
+        if (p_dtype == CTREX_F32)
+            norm_tiles_kernel<<<ctas, 256, 0, a.stream>>>(*a.grid, a.view_idx, fg,
+                                                          static_cast<const float *>(p), partials + 2 * (size_t)n);
+        else
+            norm_tiles_kernel<<<ctas, 256, 0, a.stream>>>(*a.grid, a.view_idx, fg,
+                                                          static_cast<const __nv_bfloat16 *>(p), partials + 2 * (size_t)n);
+    }
     if (n <= FINISH_ONE) {
-        finish_sums_kernel<<<1, 512, 0, a.stream>>>(partials, (size_t)n, sums);
+        finish_sums_kernel<<<1, 512, 0, a.stream>>>(partials, (size_t)n, sums, (size_t)n, nt);
     } else {  // the intermediate sums lie behind the partials
         double *mid = reinterpret_cast<double *>(partials + 2 * ((size_t)n_partials_cap - 2 * FINISH_CTAS));
-        finish_sums_kernel<<<FINISH_CTAS, 512, 0, a.stream>>>(partials, (size_t)n, mid);
+        finish_sums_kernel<<<FINISH_CTAS, 512, 0, a.stream>>>(partials, (size_t)n, mid, (size_t)n, nt);
         finish_sums_kernel<<<1, 512, 0, a.stream>>>(mid, (size_t)FINISH_CTAS, sums);
     }
     return cudaGetLastError();

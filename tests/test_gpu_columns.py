@@ -293,3 +293,36 @@ def test_flat_backprojection_matches_oracle(n, det, views, sub, turn, width):
     got = c.back_project(r16, alpha=0.7, vol_dtype=torch.bfloat16)
     assert rel_l2(_np(got), want) <= 2.0 ** -8
     c.close()
+
+
+# |p|^2 of fwd_correct: FP32 in tiles of 32 x 4 pixels (a butterfly over each
+# row of 32, then row by row), FP64 over the tiles; the last sum's order is
+# free: 1e-13.
+@pytest.mark.parametrize("det,dtype", [((45, 31), torch.float32), ((64, 33), torch.bfloat16), ((31, 66), torch.float32)])
+def test_correction_norm_by_tiles(det, dtype):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    nu, nv = det
+    views, shape = 5, (40, 22, 24)
+    c = ctrex.Context()
+    c.set_geometry(_matrices(views, 1, 0.2, nu, nv, 96.0, 200.0), shape, (1.0, 1.0, 1.0), (-11.5, -10.5, -19.5), det)
+    rng = np.random.default_rng(3)
+    p = _t(rng.uniform(0.0, 2.0, size=(views, nv, nu)), dtype)
+    x = _t(rng.uniform(size=shape))
+    sums = torch.empty(2, dtype=torch.float64, device="cuda")
+    vi = np.array([4, 1, 3], dtype=np.int32)
+    for k, idx in ((views, None), (3, vi)):
+        c.fwd_correct(x, p[:k].contiguous(), sums=sums, view_idx=idx)
+        q = np.zeros((k, -(-nv // 4) * 4, -(-nu // 32) * 32), dtype=np.float32)
+        q[:, :nv, :nu] = p[:k].float().cpu().numpy()
+        v = (q * q).reshape(k, -1, 4, q.shape[2] // 32, 32)
+        for off in (16, 8, 4, 2, 1):
+            v = v[..., :off] + v[..., off:2 * off]
+        t = np.zeros(v.shape[:2] + v.shape[3:4], dtype=np.float32)
+        for r in range(4):
+            t = t + v[:, :, r, :, 0]
+        want = t.astype(np.float64).sum()
+        assert abs(sums[1].item() - want) <= 1e-13 * want
+    c.close()
+
