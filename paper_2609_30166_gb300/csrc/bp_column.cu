@@ -15,6 +15,7 @@ constexpr int BPC_THREADS = 32 * BPC_COLS;
 constexpr int BPC_CHUNK = 128;  // views staged at a time
 constexpr int BPC_MIN_BLOCKS = 5;  // 48 registers (4 and 6: 21.1 and 21.8 ms where 5 takes 18.8)
 constexpr int BPC_SUBV_MIN_BLOCKS = 4;
+constexpr size_t BPC_DEEP_MAX = 4 * 152;  // 4 CTAs on each of 152 SMs
 
 // The correction images [n][nu][nv] in column layout: pair (u, v) of image k,
 // padded indices (u + 1, v + 1), at k view + (v >> 4) sv + (u << 4) + v.
@@ -347,8 +348,10 @@ __global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR
 // slower (256^3, 90 views: 2.57 ms for 2.31), which stays there.  u and v
 // count from a whole column and a chunk of rows below them (the image pointer
 // takes the rest), so that they round less.
-template <typename TV, int VZ>
-__global__ void __launch_bounds__(BPC_THREADS, BPC_MIN_BLOCKS)
+// DEEP: a grid of few CTAs (bpc_launch), which waits for its loads: four terms
+// in flight, 64 registers.
+template <typename TV, int VZ, bool DEEP>
+__global__ void __launch_bounds__(BPC_THREADS, DEEP ? 4 : BPC_MIN_BLOCKS)
     bp_flat_kernel(Grid G, const ViewGPU *__restrict__ views, const int *__restrict__ view_idx, int n_idx,
                    const ColImages I, TV *__restrict__ vol, const float *__restrict__ w, float alpha, int normalize,
                    int accumulate)
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(BPC_THREADS, BPC_MIN_BLOCKS)
         }
         __syncwarp();
         count += n;
-#pragma unroll 1  // (2: 18.8 ms, out of registers)
+#pragma unroll DEEP ? 4 : 1  // (2 at 48 registers: 18.8 ms)
         for (int i = 0; i < n; ++i) {
             const float4 f = sh.term.f[warp][i];
             const float2 *img = sh.term.img[warp][i];
@@ -425,7 +428,11 @@ static cudaError_t bpc_launch(const BpArgs &a)
     const float *tau = a.dyr ? a.dyr->tau : nullptr, *tv = a.dyr ? a.dyr->t_view : nullptr;
     if constexpr (!SUBV && !CYL && !DYR)
         if (a.flat && !a.window) {
-            bp_flat_kernel<TV, VZ><<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
+            // up to one wave of the deep form's CTAs (64^3 x 90 views: 0.044 ->
+            // 0.042 ms; 512^3: 17.5 -> 19.6)
+            const bool deep = (size_t)grid.x * grid.y * grid.z <= BPC_DEEP_MAX;
+            auto *kernel = deep ? bp_flat_kernel<TV, VZ, true> : bp_flat_kernel<TV, VZ, false>;
+            kernel<<<grid, dim3(32, BPC_COLS), 0, a.stream>>>(
                 G, a.views, a.view_idx, a.n_idx, I, static_cast<TV *>(a.vol), a.w, a.alpha, a.normalize, a.accumulate);
             return cudaGetLastError();
         }

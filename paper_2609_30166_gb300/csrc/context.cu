@@ -40,6 +40,8 @@ struct ctrex_ctx {
     float *d_partials = nullptr;
     int partials_cap = 0;
     double *d_sums = nullptr;
+    double *h_sums = nullptr;         // the SIRT loop's residual on the host (pinned)
+    cudaEvent_t sums_done = nullptr;  // and its arrival
     unsigned *d_devcheck = nullptr;
     unsigned long long *d_count = nullptr;
     void *d_r = nullptr;  // SIRT correction images
@@ -531,6 +533,8 @@ int ctrex_destroy(ctrex_ctx *c)
         if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
         if (c->ev_vol) cudaEventDestroy(c->ev_vol);
         if (c->ev_p) cudaEventDestroy(c->ev_p);
+        if (c->sums_done) cudaEventDestroy(c->sums_done);
+        if (c->h_sums) cudaFreeHost(c->h_sums);
         dfree(c->d_subset_views);
         dfree(c->d_window);
         dfree(c->d_subset_sums);
@@ -1087,35 +1091,9 @@ int ctrex_fwd_correct(ctrex_ctx *c, const void *vol, int vdt, const void *p, int
     return CTREX_OK;
 }
 
-int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt, const float *w, float alpha,
-                       int normalize, int accumulate, const int *view_idx, int n_idx)
+// The images of a backprojection into the layout that it reads.
+static int bp_images(ctrex_ctx *c, BpArgs &a, const void *r, int rdt, int n_idx)
 {
-    if (!c) return CTREX_E_ARG;
-    int e = check_views(c, view_idx, n_idx);
-    if (e) return e;
-    if (!vol || (!r && n_idx > 0)) return fail(c, CTREX_E_ARG, "back_project: NULL buffer");
-    if (!dtype_ok(vdt) || !dtype_ok(rdt)) return fail(c, CTREX_E_DTYPE, "back_project: bad dtype");
-    if (!isfinite(alpha)) return fail(c, CTREX_E_ARG, "back_project: alpha not finite");
-    DeviceGuard g(c->device);
-    BpArgs a;
-    a.grid = &c->grid;
-    a.views = c->d_views;
-    a.view_idx = view_idx;
-    a.n_idx = n_idx;
-    a.r = r;
-    a.r_dtype = rdt;
-    a.vol = vol;
-    a.vol_dtype = vdt;
-    a.w = w;
-    a.alpha = alpha;
-    a.normalize = normalize ? 1 : 0;
-    a.accumulate = accumulate ? 1 : 0;
-    a.stream = c->stream;
-    a.window = c->has_window ? c->d_window : nullptr;
-    a.subvox = c->bp_subvoxel;
-    a.cyl = c->cyl ? &c->cylg : nullptr;
-    a.dyr = c->dyr ? &c->dyra : nullptr;
-    a.flat = c->bp_flat && !c->cyl;
     if (n_idx > 0 && column_backproject(c)) {
         cudaError_t ae = col_ensure_images(c->img_col, c->grid.nu, c->grid.nv, n_idx, c->stream);
         if (ae == cudaSuccess) {
@@ -1140,6 +1118,31 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
             a.atlas = &c->img_atlas_view;
         }
     }
+    return CTREX_OK;
+}
+
+// The backprojection of images that bp_images() has laid out in `a`.
+static int bp_run(ctrex_ctx *c, BpArgs &a, const void *r, int rdt, void *vol, int vdt, const float *w, float alpha,
+                  int normalize, int accumulate, const int *view_idx, int n_idx)
+{
+    a.grid = &c->grid;
+    a.views = c->d_views;
+    a.view_idx = view_idx;
+    a.n_idx = n_idx;
+    a.r = r;
+    a.r_dtype = rdt;
+    a.vol = vol;
+    a.vol_dtype = vdt;
+    a.w = w;
+    a.alpha = alpha;
+    a.normalize = normalize ? 1 : 0;
+    a.accumulate = accumulate ? 1 : 0;
+    a.stream = c->stream;
+    a.window = c->has_window ? c->d_window : nullptr;
+    a.subvox = c->bp_subvoxel;
+    a.cyl = c->cyl ? &c->cylg : nullptr;
+    a.dyr = c->dyr ? &c->dyra : nullptr;
+    a.flat = c->bp_flat && !c->cyl;
     cudaError_t ce = launch_backproject(a);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "back_project launch");
     if (c->roi) {  // the ROI grid's voxels follow the context grid's
@@ -1153,6 +1156,21 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
         if (ce != cudaSuccess) return cuda_fail(c, ce, "back_project launch (ROI grid)");
     }
     return CTREX_OK;
+}
+
+int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt, const float *w, float alpha,
+                       int normalize, int accumulate, const int *view_idx, int n_idx)
+{
+    if (!c) return CTREX_E_ARG;
+    int e = check_views(c, view_idx, n_idx);
+    if (e) return e;
+    if (!vol || (!r && n_idx > 0)) return fail(c, CTREX_E_ARG, "back_project: NULL buffer");
+    if (!dtype_ok(vdt) || !dtype_ok(rdt)) return fail(c, CTREX_E_DTYPE, "back_project: bad dtype");
+    if (!isfinite(alpha)) return fail(c, CTREX_E_ARG, "back_project: alpha not finite");
+    DeviceGuard g(c->device);
+    BpArgs a;
+    e = bp_images(c, a, r, rdt, n_idx);
+    return e ? e : bp_run(c, a, r, rdt, vol, vdt, w, alpha, normalize, accumulate, view_idx, n_idx);
 }
 
 int ctrex_adjoint_project(ctrex_ctx *c, const float *proj, float *vol, const int *view_idx, int n_idx)
@@ -1226,21 +1244,30 @@ int ctrex_sirt_iterate(ctrex_ctx *c, void *vol, int vdt, const void *p, int pdt,
     if (e) return e;
     e = ensure_partials(c, V);
     if (e) return e;
+    if (!c->sums_done) CT_CUDA(c, cudaEventCreateWithFlags(&c->sums_done, cudaEventDisableTiming));
+    if (!c->h_sums) CT_CUDA(c, cudaMallocHost((void **)&c->h_sums, 2 * sizeof(double)));
     for (int k = 0; k < max_iter; ++k) {
         FwdArgs a = fwd_args(c, vol, vdt, nullptr, V);
         e = prepare_atlas(c, a, vol, vdt);
         if (e) return e;
         cudaError_t ce = launch_forward_correct(a, p, pdt, c->d_r, pdt, c->d_partials, c->partials_cap, c->d_sums);
         if (ce != cudaSuccess) return cuda_fail(c, ce, "sirt: fwd_correct");
-        double s[2];
-        CT_CUDA(c, cudaMemcpyAsync(s, c->d_sums, sizeof s, cudaMemcpyDeviceToHost, c->stream));
-        CT_CUDA(c, cudaStreamSynchronize(c->stream));
+        // the images' layout for the backprojection is under way while the host
+        // waits for the residual
+        CT_CUDA(c, cudaMemcpyAsync(c->h_sums, c->d_sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        CT_CUDA(c, cudaEventRecord(c->sums_done, c->stream));
+        BpArgs b;
+        const int be = bp_images(c, b, c->d_r, pdt, V);
+        CT_CUDA(c, cudaEventSynchronize(c->sums_done));
+        const double s[2] = {c->h_sums[0], c->h_sums[1]};
         const double rho = s[1] > 0.0 ? sqrt(s[0] / s[1]) : sqrt(s[0]);
         if (hist) hist[k] = (float)rho;
         if (!isfinite(rho)) return fail(c, CTREX_E_DIVERGED, "sirt: residual not finite at iteration %d", k);
         if (rho <= (double)tol) break;
-        int be = ctrex_back_project(c, c->d_r, pdt, vol, vdt, w, alpha, 1, 1, nullptr, V);
         if (be) return be;
+        if (!isfinite(alpha)) return fail(c, CTREX_E_ARG, "back_project: alpha not finite");
+        e = bp_run(c, b, c->d_r, pdt, vol, vdt, w, alpha, 1, 1, nullptr, V);
+        if (e) return e;
         if (iters_done) *iters_done = k + 1;
     }
     return ctrex_device_status(c);
