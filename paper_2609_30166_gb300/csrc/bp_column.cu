@@ -448,11 +448,22 @@ static cudaError_t bpc_launch(const BpArgs &a)
 }
 
 // Voxels per thread: 4 where 128-slice blocks fit the volume to within 14 %
-// of 64-slice ones (144 views at 512^3: 21.7 ms with 4, 24.7 with 2, 27 with 8).
+// of 64-slice ones (144 views at 512^3: 21.7 ms with 4, 24.7 with 2, 27 with 8;
+// 180 x 180 x 130, 100 views: 0.69 ms with 2, 0.83 with 1).  Four only from 128
+// slices on: a block that reaches beyond the volume reaches beyond the
+// detector (85 x 98 x 82, 34 helical views of 3 sub-angles: 0.32 ms with 4,
+// 0.16 with 2).
 static bool four_voxels(int nz)
 {
     const int n4 = (nz + 127) / 128 * 128, n2 = (nz + 63) / 64 * 64;
-    return 100 * n4 < 114 * n2;
+    return nz >= 128 && 100 * n4 < 114 * n2;
+}
+
+// Slices that the kernel works through, the last block's repeats among them.
+int backproject_column_slices(const Grid &G)
+{
+    const int b = four_voxels(G.nz) ? 128 : 64;
+    return (G.nz + b - 1) / b * b;
 }
 
 template <typename TV, bool CYL> static cudaError_t bpc_plain(const BpArgs &a)

@@ -276,6 +276,13 @@ bool column_forward(const ctrex_ctx *c, int vdt)
 
 bool column_backproject(const ctrex_ctx *c)
 {
+    // blocks of slices that repeat or leave empty a third and more (FP32 / BF16
+    // images, us by columns, by gathers): 60 x 60 x 20, 100 views 105, 86 / 105,
+    // 82; 50 x 50 x 40 91, 85 / 92, 81; 180 x 180 x 70 476, 486 / 476, 422; 74 x
+    // 87 x 84, 132 views 155, 237 / 156, 218
+    if (!c->cyl && !c->roi && !c->dyr && c->bp_subvoxel == 1 &&
+        100.0 * backproject_column_slices(c->grid) > 155.0 * c->grid.nz)
+        return false;
     return c->col_lean <= COL_LEAN_BP && c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(c->grid) &&
            (!c->roi || backproject_column_fits(c->roi_grid));
 }
