@@ -137,16 +137,17 @@ class ClockSampler:
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one full-size
 # launch of the fused forward kernel, from one-pass ncu captures of that
 # kernel on 16 and 180 views of the workload (summary kept under profiles/):
-# the launch reads the volume atlas once and each view's measured image and
-# writes its correction image, so traffic = a + b * views, with a and b from
-# the two captures, evaluated at 720 views.  Valid only for the kernel
+# the launch reads the volume's columns a few times over (a strip of detector
+# columns at a time) and each view's measured image, and writes its correction
+# image, so traffic = a + b * views, with a and b from the two captures,
+# evaluated at 720 views.  Valid only for the kernel
 # sources it was taken on (hash below) and for the FP32 workload; otherwise
 # null.
-_T16, _T180 = 585831936 + 33430016, 982422528 + 395699200
+_T16, _T180 = 8918335232 + 230262272, 11976001024 + 1530899200
 FWD_TRAFFIC_BYTES = int(_T16 + (_T180 - _T16) * (720 - 16) / (180 - 16))
-FWD_TRAFFIC_SOURCES = ("project.cu", "atlas.cuh", "ray.cuh", "cylinder.cuh", "joseph.cuh", "roi.cuh", "fwd_common.cuh",
-                       "ctrex_internal.cuh", "dyrect.cuh")
-FWD_TRAFFIC_HASH = "ffcabe5e01f8bb0a"
+FWD_TRAFFIC_SOURCES = ("fwd_column.cu", "fwd_column.cuh", "column.cuh", "column.cu", "ray.cuh", "fwd_common.cuh",
+                       "ctrex_internal.cuh")
+FWD_TRAFFIC_HASH = "92917f68f57cff6e"
 
 
 def fwd_traffic(dtype, views):
@@ -625,7 +626,7 @@ def run_ours(args):
         "residual_after": res,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None if (cyl or args.projector != "trilinear") else fwd_traffic(args.dtype, args.views),
-                     "kernel": "fwd_kernel (fused forward + correction)",
+                     "kernel": "fwd_column_kernel (fused forward + correction, volume as z columns)",
                      "l2_gather": {"achieved": achieved, "peak": l2_peak, "unit": "GB/s", "frac": achieved / l2_peak,
                                    "peak_method": "ctrex_probe_l2_read_bandwidth: 16-byte L2-only loads "
                                                   "(ld.global.cg) over half of L2, 512 passes"},
@@ -639,13 +640,15 @@ def run_ours(args):
                      "note": f"algorithmic gather bytes = 8 taps x {elt} B per sample; peak = HBM copy "
                              f"bandwidth ({peak_kind}). The taps are served from L1/TEX and L2 (DRAM traffic "
                              "is ~1x the compulsory bytes), so the HBM figure cannot bound this kernel: "
-                             "frac > 1 is expected. Its binding ceiling is tex_gather (texture return "
-                             "path, 2 gathers per FP32 sample); l2_gather and l1_gather give the graded "
-                             "gather roofline against the measured L2 read bandwidth and the L1 ceiling"},
-        # per step: volume atlas upload (two kernels for the Joseph atlas),
-        # fused forward + correction, residual finish, correction-image atlas
-        # upload, backprojection + update
-        "gpu_launches": (6 if args.projector == "joseph" else 5) * args.steps,
+                             "frac > 1 is expected. Its binding ceiling is L1's data path (l1_gather; 86 % "
+                             "busy in ncu, as the loads of a warp straddle 128-byte lines); l2_gather gives "
+                             "the gather roofline against the measured L2 read bandwidth, and tex_gather "
+                             "what texture gathers (2 per FP32 sample) could do at most: above 1 since the "
+                             "column loads do not use them"},
+        # per step: volume column upload (and the cylinder's repeated sector),
+        # fused forward + correction, residual finish in two levels,
+        # correction-image column upload, backprojection + update
+        "gpu_launches": (7 if cyl else 6) * args.steps,
         "e2e": e2e,
         "clocks": clk,
     }

@@ -152,8 +152,8 @@ int ctrex_set_geometry(ctrex_ctx *ctx, const double *P, int n_views, int n_sub,
  *            pose is folded into them, so they are copied.
  *   cyl      HOST grid and pose (pose rotation orthonormal within 1e-9,
  *            det +1, else CTREX_E_ARG); n_phi >= 3.
- * Volumes are sampled through a texture atlas; one that exceeds the
- * device's 2D texture limits fails at the first projection with
+ * Volumes are sampled through a texture atlas or a column store; one that
+ * exceeds the device's 2D texture limits fails at the first projection with
  * CTREX_E_SHAPE.  set_motion (with parameters), adjoint_project and
  * motion_grad return CTREX_E_STATE on this domain.  Clears any motion, BP
  * window and earlier geometry; ctrex_set_geometry switches back.
@@ -225,8 +225,8 @@ int ctrex_set_bp_subvoxel(ctrex_ctx *ctx, int s);
  *       the unit direction), the path length between neighbouring planes.
  *       Row sums are the same sum of in-range weights.  count_samples then
  *       counts slice crossings with a tap inside the grid.  The context keeps
- *       the volume as x-, y- and z-slice stacks in one texture atlas (three
- *       copies; CTREX_E_SHAPE at the first projection if it exceeds the
+ *       the volume as columns along z, or as x-, y- and z-slice stacks in one
+ *       texture atlas (three copies; CTREX_E_SHAPE at the first projection if it exceeds the
  *       device's 2D texture limits).
  * Joseph is defined on the Cartesian grid without motion: CTREX_E_STATE if
  * the cylindrical domain or motion is set, and set_motion, adjoint_project
@@ -255,7 +255,7 @@ int ctrex_set_bp_subvoxel(ctrex_ctx *ctx, int s);
  * motion: CTREX_E_STATE on the cylindrical domain, with motion or with the
  * Joseph projector (and set_motion, set_projector(JOSEPH) and
  * adjoint_project return CTREX_E_STATE while an ROI is set).  Both grids are
- * sampled through texture atlases (CTREX_E_SHAPE at the first projection if
+ * sampled through texture atlases or column stores (CTREX_E_SHAPE at the first projection if
  * one exceeds the device's 2D texture limits).  NULL removes the ROI;
  * set_geometry and set_geometry_cylinder remove it too.
  */
@@ -281,7 +281,7 @@ int ctrex_set_roi(ctrex_ctx *ctx, const ctrex_vol_grid *roi);
  *   t_view  DEVICE float [n_views] acquisition time of each view (same
  *           unit as tau).
  * Both are copied on the stream (the caller may free them once the stream
- * has passed this call).  The context also keeps tau as a texture atlas and
+ * has passed this call).  The context also keeps tau as a texture atlas (column store) and
  * the smallest and largest tau of each 8^3 brick (over the brick and the
  * voxel past each upper face; 8 bytes per brick), with which the projector
  * takes one field for a whole footprint when the view's time lies on one
