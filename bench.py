@@ -288,10 +288,12 @@ def _time(fn, reps=3, warm=1):
     return s.elapsed_time(e) / 1e3 / reps
 
 
-# FP32 operations per motion-warped sample: 64-control-point cubic B-spline
-# (per point one weight product and three FMAs, plus per-axis weights), the
-# pose (9 FMA + 3), trilinear interpolation; counted from ray.cuh.
-MOTION_OPS_PER_SAMPLE = 64 * 4 + 16 + 3 * 10 + 12 + 30
+# FP32 operations per motion-warped sample of the 256^3 workload, by runs of
+# one spline cell (about 100 samples): Chebyshev values (8) and their sum with
+# the 10 coefficients (30), position under the pose (15), trilinear
+# interpolation (30), index and weight (12), and the run's fit, 10 passes over
+# the cell's 64 control points (25 a sample); counted from ray.cuh.
+MOTION_OPS_PER_SAMPLE = 8 + 30 + 15 + 30 + 12 + 25
 
 
 def sirt_50_iterations(ctx, cfg, p, device):
