@@ -104,7 +104,12 @@ int ctrex_create(ctrex_ctx **out, int device, void *cuda_stream);
 /* Free the context and every buffer it owns (synchronises its stream). */
 int ctrex_destroy(ctrex_ctx *ctx);
 
-/* Change the stream later calls enqueue on. */
+/*
+ * Change the stream later calls enqueue on.  The buffers that the context
+ * keeps for adjoint_project and motion_grad, and the column layouts of
+ * volumes and images, are ordered across streams: a call waits for the one
+ * that used them last.  The caller orders everything else.
+ */
 int ctrex_set_stream(ctrex_ctx *ctx, void *cuda_stream);
 
 /* Message of the last failed call on ctx (static text if ctx is NULL). */

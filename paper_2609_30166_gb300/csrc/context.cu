@@ -59,6 +59,9 @@ struct ctrex_ctx {
     float *d_adj = nullptr;  // the adjoint's scatter volume
     size_t adj_elems = 0;
     ColStore img_col;  // the correction images
+    // the last use of the stores and the scatter volume (ScratchUse)
+    cudaEvent_t scratch_done = nullptr;
+    bool scratch_open = false;
     // texture atlas of the correction images read by the backprojector
     AtlasStore img_atlas;
     Atlas img_atlas_view;
@@ -154,6 +157,41 @@ struct DeviceGuard {
     ~DeviceGuard()
     {
         if (prev >= 0) cudaSetDevice(prev);
+    }
+};
+
+// The column stores and the adjoint's scatter volume belong to the context,
+// while calls may run on different streams (ctrex_set_stream) with nothing
+// that orders them: a call waits for the last one's use before its own
+// (scratch_begin) and leaves an event behind it (ScratchUse, at the end of
+// the entry point).  A capturing stream can wait for no event outside its
+// graph; work replayed from a graph is ordered by the caller.
+bool capturing(const ctrex_ctx *c)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the legacy stream while another one captures
+    return true;
+}
+
+cudaError_t scratch_begin(ctrex_ctx *c)
+{
+    if (c->scratch_open || capturing(c)) return cudaSuccess;
+    c->scratch_open = true;
+    return cudaStreamWaitEvent(c->stream, c->scratch_done, 0);
+}
+
+struct ScratchUse {
+    ctrex_ctx *c;
+    explicit ScratchUse(ctrex_ctx *ctx) : c(ctx) {}
+    ~ScratchUse()
+    {
+        if (!c->scratch_open) return;
+        c->scratch_open = false;
+        if (cudaEventRecord(c->scratch_done, c->stream) != cudaSuccess) {
+            cudaGetLastError();
+            cudaStreamSynchronize(c->stream);
+        }
     }
 };
 
@@ -325,7 +363,9 @@ int prepare_columns(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     if ((c->cyl && !atlas_fits(nx, ny + 1, nz, d)) || (c->dyr && !atlas_fits(nx, ny, nz, d)) ||
         (c->roi && !(atlas_fits(nx, ny, nz, d) && atlas_fits(rx, ry, rz, d))))
         return CTREX_OK;
-    cudaError_t e = col_ensure(c->vol_col, nx, ny, nz, c->stream, c->cyl);
+    cudaError_t e = scratch_begin(c);
+    if (e != cudaSuccess) return cuda_fail(c, e, "column scratch");
+    e = col_ensure(c->vol_col, nx, ny, nz, c->stream, c->cyl);
     if (e == cudaSuccess && c->dyr) e = col_ensure(c->col1, nx, ny, nz, c->stream);
     if (e == cudaSuccess && c->roi) e = col_ensure(c->col1, rx, ry, rz, c->stream);
     if (e == cudaSuccess && c->dyr && !c->tau_col_set) {
@@ -501,7 +541,8 @@ int ctrex_create(ctrex_ctx **out, int device, void *stream)
     DeviceGuard g(device);
     if (cudaMalloc((void **)&c->d_sums, 2 * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_devcheck, sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc((void **)&c->d_count, sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMalloc((void **)&c->d_count, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         ctrex_destroy(c);
         return CTREX_E_NOMEM;
@@ -540,6 +581,7 @@ int ctrex_destroy(ctrex_ctx *c)
         if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
         if (c->ev_vol) cudaEventDestroy(c->ev_vol);
         if (c->ev_p) cudaEventDestroy(c->ev_p);
+        if (c->scratch_done) cudaEventDestroy(c->scratch_done);
         if (c->sums_done) cudaEventDestroy(c->sums_done);
         if (c->h_sums) cudaFreeHost(c->h_sums);
         dfree(c->d_subset_views);
@@ -1054,6 +1096,7 @@ int ctrex_fwd_project(ctrex_ctx *c, const void *vol, int vdt, void *proj, int pd
     if (!vol || !proj) return fail(c, CTREX_E_ARG, "fwd_project: NULL buffer");
     if (!dtype_ok(vdt) || !dtype_ok(pdt)) return fail(c, CTREX_E_DTYPE, "fwd_project: bad dtype");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     FwdArgs a = fwd_args(c, vol, vdt, view_idx, n_idx);
     e = prepare_atlas(c, a, vol, vdt);
     if (e) return e;
@@ -1087,6 +1130,7 @@ int ctrex_fwd_correct(ctrex_ctx *c, const void *vol, int vdt, const void *p, int
     if (!dtype_ok(vdt) || !dtype_ok(pdt) || !dtype_ok(rdt)) return fail(c, CTREX_E_DTYPE, "fwd_correct: bad dtype");
     if (pdt != rdt) return fail(c, CTREX_E_DTYPE, "fwd_correct: p and r must share one dtype");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     e = ensure_partials(c, n_idx);
     if (e) return e;
     FwdArgs a = fwd_args(c, vol, vdt, view_idx, n_idx);
@@ -1102,6 +1146,7 @@ int ctrex_fwd_correct(ctrex_ctx *c, const void *vol, int vdt, const void *p, int
 static int bp_images(ctrex_ctx *c, BpArgs &a, const void *r, int rdt, int n_idx)
 {
     if (n_idx > 0 && column_backproject(c)) {
+        CT_CUDA(c, scratch_begin(c));
         cudaError_t ae = col_ensure_images(c->img_col, c->grid.nu, c->grid.nv, n_idx, c->stream);
         if (ae == cudaSuccess) {
             ae = col_upload_images(c->img_col, r, rdt, n_idx, c->stream);
@@ -1175,6 +1220,7 @@ int ctrex_back_project(ctrex_ctx *c, const void *r, int rdt, void *vol, int vdt,
     if (!dtype_ok(vdt) || !dtype_ok(rdt)) return fail(c, CTREX_E_DTYPE, "back_project: bad dtype");
     if (!isfinite(alpha)) return fail(c, CTREX_E_ARG, "back_project: alpha not finite");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     BpArgs a;
     e = bp_images(c, a, r, rdt, n_idx);
     return e ? e : bp_run(c, a, r, rdt, vol, vdt, w, alpha, normalize, accumulate, view_idx, n_idx);
@@ -1191,11 +1237,13 @@ int ctrex_adjoint_project(ctrex_ctx *c, const float *proj, float *vol, const int
     if (n_idx == 0) return CTREX_OK;
     if (!proj || !vol) return fail(c, CTREX_E_ARG, "adjoint_project: NULL buffer");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     const FwdArgs a = fwd_args(c, nullptr, CTREX_F32, view_idx, n_idx);
     cudaError_t ce;
-    if (column_adjoint(c, n_idx))
+    if (column_adjoint(c, n_idx)) {
+        CT_CUDA(c, scratch_begin(c));
         ce = launch_adjoint_column(a, c->col_lean <= COL_LEAN_ADJ, proj, vol, c->d_adj);
-    else
+    } else
         ce = launch_adjoint(a, proj, vol);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "adjoint_project launch");
     return CTREX_OK;
@@ -1216,7 +1264,9 @@ int ctrex_motion_grad(ctrex_ctx *c, const void *vol, int vdt, const float *gproj
     if (grad_coef && !c->coef_valid)
         return fail(c, CTREX_E_STATE, "motion_grad: grad_coef requested but no coefficients were set");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     const int V = c->grid.n_views;
+    CT_CUDA(c, scratch_begin(c));
     CT_CUDA(c, cudaMemsetAsync(c->d_gM, 0, sizeof(double) * 9 * (size_t)V, c->stream));
     CT_CUDA(c, cudaMemsetAsync(c->d_gb, 0, sizeof(double) * 3 * (size_t)V, c->stream));
     CT_CUDA(c, cudaMemsetAsync(c->d_gcoef, 0, sizeof(double) * 1536, c->stream));
@@ -1245,6 +1295,7 @@ int ctrex_sirt_iterate(ctrex_ctx *c, void *vol, int vdt, const void *p, int pdt,
     if (!dtype_ok(vdt) || !dtype_ok(pdt)) return fail(c, CTREX_E_DTYPE, "sirt_iterate: bad dtype");
     if (max_iter < 0) return fail(c, CTREX_E_ARG, "sirt_iterate: max_iter < 0");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     const int V = c->grid.n_views;
     const size_t rb = (size_t)V * c->grid.nu * c->grid.nv * dtype_size(pdt);
     e = ensure(c, &c->d_r, &c->r_bytes, rb, "SIRT correction images");
@@ -1303,6 +1354,7 @@ int ctrex_os_sirt_iterate(ctrex_ctx *c, void *vol, int vdt, const void *p, int p
         if (subset_views[i] < 0 || subset_views[i] >= V)
             return fail(c, CTREX_E_SHAPE, "os_sirt: view %d out of range", subset_views[i]);
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     int e = ensure(c, (void **)&c->d_subset_views, &c->subset_views_bytes, sizeof(int) * (size_t)(total > 0 ? total : 1),
                    "subset view lists");
     if (e) return e;
@@ -1360,6 +1412,7 @@ int ctrex_sirt_host(ctrex_ctx *c, void *vol_h, int vdt, const void *p_h, int pdt
     if (!vol_h || !p_h) return fail(c, CTREX_E_ARG, "sirt_host: NULL buffer");
     if (!dtype_ok(vdt) || !dtype_ok(pdt)) return fail(c, CTREX_E_DTYPE, "sirt_host: bad dtype");
     DeviceGuard g(c->device);
+    ScratchUse use(c);
     const Grid &G = c->grid;
     const size_t nvox = volume_elems(c);
     const size_t vb = nvox * dtype_size(vdt);
