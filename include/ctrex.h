@@ -351,7 +351,10 @@ int ctrex_back_project(ctrex_ctx *ctx, const void *r, int r_dtype, void *vol, in
  * Matched adjoint of ctrex_fwd_project (exact transpose, motion included):
  * vol += A^T proj, scattered with FP32 atomics (summation order is not
  * reproducible bit for bit).  The paper has no such operator; it is the
- * transpose of its Sec. 4.1 projector, used for gradients.
+ * transpose of its Sec. 4.1 projector, used for gradients.  The context keeps
+ * a zeroed volume that it scatters through (4 bytes a voxel, allocated by the
+ * first call; at most half of the free memory, else vol itself); while the
+ * stream captures, vol itself takes the reductions and nothing is allocated.
  *   proj     DEVICE float [n_idx][nv][nu];  vol  DEVICE float [nz][ny][nx].
  */
 int ctrex_adjoint_project(ctrex_ctx *ctx, const float *proj, float *vol, const int *view_idx,
@@ -364,6 +367,9 @@ int ctrex_adjoint_project(ctrex_ctx *ctx, const float *proj, float *vol, const i
  *   grad_proj   DEVICE float [n_idx][nv][nu] (= g).
  *   grad_theta  DEVICE float [n_views][15], accumulated (+=), or NULL.
  *   grad_coef   DEVICE float [8][8][8][3], accumulated (+=), or NULL.
+ * vol is read through the context's column store (8 bytes a voxel, allocated
+ * by the first call; at most half of the free memory, else vol itself); while
+ * the stream captures, vol itself is read and nothing is allocated.
  */
 int ctrex_motion_grad(ctrex_ctx *ctx, const void *vol, int vol_dtype, const float *grad_proj,
                       float *grad_theta, float *grad_coef, const int *view_idx, int n_idx);

@@ -9,9 +9,11 @@ void col_release(ColStore &s)
     s = ColStore();
 }
 
-// At least n zeroed pairs.
+// At least n zeroed pairs.  Not in a capture, where the zeros would be written
+// by the replay while the store counts as laid out at once.
 static cudaError_t col_alloc(ColStore &s, size_t n, cudaStream_t stream)
 {
+    if (stream_capturing(stream)) return cudaErrorInvalidValue;
     const size_t bytes = n * sizeof(float2);
     s.nx = 0;
     if (bytes > s.bytes) {

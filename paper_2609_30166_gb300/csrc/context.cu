@@ -137,6 +137,7 @@ int fail(ctrex_ctx *c, int code, const char *fmt, ...)
 
 int cuda_fail(ctrex_ctx *c, cudaError_t e, const char *where)
 {
+    cudaGetLastError();  // not for the next call to find after its launches
     return fail(c, e == cudaErrorMemoryAllocation ? CTREX_E_NOMEM : CTREX_E_CUDA, "%s: %s (%s)", where,
                 cudaGetErrorString(e), cudaGetErrorName(e));
 }
@@ -165,14 +166,9 @@ struct DeviceGuard {
 // that orders them: a call waits for the last one's use before its own
 // (scratch_begin) and leaves an event behind it (ScratchUse, at the end of
 // the entry point).  A capturing stream can wait for no event outside its
-// graph; work replayed from a graph is ordered by the caller.
-bool capturing(const ctrex_ctx *c)
-{
-    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
-    cudaGetLastError();  // the legacy stream while another one captures
-    return true;
-}
+// graph, nor allocate: what read the caller's buffers alone before there were
+// stores does so there, and work replayed from a graph is ordered by the caller.
+bool capturing(const ctrex_ctx *c) { return stream_capturing(c->stream); }
 
 cudaError_t scratch_begin(ctrex_ctx *c)
 {
@@ -331,7 +327,7 @@ bool column_backproject(const ctrex_ctx *c)
 bool column_adjoint(ctrex_ctx *c, int n_idx)
 {
     const Grid &G = c->grid;
-    if (c->dyr) return false;
+    if (c->dyr || capturing(c)) return false;
     const double reach = fmax(G.nx, fmax(G.ny, G.nz));  // voxels of a ray, about
     if ((double)n_idx * G.n_sub * G.nu * G.nv * reach < 0.03 * (double)grid_voxels(G)) return false;
     const size_t n = adjoint_column_elems(G);
@@ -369,7 +365,7 @@ int prepare_columns(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     if (e == cudaSuccess && c->dyr) e = col_ensure(c->col1, nx, ny, nz, c->stream);
     if (e == cudaSuccess && c->roi) e = col_ensure(c->col1, rx, ry, rz, c->stream);
     if (e == cudaSuccess && c->dyr && !c->tau_col_set) {
-        e = col_ensure(c->tau_col, nx, ny, nz, c->stream);
+        e = capturing(c) ? cudaErrorInvalidValue : col_ensure(c->tau_col, nx, ny, nz, c->stream);
         if (e == cudaSuccess) e = col_upload(c->tau_col, c->d_tau, CTREX_F32, c->stream, true);
         c->tau_col_set = e == cudaSuccess;
     }
@@ -1272,7 +1268,7 @@ int ctrex_motion_grad(ctrex_ctx *c, const void *vol, int vdt, const float *gproj
     CT_CUDA(c, cudaMemsetAsync(c->d_gcoef, 0, sizeof(double) * 1536, c->stream));
     FwdArgs a = fwd_args(c, vol, vdt, view_idx, n_idx);
     // the volume from its column store if that can be had, row-major otherwise
-    if (col_ensure(c->vol_col, c->grid.nx, c->grid.ny, c->grid.nz, c->stream) == cudaSuccess) {
+    if (!capturing(c) && col_ensure(c->vol_col, c->grid.nx, c->grid.ny, c->grid.nz, c->stream) == cudaSuccess) {
         CT_CUDA(c, col_upload(c->vol_col, vol, vdt, c->stream));
         a.column = &c->vol_col;
     }

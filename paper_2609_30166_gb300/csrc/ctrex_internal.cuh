@@ -96,6 +96,16 @@ template <> struct Storage<__nv_bfloat16> {
 __device__ __forceinline__ float2 two(float x) { return make_float2(x, x); }
 #endif
 
+// Whether a stream captures its work into a graph (true also where that
+// cannot be told: the legacy stream while another stream captures).
+inline bool stream_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Status word written by kernels whose own bounds checks fire (never trap).
 enum : unsigned { DEVCHECK_OOB = 1u };
 
