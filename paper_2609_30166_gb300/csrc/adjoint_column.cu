@@ -231,15 +231,29 @@ size_t adjoint_column_elems(const Grid &G)
     return n < (1ull << 32) && (G.nz + 31) / 32 <= 65535 ? n : 0;
 }
 
+// Tiles of a strip, list entries, strips x bands, with lv lanes along v.
+static dim3 adj_grid(const Grid &G, int n_idx, int lv, int &n_strips)
+{
+    const int tu = 4 * (32 / lv);  // columns per CTA
+    const int tiles = (G.nu + tu - 1) / tu, strip = 128 / tu, per = tiles < strip ? tiles : strip;
+    n_strips = (tiles + per - 1) / per;
+    return dim3(per, n_idx, (unsigned)n_strips * (unsigned)((G.nv + lv - 1) / lv));
+}
+
+static int adj_lanes(bool motion, bool along_z) { return !motion && along_z ? ADJ_LV : ADJ_LV_PATCH; }
+
+bool adjoint_column_fits(const Grid &G, bool motion, bool along_z)
+{
+    int n_strips;
+    return adj_grid(G, 1, adj_lanes(motion, along_z), n_strips).z <= 65535;
+}
+
 template <bool MOTION, int LV, bool RUNS = false>
 static cudaError_t adj_launch(const FwdArgs &a, const float *proj, const AdjVolume &V)
 {
     const Grid &G = *a.grid;
-    constexpr int TU = 4 * (32 / LV);  // columns per CTA
-    const int tiles = (G.nu + TU - 1) / TU, strip = 128 / TU, per = tiles < strip ? tiles : strip;
-    const int n_strips = (tiles + per - 1) / per;
-    const dim3 grid(per, a.n_idx, n_strips * ((G.nv + LV - 1) / LV));
-    if (grid.z > 65535) return cudaErrorNotSupported;
+    int n_strips;
+    const dim3 grid = adj_grid(G, a.n_idx, LV, n_strips);
     adjoint_column_kernel<MOTION, LV, RUNS><<<grid, 128, 0, a.stream>>>(
         G, a.views, MOTION ? a.motion : nullptr, MOTION ? a.spline : nullptr, a.view_idx, proj, V, a.devcheck, n_strips);
     return cudaGetLastError();

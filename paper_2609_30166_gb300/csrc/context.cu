@@ -321,13 +321,16 @@ bool column_backproject(const ctrex_ctx *c)
            (!c->roi || backproject_column_fits(c->roi_grid));
 }
 
-// The adjoint through a scatter volume, if that can be had: it is zeroed and
+bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ; }
+
+// The adjoint through a scatter volume, if that can be had (and the launch, an
+// 8192^2 detector with motion is beyond it): it is zeroed and
 // added once per call, so the call's rays have to outweigh it (one view of
 // 64^2 pixels on 512^3: 0.71 ms, 0.65 in place; 768^2: 1.7, 3.6 in place).
 bool column_adjoint(ctrex_ctx *c, int n_idx)
 {
     const Grid &G = c->grid;
-    if (c->dyr || capturing(c)) return false;
+    if (c->dyr || capturing(c) || !adjoint_column_fits(G, c->has_motion, adjoint_along_z(c))) return false;
     const double reach = fmax(G.nx, fmax(G.ny, G.nz));  // voxels of a ray, about
     if ((double)n_idx * G.n_sub * G.nu * G.nv * reach < 0.03 * (double)grid_voxels(G)) return false;
     const size_t n = adjoint_column_elems(G);
@@ -1238,9 +1241,10 @@ int ctrex_adjoint_project(ctrex_ctx *c, const float *proj, float *vol, const int
     cudaError_t ce;
     if (column_adjoint(c, n_idx)) {
         CT_CUDA(c, scratch_begin(c));
-        ce = launch_adjoint_column(a, c->col_lean <= COL_LEAN_ADJ, proj, vol, c->d_adj);
-    } else
+        ce = launch_adjoint_column(a, adjoint_along_z(c), proj, vol, c->d_adj);
+    } else {
         ce = launch_adjoint(a, proj, vol);
+    }
     if (ce != cudaSuccess) return cuda_fail(c, ce, "adjoint_project launch");
     return CTREX_OK;
 }

@@ -326,3 +326,37 @@ def test_correction_norm_by_tiles(det, dtype):
         assert abs(sums[1].item() - want) <= 1e-13 * want
     c.close()
 
+
+
+# Detectors whose 8-row bands are more than a launch holds: 300 x 262140 pixels,
+# of which the object's shadow takes the middle rows (rays are formed relative
+# to the detector's middle in FP32).  Reference: the same rays on a detector of
+# those rows alone.
+@pytest.mark.parametrize("motion,turn", [(True, 0.0), (False, 20.0)])
+def test_adjoint_of_tall_detector(motion, turn):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    nu, nv, shadow, shape = 300, 262140, 100, (20, 18, 16)
+    vox, org = (1.0, 1.0, 1.0), tuple(-0.5 * (m - 1) for m in shape[::-1])
+    P = _matrices(1, 1, turn, nu, shadow, 96.0, 200.0)
+    first = (nv - shadow) // 2
+    rng = np.random.default_rng(8)
+    pb = oracle.Problem(P, shape, vox, org, (nu, shadow), 0.5)
+    c = ctrex.Context()
+    shift = np.array([[1.0, 0.0, 0.0], [0.0, 1.0, first], [0.0, 0.0, 1.0]])
+    c.set_geometry(shift @ P, shape, vox, org, (nu, nv))  # the same rows, and more on both sides
+    if motion:
+        theta = np.zeros((1, 15))
+        theta[:, :6] = rng.uniform(-0.02, 0.02, (1, 6))
+        theta[:, 6:] = np.eye(3).ravel()
+        coef, sv = rng.uniform(-1, 1, (8, 8, 8, 3)), np.ones(1)
+        theta, coef = _np(_t(theta)), _np(_t(coef))
+        pb = pb.with_motion(theta, coef, sv, margin=0.5)
+        c.set_motion(_t(theta), _t(coef), _t(sv), 0.5)
+    y = torch.zeros((1, nv, nu), device="cuda")
+    rows = y[:, first:first + shadow]
+    rows.copy_(_t(rng.uniform(0.5, 1.5, size=(1, shadow, nu))))
+    want = oracle.adjoint(pb, _np(rows))
+    assert rel_l2(_np(c.adjoint_project(y)), want) <= TOL32
+    c.close()
