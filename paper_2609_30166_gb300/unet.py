@@ -131,6 +131,9 @@ class UNet3D(torch.nn.Module):
             return None
         if torch.is_autocast_enabled() or torch.jit.is_tracing() or torch.compiler.is_compiling():
             return None
+        # a dual (forward-mode) tensor is a plain tensor without requires_grad
+        if any(torch.autograd.forward_ad.unpack_dual(t).tangent is not None for t in tensors):
+            return None
         if torch._C._functorch.peek_interpreter_stack() is not None or torch._C._len_torch_dispatch_stack() \
                 or torch._C._len_torch_function_stack():
             return None

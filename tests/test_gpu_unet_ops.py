@@ -70,3 +70,31 @@ def test_one_call_forward(mods, shape, base):
         assert net._one_call(x.transpose(1, 2)) is None and net._one_call(x.double()) is None
     assert net._one_call(x) is None
     ctrex.conv_status_check()
+
+
+def _net(unet):
+    return unet.UNet3D(base=8, seed=3).cuda(), torch.rand((1, 8, 8, 8), device="cuda")
+
+
+def test_forward_mode_is_refused(mods):
+    """The layers have no forward-mode derivative: a dual input or parameter
+    raises, as it does with gradients enabled, and is never taken for a
+    constant."""
+    _, unet = mods
+    import torch.autograd.forward_ad as fwd
+
+    net, x = _net(unet)
+    with torch.no_grad(), fwd.dual_level():
+        for name, grad in ((None, False), ("e1.0.w", False), ("head_b", False)):
+            if name is None:
+                with pytest.raises(NotImplementedError):
+                    net(fwd.make_dual(x, torch.ones_like(x)))
+            else:
+                p = dict(net.named_parameters())[name]
+                dual = fwd.make_dual(p.detach(), torch.ones_like(p))
+                if name == "head_b":  # the head alone is made of differentiable operations
+                    y = torch.func.functional_call(net, {name: dual}, (x,))
+                    assert fwd.unpack_dual(y).tangent is not None
+                else:
+                    with pytest.raises(NotImplementedError):
+                        torch.func.functional_call(net, {name: dual}, (x,))
