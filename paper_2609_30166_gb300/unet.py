@@ -113,8 +113,11 @@ class UNet3D(torch.nn.Module):
 
     def _one_call(self, x):
         """The layers' parameters if the whole pass can run as one native call:
-        plain inference of an unmodified network (no gradients, hooks, tracing
-        or tensor subclasses that would have to see the single operations)."""
+        plain inference of an unmodified network (no subclass, replaced method,
+        gradients, hooks, tracing or tensor subclasses that would have to see
+        the single operations)."""
+        if type(self) is not UNet3D or not self.__dict__.keys().isdisjoint(("forward", "_block", "_layers")):
+            return None
         layers = self._layers()
         params = list(self.parameters())
         tensors = [x] + params
@@ -123,7 +126,8 @@ class UNet3D(torch.nn.Module):
         if any(type(t) not in (torch.Tensor, torch.nn.Parameter) or t.dtype != torch.float32 or t.device != x.device
                or not t.is_contiguous() for t in tensors) or x.device.type != "cuda" or x.dim() != 4:
             return None
-        if len(layers) != 14 or len(params) != 30 or any(type(c) is not Conv3 or not c.relu for c in layers):
+        if len(layers) != 14 or len(params) != 30 or any(
+                type(c) is not Conv3 or "forward" in c.__dict__ or not c.relu for c in layers):
             return None
         m = torch.nn.modules.module
         if m._global_forward_hooks or m._global_forward_pre_hooks or any(

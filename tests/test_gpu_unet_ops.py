@@ -98,3 +98,40 @@ def test_forward_mode_is_refused(mods):
                 else:
                     with pytest.raises(NotImplementedError):
                         torch.func.functional_call(net, {name: dual}, (x,))
+
+
+def test_replaced_layers_are_called(mods):
+    """Offloading and instrumentation replace a layer's forward on the
+    instance, or override a part of the network in a subclass."""
+    _, unet = mods
+    net, x = _net(unet)
+    seen = []
+    layer = net.e1[0]
+    plain = layer.forward
+
+    def wrapped(v):
+        seen.append("forward")
+        return plain(v)
+
+    class Sub(unet.UNet3D):
+        @staticmethod
+        def _block(convs, v):
+            seen.append("subclass")
+            return unet.UNet3D._block(convs, v)
+
+    def block(convs, v):
+        seen.append("block")
+        return unet.UNet3D._block(convs, v)
+
+    with torch.no_grad():
+        layer.forward = wrapped
+        net(x)
+        assert seen == ["forward"]
+        del layer.forward, seen[:]
+        sub = Sub(base=8, seed=3).cuda()
+        sub(x)
+        assert seen == ["subclass"] * 7
+        del seen[:]
+        net._block = block
+        net(x)
+        assert seen == ["block"] * 7
