@@ -138,8 +138,12 @@ class UNet3D(torch.nn.Module):
         # a dual (forward-mode) tensor is a plain tensor without requires_grad
         if any(torch.autograd.forward_ad.unpack_dual(t).tangent is not None for t in tensors):
             return None
-        if torch._C._functorch.peek_interpreter_stack() is not None or torch._C._len_torch_dispatch_stack() \
-                or torch._C._len_torch_function_stack():
+        try:  # transforms and modes; private names, which another torch may not have
+            c = torch._C
+            if c._functorch.peek_interpreter_stack() is not None or c._len_torch_dispatch_stack() \
+                    or c._len_torch_function_stack():
+                return None
+        except AttributeError:
             return None
         nb, d, h, w = x.shape
         c1 = self.head_w.numel()

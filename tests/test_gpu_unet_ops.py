@@ -135,3 +135,18 @@ def test_replaced_layers_are_called(mods):
         net._block = block
         net(x)
         assert seen == ["block"] * 7
+
+
+@pytest.mark.parametrize("where,name", [("_functorch", "peek_interpreter_stack"), (None, "_len_torch_dispatch_stack"),
+                                        (None, "_len_torch_function_stack")])
+def test_inference_without_private_names(mods, monkeypatch, where, name):
+    """A torch that does not tell what is active keeps the layers."""
+    _, unet = mods
+    net, x = _net(unet)
+    with torch.no_grad():
+        want = net(x)
+        monkeypatch.delattr(getattr(torch._C, where) if where else torch._C, name)
+        assert net._one_call(x) is None
+        got = net(x)
+    monkeypatch.undo()
+    assert torch.allclose(got, want, rtol=0, atol=1e-5)
