@@ -37,8 +37,10 @@ class _Conv3(torch.autograd.Function):
     def backward(actx, dy):
         x, wb, y = actx.saved_tensors
         dy = dy.to(torch.bfloat16).contiguous()
-        # ReLU mask and bias gradient in one pass
-        both = ctrex.conv3d_bias_grad(dy, y if actx.relu else None) if actx.needs_input_grad[2] else None
+        # ReLU mask and bias gradient in one pass; with create_graph (gradients
+        # enabled here) by operations that can be differentiated again
+        fused = actx.needs_input_grad[2] and not torch.is_grad_enabled()
+        both = ctrex.conv3d_bias_grad(dy, y if actx.relu else None) if fused else None
         if both is not None:
             dy, db = both
         else:

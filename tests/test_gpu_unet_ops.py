@@ -150,3 +150,20 @@ def test_inference_without_private_names(mods, monkeypatch, where, name):
         got = net(x)
     monkeypatch.undo()
     assert torch.allclose(got, want, rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("relu", [True, False])
+def test_second_derivative_through_the_bias_gradient(mods, relu):
+    """With create_graph the bias gradient is a function of the output's
+    gradient: sum over the voxels of dy (where the ReLU passes)."""
+    _, unet = mods
+    layer = unet.Conv3(16, 16, relu=relu, gen=torch.Generator().manual_seed(2)).cuda()
+    x = torch.randn((1, 4, 6, 8, 16), device="cuda").to(torch.bfloat16)
+    y = layer(x)
+    dy = torch.randn(y.shape, device="cuda").to(torch.bfloat16).requires_grad_(True)
+    (db,) = torch.autograd.grad(y, layer.b, grad_outputs=dy, create_graph=True)
+    assert db.requires_grad
+    k = torch.arange(1.0, 17.0, device="cuda")
+    (g,) = torch.autograd.grad((db * k).sum(), dy)
+    mask = (y > 0) if relu else torch.ones_like(y)
+    assert torch.equal(g, (mask * k).to(g.dtype))
