@@ -546,11 +546,19 @@ def conv3d_bias_grad(dy, y=None):
     """(g, db) of a layer's activation and bias for the output gradient dy
     (bf16, channels last): g = dy * (y > 0) with the layer's output y (its
     ReLU's), dy itself without; db [channels] float32 = g summed over the
-    voxels.  None if the layer's channel count is not one the kernel takes."""
+    voxels.  None if the kernel does not take the layer's channel count, the
+    tensors' layout, or tensors without memory of their own (vmap's)."""
     c = dy.shape[-1]
-    if c % 8 or (c // 8) & (c // 8 - 1) or c // 8 > 256 or dy.numel() == 0 or dy.data_ptr() % 16:
+    if c % 8 or (c // 8) & (c // 8 - 1) or c // 8 > 256 or dy.numel() == 0:
         return None
-    if y is not None and (y.shape != dy.shape or y.dtype != dy.dtype or not y.is_contiguous() or y.data_ptr() % 16):
+    if dy.dtype != torch.bfloat16 or dy.device.type != "cuda" or not dy.is_contiguous():
+        return None
+    if y is not None and (y.shape != dy.shape or y.dtype != dy.dtype or not y.is_contiguous()):
+        return None
+    try:
+        if dy.data_ptr() % 16 or y is not None and y.data_ptr() % 16:
+            return None
+    except RuntimeError:
         return None
     lib = load_library()
     g = dy if y is None else torch.empty_like(dy)

@@ -22,6 +22,18 @@ import torch
 from . import ctrex, inputs
 
 
+def _observed():
+    """Whether a function transform (vmap and the like) or a mode is active
+    that has to see single torch operations.  The queries are private names:
+    a torch that lacks one counts as observed."""
+    try:
+        c = torch._C
+        return (c._functorch.peek_interpreter_stack() is not None or c._len_torch_dispatch_stack() > 0
+                or c._len_torch_function_stack() > 0)
+    except AttributeError:
+        return True
+
+
 class _Conv3(torch.autograd.Function):
     """y = act(conv3x3x3(x, w) + b), act = ReLU or identity."""
 
@@ -38,8 +50,8 @@ class _Conv3(torch.autograd.Function):
         x, wb, y = actx.saved_tensors
         dy = dy.to(torch.bfloat16).contiguous()
         # ReLU mask and bias gradient in one pass; with create_graph (gradients
-        # enabled here) by operations that can be differentiated again
-        fused = actx.needs_input_grad[2] and not torch.is_grad_enabled()
+        # enabled here) and under a transform by torch operations
+        fused = actx.needs_input_grad[2] and not torch.is_grad_enabled() and not _observed()
         both = ctrex.conv3d_bias_grad(dy, y if actx.relu else None) if fused else None
         if both is not None:
             dy, db = both
@@ -140,12 +152,7 @@ class UNet3D(torch.nn.Module):
         # a dual (forward-mode) tensor is a plain tensor without requires_grad
         if any(torch.autograd.forward_ad.unpack_dual(t).tangent is not None for t in tensors):
             return None
-        try:  # transforms and modes; private names, which another torch may not have
-            c = torch._C
-            if c._functorch.peek_interpreter_stack() is not None or c._len_torch_dispatch_stack() \
-                    or c._len_torch_function_stack():
-                return None
-        except AttributeError:
+        if _observed():
             return None
         nb, d, h, w = x.shape
         c1 = self.head_w.numel()

@@ -167,3 +167,18 @@ def test_second_derivative_through_the_bias_gradient(mods, relu):
     (g,) = torch.autograd.grad((db * k).sum(), dy)
     mask = (y > 0) if relu else torch.ones_like(y)
     assert torch.equal(g, (mask * k).to(g.dtype))
+
+
+@pytest.mark.parametrize("relu", [True, False])
+def test_batched_bias_gradient(mods, relu):
+    """Several output gradients at once (vmap over the backward pass), where
+    only the bias asks for a gradient."""
+    _, unet = mods
+    layer = unet.Conv3(16, 16, relu=relu, gen=torch.Generator().manual_seed(2)).cuda()
+    layer.w.requires_grad_(False)
+    y = layer(torch.randn((1, 4, 6, 8, 16), device="cuda").to(torch.bfloat16))
+    dy = torch.randn((3,) + y.shape, device="cuda").to(torch.bfloat16)
+    (db,) = torch.autograd.grad(y, layer.b, grad_outputs=dy, is_grads_batched=True, retain_graph=True)
+    for k in range(3):
+        (want,) = torch.autograd.grad(y, layer.b, grad_outputs=dy[k], retain_graph=True)
+        assert torch.allclose(db[k], want, rtol=0, atol=8 * 2.0 ** -24 * float(dy[k].float().abs().sum()))
