@@ -10,6 +10,8 @@
 // tiles): the CTAs resident at one time cover a band of detector rows across
 // many views, whose rays all cross the same z-slab of the volume, so that
 // slab stays in L2 while it is being sampled.
+#include <cooperative_groups.h>
+
 #include "atlas.cuh"
 #include "cylinder.cuh"
 #include "dyrect.cuh"
@@ -257,49 +259,32 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY, Sampler::MIN_BLOCKS > 0 ? Samp
                                        devcheck, p_by_view);
 }
 
-// Second pass of the residual reduction, FP64 in a fixed order: CTA b sums a
-// contiguous part of the n pairs; a single CTA writes the result, several
-// write theirs for a last launch to sum.  (FP64 from the first add on
-// took 12 us for the 6480 pairs of a 64^3 iteration, this 8 us.)
-struct SumFloat {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x)  // Knuth's two-sum
-    {
-        const float s = __fadd_rn(hi, x), t = __fadd_rn(s, -hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -t)), __fadd_rn(x, -t)));
-        hi = s;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-struct SumDouble {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <typename T> struct SumPart { typedef SumDouble type; };
-template <> struct SumPart<float> { typedef SumFloat type; };
+// Second pass of the residual reduction, FP64 from the first add in a fixed
+// order: CTA b sums a contiguous part of the n pairs, a cluster of CTAs adds
+// its parts in order and writes one pair (several clusters leave theirs for a
+// last launch).  FP64 adds and conversions run at two per clock and SM, so the
+// single CTA that a 64^3 iteration's 6480 pairs would fill is bound by them:
+// FINISH_TIMES.
+constexpr int FINISH_CLUSTER = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ pairs, size_t n, double *__restrict__ out,
-                                                          size_t second = 0, size_t n2 = 0)
+__global__ void __cluster_dims__(FINISH_CLUSTER, 1, 1) __launch_bounds__(512)
+    finish_sums_kernel(const T *__restrict__ pairs, size_t n, double *__restrict__ out, size_t second = 0, size_t n2 = 0)
 {
-    __shared__ double s[2][16];
+    namespace cg = cooperative_groups;
+    __shared__ double s[2][16], part[2];
     const size_t per = (n + gridDim.x - 1) / gridDim.x, i0 = per * blockIdx.x, i1 = min(i0 + per, n);
-    // per thread in compensated FP32 (exact to ~2^-48 over a few dozen
-    // terms: FP64 adds and conversions run at a fraction of the rate)
-    typedef typename SumPart<T>::type S;
-    S sa, sb;
+    double a = 0.0, b = 0.0;
 #pragma unroll 4
     for (size_t i = i0 + threadIdx.x; i < i1; i += 512) {
-        sa.add(pairs[2 * i]);
-        if (n2 == 0) sb.add(pairs[2 * i + 1]);
+        a += (double)pairs[2 * i];
+        if (n2 == 0) b += (double)pairs[2 * i + 1];
     }
     // n2: the second sum is that of the n2 pairs from `second` on
     const size_t per2 = (n2 + gridDim.x - 1) / gridDim.x, j0 = second + per2 * blockIdx.x,
                  j1 = min(j0 + per2, second + n2);
 #pragma unroll 4
-    for (size_t i = j0 + threadIdx.x; i < j1; i += 512) sb.add(pairs[2 * i + 1]);
-    double a = sa.value(), b = sb.value();
+    for (size_t i = j0 + threadIdx.x; i < j1; i += 512) b += (double)pairs[2 * i + 1];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, off);
@@ -313,8 +298,16 @@ __global__ void __launch_bounds__(512) finish_sums_kernel(const T *__restrict__ 
     if (threadIdx.x < 2) {
         double t = 0.0;
         for (int w = 0; w < 16; ++w) t += s[threadIdx.x][w];
-        out[2 * blockIdx.x + threadIdx.x] = t;
+        part[threadIdx.x] = t;
     }
+    const cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x < 2) {
+        double t = 0.0;
+        for (int r = 0; r < FINISH_CLUSTER; ++r) t += *cluster.map_shared_rank(part + threadIdx.x, r);
+        out[2 * (blockIdx.x / FINISH_CLUSTER) + threadIdx.x] = t;
+    }
+    cluster.sync();  // the parts are read before their CTAs end
 }
 
 // |p|^2 in the texture kernel's tiles of 32 x 4 pixels and its order of
@@ -388,7 +381,10 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY)
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(out, n);
 }
 
-constexpr int FINISH_ONE = 16384, FINISH_CTAS = 152;
+// Pairs up to which one cluster sums alone (one launch / two: 25,600 pairs 9.3 /
+// 12.8 us, 51,200 12.8 / 13.1, 102,400 20.7 / 14.6), and the CTAs beyond.
+constexpr int FINISH_ONE = 49152, FINISH_CTAS = 152;
+static_assert(FINISH_CTAS % FINISH_CLUSTER == 0, "whole clusters");
 
 static dim3 fwd_grid(const Grid &G, int n_idx)
 {
@@ -512,11 +508,11 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
                                                           static_cast<const __nv_bfloat16 *>(p), partials + 2 * (size_t)n);
     }
     if (n <= FINISH_ONE) {
-        finish_sums_kernel<<<1, 512, 0, a.stream>>>(partials, (size_t)n, sums, (size_t)n, nt);
+        finish_sums_kernel<<<FINISH_CLUSTER, 512, 0, a.stream>>>(partials, (size_t)n, sums, (size_t)n, nt);
     } else {  // the intermediate sums lie behind the partials
         double *mid = reinterpret_cast<double *>(partials + 2 * ((size_t)n_partials_cap - 2 * FINISH_CTAS));
         finish_sums_kernel<<<FINISH_CTAS, 512, 0, a.stream>>>(partials, (size_t)n, mid, (size_t)n, nt);
-        finish_sums_kernel<<<1, 512, 0, a.stream>>>(mid, (size_t)FINISH_CTAS, sums);
+        finish_sums_kernel<<<FINISH_CLUSTER, 512, 0, a.stream>>>(mid, (size_t)(FINISH_CTAS / FINISH_CLUSTER), sums);
     }
     return cudaGetLastError();
 }
