@@ -323,7 +323,8 @@ int ctrex_fwd_project(ctrex_ctx *ctx, const void *vol, int vol_dtype, void *proj
  * kernel): r_i = R_i (p_i - (A x)_i) with R_i = 1 / (A 1)_i if that row sum
  * exceeds 1e-6 * (smallest voxel pitch), else 0.  A x is never stored.
  *   p        DEVICE measured images [n_idx][nv][nu] of p_dtype.
- *   r        DEVICE output [n_idx][nv][nu] of r_dtype (may alias nothing).
+ *   r        DEVICE output [n_idx][nv][nu] of r_dtype (may be p itself; may
+ *            alias nothing else).
  *   sums     DEVICE double [2] receiving (sum (p - Ax)^2, sum p^2) over all
  *            pixels of the listed views (fixed-order reduction: bitwise
  *            reproducible), or NULL.

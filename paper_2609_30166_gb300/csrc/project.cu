@@ -496,9 +496,7 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
     const bool norm = a.column && a.norm_tiles && sums;
     const size_t nt = norm ? (size_t)fg.x * fg.y * fg.z : 0;
     if (n + nt + 2 * FINISH_CTAS > (size_t)n_partials_cap) return cudaErrorInvalidValue;
-    cudaError_t e = fwd_dispatch<MODE_CORRECT>(a, p_dtype, r, nullptr, p, partials);
-    if (e != cudaSuccess || sums == nullptr) return e;
-    if (norm) {
+    if (norm) {  // first: r may be p itself
         const unsigned ctas = (unsigned)((nt + 7) / 8);
         if (p_dtype == CTREX_F32)
             norm_tiles_kernel<<<ctas, 256, 0, a.stream>>>(*a.grid, a.view_idx, fg,
@@ -507,6 +505,8 @@ cudaError_t launch_forward_correct(const FwdArgs &a, const void *p, int p_dtype,
             norm_tiles_kernel<<<ctas, 256, 0, a.stream>>>(*a.grid, a.view_idx, fg,
                                                           static_cast<const __nv_bfloat16 *>(p), partials + 2 * (size_t)n);
     }
+    cudaError_t e = fwd_dispatch<MODE_CORRECT>(a, p_dtype, r, nullptr, p, partials);
+    if (e != cudaSuccess || sums == nullptr) return e;
     if (n <= FINISH_ONE) {
         finish_sums_kernel<<<FINISH_CLUSTER, 512, 0, a.stream>>>(partials, (size_t)n, sums, (size_t)n, nt);
     } else {  // the intermediate sums lie behind the partials
