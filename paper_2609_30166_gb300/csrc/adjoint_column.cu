@@ -142,6 +142,18 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
                 L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
             }
             const float kl = last_kappa(G, R);
+            if (mo.s == 0.0f) {  // the view sees no deformation, whatever the coefficients are
+#pragma unroll 1
+                for (int k = 0; k < R.K; ++k) {
+                    const bool last = k == R.K - 1;
+                    const float kap = last ? kl : (float)k, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
+                    float q[3];
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) q[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(kap, ds[r], d0[r]);
+                    point(cen, q, y * w);
+                }
+                continue;
+            }
             for (int k = 0; k < R.K;) {
                 SplineRun run;
                 const int end = run.find(L, k, R.K, kl);

@@ -65,6 +65,19 @@ __device__ __forceinline__ void motion_runs_integral(const Grid &G, const ViewGP
         L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
     }
     const float kl = last_kappa(G, R);
+    if (mo.s == 0.0f) {  // the view sees no deformation, whatever the coefficients are
+#pragma unroll 1
+        for (int k = 0; k < R.K; ++k) {
+            const bool last = k == R.K - 1;
+            const float kap = last ? kl : (float)k, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
+            float q[3], ws;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) q[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(kap, ds[r], d0[r]) + cen[r];
+            a = fmaf(w, vol(q[0], q[1], q[2], ws), a);
+            ars = fmaf(w, ws, ars);
+        }
+        return;
+    }
     for (int k = 0; k < R.K;) {
         SplineRun run;
         const int end = run.find(L, k, R.K, kl);

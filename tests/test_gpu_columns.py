@@ -360,3 +360,32 @@ def test_adjoint_of_tall_detector(motion, turn):
     want = oracle.adjoint(pb, _np(rows))
     assert rel_l2(_np(c.adjoint_project(y)), want) <= TOL32
     c.close()
+
+
+# Views whose time scale is 0 see no deformation, whatever its coefficients
+# are, sample by sample and by runs.
+@pytest.mark.parametrize("step", [0.5, 0.08])
+def test_views_without_deformation(step):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    n, det, views = (30, 41, 35), (37, 22), 4
+    P = _matrices(views, 1, 0.4, det[0], det[1], 60.0, 200.0)
+    vox, shape = (0.7, 0.7, 0.7), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(12)
+    theta = np.zeros((views, 15))
+    theta[:, :6] = rng.uniform(-0.03, 0.03, (views, 6))
+    theta[:, 6:] = np.eye(3).ravel()
+    theta = _np(_t(theta))
+    coef = np.full((8, 8, 8, 3), np.inf)
+    coef[::2] = np.nan
+    pb = oracle.Problem(P, shape, vox, org, det, step).with_motion(theta, None, None, margin=0.5)
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det, step_vox=step)
+    c.set_motion(_t(theta), _t(coef), _t(np.array([0.0, 1.0, 0.0, 1.0])), 0.5)
+    x, y = rng.uniform(0.2, 1.0, size=shape), rng.uniform(0.5, 1.5, size=(2, det[1], det[0]))
+    vi = np.array([0, 2], dtype=np.int32)
+    assert rel_l2(_np(c.fwd_project(_t(x), view_idx=vi)), oracle.forward(pb, _np(_t(x)), views=vi)[0]) <= TOL32
+    assert rel_l2(_np(c.adjoint_project(_t(y), view_idx=vi)), oracle.adjoint(pb, _np(_t(y)), views=vi)) <= TOL32
+    c.close()
