@@ -90,6 +90,52 @@ __device__ __forceinline__ void bp_edge(const ColImages &I, const float2 *img, f
     c += (wu0 + wu1) * (wv0 + wv1);
 }
 
+// A voxel's sums over the views (field 0: b, c; field 1: b, c), each term in
+// general position.  bp_interp's differences turn a mean with infinite values,
+// or with values too far apart for FP32, into NaN or an infinity, so a voxel
+// whose sum is not finite takes its terms again here.  Not inlined: within
+// the kernels it cost their loops 2 to 4 %.
+template <bool WINDOW, bool SUBV, bool CYL, bool DYR>
+__device__ __noinline__ float4 bp_voxel(const ViewGPU *__restrict__ views, const int *__restrict__ view_idx, int total,
+                                        int n_sub, int n_views, ColImages I, const int4 *__restrict__ window, float4 det,
+                                        int ix, int iy, int iz, int sv, CylGPU cyl, float tau,
+                                        const float *__restrict__ t_view)
+{
+    const int points = SUBV ? sv * sv * sv : 1;
+    const float d = 1.0f / (float)sv, o = SUBV ? 0.5f * d - 0.5f : 0.0f;
+    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int m = 0; m < total; ++m) {
+        const int k = m / n_sub, view = view_idx ? view_idx[k] : k;
+        if (view < 0 || view >= n_views) continue;
+        const float *P = views[view * n_sub + (m - k * n_sub)].P;
+        float4 win = det;
+        if (WINDOW) {
+            const int4 w = window[view];
+            win = make_float4((float)w.x, (float)w.y, (float)w.z, (float)w.w);
+        }
+        float b = 0.0f, c = 0.0f;
+        for (int i = 0; i < points; ++i) {
+            float x = (float)ix, y = (float)iy, z = (float)iz;
+            if (SUBV) {
+                x += fmaf((float)(i % sv), d, o);
+                y += fmaf((float)(i / sv % sv), d, o);
+                z += fmaf((float)(i / (sv * sv)), d, o);
+            }
+            if (CYL) cyl_point(cyl, x, y, z, x, y, z);
+            auto row = [&](const float *p) { return fmaf(p[0], x, fmaf(p[1], y, fmaf(p[2], z, p[3]))); };
+            bp_edge(I, I.p + (size_t)k * I.view, row(P), row(P + 4), row(P + 8), win, b, c);
+        }
+        if (DYR && !(t_view[view] < tau)) {
+            sum.z += b;
+            sum.w += c;
+        } else {
+            sum.x += b;
+            sum.y += c;
+        }
+    }
+    return sum;
+}
+
 // ColView::inside of the points of a box: its corners decide (the image of a
 // box in front of the source is the hull of its corners' images), by a margin
 // that covers the rounding of u and v, bounded from the size of the terms
@@ -204,7 +250,7 @@ __global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR
             lo[a] -= 0.5f;
             hi[a] += 0.5f;
         }
-    float ta[VZ];
+    float ta[VZ] = {};
     if (DYR)
 #pragma unroll
         for (int q = 0; q < VZ; ++q)
@@ -328,6 +374,18 @@ __global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR
 #pragma unroll
             for (int q = 0; q < VZ; ++q) c[0][q] += (float)cnt;
     }
+#pragma unroll
+    for (int q = 0; q < VZ; ++q)
+        if (!isfinite(b[0][q]) || !isfinite(b[NP - 1][q])) {
+            const float4 s = bp_voxel<WINDOW, SUBV, CYL, DYR>(views, view_idx, total, G.n_sub, G.n_views, I, window, det,
+                                                              ix, iy, iz + 32 * q, sv, CYL ? cyl : CylGPU{}, ta[q], t_view);
+            b[0][q] = s.x;
+            c[0][q] = s.y;
+            if (DYR) {
+                b[NP - 1][q] = s.z;
+                c[NP - 1][q] = s.w;
+            }
+        }
     const float mean = SUBV ? G.inv_sub / (float)(sv * sv * sv) : G.inv_sub;
 #pragma unroll
     for (int f = 0; f < NP; ++f) {
@@ -406,6 +464,14 @@ __global__ void __launch_bounds__(BPC_THREADS, DEEP ? 4 : BPC_MIN_BLOCKS)
             for (int q = 0; q < VZ; ++q) b[q] += bp_interp(t[q]);
         }
     }
+#pragma unroll
+    for (int q = 0; q < VZ; ++q)
+        if (!isfinite(b[q]))
+            b[q] = bp_voxel<false, false, false, false>(
+                       views, view_idx, total, G.n_sub, G.n_views, I, nullptr,
+                       make_float4(0.0f, (float)(G.nu - 1), 0.0f, (float)(G.nv - 1)), ix, iy, z0 + lane + 32 * q, 1,
+                       CylGPU{}, 0.0f, nullptr)
+                       .x;
     const float mean = G.inv_sub;
 #pragma unroll
     for (int q = 0; q < VZ; ++q) c[q] = (float)count * mean;
