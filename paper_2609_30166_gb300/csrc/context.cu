@@ -287,6 +287,7 @@ void dyr_release(ctrex_ctx *c)
 //   11.7 / 10.9, 19.4 / 7.8 ms;
 // - fine pixels spread a warp's voxels (768^2 pixels, 90 views, voxel steps
 //   of 2 and 4 pixels): backprojection 2.0 / 3.0 ms, 0.66 / 0.62 ms.
+// The other models and BF16 volumes: see column_forward.
 constexpr double COL_LEAN_FWD = 1.0, COL_LEAN_BP = 0.55, COL_STEP_FP32 = 6.0, COL_STEP_BF16 = 3.0;
 constexpr double COL_STEP_BP_MIN = 0.3;
 // The adjoint's warps: 32 rows of a detector column up to this lean, 8 x 4
@@ -295,9 +296,21 @@ constexpr double COL_STEP_BP_MIN = 0.3;
 constexpr double COL_LEAN_ADJ = 0.12;
 
 // The forward projector: also the lanes that each kernel's tiles (4 x 32
-// columns x rows here, 32 x 4 there) waste on a ragged detector, against the
-// kernels' speeds (2.4 : 1 with FP32 volumes, whose gathers carry one slice,
-// and 1.27 : 1 with BF16 ones).
+// columns x rows here, 32 x 4 there) waste on a ragged detector, against what
+// the columns gain over the gathers.  90 views of 256^3, 384^2 pixels, ms
+// columns / gathers at 0, 5, 10, 15, 20, 30, 44 degrees:
+//   static, FP32  6.3/16.6 7.6/16.7 9.2/16.8 10.7/16.9 12.0/17.0 14.0/17.8 16.5/20.3
+//   static, BF16  6.3/8.6  7.7/8.8  9.3/9.0  10.7/9.0  12.0/9.1  14.0/9.2  16.5/9.7
+//   event, FP32   8.3/24.4 9.2/25.0 10.7/25.7 12.3/26.4 13.8/27.1 16.6/28.3 19.9/30.1
+//   ROI, FP32     9.1/20.3 11.1/20.6 12.9/21.0 14.7/21.3 16.4/21.8 19.2/23.3 22.3/26.5
+//   cylinder      11.0/15.4 11.1/15.6 11.2/15.8 11.2/15.8 11.4/15.8 11.9/15.9 13.4/17.0
+//   Joseph, FP32  2.7/3.8  2.8/3.9  3.2/3.9  3.6/3.9   3.9/3.9   4.4/3.9   5.1/3.9
+//   Joseph, BF16  2.6/3.7  2.8/3.8  3.2/3.8  3.6/3.8   3.9/3.8   4.4/3.8   5.1/3.7
+// (event and ROI in BF16 gain as in FP32).  Coarse pixels spread a leaning
+// warp further.  Of 376 ragged detectors for each model and type (96^3 and
+// 256^3, pixel steps of 1 to 4.5 voxels, 0 to 44 degrees) the choice below is
+// slower than gathers by more than 3 % on 5 Joseph ones (8 % at most, 86 us for
+// 79) and no other; with one limit per type for all models it was on 370.
 bool column_forward(const ctrex_ctx *c, int vdt)
 {
     if (!(c->col_lean <= COL_LEAN_FWD && column_grid_fits(c->grid))) return false;
@@ -305,7 +318,15 @@ bool column_forward(const ctrex_ctx *c, int vdt)
     if (step > (vdt == CTREX_F32 ? COL_STEP_FP32 : COL_STEP_BF16)) return false;
     const double u4 = (c->grid.nu + 3) / 4 * 4.0, u32 = (c->grid.nu + 31) / 32 * 32.0;
     const double v4 = (c->grid.nv + 3) / 4 * 4.0, v32 = (c->grid.nv + 31) / 32 * 32.0;
-    return u4 * v32 <= u32 * v4 * (vdt == CTREX_F32 ? 2.2 : 1.2);
+    const double spread = c->col_lean * fmax(step, 1.0);
+    double gain = vdt == CTREX_F32 ? 2.2 : 1.2;
+    if (c->projector == CTREX_PROJ_JOSEPH)
+        gain = fmin(gain, 2.1 - 0.1 * step - 3.0 * spread);
+    else if (c->cyl)
+        gain = fmin(gain, 1.6);
+    else if (vdt == CTREX_BF16 && !c->dyr && !c->roi)
+        gain = fmin(gain, 1.75 - 5.0 * spread);
+    return u4 * v32 <= u32 * v4 * gain;
 }
 
 bool column_backproject(const ctrex_ctx *c)

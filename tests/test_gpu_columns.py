@@ -389,3 +389,36 @@ def test_views_without_deformation(step):
     assert rel_l2(_np(c.fwd_project(_t(x), view_idx=vi)), oracle.forward(pb, _np(_t(x)), views=vi)[0]) <= TOL32
     assert rel_l2(_np(c.adjoint_project(_t(y), view_idx=vi)), oracle.adjoint(pb, _np(_t(y)), views=vi)) <= TOL32
     c.close()
+
+
+# Detectors on both sides of the lean at which a model and a storage type
+# change from columns to gathers (static BF16 about 8 degrees, Joseph about 17),
+# and rows of which columns waste too many lanes on the cylinder (33).
+@pytest.mark.parametrize("model,turn,nv", [("static", 6.0, 60), ("static", 11.0, 60), ("joseph", 14.0, 60),
+                                           ("joseph", 21.0, 60), ("cylinder", 0.3, 33), ("cylinder", 30.0, 60)])
+def test_lean_limits_of_models(model, turn, nv):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    n, det, views = (22, 27, 41), (37, nv), 5
+    P = _matrices(views, 1, turn, det[0], det[1], 80.0, 200.0)
+    shape = n[::-1]
+    c = ctrex.Context()
+    if model == "cylinder":
+        shape = (41, 30, 17)  # slices, sectors, rings
+        args = dict(n_r=17, n_phi=30, n_z=41, dr=0.8, dz=0.8)
+        c.set_geometry_cylinder(P, det=det, **args)
+        pb = oracle.cylinder_problem(P, det=det, **args)
+    else:
+        vox = (1.0, 0.9, 0.8)
+        org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+        c.set_geometry(P, shape, vox, org, det)
+        pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    if model == "joseph":
+        c.set_projector("joseph")
+        pb = pb.with_joseph()
+    x = np.random.default_rng(4).uniform(0.2, 1.0, size=shape)
+    for dt in (torch.float32, torch.bfloat16):
+        ref, _ = oracle.forward(pb, _np(_t(x, dt)))
+        assert rel_l2(_np(c.fwd_project(_t(x, dt), out_dtype=torch.float32)), ref) <= TOL32
+    c.close()
