@@ -525,10 +525,11 @@ static bool four_voxels(int nz)
     return nz >= 128 && 100 * n4 < 114 * n2;
 }
 
-// Slices that the kernel works through, the last block's repeats among them.
-int backproject_column_slices(const Grid &G)
+// Slices that the kernel works through, the last block's repeats among them
+// (two: the event model and sub-voxels always take two voxels per thread).
+int backproject_column_slices(const Grid &G, bool two)
 {
-    const int b = four_voxels(G.nz) ? 128 : 64;
+    const int b = !two && four_voxels(G.nz) ? 128 : 64;
     return (G.nz + b - 1) / b * b;
 }
 

@@ -288,8 +288,8 @@ void dyr_release(ctrex_ctx *c)
 // - fine pixels spread a warp's voxels (768^2 pixels, 90 views, voxel steps
 //   of 2 and 4 pixels): backprojection 2.0 / 3.0 ms, 0.66 / 0.62 ms.
 // The other models and BF16 volumes: see column_forward.
-constexpr double COL_LEAN_FWD = 1.0, COL_LEAN_BP = 0.55, COL_STEP_FP32 = 6.0, COL_STEP_BF16 = 3.0;
-constexpr double COL_STEP_BP_MIN = 0.3;
+constexpr double COL_LEAN_FWD = 1.0, COL_STEP_FP32 = 6.0, COL_STEP_BF16 = 3.0;
+constexpr double COL_STEP_BP_MIN = 0.3;  // (and see column_backproject)
 // The adjoint's warps: 32 rows of a detector column up to this lean, 8 x 4
 // patches beyond (45 views of 384^2 on 256^3, ms column / patch at 0, 6, 8, 45
 // degrees: 5.7 / 7.8, 12.0 / 12.4, 13.8 / 13.4, 29 / 17; in place 16.6 .. 18.3).
@@ -329,17 +329,55 @@ bool column_forward(const ctrex_ctx *c, int vdt)
     return u4 * v32 <= u32 * v4 * gain;
 }
 
-bool column_backproject(const ctrex_ctx *c)
+// The backprojector: time by columns over time by gathers, fitted to 8638 scans
+// of all kinds and both image types (64^2 to 512^2 voxels in x and y, 8 to 512
+// slices, pixel steps of 0.3 to 3.5 voxels, 0 to 38 degrees of lean).  A pixel
+// step of s voxels spreads a warp's 32 voxels over 32 / s rows and lean * 32 / s
+// columns, each one more line; blocks of 64 or 128 slices repeat slices, and a
+// block beyond the volume, or a turned detector that cuts the object off, takes
+// terms to the general path.  90 views, 256 x 256 in x and y, 0.8 voxels a
+// pixel, static FP32, ms columns / gathers: 256 slices 1.64 / 2.89, 130 1.43 /
+// 1.50, 70 0.95 / 0.82, 50 0.89 / 0.60, 20 0.73 / 0.28; 256 slices at 8, 15, 22
+// degrees 2.1 / 2.9, 2.5 / 2.9, 2.9 / 2.9.  The choice takes more than 3 %
+// longer than gathers on 132 of the scans (18 % at most without a detector
+// window, 29 % with one); with one lean limit for all, and thin volumes left to
+// gathers for the static model only, on 3265, up to seven times as long.
+double bp_column_cost(const ctrex_ctx *c, const Grid &G, int rdt, double step, bool tiny)
 {
-    // blocks of slices that repeat or leave empty a third and more (FP32 / BF16
-    // images, us by columns, by gathers): 60 x 60 x 20, 100 views 105, 86 / 105,
-    // 82; 50 x 50 x 40 91, 85 / 92, 81; 180 x 180 x 70 476, 486 / 476, 422; 74 x
-    // 87 x 84, 132 views 155, 237 / 156, 218
-    if (!c->cyl && !c->roi && !c->dyr && c->bp_subvoxel == 1 &&
-        100.0 * backproject_column_slices(c->grid) > 155.0 * c->grid.nz)
+    struct {
+        double base, rows, cols, bf16;
+    } k = {0.49, 0.13, 0.63, 1.2};  // static, cylinder
+    if (c->bp_subvoxel > 1)
+        k = {0.56, 0.10, 0.24, 1.02};
+    else if (c->dyr)
+        k = {0.55, 0.07, 0.59, 1.2};
+    else if (c->has_window)
+        k = {0.70, 0.06, 0.70, 1.12};
+    const double slices = backproject_column_slices(G, c->dyr || c->bp_subvoxel > 1);
+    const double blocks = tiny ? 1.0 : slices / G.nz * (G.nz < 64 ? 1.5 : 1.0);
+    // what a turn moves the volume's sides along the detector's rows by, over its height
+    const double width = c->cyl ? 2.0 * G.nx * c->cylg.dr / c->cylg.dz : (double)(G.nx > G.ny ? G.nx : G.ny);
+    return blocks * (rdt == CTREX_BF16 ? k.bf16 : 1.0) *
+           (k.base + k.rows / step + k.cols * fmin(c->col_lean / step, 0.35) +
+            0.25 * fmin(c->col_lean * width / G.nz, 3.0));
+}
+
+bool column_backproject(const ctrex_ctx *c, int rdt)
+{
+    const Grid &G = c->grid;
+    if (!(c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(G) && (!c->roi || backproject_column_fits(c->roi_grid))))
         return false;
-    return c->col_lean <= COL_LEAN_BP && c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(c->grid) &&
-           (!c->roi || backproject_column_fits(c->roi_grid));
+    // a launch of less than a wave waits for its loads, however little of it
+    // is of use (64 x 64 x 20, 90 views: 78 us by columns, 86 by gathers)
+    auto tiny = [](const Grid &g, int nz) { return (g.nx + 7) / 8 * (double)g.ny <= 760.0 && g.nz <= nz; };
+    if (c->bp_subvoxel == 1 && !c->roi && tiny(G, 24)) return c->col_lean <= 0.55;
+    double cost = bp_column_cost(c, G, rdt, c->col_step, c->roi && tiny(G, 128));
+    if (c->roi) {
+        const Grid &R = c->roi_grid;
+        const double v = (double)grid_voxels(G), w = (double)grid_voxels(R);
+        cost = (cost * v + bp_column_cost(c, R, rdt, c->col_step * c->roig.sc[2], tiny(R, 128)) * w) / (v + w);
+    }
+    return cost <= 1.0;
 }
 
 bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ; }
@@ -1165,7 +1203,7 @@ int ctrex_fwd_correct(ctrex_ctx *c, const void *vol, int vdt, const void *p, int
 // The images of a backprojection into the layout that it reads.
 static int bp_images(ctrex_ctx *c, BpArgs &a, const void *r, int rdt, int n_idx)
 {
-    if (n_idx > 0 && column_backproject(c)) {
+    if (n_idx > 0 && column_backproject(c, rdt)) {
         CT_CUDA(c, scratch_begin(c));
         cudaError_t ae = col_ensure_images(c->img_col, c->grid.nu, c->grid.nv, n_idx, c->stream);
         if (ae == cudaSuccess) {

@@ -205,7 +205,7 @@ cudaError_t launch_backproject(const BpArgs &a);
 // The same on a.column (bp_column.cu).
 cudaError_t launch_backproject_column(const BpArgs &a);
 bool backproject_column_fits(const Grid &g);  // its launch shape stays within the grid limits
-int backproject_column_slices(const Grid &g);  // slices it works through (>= nz)
+int backproject_column_slices(const Grid &g, bool two);  // slices it works through
 // Whether every one of n views (on the host) has the whole volume inside the
 // detector and every z column at one depth, to FP32 rounding.
 bool backproject_flat(const Grid &g, const ViewGPU *views, int n);
