@@ -40,9 +40,41 @@ __device__ __forceinline__ float LinearSampler<TV>::interior(float gx, float gy,
     return trilinear(vol, nx, ny, nz, gx, gy, gz, ws);
 }
 
-// One ray's integral and row sum under motion, run by run (SplineRun).
+// How a motion projector forms its samples' positions: not at all, by the
+// pose alone, with the spline two samples at a time, or run by run (SplineRun).
+enum FwdMotion { MOTION_NONE, MOTION_POSE, MOTION_PAIRS, MOTION_RUNS };
+
+// The samples of a ray (positions relative to the grid centre `cen`) displaced
+// by the pose alone, linear in the sample index.  In a kernel without the
+// spline's registers (60 views of 128^3, pixels of a voxel, 1.18 ms; as pairs
+// in the spline's kernel 2.04; unrolled by 2 or 4, 1.23).
 template <typename Sampler>
-__device__ __forceinline__ void motion_runs_integral(const Grid &G, const ViewGPU &V, const MotionGPU &mo,
+__device__ __forceinline__ void pose_samples(const Grid &G, const Ray &R, const float d0[3], const float ds[3],
+                                             const float cen[3], const Sampler &vol, float &a, float &ars)
+{
+    auto sample = [&](float kap, float &ws) {
+        float q[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) q[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(kap, ds[r], d0[r]) + cen[r];
+        return vol(q[0], q[1], q[2], ws);
+    };
+    float ws;
+#pragma unroll 1
+    for (int k = 0; k < R.K - 1; ++k) {
+        a += sample((float)k, ws);
+        ars += ws;
+    }
+    a *= G.step_mm;
+    ars *= G.step_mm;
+    if (R.w_last > 0.0f) {
+        a = fmaf(R.w_last, sample(last_kappa(G, R), ws), a);
+        ars = fmaf(R.w_last, ws, ars);
+    }
+}
+
+// One ray's integral and row sum under motion, by the pose alone or run by run.
+template <typename Sampler, bool RUNS>
+__device__ __forceinline__ void motion_line_integral(const Grid &G, const ViewGPU &V, const MotionGPU &mo,
                                                      const float4 *spline, const Sampler &vol, float u, float v,
                                                      float &a, float &ars)
 {
@@ -52,32 +84,20 @@ __device__ __forceinline__ void motion_runs_integral(const Grid &G, const ViewGP
     grid_centre(G, cen);
     Ray R;
     if (!setup_ray(G, V, u, v, R, cen)) return;
-    // displacement by the pose at sample index kappa, linear; positions
-    // relative to the grid centre (R's), see MotionGPU
     float d0[3], ds[3];
+    pose_line(mo, R, d0, ds);
+    // (a view whose time scale is 0 sees no deformation, whatever the coefficients are)
+    if (!RUNS || mo.s == 0.0f) {
+        pose_samples(G, R, d0, ds, cen, vol, a, ars);
+        return;
+    }
     SplineLine L;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-        const float *D = mo.D + 3 * r;
-        d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], mo.bc[r])));
-        ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
         L.x0[r] = fmaf(R.g0[r] + d0[r] + cen[r] + 0.5f, G.spl_scale[r], 1.0f);
         L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
     }
     const float kl = last_kappa(G, R);
-    if (mo.s == 0.0f) {  // the view sees no deformation, whatever the coefficients are
-#pragma unroll 1
-        for (int k = 0; k < R.K; ++k) {
-            const bool last = k == R.K - 1;
-            const float kap = last ? kl : (float)k, w = last ? fmaxf(R.w_last, 0.0f) : G.step_mm;
-            float q[3], ws;
-#pragma unroll
-            for (int r = 0; r < 3; ++r) q[r] = fmaf(kap, R.sg[r], R.g0[r]) + fmaf(kap, ds[r], d0[r]) + cen[r];
-            a = fmaf(w, vol(q[0], q[1], q[2], ws), a);
-            ars = fmaf(w, ws, ars);
-        }
-        return;
-    }
     for (int k = 0; k < R.K;) {
         SplineRun run;
         const int end = run.find(L, k, R.K, kl);
@@ -107,8 +127,7 @@ __device__ __forceinline__ void motion_runs_integral(const Grid &G, const ViewGP
 // Integral of one pixel (mean over its sub-angle rays): value and row sum.
 // On the cylindrical domain the ray is clipped to the bounding cylinder and
 // every sample is mapped to (r, phi, z) by the sampler; the rest is shared.
-// RUNS (motion): the deformation run by run (SplineRun), else pair by pair.
-template <typename Sampler, bool MOTION, bool RUNS>
+template <typename Sampler, int MOTION>
 __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__restrict__ views,
                                                const MotionGPU &mo, const float4 *spline,
                                                const Sampler &vol, int view, float u,
@@ -131,9 +150,9 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
             acc_rs += ars;
             continue;
         }
-        if constexpr (RUNS) {
+        if constexpr (MOTION == MOTION_POSE || MOTION == MOTION_RUNS) {
             float a, ars;
-            motion_runs_integral(G, V, mo, spline, vol, u, v, a, ars);
+            motion_line_integral<Sampler, MOTION == MOTION_RUNS>(G, V, mo, spline, vol, u, v, a, ars);
             acc += a;
             acc_rs += ars;
             continue;
@@ -148,7 +167,7 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
         const int Km1 = R.K - 1;
         int ka = Km1, kb = Km1;
         if (!MOTION && !Sampler::CYLINDER) interior_range(G, R, ka, kb);
-        if constexpr (MOTION) {
+        if constexpr (MOTION == MOTION_PAIRS) {
             for (int k = 0; k < R.K; k += 2) {
                 float g[2][3], w[2], y[2][3];
                 sample_pair(G, R, k, g, w);
@@ -190,7 +209,7 @@ __device__ __forceinline__ void pixel_integral(const Grid &G, const ViewGPU *__r
     rs = acc_rs * G.inv_sub;
 }
 
-template <typename Sampler, typename TP, int MODE, bool MOTION, bool RUNS = false>
+template <typename Sampler, typename TP, int MODE, int MOTION>
 __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ views,
                                          const MotionGPU *__restrict__ motion, const float4 *spline,
                                          const Sampler &vol_in, const int *__restrict__ view_idx,
@@ -212,26 +231,25 @@ __device__ __forceinline__ void fwd_body(Grid G, const ViewGPU *__restrict__ vie
     }
     if constexpr (Sampler::DYRECT) vol.set_view(view);  // the view's acquisition time
     MotionGPU mo;
-    __shared__ float4 s_spline[MOTION ? SPLINE_TABLE : 1];
-    if (MOTION) {
-        mo = motion[view];
-        if (spline != nullptr) {
-            load_spline(s_spline, spline, threadIdx.y * FWD_TX + threadIdx.x, FWD_TX * FWD_TY);
-            spline = s_spline;
-        }
-        __syncthreads();
+    constexpr bool SPLINE = MOTION == MOTION_PAIRS || MOTION == MOTION_RUNS;
+    __shared__ float4 s_spline[SPLINE ? SPLINE_TABLE : 1];
+    if (MOTION) mo = motion[view];
+    if (SPLINE) {
+        load_spline(s_spline, spline, threadIdx.y * FWD_TX + threadIdx.x, FWD_TX * FWD_TY);
+        spline = s_spline;
     }
+    if (MOTION) __syncthreads();
     int iu, iv;
-    tile_pixel<MOTION>(blockIdx.x * FWD_TX, blockIdx.z * FWD_TY, iu, iv);
+    tile_pixel<MOTION != MOTION_NONE>(blockIdx.x * FWD_TX, blockIdx.z * FWD_TY, iu, iv);
     const bool in_pix = iu < G.nu && iv < G.nv;
     const bool inside = ok && in_pix;
     float val = 0.0f, rs = 0.0f;
-    if (inside) pixel_integral<Sampler, MOTION, RUNS>(G, views, mo, spline, vol, view, (float)iu, (float)iv, val, rs);
+    if (inside) pixel_integral<Sampler, MOTION>(G, views, mo, spline, vol, view, (float)iu, (float)iv, val, rs);
     fwd_epilogue<TP, MODE>(G, k, view, ok, in_pix, iu, iv, val, rs, out, rowsum_out, p, partials, p_by_view,
                            s_red);
 }
 
-template <typename Sampler, typename TP, int MODE, bool MOTION>
+template <typename Sampler, typename TP, int MODE, int MOTION>
 __global__ void __launch_bounds__(FWD_TX *FWD_TY)
     fwd_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                const float4 *spline, const Sampler vol_in, const int *__restrict__ view_idx,
@@ -253,8 +271,8 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY, 4)
                    TP *__restrict__ out, float *__restrict__ rowsum_out, const TP *__restrict__ p,
                    float *__restrict__ partials, unsigned *devcheck, int p_by_view)
 {
-    fwd_body<Sampler, TP, MODE, true, true>(G, views, motion, spline, vol_in, view_idx, out, rowsum_out, p, partials,
-                                            devcheck, p_by_view);
+    fwd_body<Sampler, TP, MODE, MOTION_RUNS>(G, views, motion, spline, vol_in, view_idx, out, rowsum_out, p, partials,
+                                             devcheck, p_by_view);
 }
 
 // Projectors whose sampler declares MIN_BLOCKS > 0 (the event model and
@@ -268,8 +286,8 @@ __global__ void __launch_bounds__(FWD_TX *FWD_TY, Sampler::MIN_BLOCKS > 0 ? Samp
                   TP *__restrict__ out, float *__restrict__ rowsum_out, const TP *__restrict__ p,
                   float *__restrict__ partials, unsigned *devcheck, int p_by_view)
 {
-    fwd_body<Sampler, TP, MODE, false>(G, views, nullptr, nullptr, vol_in, view_idx, out, rowsum_out, p, partials,
-                                       devcheck, p_by_view);
+    fwd_body<Sampler, TP, MODE, MOTION_NONE>(G, views, nullptr, nullptr, vol_in, view_idx, out, rowsum_out, p,
+                                             partials, devcheck, p_by_view);
 }
 
 // Second pass of the residual reduction, FP64 from the first add in a fixed
@@ -425,9 +443,10 @@ static cudaError_t fwd_launch(const FwdArgs &a, const Sampler &smp, TP *out, flo
             return cudaGetLastError();
         }
         if (a.motion) {
-            fwd_kernel<Sampler, TP, MODE, true><<<grid, block, 0, a.stream>>>(
-                G, a.views, a.motion, a.spline, smp, a.view_idx, out, rowsum, p, partials, a.devcheck,
-                a.p_by_view);
+            auto *kernel = a.spline ? fwd_kernel<Sampler, TP, MODE, MOTION_PAIRS>
+                                    : fwd_kernel<Sampler, TP, MODE, MOTION_POSE>;
+            kernel<<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, smp, a.view_idx, out, rowsum, p,
+                                                 partials, a.devcheck, a.p_by_view);
             return cudaGetLastError();
         }
     } else if (a.motion) {
@@ -437,7 +456,7 @@ static cudaError_t fwd_launch(const FwdArgs &a, const Sampler &smp, TP *out, flo
         fwd_kernel_mb<Sampler, TP, MODE><<<grid, block, 0, a.stream>>>(G, a.views, smp, a.view_idx, out, rowsum, p,
                                                                       partials, a.devcheck, a.p_by_view);
     else
-        fwd_kernel<Sampler, TP, MODE, false><<<grid, block, 0, a.stream>>>(
+        fwd_kernel<Sampler, TP, MODE, MOTION_NONE><<<grid, block, 0, a.stream>>>(
             G, a.views, nullptr, nullptr, smp, a.view_idx, out, rowsum, p, partials, a.devcheck, a.p_by_view);
     return cudaGetLastError();
 }

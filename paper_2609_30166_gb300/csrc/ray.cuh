@@ -534,6 +534,18 @@ __device__ __forceinline__ float last_kappa(const Grid &G, const Ray &R)
     return (float)(R.K - 1) + 0.5f * (R.w_last / G.step_mm - 1.0f);
 }
 
+// Displacement of a ray's samples by the pose, D g + bc (g relative to the
+// grid centre, as R's positions): d0 + kappa ds at sample index kappa.
+__device__ __forceinline__ void pose_line(const MotionGPU &m, const Ray &R, float d0[3], float ds[3])
+{
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const float *D = m.D + 3 * r;
+        d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], m.bc[r])));
+        ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
+    }
+}
+
 // Samples kk and kk + 1 of a ray and their weights (mm): the last one is the
 // clipped segment's remainder, one past it weighs nothing (and repeats it).
 __device__ __forceinline__ void sample_pair(const Grid &G, const Ray &R, int kk, float g[2][3], float w[2])

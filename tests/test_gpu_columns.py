@@ -422,3 +422,45 @@ def test_lean_limits_of_models(model, turn, nv):
         ref, _ = oracle.forward(pb, _np(_t(x, dt)))
         assert rel_l2(_np(c.fwd_project(_t(x, dt), out_dtype=torch.float32)), ref) <= TOL32
     c.close()
+
+
+# Motion by the pose alone: straight displaced rays, in every operator, and
+# the gradient with respect to the pose with and without a deformation beside
+# it; tolerances as in test_motion_runs_match_oracle.
+@pytest.mark.parametrize("n,det,views,sub,turn,step", [
+    ((30, 41, 35), (37, 22), 4, 1, 0.4, 0.5),
+    ((33, 32, 70), (21, 33), 3, 2, 30.0, 0.08),
+    ((5, 40, 8), (70, 5), 5, 1, 0.0, 0.5),
+    ((64, 64, 64), (12, 5), 1, 1, 60.0, 0.5),   # few rays
+])
+def test_pose_only_matches_oracle(n, det, views, sub, turn, step):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    P = _matrices(views, sub, turn, det[0], det[1], 60.0, 200.0)
+    pitch = 30.0 / max(n)
+    vox, shape = (pitch, 0.95 * pitch, 1.05 * pitch), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(34)
+    theta = np.zeros((views, 15))
+    theta[:, :6] = rng.uniform(-0.03, 0.03, (views, 6))
+    theta[:, 6:] = np.eye(3).ravel() + rng.uniform(-0.01, 0.01, (views, 9))
+    coef = rng.uniform(-1, 1, (8, 8, 8, 3)) * 0.05 * max(n) * pitch
+    theta, coef = (_np(_t(a)) for a in (theta, coef))  # as the GPU sees them
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det, step_vox=step)
+    axes = [(np.arange(m) + 1.0) * (m - np.arange(m)) / (m + 1.0) ** 2 for m in shape]
+    x = _np(_t(64.0 * axes[0][:, None, None] * axes[1][:, None] * axes[2]))
+    y = _np(_t(rng.uniform(0.5, 1.5, size=(views, det[1], det[0]))))
+    plain = oracle.Problem(P, shape, vox, org, det, step)
+    for co, sv in ((None, None), (coef, np.ones(views))):
+        pb = plain.with_motion(theta, co, sv, margin=0.5)
+        c.set_motion(_t(theta), None if co is None else _t(co), None if sv is None else _t(sv), 0.5)
+        rows = torch.empty((views, det[1], det[0]), device="cuda")
+        ref, rs = oracle.forward(pb, x)
+        assert rel_l2(_np(c.fwd_project(_t(x), rowsum=rows)), ref) <= TOL32
+        assert rel_l2(_np(rows), rs) <= TOL32
+        assert rel_l2(_np(c.adjoint_project(_t(y))), oracle.adjoint(pb, y)) <= TOL32
+        gt, _ = oracle.motion_grad(pb, x, y)
+        assert rel_l2(_np(c.motion_grad(_t(x), _t(y), want_coef=False)[0]), gt) <= 1e-4
+    c.close()
