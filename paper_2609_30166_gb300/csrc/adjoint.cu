@@ -16,13 +16,16 @@ constexpr int ADJ_TX = 32, ADJ_TY = 4;
 // Motion gradient CTA: four warps on 8 x 4 pixel patches side by side, which
 // share the spline table and the CTA's partial sums; three CTAs per SM (168
 // registers), by runs and sample by sample (45 views of the 256^3 motion
-// workload: 40.4 and 94.7 ms; two warps, six CTAs: 50.5 and 106 ms).
-constexpr int MG_WARPS = 4, MG_THREADS = 32 * MG_WARPS, MG_MIN_BLOCKS = 3;
+// workload: 40.4 and 94.7 ms; two warps, six CTAs: 50.5 and 106 ms).  The pose
+// alone needs none of that: eight CTAs, sums in registers (60 views of 128^3
+// 1.82 ms; in the spline's kernel with sums in shared memory 4.0).
+constexpr int MG_WARPS = 4, MG_THREADS = 32 * MG_WARPS, MG_MIN_BLOCKS = 3, MG_POSE_BLOCKS = 8;
 // Samples per spline cell from which the gradient goes by runs.  60 views at
-// 64^3 / 80^3 / 96^3 / 128^3 (26 / 32 / 38 / 51 samples), by samples: 4.6 /
-// 7.4 / 10.9 / 21.9 ms, by runs: 4.8 / 6.7 / 8.7 / 14.1 ms; pose only: 1.37 /
-// 2.40 / 3.79 / 8.14 and 1.80 / 2.73 / 3.82 / 6.89 ms.
-constexpr float MG_RUN_MIN = 30.0f, MG_RUN_MIN_POSE = 40.0f;
+// 64^3 / 80^3 / 96^3 / 112^3 / 128^3 (26 / 32 / 38 / 45 / 51 samples), by
+// samples: 4.8 / 7.7 / 11.1 / 16.3 / 22.1 ms, by runs: 4.9 / 6.8 / 8.8 / 11.8 /
+// 14.5 ms; the pose's alone: 1.18 / 2.09 / 3.30 / 5.02 / 7.20 and 1.81 / 2.76 /
+// 3.87 / 5.34 / 7.01 ms.
+constexpr float MG_RUN_MIN = 30.0f, MG_RUN_MIN_POSE = 50.0f;
 constexpr int NCOEF = 8 * 8 * 8 * 3;
 
 // ---------------------------------------------------------------------------
@@ -510,19 +513,24 @@ struct ColumnVolume {
 // step run per node.  45 views of the 256^3 motion workload: sample by sample
 // with the volume row-major 104.3 ms (spline loads and the tensor-core step's
 // shuffles), from the columns 94.7, by runs 40.4 (pose only 60.3, 42.6, 25.1).
-// RUNS: as above; without, sample by sample (short runs, MG_RUN_MIN).
-template <typename Volume, bool RUNS>
-__global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
+// What a launch has to form: MG_POSE: no deformation; MG_WARPED: the pose's
+// gradient under a deformation; MG_SAMPLES: the coefficients' too, sample by
+// sample (short runs, MG_RUN_MIN); MG_RUNS: either of the last two, as above.
+enum MotionGradKind { MG_POSE, MG_WARPED, MG_SAMPLES, MG_RUNS };
+
+template <typename Volume, int KIND>
+__global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS : MG_MIN_BLOCKS)
     motion_grad_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                        const float4 *table, const int *__restrict__ view_idx, const Volume vol,
                        const float *__restrict__ gproj, double *__restrict__ grad_M, double *__restrict__ grad_b,
                        double *__restrict__ grad_coef, unsigned *devcheck)
 {
-    __shared__ float4 s_spline[SPLINE_TABLE];
-    __shared__ double s_g64[NCOEF];       // the CTA's coefficient-gradient partials
+    constexpr bool RUNS = KIND == MG_RUNS, COEF = KIND == MG_SAMPLES || RUNS;
+    __shared__ float4 s_spline[KIND == MG_POSE ? 1 : SPLINE_TABLE];
+    __shared__ double s_g64[COEF ? NCOEF : 1];  // the CTA's coefficient-gradient partials
     __shared__ double s_red[12][MG_WARPS];
     __shared__ float4 s_piece[4];
-    __shared__ float s_pose[12][MG_THREADS];
+    __shared__ float s_pose[COEF ? 12 : 1][MG_THREADS];
     extern __shared__ float s_V[][MG_THREADS];  // RUNS: the nodes' dL/dy of each thread's run, 3 CHEB_N
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const int lane = tid & 31;
@@ -533,12 +541,12 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
         return;  // uniform over the CTA
     }
     const float mos = motion[view].s;
-    const bool spline = table != nullptr && mos != 0.0f;
-    const bool want_coef = spline && grad_coef != nullptr;
+    const bool spline = KIND != MG_POSE && mos != 0.0f;
+    const bool want_coef = COEF && spline && grad_coef != nullptr;
     if (spline) load_spline(s_spline, table, tid, MG_THREADS);
     if (want_coef)
         for (int i = tid; i < NCOEF; i += MG_THREADS) s_g64[i] = 0.0;
-    if (tid < 4) s_piece[tid] = bspline_piece(tid);
+    if (COEF && tid < 4) s_piece[tid] = bspline_piece(tid);
     __syncthreads();
     float cen[3];
     grid_centre(G, cen);
@@ -548,10 +556,20 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
 #pragma unroll
         for (int e = 0; e < 4; ++e) CA.acc[h][e] = 0.0f;
     CA.cell = -1;
-    // this thread's 12 pose sums (9 of dL/dM, 3 of dL/db): in shared memory,
-    // for want of registers
+    // this thread's 12 pose sums (9 of dL/dM, 3 of dL/db): in registers, or in
+    // shared memory beside the coefficients' sums
+    float pose_reg[12];
 #pragma unroll
-    for (int q = 0; q < 12; ++q) s_pose[q][tid] = 0.0f;
+    for (int q = 0; q < 12; ++q) {
+        pose_reg[q] = 0.0f;
+        if (COEF) s_pose[q][tid] = 0.0f;
+    }
+    auto pose_add = [&](int q, float a, float b) {
+        if (COEF)
+            s_pose[q][tid] = fmaf(a, b, s_pose[q][tid]);
+        else
+            pose_reg[q] = fmaf(a, b, pose_reg[q]);
+    };
     int iu, iv;
     tile_pixel<true>(blockIdx.x * 8 * MG_WARPS, blockIdx.z * 4, iu, iv);
     const bool pix_ok = iu < G.nu && iv < G.nv;
@@ -591,9 +609,9 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
             for (int r = 0; r < 3; ++r) gc[r] = fmaf(kap, R.sg[r], R.g0[r]);
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
-                s_pose[9 + r][tid] += gg[r];
+                pose_add(9 + r, gg[r], 1.0f);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) s_pose[3 * r + c][tid] = fmaf(gg[r], gc[c], s_pose[3 * r + c][tid]);
+                for (int c = 0; c < 3; ++c) pose_add(3 * r + c, gg[r], gc[c]);
             }
         };
         // pose sums of dL/dy = gy at kappa: dL/dg' = dL/dy (I + s J), J[c][a] =
@@ -608,12 +626,30 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
             pose(kap, gg);
         };
         if (!spline) {  // CTA-uniform: the pose alone
-            const float u[3] = {0.f, 0.f, 0.f};
+            // the ray's sums of dL/dy and of dL/dy (kappa - mid): the position
+            // is linear in kappa
+            const float u[3] = {0.f, 0.f, 0.f}, mid = 0.5f * kl;
+            float S[3] = {0.f, 0.f, 0.f}, S1[3] = {0.f, 0.f, 0.f};
             for (int kk = 0; kk < K; ++kk) {
                 float g[3];
                 sample(kk, u, g);
-                pose(kk == K - 1 ? kl : (float)kk, g);
+                const float t = (kk == K - 1 ? kl : (float)kk) - mid;
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    S[r] += g[r];
+                    S1[r] = fmaf(t, g[r], S1[r]);
+                }
             }
+            if (K > 0)
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    pose_add(9 + r, S[r], 1.0f);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        pose_add(3 * r + c, S[r], fmaf(mid, R.sg[c], R.g0[c]));
+                        pose_add(3 * r + c, S1[r], R.sg[c]);
+                    }
+                }
             continue;
         }
         SplineLine L;
@@ -626,8 +662,9 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
             // the coefficient step is collective: lanes without work run the
             // loop with zero weight up to the warp's longest ray
             int Kmax = K;
+            if (COEF)
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) Kmax = max(Kmax, __shfl_xor_sync(0xffffffffu, Kmax, off));
+                for (int off = 16; off > 0; off >>= 1) Kmax = max(Kmax, __shfl_xor_sync(0xffffffffu, Kmax, off));
             for (int kk = 0; kk < Kmax; ++kk) {
                 const float kap = kk == K - 1 ? kl : (float)kk;
                 int i0[3];
@@ -640,7 +677,7 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
                     sample(kk, u, gy);
                     point(kap, gy, on, Jx, Jy, Jz);
                 }
-                if (want_coef) {  // CTA-uniform
+                if (COEF && want_coef) {  // CTA-uniform
                     const float v[3] = {mos * gy[0], mos * gy[1], mos * gy[2]};
                     coef_step(CA, s_g64, (i0[2] * 8 + i0[1]) * 8 + i0[0], f, v,
                               kk < K && (v[0] != 0.0f || v[1] != 0.0f || v[2] != 0.0f), s_piece);
@@ -731,7 +768,7 @@ __global__ void __launch_bounds__(MG_THREADS, MG_MIN_BLOCKS)
     // the warps and across CTAs
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-        float v = s_pose[q][tid];
+        float v = COEF ? s_pose[q][tid] : pose_reg[q];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
         if (lane == 0) s_red[q][tid >> 5] = (double)v;
@@ -760,10 +797,13 @@ cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *gra
     const dim3 grid((G.nu + 8 * MG_WARPS - 1) / (8 * MG_WARPS), a.n_idx, (G.nv + 3) / 4);
     const dim3 block(32, MG_WARPS);
     cudaError_t err = cudaSuccess;
-    const bool runs = spline_runs(G, a.spline && grad_coef_idx ? MG_RUN_MIN : MG_RUN_MIN_POSE);
+    const bool runs = a.spline && spline_runs(G, grad_coef_idx ? MG_RUN_MIN : MG_RUN_MIN_POSE);
     auto launch = [&](const auto &vol) {
         typedef std::decay_t<decltype(vol)> V;
-        auto *kernel = runs ? motion_grad_kernel<V, true> : motion_grad_kernel<V, false>;
+        auto *kernel = !a.spline       ? motion_grad_kernel<V, MG_POSE>
+                       : runs          ? motion_grad_kernel<V, MG_RUNS>
+                       : grad_coef_idx ? motion_grad_kernel<V, MG_SAMPLES>
+                                       : motion_grad_kernel<V, MG_WARPED>;
         const int nodes = runs ? 3 * CHEB_N * MG_THREADS * (int)sizeof(float) : 0;  // 53 KB with the static part
         if (runs) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nodes);
         if (err != cudaSuccess) return;
