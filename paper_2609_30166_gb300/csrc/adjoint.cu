@@ -20,6 +20,7 @@ constexpr int ADJ_TX = 32, ADJ_TY = 4;
 // alone needs none of that: eight CTAs, sums in registers (60 views of 128^3
 // 1.82 ms; in the spline's kernel with sums in shared memory 4.0).
 constexpr int MG_WARPS = 4, MG_THREADS = 32 * MG_WARPS, MG_MIN_BLOCKS = 3, MG_POSE_BLOCKS = 8;
+constexpr int MG_POSE_WARPS = 4, MG_WARPED_WARPS = 4;
 // Samples per spline cell from which the gradient goes by runs.  60 views at
 // 64^3 / 80^3 / 96^3 / 112^3 / 128^3 (26 / 32 / 38 / 45 / 51 samples), by
 // samples: 4.8 / 7.7 / 11.1 / 16.3 / 22.1 ms, by runs: 4.9 / 6.8 / 8.8 / 11.8 /
@@ -518,19 +519,20 @@ struct ColumnVolume {
 // sample (short runs, MG_RUN_MIN); MG_RUNS: either of the last two, as above.
 enum MotionGradKind { MG_POSE, MG_WARPED, MG_SAMPLES, MG_RUNS };
 
-template <typename Volume, int KIND>
-__global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS : MG_MIN_BLOCKS)
+template <typename Volume, int KIND, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, (KIND == MG_POSE ? MG_POSE_BLOCKS : MG_MIN_BLOCKS) * MG_WARPS / WARPS)
     motion_grad_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                        const float4 *table, const int *__restrict__ view_idx, const Volume vol,
                        const float *__restrict__ gproj, double *__restrict__ grad_M, double *__restrict__ grad_b,
                        double *__restrict__ grad_coef, unsigned *devcheck)
 {
+    constexpr int THREADS = 32 * WARPS;
     constexpr bool RUNS = KIND == MG_RUNS, COEF = KIND == MG_SAMPLES || RUNS;
     __shared__ float4 s_spline[KIND == MG_POSE ? 1 : SPLINE_TABLE];
     __shared__ double s_g64[COEF ? NCOEF : 1];  // the CTA's coefficient-gradient partials
-    __shared__ double s_red[12][MG_WARPS];
+    __shared__ double s_red[12][WARPS];
     __shared__ float4 s_piece[4];
-    __shared__ float s_pose[COEF ? 12 : 1][MG_THREADS];
+    __shared__ float s_pose[COEF ? 12 : 1][THREADS];
     extern __shared__ float s_V[][MG_THREADS];  // RUNS: the nodes' dL/dy of each thread's run, 3 CHEB_N
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const int lane = tid & 31;
@@ -543,9 +545,9 @@ __global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS :
     const float mos = motion[view].s;
     const bool spline = KIND != MG_POSE && mos != 0.0f;
     const bool want_coef = COEF && spline && grad_coef != nullptr;
-    if (spline) load_spline(s_spline, table, tid, MG_THREADS);
+    if (spline) load_spline(s_spline, table, tid, THREADS);
     if (want_coef)
-        for (int i = tid; i < NCOEF; i += MG_THREADS) s_g64[i] = 0.0;
+        for (int i = tid; i < NCOEF; i += THREADS) s_g64[i] = 0.0;
     if (COEF && tid < 4) s_piece[tid] = bspline_piece(tid);
     __syncthreads();
     float cen[3];
@@ -571,7 +573,7 @@ __global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS :
             pose_reg[q] = fmaf(a, b, pose_reg[q]);
     };
     int iu, iv;
-    tile_pixel<true>(blockIdx.x * 8 * MG_WARPS, blockIdx.z * 4, iu, iv);
+    tile_pixel<true>(blockIdx.x * 8 * WARPS, blockIdx.z * 4, iu, iv);
     const bool pix_ok = iu < G.nu && iv < G.nv;
     const float y = pix_ok ? gproj[((size_t)k * G.nv + iv) * G.nu + iu] * G.inv_sub : 0.0f;
     for (int s = 0; s < G.n_sub; ++s) {
@@ -652,6 +654,7 @@ __global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS :
                 }
             continue;
         }
+        if constexpr (KIND != MG_POSE) {
         SplineLine L;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -762,6 +765,7 @@ __global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS :
                 }
             }
         }
+        }
     }
     if (want_coef) coef_flush(CA, s_g64, lane);
     // CTA reduction of the 12 pose-gradient entries: FP32 warp sums, FP64 over
@@ -777,12 +781,12 @@ __global__ void __launch_bounds__(MG_THREADS, KIND == MG_POSE ? MG_POSE_BLOCKS :
     if (tid < 12) {
         double v = 0.0;
 #pragma unroll
-        for (int w = 0; w < MG_WARPS; ++w) v += s_red[tid][w];
+        for (int w = 0; w < WARPS; ++w) v += s_red[tid][w];
         if (grad_M && tid < 9) atomicAdd(grad_M + 9 * view + tid, v);
         if (grad_b && tid >= 9) atomicAdd(grad_b + 3 * view + (tid - 9), v);
     }
     if (want_coef) {
-        for (int i = tid; i < NCOEF; i += MG_THREADS) {
+        for (int i = tid; i < NCOEF; i += THREADS) {
             const double v = s_g64[i];
             if (v != 0.0) atomicAdd(grad_coef + i, v);
         }
@@ -794,16 +798,17 @@ cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *gra
 {
     if (a.n_idx == 0) return cudaSuccess;
     const Grid &G = *a.grid;
-    const dim3 grid((G.nu + 8 * MG_WARPS - 1) / (8 * MG_WARPS), a.n_idx, (G.nv + 3) / 4);
-    const dim3 block(32, MG_WARPS);
-    cudaError_t err = cudaSuccess;
     const bool runs = a.spline && spline_runs(G, grad_coef_idx ? MG_RUN_MIN : MG_RUN_MIN_POSE);
+    const int warps = !a.spline ? MG_POSE_WARPS : runs || grad_coef_idx ? MG_WARPS : MG_WARPED_WARPS;
+    const dim3 grid((G.nu + 8 * warps - 1) / (8 * warps), a.n_idx, (G.nv + 3) / 4);
+    const dim3 block(32, warps);
+    cudaError_t err = cudaSuccess;
     auto launch = [&](const auto &vol) {
         typedef std::decay_t<decltype(vol)> V;
-        auto *kernel = !a.spline       ? motion_grad_kernel<V, MG_POSE>
-                       : runs          ? motion_grad_kernel<V, MG_RUNS>
-                       : grad_coef_idx ? motion_grad_kernel<V, MG_SAMPLES>
-                                       : motion_grad_kernel<V, MG_WARPED>;
+        auto *kernel = !a.spline       ? motion_grad_kernel<V, MG_POSE, MG_POSE_WARPS>
+                       : runs          ? motion_grad_kernel<V, MG_RUNS, MG_WARPS>
+                       : grad_coef_idx ? motion_grad_kernel<V, MG_SAMPLES, MG_WARPS>
+                                       : motion_grad_kernel<V, MG_WARPED, MG_WARPED_WARPS>;
         const int nodes = runs ? 3 * CHEB_N * MG_THREADS * (int)sizeof(float) : 0;  // 53 KB with the static part
         if (runs) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nodes);
         if (err != cudaSuccess) return;
@@ -917,16 +922,16 @@ __global__ void motion_setup_kernel(const float *__restrict__ theta, const float
 }
 
 // The spline's table (ray.cuh), FP64: thread = (z, y, cell, power).
-__global__ void __launch_bounds__(SPL_PLANE) spline_table_kernel(const float *__restrict__ coef, Frame F,
+__global__ void __launch_bounds__(160) spline_table_kernel(const float *__restrict__ coef, Frame F,
                                                                  float4 *__restrict__ table)
 {
     // f^p coefficients of piece m (B-spline matrix times 6)
     const double B[4][4] = {{1, -3, 3, -1}, {4, 0, -6, 3}, {1, 3, 3, -3}, {0, 0, 0, 1}};
-    const int p = threadIdx.x & 3, cell = threadIdx.x / 4 % 5, y = threadIdx.x / SPL_ROW, z = blockIdx.x;
+    const int p = threadIdx.x & 3, cell = threadIdx.x / 4 % 5, y = threadIdx.x / 20, z = blockIdx.x;
     double s[3] = {0.0, 0.0, 0.0};
     for (int m = 0; m < 4; ++m)
         for (int a = 0; a < 3; ++a) s[a] += B[m][p] / 6.0 * (double)coef[3 * ((z * 8 + y) * 8 + cell + m) + a];
-    table[z * SPL_PLANE + threadIdx.x] =
+    table[z * SPL_PLANE + y * SPL_ROW + cell * 4 + p] =
         make_float4((float)(s[0] / F.vox[0]), (float)(s[1] / F.vox[1]), (float)(s[2] / F.vox[2]), 0.f);
 }
 
@@ -945,7 +950,7 @@ cudaError_t launch_motion_setup(const float *theta, const float *coef, const flo
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (coef) {
-        spline_table_kernel<<<8, SPL_PLANE, 0, stream>>>(coef, F, spline);
+        spline_table_kernel<<<8, 160, 0, stream>>>(coef, F, spline);
         e = cudaGetLastError();
     }
     return e;

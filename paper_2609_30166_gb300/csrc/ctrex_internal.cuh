@@ -219,7 +219,7 @@ size_t adjoint_column_elems(const Grid &g);
 bool adjoint_column_fits(const Grid &g, bool motion, bool along_z);  // its launch shape stays within the grid limits
 cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *grad_M, double *grad_b,
                                double *grad_coef_idx);
-constexpr int SPLINE_TABLE = 8 * 8 * 5 * 4;  // float4 elements of the deformation's table (ray.cuh)
+constexpr int SPLINE_TABLE = 8 * (8 * (5 * 4 + 1) + 1);  // float4 elements of the deformation's table (ray.cuh)
 cudaError_t launch_motion_setup(const float *theta, const float *coef, const float *s_view,
                                 int n_views, const Grid &g, const double vox[3],
                                 const double origin[3], MotionGPU *motion, float4 *spline,

@@ -162,12 +162,15 @@ __device__ __forceinline__ float trilinear(const TV *__restrict__ vol, int nx, i
 // over a cell's 64 coefficients serves two samples of a ray (their loads are
 // what bounds it: a vector load fills a register of every lane, shared
 // address or not).  Table: [z 8][y 8][cell 5][power of f 4] float4 (x, y, z
-// components in voxels), 20 KB, copied to shared memory by each CTA.
+// components in voxels), 21 KB, copied to shared memory by each CTA.
 //
 // 45 views of the 256^3 motion workload, basis functions on three axes and a
 // pass per sample / this: projector 29.7 / 23.8 ms, gradient 118.7 / 104.3 ms
 // (all 64 monomials per cell from a 125 KB table in global memory: 39.5 ms).
-constexpr int SPL_ROW = 5 * 4, SPL_PLANE = 8 * SPL_ROW;
+// Rows and planes are padded to 5 and 1 mod 8 elements, so that lanes in
+// different cells read different banks (unpadded, cells above one another hit
+// the same ones: adjoint with motion, 128 x 128 x 8, 60 views, 1.37 -> 0.64 ms).
+constexpr int SPL_ROW = 5 * 4 + 1, SPL_PLANE = 8 * SPL_ROW + 1;
 static_assert(SPLINE_TABLE == 8 * SPL_PLANE, "spline table size");
 
 __device__ __forceinline__ void load_spline(float4 *s, const float4 *__restrict__ table, int tid, int nthreads)
