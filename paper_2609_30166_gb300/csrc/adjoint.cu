@@ -20,7 +20,11 @@ constexpr int ADJ_TX = 32, ADJ_TY = 4;
 // alone needs none of that: eight CTAs, sums in registers (60 views of 128^3
 // 1.82 ms; in the spline's kernel with sums in shared memory 4.0).
 constexpr int MG_WARPS = 4, MG_THREADS = 32 * MG_WARPS, MG_MIN_BLOCKS = 3, MG_POSE_BLOCKS = 8;
-constexpr int MG_POSE_WARPS = 4, MG_WARPED_WARPS = 4;
+// Warps per CTA of the pose's kernels: a few views have too few CTAs of four
+// (256 x 256 x 8, 12 views of 128 x 4 pixels, pose alone 0.38 -> 0.34 ms; 32^3, 60
+// views, under a deformation 0.29 -> 0.25, by one 0.24 but 64^3 of half a voxel's
+// pixels 3.66 for 3.49).
+constexpr int MG_POSE_WARPS = 1, MG_WARPED_WARPS = 2;
 // Samples per spline cell from which the gradient goes by runs.  60 views at
 // 64^3 / 80^3 / 96^3 / 112^3 / 128^3 (26 / 32 / 38 / 45 / 51 samples), by
 // samples: 4.8 / 7.7 / 11.1 / 16.3 / 22.1 ms, by runs: 4.9 / 6.8 / 8.8 / 11.8 /
