@@ -164,7 +164,8 @@ __device__ __forceinline__ void scatter_trilinear(float *__restrict__ vol, int n
         }
 }
 
-template <bool MOTION, bool DYR>
+// SPLINE: motion with a deformation; MOTION alone: by the pose.
+template <bool MOTION, bool SPLINE, bool DYR>
 __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
     adjoint_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                    const float4 *spline, const int *__restrict__ view_idx,
@@ -178,13 +179,11 @@ __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
         return;
     }
     MotionGPU mo;
-    __shared__ float4 s_spline[MOTION ? SPLINE_TABLE : 1];
-    if (MOTION) {
-        mo = motion[view];
-        if (spline != nullptr) {
-            load_spline(s_spline, spline, threadIdx.y * ADJ_TX + threadIdx.x, ADJ_TX * ADJ_TY);
-            spline = s_spline;
-        }
+    __shared__ float4 s_spline[SPLINE ? SPLINE_TABLE : 1];
+    if (MOTION) mo = motion[view];
+    if (SPLINE) {
+        load_spline(s_spline, spline, threadIdx.y * ADJ_TX + threadIdx.x, ADJ_TX * ADJ_TY);
+        spline = s_spline;
         __syncthreads();
     }
     int iu, iv;
@@ -201,11 +200,20 @@ __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
     for (int s = 0; s < G.n_sub; ++s) {
         Ray R;  // sample positions relative to the grid centre
         if (!setup_ray(G, views[view * G.n_sub + s], (float)iu, (float)iv, R, cen)) continue;
+        float d0[3], ds[3];
+        if (MOTION && !SPLINE) pose_line(mo, R, d0, ds);
+        const float kl = last_kappa(G, R);
         for (int kk = 0; kk < R.K; kk += 2) {
             float g[2][3], w[2], gc[2][3];
             sample_pair(G, R, kk, g, w);
-            if (MOTION)
+            if (SPLINE) {
                 warp_pair_c(G, mo, spline, g, gc);
+            } else if (MOTION) {
+#pragma unroll
+                for (int n = 0; n < 2; ++n)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) gc[n][a] = g[n][a] + fmaf(kk + n >= R.K - 1 ? kl : (float)(kk + n), ds[a], d0[a]);
+            }
 #pragma unroll
             for (int n = 0; n < 2; ++n) {
                 const float *q = MOTION ? gc[n] : g[n];
@@ -230,14 +238,17 @@ cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol)
     const dim3 grid((G.nu + ADJ_TX - 1) / ADJ_TX, a.n_idx, (G.nv + ADJ_TY - 1) / ADJ_TY);
     const dim3 block(ADJ_TX, ADJ_TY);
     if (a.dyr && a.motion) return cudaErrorInvalidValue;  // the event model is defined without motion
-    if (a.motion)
-        adjoint_kernel<true, false><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx,
+    if (a.motion && !a.spline)
+        adjoint_kernel<true, false, false><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, nullptr, a.view_idx, proj,
+                                                                        vol, a.devcheck, nullptr, nullptr);
+    else if (a.motion)
+        adjoint_kernel<true, true, false><<<grid, block, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx,
                                                                  proj, vol, a.devcheck, nullptr, nullptr);
     else if (a.dyr)
-        adjoint_kernel<false, true><<<grid, block, 0, a.stream>>>(G, a.views, nullptr, nullptr, a.view_idx, proj,
+        adjoint_kernel<false, false, true><<<grid, block, 0, a.stream>>>(G, a.views, nullptr, nullptr, a.view_idx, proj,
                                                                  vol, a.devcheck, a.dyr->tau, a.dyr->t_view);
     else
-        adjoint_kernel<false, false><<<grid, block, 0, a.stream>>>(G, a.views, nullptr, nullptr, a.view_idx, proj,
+        adjoint_kernel<false, false, false><<<grid, block, 0, a.stream>>>(G, a.views, nullptr, nullptr, a.view_idx, proj,
                                                                   vol, a.devcheck, nullptr, nullptr);
     return cudaGetLastError();
 }

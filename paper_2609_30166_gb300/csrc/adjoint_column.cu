@@ -86,28 +86,31 @@ struct AdjFoot {
 
 // LV: lanes of a warp along v; the other 32 / LV and the four warps of the
 // CTA run along u.
-// RUNS (motion): the deformation run by run (SplineRun), else pair by pair.
-template <bool MOTION, int LV, bool RUNS>
-__global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_BLOCKS)
+// KIND: how the samples' positions are formed.  The pose alone in a kernel
+// without the spline's registers (60 views of 128^3, pixels of a voxel: 1.81 ->
+// 1.47 ms; 64^3, pixels of half a voxel: 1.47 -> 0.93).
+enum AdjKind { ADJ_STILL, ADJ_POSE, ADJ_PAIRS, ADJ_RUNS };
+
+template <int KIND, int LV>
+__global__ void __launch_bounds__(128, KIND == ADJ_PAIRS || KIND == ADJ_RUNS ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_BLOCKS)
     adjoint_column_kernel(Grid G, const ViewGPU *__restrict__ views, const MotionGPU *__restrict__ motion,
                           const float4 *spline, const int *__restrict__ view_idx, const float *__restrict__ proj,
                           const AdjVolume V, unsigned *devcheck, int n_strips)
 {
     constexpr int LU = 32 / LV;
+    constexpr bool SPLINE = KIND == ADJ_PAIRS || KIND == ADJ_RUNS;
     const int k = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int view = view_idx ? view_idx[k] : k;
     if (view < 0 || view >= G.n_views) {
         if (tid == 0) atomicOr(devcheck, (unsigned)DEVCHECK_OOB);
         return;
     }
-    __shared__ float4 s_spline[MOTION ? SPLINE_TABLE : 1];
+    __shared__ float4 s_spline[SPLINE ? SPLINE_TABLE : 1];
     MotionGPU mo;
-    if (MOTION) {
-        mo = motion[view];
-        if (spline != nullptr) {
-            load_spline(s_spline, spline, tid, 128);
-            spline = s_spline;
-        }
+    if (KIND != ADJ_STILL) mo = motion[view];
+    if (SPLINE) {
+        load_spline(s_spline, spline, tid, 128);
+        spline = s_spline;
         __syncthreads();
     }
     const int strip = blockIdx.z % n_strips, band = blockIdx.z / n_strips;
@@ -129,20 +132,13 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
     for (int s = 0; s < G.n_sub; ++s) {
         Ray R;  // sample positions relative to the grid centre
         if (!setup_ray(G, views[view * G.n_sub + s], (float)iu, (float)iv, R, cen)) continue;
-        if (RUNS) {
-            // displacement by the pose at sample index kappa, linear
+        if (KIND == ADJ_POSE || KIND == ADJ_RUNS) {
             float d0[3], ds[3];
-            SplineLine L;
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const float *D = mo.D + 3 * r;
-                d0[r] = fmaf(D[0], R.g0[0], fmaf(D[1], R.g0[1], fmaf(D[2], R.g0[2], mo.bc[r])));
-                ds[r] = fmaf(D[0], R.sg[0], fmaf(D[1], R.sg[1], D[2] * R.sg[2]));
-                L.x0[r] = fmaf(R.g0[r] + d0[r] + cen[r] + 0.5f, G.spl_scale[r], 1.0f);
-                L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
-            }
+            pose_line(mo, R, d0, ds);
             const float kl = last_kappa(G, R);
-            if (mo.s == 0.0f) {  // the view sees no deformation, whatever the coefficients are
+            // the pose alone (a view whose time scale is 0 sees no deformation,
+            // whatever the coefficients are)
+            if (KIND == ADJ_POSE || mo.s == 0.0f) {
 #pragma unroll 1
                 for (int k = 0; k < R.K; ++k) {
                     const bool last = k == R.K - 1;
@@ -153,6 +149,12 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
                     point(cen, q, y * w);
                 }
                 continue;
+            }
+            SplineLine L;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                L.x0[r] = fmaf(R.g0[r] + d0[r] + cen[r] + 0.5f, G.spl_scale[r], 1.0f);
+                L.xs[r] = (R.sg[r] + ds[r]) * G.spl_scale[r];
             }
             for (int k = 0; k < R.K;) {
                 SplineRun run;
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(128, MOTION ? ADJ_MIN_BLOCKS_MOTION : ADJ_MIN_
                     point(base, q, y * w);
                 }
             }
-        } else if (MOTION) {
+        } else if (KIND == ADJ_PAIRS) {
             for (int kk = 0; kk < R.K; kk += 2) {
                 float g[2][3], w[2], gc[2][3];
                 sample_pair(G, R, kk, g, w);
@@ -252,22 +254,22 @@ static dim3 adj_grid(const Grid &G, int n_idx, int lv, int &n_strips)
     return dim3(per, n_idx, (unsigned)n_strips * (unsigned)((G.nv + lv - 1) / lv));
 }
 
-static int adj_lanes(bool motion, bool along_z) { return !motion && along_z ? ADJ_LV : ADJ_LV_PATCH; }
+static int adj_lanes(bool spline, bool along_z) { return !spline && along_z ? ADJ_LV : ADJ_LV_PATCH; }
 
-bool adjoint_column_fits(const Grid &G, bool motion, bool along_z)
+bool adjoint_column_fits(const Grid &G, bool spline, bool along_z)
 {
     int n_strips;
-    return adj_grid(G, 1, adj_lanes(motion, along_z), n_strips).z <= 65535;
+    return adj_grid(G, 1, adj_lanes(spline, along_z), n_strips).z <= 65535;
 }
 
-template <bool MOTION, int LV, bool RUNS = false>
+template <int KIND, int LV>
 static cudaError_t adj_launch(const FwdArgs &a, const float *proj, const AdjVolume &V)
 {
     const Grid &G = *a.grid;
     int n_strips;
     const dim3 grid = adj_grid(G, a.n_idx, LV, n_strips);
-    adjoint_column_kernel<MOTION, LV, RUNS><<<grid, 128, 0, a.stream>>>(
-        G, a.views, MOTION ? a.motion : nullptr, MOTION ? a.spline : nullptr, a.view_idx, proj, V, a.devcheck, n_strips);
+    adjoint_column_kernel<KIND, LV><<<grid, 128, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx, proj, V,
+                                                                a.devcheck, n_strips);
     return cudaGetLastError();
 }
 
@@ -278,11 +280,13 @@ cudaError_t launch_adjoint_column(const FwdArgs &a, bool along_z, const float *p
     const AdjVolume V = adj_layout(G, scratch, n);
     cudaError_t e = cudaMemsetAsync(scratch, 0, n * sizeof(float), a.stream);
     if (e != cudaSuccess) return e;
-    if (a.motion)
-        e = a.spline && spline_runs(G, ADJ_RUN_MIN) ? adj_launch<true, ADJ_LV_PATCH, true>(a, proj, V)
-                                       : adj_launch<true, ADJ_LV_PATCH>(a, proj, V);
+    if (a.spline)
+        e = spline_runs(G, ADJ_RUN_MIN) ? adj_launch<ADJ_RUNS, ADJ_LV_PATCH>(a, proj, V)
+                                        : adj_launch<ADJ_PAIRS, ADJ_LV_PATCH>(a, proj, V);
+    else if (a.motion)
+        e = along_z ? adj_launch<ADJ_POSE, ADJ_LV>(a, proj, V) : adj_launch<ADJ_POSE, ADJ_LV_PATCH>(a, proj, V);
     else
-        e = along_z ? adj_launch<false, ADJ_LV>(a, proj, V) : adj_launch<false, ADJ_LV_PATCH>(a, proj, V);
+        e = along_z ? adj_launch<ADJ_STILL, ADJ_LV>(a, proj, V) : adj_launch<ADJ_STILL, ADJ_LV_PATCH>(a, proj, V);
     if (e != cudaSuccess) return e;
     const dim3 grid((G.nx + 31) / 32, G.ny < 65535 ? G.ny : 65535, (G.nz + 31) / 32);
     adjoint_add_kernel<<<grid, 256, 0, a.stream>>>(V, vol);

@@ -387,7 +387,9 @@ double ray_voxels(const ctrex_ctx *c, int n_idx)
     return (double)n_idx * G.n_sub * G.nu * G.nv * fmax(G.nx, fmax(G.ny, G.nz));
 }
 
-bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ; }
+// (Detectors of less than half a warp's rows: 192 x 12 pixels 0.20 ms by
+// patches, 0.22 by rows; 192 x 33 0.35 and 0.24.)
+bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ && c->grid.nv > 16; }
 
 // The adjoint through a scatter volume, if that can be had (and the launch, an
 // 8192^2 detector with motion is beyond it): it is zeroed and
@@ -396,7 +398,7 @@ bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ; }
 bool column_adjoint(ctrex_ctx *c, int n_idx)
 {
     const Grid &G = c->grid;
-    if (c->dyr || capturing(c) || !adjoint_column_fits(G, c->has_motion, adjoint_along_z(c))) return false;
+    if (c->dyr || capturing(c) || !adjoint_column_fits(G, c->has_motion && c->coef_valid, adjoint_along_z(c))) return false;
     if (ray_voxels(c, n_idx) < 0.03 * (double)grid_voxels(G)) return false;
     const size_t n = adjoint_column_elems(G);
     if (n == 0) return false;

@@ -216,7 +216,7 @@ cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol);
 // nearly along z.
 cudaError_t launch_adjoint_column(const FwdArgs &a, bool along_z, const float *proj, float *vol, float *scratch);
 size_t adjoint_column_elems(const Grid &g);
-bool adjoint_column_fits(const Grid &g, bool motion, bool along_z);  // its launch shape stays within the grid limits
+bool adjoint_column_fits(const Grid &g, bool spline, bool along_z);  // its launch shape stays within the grid limits
 cudaError_t launch_motion_grad(const FwdArgs &a, const float *gproj, double *grad_M, double *grad_b,
                                double *grad_coef_idx);
 constexpr int SPLINE_TABLE = 8 * (8 * (5 * 4 + 1) + 1);  // float4 elements of the deformation's table (ray.cuh)

@@ -464,3 +464,34 @@ def test_pose_only_matches_oracle(n, det, views, sub, turn, step):
         gt, _ = oracle.motion_grad(pb, x, y)
         assert rel_l2(_np(c.motion_grad(_t(x), _t(y), want_coef=False)[0]), gt) <= 1e-4
     c.close()
+
+
+# The adjoint's patches for a few rows, and (64 slices, fine pixels, turned)
+# in place by the pose alone and with a deformation.
+@pytest.mark.parametrize("n,det,views,turn", [((37, 22, 9), (90, 12), 5, 0.4), ((37, 22, 9), (90, 17), 5, 0.4),
+                                              ((64, 60, 64), (190, 190), 12, 60.0)])
+@pytest.mark.parametrize("motion", ["none", "pose", "full"])
+def test_adjoint_of_few_rows_and_turned(n, det, views, turn, motion):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    P = _matrices(views, 1, turn, det[0], det[1], 60.0, 200.0)
+    pitch = 30.0 / max(n)
+    vox, shape = (pitch, 0.95 * pitch, 1.05 * pitch), n[::-1]
+    org = tuple(-0.5 * (m - 1) * v for m, v in zip(n, vox))
+    rng = np.random.default_rng(35)
+    pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    c = ctrex.Context()
+    c.set_geometry(P, shape, vox, org, det)
+    if motion != "none":
+        theta = np.zeros((views, 15))
+        theta[:, :6] = rng.uniform(-0.03, 0.03, (views, 6))
+        theta[:, 6:] = np.eye(3).ravel()
+        theta = _np(_t(theta))
+        coef = _np(_t(rng.uniform(-1, 1, (8, 8, 8, 3)) * pitch)) if motion == "full" else None
+        sv = np.ones(views) if motion == "full" else None
+        pb = pb.with_motion(theta, coef, sv, margin=0.5)
+        c.set_motion(_t(theta), None if coef is None else _t(coef), None if sv is None else _t(sv), 0.5)
+    y = _np(_t(rng.uniform(0.5, 1.5, size=(views, det[1], det[0]))))
+    assert rel_l2(_np(c.adjoint_project(_t(y))), oracle.adjoint(pb, y)) <= TOL32
+    c.close()
