@@ -20,6 +20,11 @@ constexpr int ADJ_LV = 32, ADJ_LV_PATCH = 8;
 // CTAs per SM: the spline needs 168 registers to keep out of local memory (4
 // CTAs at 128: 30.3 ms, 2: 26.6).
 constexpr int ADJ_MIN_BLOCKS = 8, ADJ_MIN_BLOCKS_MOTION = 3;
+// Shared memory that a CTA of the pose's patches asks for and leaves alone: three
+// CTAs per SM, as with the spline.  More warps at a time reduce into lines
+// further apart (256 x 256 x 24, 4 views turned by 20 degrees, 0.7 voxels a
+// pixel: 0.32 ms; with 64 registers and as many CTAs as fit 0.65).
+constexpr int ADJ_POSE_SHARED = 72 * 1024;
 // Samples per spline cell from which the deformation goes by runs.  60 views
 // at 64^3 / 80^3 / 96^3 (26 / 32 / 38 samples), by pairs: 0.76 / 1.36 / 2.14
 // ms, by runs: 0.82 / 1.30 / 1.90 ms.
@@ -268,8 +273,14 @@ static cudaError_t adj_launch(const FwdArgs &a, const float *proj, const AdjVolu
     const Grid &G = *a.grid;
     int n_strips;
     const dim3 grid = adj_grid(G, a.n_idx, LV, n_strips);
-    adjoint_column_kernel<KIND, LV><<<grid, 128, 0, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx, proj, V,
-                                                                a.devcheck, n_strips);
+    const int shared = KIND == ADJ_POSE && LV == ADJ_LV_PATCH ? ADJ_POSE_SHARED : 0;
+    if (shared) {
+        const cudaError_t e = cudaFuncSetAttribute(adjoint_column_kernel<KIND, LV>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, shared);
+        if (e != cudaSuccess) return e;
+    }
+    adjoint_column_kernel<KIND, LV><<<grid, 128, shared, a.stream>>>(G, a.views, a.motion, a.spline, a.view_idx, proj,
+                                                                     V, a.devcheck, n_strips);
     return cudaGetLastError();
 }
 

@@ -387,9 +387,11 @@ double ray_voxels(const ctrex_ctx *c, int n_idx)
     return (double)n_idx * G.n_sub * G.nu * G.nv * fmax(G.nx, fmax(G.ny, G.nz));
 }
 
-// (Detectors of less than half a warp's rows: 192 x 12 pixels 0.20 ms by
-// patches, 0.22 by rows; 192 x 33 0.35 and 0.24.)
-bool adjoint_along_z(const ctrex_ctx *c) { return c->col_lean <= COL_LEAN_ADJ && c->grid.nv > 16; }
+// (By the pose and a few rows, patches: 192 x 12 pixels 0.23 ms, rows 0.28.)
+bool adjoint_along_z(const ctrex_ctx *c)
+{
+    return c->col_lean <= COL_LEAN_ADJ && (!c->has_motion || c->grid.nv > 16);
+}
 
 // The adjoint through a scatter volume, if that can be had (and the launch, an
 // 8192^2 detector with motion is beyond it): it is zeroed and
