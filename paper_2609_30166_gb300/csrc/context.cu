@@ -61,6 +61,7 @@ struct ctrex_ctx {
     ColStore img_col;  // the correction images
     // the last use of the stores and the scatter volume (ScratchUse)
     cudaEvent_t scratch_done = nullptr;
+    unsigned long long scratch_stream = 0;  // its id (unique among all streams ever made)
     bool scratch_open = false;
     // texture atlas of the correction images read by the backprojector
     AtlasStore img_atlas;
@@ -174,7 +175,11 @@ cudaError_t scratch_begin(ctrex_ctx *c)
 {
     if (c->scratch_open || capturing(c)) return cudaSuccess;
     c->scratch_open = true;
-    return cudaStreamWaitEvent(c->stream, c->scratch_done, 0);
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamGetId(c->stream, &id);
+    if (e == cudaSuccess && id != c->scratch_stream) e = cudaStreamWaitEvent(c->stream, c->scratch_done, 0);
+    c->scratch_stream = id;
+    return e;
 }
 
 struct ScratchUse {
