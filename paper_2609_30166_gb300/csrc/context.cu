@@ -50,7 +50,7 @@ struct ctrex_ctx {
     AtlasStore vol_atlas;
     Atlas vol_atlas_view;
     // the volume in column layout, where the scan's detector columns run along z
-    double col_lean = 10.0, col_step = 1.0;  // detector_column_step
+    double col_lean = 10.0, col_step = 1.0, col_pixel = 1.0;  // detector_column_step
     bool bp_flat = false, bp_flat_roi = false;  // backproject_flat (Cartesian grids)
     ColStore vol_col;
     ColStore col1;     // the ROI grid, or the event model's final values
@@ -406,7 +406,24 @@ bool column_adjoint(ctrex_ctx *c, int n_idx)
 {
     const Grid &G = c->grid;
     if (c->dyr || capturing(c) || !adjoint_column_fits(G, c->has_motion && c->coef_valid, adjoint_along_z(c))) return false;
-    if (ray_voxels(c, n_idx) < 0.03 * (double)grid_voxels(G)) return false;
+    const double rays = ray_voxels(c, n_idx), vox = (double)grid_voxels(G);
+    if (rays < 0.03 * vox) return false;
+    // Turned detectors (no deformation, enough rays to fill the GPU): the rays
+    // of a warp drift apart, with fine pixels soonest, while in place they share
+    // footprints; large volumes with coarse pixels miss the L2 by way of the
+    // scatter volume.  256^3, 16 views, ms here / in place at 10, 35, 60
+    // degrees: 0.4 voxels a pixel 37.9 / 41.1, 46.3 / 42.8, 53.1 / 42.5; 2 voxels
+    // 2.25 / 2.01, 2.67 / 2.01, 2.77 / 2.00 (by the pose, whose patches keep to
+    // three CTAs per SM, fine pixels only).  Of 4872 scans (32^2 to 256^2 in x and
+    // y, 8 to 256 slices, 1 to 60 views, 0 to 88 degrees) 157 take more than 3 %
+    // longer than in place before there was a scatter volume; 330 with columns
+    // throughout.
+    const double pixel = c->col_pixel;
+    if (!(c->has_motion && c->coef_valid) && G.nz >= 32 && rays >= 2e7) {
+        if (pixel < 0.55 && c->col_lean > 0.45) return false;
+        if (!c->has_motion && pixel < 1.0 && c->col_lean > 1.0) return false;
+        if (!c->has_motion && pixel >= 1.6 && vox > 6e6 && rays >= 3e7 && c->col_lean > 0.1) return false;
+    }
     const size_t n = adjoint_column_elems(G);
     if (n == 0) return false;
     if (n > c->adj_elems) {
@@ -754,18 +771,20 @@ static int compute_views(ctrex_ctx *c, const double *P, int nvs, int n_sub, cons
 }
 
 // A pixel step along a detector column, in index coordinates at the volume's
-// depth: its sideways part over its part along z, and the latter (means over
-// the views).
-static void detector_column_step(const std::vector<ViewGPU> &hv, double &lean, double &step)
+// depth: its sideways part over its part along z, the latter, and its length
+// (means over the views).
+static void detector_column_step(const std::vector<ViewGPU> &hv, double &lean, double &step, double &pixel)
 {
-    lean = step = 0.0;
+    lean = step = pixel = 0.0;
     for (const ViewGPU &V : hv) {
         const double xy = sqrt((double)V.qv[0] * V.qv[0] + (double)V.qv[1] * V.qv[1]), z = fabs((double)V.qv[2]);
         lean += xy <= 10.0 * z ? xy / z : 10.0;
         step += z;
+        pixel += sqrt(xy * xy + z * z);
     }
     lean /= (double)hv.size();
     step /= (double)hv.size();
+    pixel /= (double)hv.size();
 }
 
 static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub, const int n[3], const double vox[3],
@@ -826,7 +845,7 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
     c->has_geom = true;
     c->atlas_unfit = false;
     c->img_atlas_unfit = false;
-    detector_column_step(hv, c->col_lean, c->col_step);
+    detector_column_step(hv, c->col_lean, c->col_step, c->col_pixel);
     c->bp_flat = backproject_flat(G, hv.data(), nvs);
     set_clip_box(c);
     return CTREX_OK;
