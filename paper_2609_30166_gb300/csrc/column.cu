@@ -9,18 +9,19 @@ void col_release(ColStore &s)
     s = ColStore();
 }
 
-// At least n zeroed pairs.  Not in a capture, where the zeros would be written
-// by the replay while the store counts as laid out at once.
+// At least n zeroed pairs; a buffer that holds them and is not twice as large
+// is kept, another one is replaced, and a refusal leaves the store as it was.
+// Not in a capture, where the zeros would be written by the replay while the
+// store counts as laid out at once.
 static cudaError_t col_alloc(ColStore &s, size_t n, cudaStream_t stream)
 {
     if (stream_capturing(stream)) return cudaErrorInvalidValue;
     const size_t bytes = n * sizeof(float2);
-    s.nx = 0;
-    if (bytes > s.bytes) {
-        col_release(s);
+    if (bytes > s.bytes || bytes < s.bytes / 2) {
         size_t free = 0, total = 0;
         cudaError_t e = cudaMemGetInfo(&free, &total);
-        if (e == cudaSuccess && bytes > free / 2) return cudaErrorInvalidValue;
+        if (e == cudaSuccess && bytes > (free + s.bytes) / 2) return cudaErrorInvalidValue;
+        col_release(s);
         if (e == cudaSuccess) e = cudaMalloc(&s.buf, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -29,6 +30,7 @@ static cudaError_t col_alloc(ColStore &s, size_t n, cudaStream_t stream)
         }
         s.bytes = bytes;
     }
+    s.nx = 0;
     return cudaMemsetAsync(s.buf, 0, bytes, stream);
 }
 

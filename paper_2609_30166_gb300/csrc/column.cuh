@@ -52,7 +52,7 @@ struct ColStore {
 };
 void col_release(ColStore &s);
 // Lays the store out for a volume (zero border written once); an allocation
-// that fits is kept.  cudaErrorInvalidValue: the layout's 32-bit indices
+// that fits, and is not twice as large, is kept.  cudaErrorInvalidValue: the layout's 32-bit indices
 // cannot hold it, it would take more than half of the free device memory, or
 // the stream is capturing (the caller keeps its other path).
 cudaError_t col_ensure(ColStore &s, int nx, int ny, int nz, cudaStream_t stream, bool wrap = false);

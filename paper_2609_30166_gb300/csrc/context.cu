@@ -63,6 +63,7 @@ struct ctrex_ctx {
     cudaEvent_t scratch_done = nullptr;
     unsigned long long scratch_stream = 0;  // its id (unique among all streams ever made)
     bool scratch_open = false;
+    bool scratch_captured = false;  // a graph may hold the stores' addresses
     // texture atlas of the correction images read by the backprojector
     AtlasStore img_atlas;
     Atlas img_atlas_view;
@@ -173,7 +174,11 @@ bool capturing(const ctrex_ctx *c) { return stream_capturing(c->stream); }
 
 cudaError_t scratch_begin(ctrex_ctx *c)
 {
-    if (c->scratch_open || capturing(c)) return cudaSuccess;
+    if (c->scratch_open) return cudaSuccess;
+    if (capturing(c)) {
+        c->scratch_captured = true;
+        return cudaSuccess;
+    }
     c->scratch_open = true;
     unsigned long long id = 0;
     cudaError_t e = cudaStreamGetId(c->stream, &id);
@@ -202,13 +207,37 @@ template <typename T> void dfree(T *&p)
     p = nullptr;
 }
 
+// Gives the column scratch back (laid out again by the next call that uses it).
+void release_columns(ctrex_ctx *c)
+{
+    col_release(c->vol_col);
+    col_release(c->col1);
+    col_release(c->tau_col);
+    c->tau_col_set = false;
+    col_release(c->img_col);
+    dfree(c->d_adj);
+    c->adj_elems = 0;
+}
+
+// An allocation, with the column scratch given back if it fails at first:
+// nothing that fits without the scratch is refused for it (unless a graph may
+// hold its addresses).
+template <typename Make> cudaError_t alloc_or_release(ctrex_ctx *c, Make make)
+{
+    cudaError_t e = make();
+    if (e != cudaErrorMemoryAllocation || c->scratch_captured) return e;
+    cudaGetLastError();
+    release_columns(c);
+    return make();
+}
+
 int ensure(ctrex_ctx *c, void **p, size_t *have, size_t need, const char *what)
 {
     if (*have >= need && *p) return CTREX_OK;
     if (*p) cudaFree(*p);
     *p = nullptr;
     *have = 0;
-    cudaError_t e = cudaMalloc(p, need);
+    cudaError_t e = alloc_or_release(c, [&] { return cudaMalloc(p, need); });
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(c, CTREX_E_NOMEM, "cannot allocate %zu bytes for %s: %s", need, what, cudaGetErrorString(e));
@@ -426,14 +455,17 @@ bool column_adjoint(ctrex_ctx *c, int n_idx)
     }
     const size_t n = adjoint_column_elems(G);
     if (n == 0) return false;
-    if (n > c->adj_elems) {
-        dfree(c->d_adj);
-        c->adj_elems = 0;
+    if (n > c->adj_elems || n < c->adj_elems / 2) {
         size_t free = 0, total = 0;
-        if (cudaMemGetInfo(&free, &total) != cudaSuccess || n * sizeof(float) > free / 2 ||
-            cudaMalloc((void **)&c->d_adj, n * sizeof(float)) != cudaSuccess) {
+        const bool fits = cudaMemGetInfo(&free, &total) == cudaSuccess &&
+                          n * sizeof(float) <= (free + c->adj_elems * sizeof(float)) / 2;
+        if (fits) {
+            dfree(c->d_adj);
+            c->adj_elems = 0;
+        }
+        if (!fits || cudaMalloc((void **)&c->d_adj, n * sizeof(float)) != cudaSuccess) {
             cudaGetLastError();
-            c->d_adj = nullptr;
+            if (fits) c->d_adj = nullptr;
             return false;
         }
         c->adj_elems = n;
@@ -463,7 +495,16 @@ int prepare_columns(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
         if (e == cudaSuccess) e = col_upload(c->tau_col, c->d_tau, CTREX_F32, c->stream, true);
         c->tau_col_set = e == cudaSuccess;
     }
-    if (e == cudaErrorInvalidValue) return CTREX_OK;
+    if (e == cudaErrorInvalidValue) {
+        // the atlases need not fit beside stores that only a part of the model got
+        if ((c->dyr || c->roi) && !c->scratch_captured) {
+            col_release(c->vol_col);
+            col_release(c->col1);
+            col_release(c->tau_col);
+            c->tau_col_set = false;
+        }
+        return CTREX_OK;
+    }
     if (e == cudaSuccess) e = col_upload(c->vol_col, vol, vdt, c->stream, c->dyr);
     if (e == cudaSuccess && (c->dyr || c->roi))
         e = col_upload(c->col1, static_cast<const char *>(vol) + grid_voxels(c->grid) * dtype_size(vdt), vdt,
@@ -486,8 +527,10 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     if (c->projector == CTREX_PROJ_JOSEPH) {
         // x-, y- and z-slice stacks in one atlas; no row-major fallback
         const int nx = c->grid.nx, ny = c->grid.ny, nz = c->grid.nz;
-        cudaError_t e = atlas_ensure(c->jos_atlas, nx > ny ? nx : ny, ny > nz ? ny : nz, nx + ny + nz,
-                                     vdt == CTREX_BF16, c->device, false);
+        cudaError_t e = alloc_or_release(c, [&] {
+            return atlas_ensure(c->jos_atlas, nx > ny ? nx : ny, ny > nz ? ny : nz, nx + ny + nz,
+                                vdt == CTREX_BF16, c->device, false);
+        });
         if (e == cudaErrorInvalidValue) {
             cudaGetLastError();
             return fail(c, CTREX_E_SHAPE, "Joseph projector: volume exceeds the 2D texture limits of the device");
@@ -506,8 +549,9 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
         AtlasStore *st[2] = {&c->vol_atlas, &c->dyr_atlas1};
         Atlas *vw[2] = {&c->vol_atlas_view, &c->dyr_atlas1_view};
         for (int i = 0; i < 2; ++i) {
-            cudaError_t e = atlas_ensure(*st[i], c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device,
-                                         false);
+            cudaError_t e = alloc_or_release(c, [&] {
+                return atlas_ensure(*st[i], c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device, false);
+            });
             if (e == cudaErrorInvalidValue) {
                 cudaGetLastError();
                 return fail(c, CTREX_E_SHAPE, "event model: the volume exceeds the 2D texture limits of the device");
@@ -529,7 +573,9 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
         AtlasStore *st[2] = {&c->vol_atlas, &c->roi_atlas};
         Atlas *vw[2] = {&c->vol_atlas_view, &c->roi_atlas_view};
         for (int i = 0; i < 2; ++i) {
-            cudaError_t e = atlas_ensure(*st[i], gs[i]->nx, gs[i]->ny, gs[i]->nz, vdt == CTREX_BF16, c->device, false);
+            cudaError_t e = alloc_or_release(c, [&] {
+                return atlas_ensure(*st[i], gs[i]->nx, gs[i]->ny, gs[i]->nz, vdt == CTREX_BF16, c->device, false);
+            });
             if (e == cudaErrorInvalidValue) {
                 cudaGetLastError();
                 return fail(c, CTREX_E_SHAPE, "ROI projection: a grid exceeds the 2D texture limits of the device");
@@ -546,8 +592,10 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     if (c->cyl) {
         // cylindrical domain: z-slice tiles of N_r x (N_phi + 1), the last row
         // repeating sector 0; no row-major fallback
-        cudaError_t e = atlas_ensure(c->vol_atlas, c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device,
-                                     false, true);
+        cudaError_t e = alloc_or_release(c, [&] {
+            return atlas_ensure(c->vol_atlas, c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device,
+                                false, true);
+        });
         if (e == cudaErrorInvalidValue) {
             cudaGetLastError();
             return fail(c, CTREX_E_SHAPE, "cylindrical volume exceeds the 2D texture limits of the device");
@@ -561,8 +609,10 @@ int prepare_atlas(ctrex_ctx *c, FwdArgs &a, const void *vol, int vdt)
     }
     if (c->atlas_unfit) return CTREX_OK;
     // BF16 volumes: slice pairs packed in 32-bit texels, one gather per sample
-    cudaError_t e = atlas_ensure(c->vol_atlas, c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device,
-                                 vdt == CTREX_BF16);
+    cudaError_t e = alloc_or_release(c, [&] {
+        return atlas_ensure(c->vol_atlas, c->grid.nx, c->grid.ny, c->grid.nz, vdt == CTREX_BF16, c->device,
+                            vdt == CTREX_BF16);
+    });
     if (e == cudaErrorInvalidValue) {
         cudaGetLastError();
         c->atlas_unfit = true;
@@ -846,6 +896,10 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
     c->atlas_unfit = false;
     c->img_atlas_unfit = false;
     detector_column_step(hv, c->col_lean, c->col_step, c->col_pixel);
+    if (c->col_lean > COL_LEAN_FWD) {  // beyond every column kernel but the adjoint's
+        col_release(c->vol_col);
+        col_release(c->img_col);
+    }
     c->bp_flat = backproject_flat(G, hv.data(), nvs);
     set_clip_box(c);
     return CTREX_OK;
@@ -1144,7 +1198,9 @@ int ctrex_set_dyrect(ctrex_ctx *c, const float *tau, const float *t_view)
     if (!c->d_tview) CT_CUDA(c, cudaMalloc((void **)&c->d_tview, sizeof(float) * V));
     CT_CUDA(c, cudaMemcpyAsync(c->d_tau, tau, sizeof(float) * nvox, cudaMemcpyDeviceToDevice, c->stream));
     CT_CUDA(c, cudaMemcpyAsync(c->d_tview, t_view, sizeof(float) * V, cudaMemcpyDeviceToDevice, c->stream));
-    cudaError_t e = atlas_ensure(c->tau_atlas, c->grid.nx, c->grid.ny, c->grid.nz, false, c->device, false);
+    cudaError_t e = alloc_or_release(c, [&] {
+        return atlas_ensure(c->tau_atlas, c->grid.nx, c->grid.ny, c->grid.nz, false, c->device, false);
+    });
     if (e == cudaErrorInvalidValue) {
         cudaGetLastError();
         dyr_release(c);
@@ -1249,7 +1305,9 @@ static int bp_images(ctrex_ctx *c, BpArgs &a, const void *r, int rdt, int n_idx)
         }
     }
     if (n_idx > 0 && !a.column && !c->img_atlas_unfit) {
-        cudaError_t ae = atlas_ensure(c->img_atlas, c->grid.nu, c->grid.nv, n_idx, rdt == CTREX_BF16, c->device);
+        cudaError_t ae = alloc_or_release(c, [&] {
+            return atlas_ensure(c->img_atlas, c->grid.nu, c->grid.nv, n_idx, rdt == CTREX_BF16, c->device);
+        });
         if (ae == cudaErrorInvalidValue) {
             cudaGetLastError();
             c->img_atlas_unfit = true;

@@ -1,0 +1,93 @@
+"""The memory of the column layouts: given back when a smaller or a turned scan
+takes the place of the one it was made for, refused where it would take more
+than half of what is free, and given back where another allocation needs it;
+every operator then runs on its other path."""
+
+import numpy as np
+import pytest
+import torch
+
+from tests.helpers import rel_l2
+from tests.test_gpu_columns import _matrices, _np, _t
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+def _geometry(c, n, det, views, turn=0.3):
+    vox = 32.0 / n
+    c.set_geometry(_matrices(views, 1, turn, *det, 96.0, 200.0), (n, n, n), (vox,) * 3, (-0.5 * (n - 1) * vox,) * 3, det)
+
+
+def _free():
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _context():
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    return ctrex.Context()
+
+
+@pytest.mark.parametrize("then", [(24, (32, 32), 5, 0.3), (256, (300, 300), 60, 60.0)])
+def test_given_back_with_the_geometry(then):
+    def scan(c, n, det, views, turn):
+        _geometry(c, n, det, views, turn)
+        x, y = torch.rand((n, n, n), device="cuda"), torch.rand((views, det[1], det[0]), device="cuda")
+        c.fwd_project(x)
+        c.back_project(y)
+        c.adjoint_project(y)
+
+    first = (256, (300, 300), 60, 0.3)
+    for shape in (first, then):  # loads the kernels
+        c = _context()
+        scan(c, *shape)
+        c.close()
+    c = _context()
+    before = _free()
+    scan(c, *first)
+    assert before - _free() > 220 * MB  # volume 139, images 50, scatter volume 73
+    scan(c, *then)
+    kept = before - _free()
+    # a turned scan keeps the scatter volume (73) beside its atlases (67 and 22)
+    assert kept < (170 * MB if then[0] == 256 else 20 * MB)
+    c.close()
+
+
+def test_refused_and_released_where_memory_is_short():
+    c = _context()
+    n, det, views = 256, (256, 256), 400
+    _geometry(c, n, det, views)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.rand((n, n, n), generator=g, device="cuda")
+    y = torch.rand((views, det[1], det[0]), generator=g, device="cuda")
+    vi = np.arange(0, views, 40, dtype=np.int32)
+    few = y[:len(vi)].contiguous()
+    ops = {"forward": lambda: c.fwd_project(x, view_idx=vi), "backproject": lambda: c.back_project(y, normalize=False),
+           "few": lambda: c.back_project(few, normalize=False, view_idx=vi),
+           "adjoint": lambda: c.adjoint_project(few, view_idx=vi)}
+    theta = torch.zeros((views, 15), device="cuda")
+    theta[:, 6] = theta[:, 10] = theta[:, 14] = 1.0
+    want = {k: _np(f()) for k, f in ops.items()}
+    c.set_motion(theta, None, None, 0.0)
+    grad = _np(c.motion_grad(x, few, view_idx=vi, want_coef=False)[0])
+    c.close()
+
+    c = _context()
+    _geometry(c, n, det, views)
+    left = 460 * MB  # half of it holds no store of 400 images (237) after the volume's (139)
+    hold = torch.empty(_free() - left, dtype=torch.uint8, device="cuda")
+    try:
+        for _ in range(2):
+            for k, f in ops.items():
+                assert rel_l2(_np(f()), want[k]) <= 1e-5
+                torch.cuda.empty_cache()
+        c.set_motion(theta, None, None, 0.0)
+        assert rel_l2(_np(c.motion_grad(x, few, view_idx=vi, want_coef=False)[0]), grad) <= 1e-4
+    finally:
+        del hold
+        c.close()
