@@ -495,3 +495,56 @@ def test_adjoint_of_few_rows_and_turned(n, det, views, turn, motion):
     y = _np(_t(rng.uniform(0.5, 1.5, size=(views, det[1], det[0]))))
     assert rel_l2(_np(c.adjoint_project(_t(y))), oracle.adjoint(pb, y)) <= TOL32
     c.close()
+
+
+# Backprojection by columns in every model, at heights whose blocks of 64 or 128
+# slices fit, overlap or (a tiny volume) reach beyond the last one; by FP32 and
+# 16-bit images, a view list, sub-angles.
+@pytest.mark.parametrize("model", ["static", "window", "event", "cylinder", "roi", "subvoxel"])
+@pytest.mark.parametrize("nz,sub,width", [(64, 4, 220.0), (100, 1, 220.0), (127, 1, 70.0), (150, 2, 220.0), (250, 1, 90.0),
+                                          (5, 1, 220.0)])
+def test_backprojection_blocks_match_oracle(model, nz, sub, width):
+    from paper_2609_30166_gb300 import _build, ctrex
+
+    _build.build_library()
+    nx, ny, det, views = 11, 9, (60, 76), 5
+    P = _matrices(views, sub, 0.3, *det, width, 200.0)
+    pitch = 30.0 / max(nz, 20)
+    shape, vox = (nz, ny, nx), (pitch, pitch, pitch)
+    org = tuple(-0.5 * (m - 1) * pitch for m in (nx, ny, nz))
+    rng = np.random.default_rng(11)
+    c = ctrex.Context()
+    if model == "cylinder":
+        shape, args = (nz, ny, 6), dict(n_r=6, n_phi=ny, n_z=nz, dr=pitch, dz=pitch)
+        c.set_geometry_cylinder(P, det=det, **args)
+        pb = oracle.cylinder_problem(P, det=det, **args)
+    else:
+        c.set_geometry(P, shape, vox, org, det)
+        pb = oracle.Problem(P, shape, vox, org, det, 0.5)
+    if model == "window":
+        win = np.stack([[3 + v, det[0] - 5, 4, det[1] - 9 + v] for v in range(views)]).astype(np.int32)
+        c.set_bp_window(win)
+        pb = pb.with_window(win)
+    elif model == "event":
+        tau, tv = rng.uniform(0.0, 1.0, size=shape), np.linspace(0, 1, views)
+        c.set_dyrect(_t(tau), _t(tv))
+        pb = pb.with_dyrect(_np(_t(tau)), _np(_t(tv)))
+    elif model == "roi":
+        roi = ((max(nz // 2, 1), 7, 8), (0.5 * pitch,) * 3, (-1.75 * pitch, -1.5 * pitch, -0.25 * (max(nz // 2, 1) - 1) * pitch))
+        c.set_roi(*roi)
+        pb = pb.with_roi(*roi)
+    elif model == "subvoxel":
+        c.set_bp_subvoxel(2)
+        pb = pb.with_subvoxel(2)
+    iu, iv = np.meshgrid(np.arange(det[0]), np.arange(det[1]))
+    r = np.stack([np.cos(0.11 * iu + k) + np.sin(0.07 * iv * (k + 1)) + 2.5 for k in range(views)])
+    x = rng.uniform(0.2, 1.0, size=c.vol_shape)
+    want, b, _ = oracle.backproject(pb, _np(_t(r)), alpha=0.7, x=_np(_t(x)))
+    assert rel_l2(_np(c.back_project(_t(r), vol=_t(x), alpha=0.7)), want) <= TOL32
+    r16 = _t(r, torch.bfloat16)
+    _, b, _ = oracle.backproject(pb, _np(r16))
+    assert rel_l2(_np(c.back_project(r16, normalize=False, accumulate=False)), b) <= TOL32
+    vi = np.array([4, 1], dtype=np.int32)
+    _, b, _ = oracle.backproject(pb, _np(_t(r[vi])), views=vi)
+    assert rel_l2(_np(c.back_project(_t(r[vi]), normalize=False, accumulate=False, view_idx=vi)), b) <= TOL32
+    c.close()
