@@ -122,19 +122,6 @@ __device__ __forceinline__ float col_interp(const ColPairs &t, float ax, float a
     return lerp(y.x, y.y, az);
 }
 
-// Trilinear interpolation at index coordinates (gx, gy, gz), each in
-// [-1, n); taps outside the grid read the border's zeros.  ax .. az: the
-// fractions.
-__device__ __forceinline__ float col_sample(const ColVolume &V, float gx, float gy, float gz, float &ax, float &ay,
-                                            float &az)
-{
-    const float fx = floorf(gx), fy = floorf(gy), fz = floorf(gz);
-    ax = gx - fx;
-    ay = gy - fy;
-    az = gz - fz;
-    return col_interp(col_load(V, V.index((int)fx + 1, (int)fy + 1, (int)fz + 1)), ax, ay, az);
-}
-
 // Fraction of a 32.32 fixed-point number from its low word: its top 23 bits
 // placed behind the exponent of 1.
 __device__ __forceinline__ float fixed_fraction(unsigned lo)

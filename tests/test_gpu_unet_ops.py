@@ -182,3 +182,15 @@ def test_batched_bias_gradient(mods, relu):
     for k in range(3):
         (want,) = torch.autograd.grad(y, layer.b, grad_outputs=dy[k], retain_graph=True)
         assert torch.allclose(db[k], want, rtol=0, atol=8 * 2.0 ** -24 * float(dy[k].float().abs().sum()))
+
+
+def test_bias_grad_of_long_sums(mods):
+    """103 terms a thread, of one sign: the bound of test_bias_grad."""
+    ctrex, _ = mods
+    g = torch.Generator(device="cuda").manual_seed(4)
+    dy = (torch.randn((2, 200, 200, 200, 16), generator=g, device="cuda") + 1.0).to(torch.bfloat16)
+    _, db = ctrex.conv3d_bias_grad(dy)
+    flat = dy.reshape(-1, 16)
+    want = sum(part.double().sum(0) for part in flat.split(1 << 21))
+    size = sum(part.double().abs().sum(0) for part in flat.split(1 << 21))
+    assert bool(((db.double() - want).abs() <= 8 * 2.0 ** -24 * size).all())
