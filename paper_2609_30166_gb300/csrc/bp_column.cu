@@ -406,10 +406,11 @@ __global__ void __launch_bounds__(BPC_THREADS, SUBV ? BPC_SUBV_MIN_BLOCKS : (DYR
 // slower (256^3, 90 views: 2.57 ms for 2.31), which stays there.  u and v
 // count from a whole column and a chunk of rows below them (the image pointer
 // takes the rest), so that they round less.
+// Two voxels a thread: six CTAs per SM (40 registers), four: five.
 // DEEP: a grid of few CTAs (bpc_launch), which waits for its loads: four terms
 // in flight, 64 registers.
 template <typename TV, int VZ, bool DEEP>
-__global__ void __launch_bounds__(BPC_THREADS, DEEP ? 4 : BPC_MIN_BLOCKS)
+__global__ void __launch_bounds__(BPC_THREADS, DEEP ? 4 : (VZ == 2 ? 6 : BPC_MIN_BLOCKS))
     bp_flat_kernel(Grid G, const ViewGPU *__restrict__ views, const int *__restrict__ view_idx, int n_idx,
                    const ColImages I, TV *__restrict__ vol, const float *__restrict__ w, float alpha, int normalize,
                    int accumulate)
@@ -558,6 +559,14 @@ cudaError_t launch_backproject_column(const BpArgs &a)
 bool backproject_column_fits(const Grid &G)
 {
     return (G.ny + BPC_WY - 1) / BPC_WY <= 65535 && (G.nz + 63) / 64 <= 65535;
+}
+
+bool backproject_box(const ViewGPU &view, const float lo[3], const float hi[3], int4 w)
+{
+    const float *P = view.P;
+    return box_inside(make_float4(P[0], P[1], P[2], P[3]), make_float4(P[4], P[5], P[6], P[7]),
+                      make_float4(P[8], P[9], P[10], P[11]), lo, hi,
+                      make_float4((float)w.x, (float)w.y, (float)w.z, (float)w.w)) > 0;
 }
 
 bool backproject_flat(const Grid &G, const ViewGPU *views, int n)

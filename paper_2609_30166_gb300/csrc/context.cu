@@ -52,6 +52,9 @@ struct ctrex_ctx {
     // the volume in column layout, where the scan's detector columns run along z
     double col_lean = 10.0, col_step = 1.0, col_pixel = 1.0;  // detector_column_step
     bool bp_flat = false, bp_flat_roi = false;  // backproject_flat (Cartesian grids)
+    std::vector<ViewGPU> hviews;     // the views, and the windows, on the host
+    std::vector<int4> hwindow;
+    double bp_inside = 0.0;          // set_bp_inside
     ColStore vol_col;
     ColStore col1;     // the ROI grid, or the event model's final values
     ColStore tau_col;  // the event model's transition times
@@ -363,32 +366,39 @@ bool column_forward(const ctrex_ctx *c, int vdt)
     return u4 * v32 <= u32 * v4 * gain;
 }
 
-// The backprojector: time by columns over time by gathers, fitted to 8638 scans
-// of all kinds and both image types (64^2 to 512^2 voxels in x and y, 8 to 512
-// slices, pixel steps of 0.3 to 3.5 voxels, 0 to 38 degrees of lean).  A pixel
-// step of s voxels spreads a warp's 32 voxels over 32 / s rows and lean * 32 / s
-// columns, each one more line; blocks of 64 or 128 slices repeat slices, and a
-// block beyond the volume, or a turned detector that cuts the object off, takes
-// terms to the general path.  90 views, 256 x 256 in x and y, 0.8 voxels a
-// pixel, static FP32, ms columns / gathers: 256 slices 1.64 / 2.89, 130 1.43 /
-// 1.50, 70 0.95 / 0.82, 50 0.89 / 0.60, 20 0.73 / 0.28; 256 slices at 8, 15, 22
-// degrees 2.1 / 2.9, 2.5 / 2.9, 2.9 / 2.9.  The choice takes more than 3 %
-// longer than gathers on 132 of the scans (18 % at most without a detector
-// window, 29 % with one); with one lean limit for all, and thin volumes left to
-// gathers for the static model only, on 3265, up to seven times as long.
-double bp_column_cost(const ctrex_ctx *c, const Grid &G, int rdt, double step, bool tiny)
+// The backprojector: time by columns over time by gathers, fitted to 12,700
+// scans of all kinds and both image types (40^2 to 512^2 voxels in x and y, 8 to
+// 512 slices, pixel steps of 0.3 to 3.5 voxels, 0 to 38 degrees of lean).
+// - A pixel step of s voxels spreads a warp's 32 voxels over 32 / s rows and
+//   lean * 32 / s columns, each one more line (256^3, 90 views, 0.8 voxels a
+//   pixel, static FP32, ms columns / gathers at 0, 8, 15, 22 degrees: 1.6 / 2.9,
+//   2.1 / 2.9, 2.5 / 2.9, 2.9 / 2.9).
+// - Blocks of 64 or 128 slices repeat slices, which costs where the launch has
+//   more than a wave or two of CTAs (`full`; 12 slices of 256 x 256 take 2.2 times
+//   the gathers' time, of 72 x 72 0.77; 70 slices 1.15 and 0.94).
+// - Terms of a block that reaches beyond the detector or a window, as the part
+//   beyond a volume of less than 64 slices may, take the general path (28 slices
+//   of 256 x 256: 1.4 -> 2.9; 96 behind a window that cuts them 0.9 -> 1.4).
+// What is chosen takes more than 3 % longer than gathers on 583 of the scans,
+// 10 % on 143; one lean limit for all, with a height rule for the static model
+// alone, was slower on 3265 of 8638 of them, up to seven times.
+double bp_column_cost(const ctrex_ctx *c, const Grid &G, int rdt, double step)
 {
     struct {
         double base, rows, cols, bf16;
-    } k = {0.49, 0.13, 0.63, 1.2};  // static, cylinder
+    } k = {0.49, 0.13, 0.63, 1.22};  // static, cylinder
     if (c->bp_subvoxel > 1)
         k = {0.56, 0.10, 0.24, 1.02};
     else if (c->dyr)
-        k = {0.55, 0.07, 0.59, 1.2};
+        k = {0.55, 0.07, 0.59, 1.12};
     else if (c->has_window)
-        k = {0.70, 0.06, 0.70, 1.12};
-    const double slices = backproject_column_slices(G, c->dyr || c->bp_subvoxel > 1);
-    const double blocks = tiny ? 1.0 : slices / G.nz * (G.nz < 64 ? 1.5 : 1.0);
+        k = {0.60 + 0.35 * (1.0 - c->bp_inside), 0.06, 0.70, 1.12};
+    const bool subv = c->bp_subvoxel > 1;
+    const double slices = backproject_column_slices(G, c->dyr || subv), ctas = (G.nx + 7) / 8 * (double)G.ny * (slices / 64.0);
+    const double wave = subv ? 1500.0 : 3000.0, full = c->col_lean > 0.1 ? 1.0 : ctas * ctas / (ctas * ctas + wave * wave);
+    const double out = fmin(2.5 * (1.0 - c->bp_inside), 1.0);
+    const double blocks = (1.0 - 0.2 * (1.0 - full) * (1.0 - out)) * (1.0 + (slices / G.nz - 1.0) * full) *
+                          (1.0 + 0.9 * out * fmin(fmax((64 - G.nz) / 24.0, 0.0), 1.0));
     // what a turn moves the volume's sides along the detector's rows by, over its height
     const double width = c->cyl ? 2.0 * G.nx * c->cylg.dr / c->cylg.dz : (double)(G.nx > G.ny ? G.nx : G.ny);
     return blocks * (rdt == CTREX_BF16 ? k.bf16 : 1.0) *
@@ -401,15 +411,10 @@ bool column_backproject(const ctrex_ctx *c, int rdt)
     const Grid &G = c->grid;
     if (!(c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(G) && (!c->roi || backproject_column_fits(c->roi_grid))))
         return false;
-    // a launch of less than a wave waits for its loads, however little of it
-    // is of use (64 x 64 x 20, 90 views: 78 us by columns, 86 by gathers)
-    auto tiny = [](const Grid &g, int nz) { return (g.nx + 7) / 8 * (double)g.ny <= 760.0 && g.nz <= nz; };
-    if (c->bp_subvoxel == 1 && !c->roi && tiny(G, 24)) return c->col_lean <= 0.55;
-    double cost = bp_column_cost(c, G, rdt, c->col_step, c->roi && tiny(G, 128));
+    double cost = bp_column_cost(c, G, rdt, c->col_step);
     if (c->roi) {
-        const Grid &R = c->roi_grid;
-        const double v = (double)grid_voxels(G), w = (double)grid_voxels(R);
-        cost = (cost * v + bp_column_cost(c, R, rdt, c->col_step * c->roig.sc[2], tiny(R, 128)) * w) / (v + w);
+        const double v = (double)grid_voxels(G), w = (double)grid_voxels(c->roi_grid);
+        cost = (cost * v + bp_column_cost(c, c->roi_grid, rdt, c->col_step * c->roig.sc[2]) * w) / (v + w);
     }
     return cost <= 1.0;
 }
@@ -837,6 +842,47 @@ static void detector_column_step(const std::vector<ViewGPU> &hv, double &lean, d
     pixel /= (double)hv.size();
 }
 
+// What share of the backprojection's blocks (columns side by side, 64 slices)
+// project inside the detector or the window and take the short path, from a
+// sample: eight views, nine places in x and y, the first, a middle and the last
+// block of slices (0.05 ms).
+static void set_bp_inside(ctrex_ctx *c)
+{
+    const Grid &G = c->grid;
+    const int n = (int)c->hviews.size(), blocks = (G.nz + 63) / 64, nv = n < 8 ? n : 8;
+    int inside = 0, all = 0;
+    for (int i = 0; i < nv; ++i) {
+        const int view = (int)((long long)i * n / nv);
+        const int4 win = c->has_window ? c->hwindow[(size_t)(view / G.n_sub)] : make_int4(0, G.nu - 1, 0, G.nv - 1);
+        for (int q = 0; q < 9; ++q)
+            for (int z = 0; z < 3 && z < blocks; ++z) {
+                const int zb = z == 0 ? 0 : (z == 1 ? (blocks - 1 + (blocks > 2)) / 2 : blocks - 1);
+                const int z0 = zb * 64 + 64 > G.nz && G.nz > 64 ? G.nz - 64 : zb * 64;
+                float lo[3], hi[3];
+                if (c->cyl) {  // the axis and eight places around it
+                    const double a = 0.25 * M_PI * q, r = q == 8 ? 0.0 : 0.7 * c->cylg.R;
+                    const double p[2] = {r * cos(a), r * sin(a)};
+                    for (int k = 0; k < 2; ++k) {
+                        lo[k] = (float)(p[k] - 4.0 * c->cylg.dr);
+                        hi[k] = (float)(p[k] + 4.0 * c->cylg.dr);
+                    }
+                    lo[2] = (z0 - c->cylg.zc) * c->cylg.dz;
+                    hi[2] = (z0 + 63 - c->cylg.zc) * c->cylg.dz;
+                } else {
+                    const int wide = G.nx < 8 ? G.nx : 8;  // the first, middle and last columns
+                    lo[0] = (float)((G.nx - wide) * (q % 3) / 2);
+                    hi[0] = lo[0] + wide - 1;
+                    lo[1] = hi[1] = (float)((G.ny - 1) * (q / 3) / 2);
+                    lo[2] = (float)z0;
+                    hi[2] = (float)(z0 + 63);
+                }
+                inside += backproject_box(c->hviews[(size_t)view], lo, hi, win);
+                ++all;
+            }
+    }
+    c->bp_inside = (double)inside / all;
+}
+
 static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub, const int n[3], const double vox[3],
                           const double origin[3], const double ctr[3], double min_pitch, const ctrex_det_grid *det,
                           double step_vox)
@@ -901,6 +947,9 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
         col_release(c->img_col);
     }
     c->bp_flat = backproject_flat(G, hv.data(), nvs);
+    c->hviews.swap(hv);
+    c->hwindow.clear();
+    set_bp_inside(c);
     set_clip_box(c);
     return CTREX_OK;
 }
@@ -1010,6 +1059,8 @@ int ctrex_set_geometry_cylinder(ctrex_ctx *c, const double *P, int n_views, int 
     c->grid.hi[2] = C.Z;
     c->cyl = true;
     c->col_step /= cyl->dz;  // frame mm to slices
+    c->col_pixel /= cyl->dz;
+    set_bp_inside(c);
     c->projector = CTREX_PROJ_TRILINEAR;
     return CTREX_OK;
 }
@@ -1073,6 +1124,7 @@ int ctrex_set_bp_window(ctrex_ctx *c, const int *window)
     if (!c->has_geom) return fail(c, CTREX_E_STATE, "set_bp_window before set_geometry");
     if (!window) {
         c->has_window = false;
+        set_bp_inside(c);
         return CTREX_OK;
     }
     const int V = c->grid.n_views;
@@ -1087,6 +1139,8 @@ int ctrex_set_bp_window(ctrex_ctx *c, const int *window)
     CT_CUDA(c, cudaMemcpyAsync(c->d_window, hw.data(), sizeof(int4) * (size_t)V, cudaMemcpyHostToDevice, c->stream));
     CT_CUDA(c, cudaStreamSynchronize(c->stream));  // hw is a local buffer
     c->has_window = true;
+    c->hwindow.swap(hw);
+    set_bp_inside(c);
     return CTREX_OK;
 }
 

@@ -209,6 +209,9 @@ int backproject_column_slices(const Grid &g, bool two);  // slices it works thro
 // Whether every one of n views (on the host) has the whole volume inside the
 // detector and every z column at one depth, to FP32 rounding.
 bool backproject_flat(const Grid &g, const ViewGPU *views, int n);
+// Whether a view has the box lo .. hi of its frame inside a detector window
+// (u_lo, u_hi, v_lo, v_hi), by a margin.
+bool backproject_box(const ViewGPU &view, const float lo[3], const float hi[3], int4 window);
 
 cudaError_t launch_adjoint(const FwdArgs &a, const float *proj, float *vol);
 // The same through a scatter volume of adjoint_column_elems(G) floats
