@@ -883,6 +883,14 @@ static void set_bp_inside(ctrex_ctx *c)
     c->bp_inside = (double)inside / all;
 }
 
+// Gives back the stores of an earlier geometry that this one does not use.
+static void drop_unused_columns(ctrex_ctx *c)
+{
+    DeviceGuard g(c->device);
+    if (!column_forward(c, CTREX_F32) && !column_forward(c, CTREX_BF16)) col_release(c->vol_col);
+    if (!column_backproject(c, CTREX_F32) && !column_backproject(c, CTREX_BF16)) col_release(c->img_col);
+}
+
 static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub, const int n[3], const double vox[3],
                           const double origin[3], const double ctr[3], double min_pitch, const ctrex_det_grid *det,
                           double step_vox)
@@ -942,10 +950,6 @@ static int build_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub,
     c->atlas_unfit = false;
     c->img_atlas_unfit = false;
     detector_column_step(hv, c->col_lean, c->col_step, c->col_pixel);
-    if (c->col_lean > COL_LEAN_FWD) {  // beyond every column kernel but the adjoint's
-        col_release(c->vol_col);
-        col_release(c->img_col);
-    }
     c->bp_flat = backproject_flat(G, hv.data(), nvs);
     c->hviews.swap(hv);
     c->hwindow.clear();
@@ -978,7 +982,9 @@ int ctrex_set_geometry(ctrex_ctx *c, const double *P, int n_views, int n_sub, co
         ctr[a] = vol->origin[a] + 0.5 * (n[a] - 1) * vol->vox[a];
         minv = fmin(minv, vol->vox[a]);
     }
-    return build_geometry(c, P, n_views, n_sub, n, vol->vox, vol->origin, ctr, minv, det, step_vox);
+    const int e = build_geometry(c, P, n_views, n_sub, n, vol->vox, vol->origin, ctr, minv, det, step_vox);
+    if (e == CTREX_OK) drop_unused_columns(c);
+    return e;
 }
 
 int ctrex_set_geometry_cylinder(ctrex_ctx *c, const double *P, int n_views, int n_sub, const ctrex_cyl_grid *cyl,
@@ -1062,6 +1068,7 @@ int ctrex_set_geometry_cylinder(ctrex_ctx *c, const double *P, int n_views, int 
     c->col_pixel /= cyl->dz;
     set_bp_inside(c);
     c->projector = CTREX_PROJ_TRILINEAR;
+    drop_unused_columns(c);
     return CTREX_OK;
 }
 

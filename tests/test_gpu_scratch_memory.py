@@ -90,4 +90,5 @@ def test_refused_and_released_where_memory_is_short():
         assert rel_l2(_np(c.motion_grad(x, few, view_idx=vi, want_coef=False)[0]), grad) <= 1e-4
     finally:
         del hold
+        torch.cuda.empty_cache()
         c.close()
