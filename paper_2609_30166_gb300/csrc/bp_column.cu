@@ -132,6 +132,7 @@ __device__ __noinline__ float4 bp_voxel(const ViewGPU *__restrict__ views, const
             sum.x += b;
             sum.y += c;
         }
+        if (!DYR && isnan(sum.x)) break;  // and stays it, whatever the weights
     }
     return sum;
 }
