@@ -143,11 +143,11 @@ class ClockSampler:
 # evaluated at 720 views.  Valid only for the kernel
 # sources it was taken on (hash below) and for the FP32 workload; otherwise
 # null.
-_T16, _T180 = 8923595520 + 230469376, 11978356480 + 1531409408
+_T16, _T180 = 8926221312 + 230551296, 11975691264 + 1530015232
 FWD_TRAFFIC_BYTES = int(_T16 + (_T180 - _T16) * (720 - 16) / (180 - 16))
 FWD_TRAFFIC_SOURCES = ("fwd_column.cu", "fwd_column.cuh", "column.cuh", "column.cu", "ray.cuh", "fwd_common.cuh",
                        "ctrex_internal.cuh")
-FWD_TRAFFIC_HASH = "553ebdd040001460"
+FWD_TRAFFIC_HASH = "ec87ff8a3d9ff1b2"
 
 
 def fwd_traffic(dtype, views):
