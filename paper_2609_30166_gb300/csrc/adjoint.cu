@@ -212,7 +212,10 @@ __global__ void __launch_bounds__(ADJ_TX *ADJ_TY)
 #pragma unroll
                 for (int n = 0; n < 2; ++n)
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) gc[n][a] = g[n][a] + fmaf(kk + n >= R.K - 1 ? kl : (float)(kk + n), ds[a], d0[a]);
+                    for (int a = 0; a < 3; ++a) {
+                        const float kap = kk + n >= R.K - 1 ? kl : (float)(kk + n);
+                        gc[n][a] = g[n][a] + fmaf(kap, ds[a], d0[a]);
+                    }
             }
 #pragma unroll
             for (int n = 0; n < 2; ++n) {

@@ -394,8 +394,9 @@ double bp_column_cost(const ctrex_ctx *c, const Grid &G, int rdt, double step)
     else if (c->has_window)
         k = {0.60 + 0.35 * (1.0 - c->bp_inside), 0.06, 0.70, 1.12};
     const bool subv = c->bp_subvoxel > 1;
-    const double slices = backproject_column_slices(G, c->dyr || subv), ctas = (G.nx + 7) / 8 * (double)G.ny * (slices / 64.0);
-    const double wave = subv ? 1500.0 : 3000.0, full = c->col_lean > 0.1 ? 1.0 : ctas * ctas / (ctas * ctas + wave * wave);
+    const double slices = backproject_column_slices(G, c->dyr || subv);
+    const double ctas = (G.nx + 7) / 8 * (double)G.ny * (slices / 64.0), wave = subv ? 1500.0 : 3000.0;
+    const double full = c->col_lean > 0.1 ? 1.0 : ctas * ctas / (ctas * ctas + wave * wave);
     const double out = fmin(2.5 * (1.0 - c->bp_inside), 1.0);
     const double blocks = (1.0 - 0.2 * (1.0 - full) * (1.0 - out)) * (1.0 + (slices / G.nz - 1.0) * full) *
                           (1.0 + 0.9 * out * fmin(fmax((64 - G.nz) / 24.0, 0.0), 1.0));
@@ -409,8 +410,8 @@ double bp_column_cost(const ctrex_ctx *c, const Grid &G, int rdt, double step)
 bool column_backproject(const ctrex_ctx *c, int rdt)
 {
     const Grid &G = c->grid;
-    if (!(c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(G) && (!c->roi || backproject_column_fits(c->roi_grid))))
-        return false;
+    if (!(c->col_step >= COL_STEP_BP_MIN && backproject_column_fits(G))) return false;
+    if (c->roi && !backproject_column_fits(c->roi_grid)) return false;
     double cost = bp_column_cost(c, G, rdt, c->col_step);
     if (c->roi) {
         const double v = (double)grid_voxels(G), w = (double)grid_voxels(c->roi_grid);
@@ -432,23 +433,23 @@ bool adjoint_along_z(const ctrex_ctx *c)
     return c->col_lean <= COL_LEAN_ADJ && (!c->has_motion || c->grid.nv > 16);
 }
 
-// The adjoint through a scatter volume, if that can be had (and the launch, an
-// 8192^2 detector with motion is beyond it): it is zeroed and
-// added once per call, so the call's rays have to outweigh it (one view of
-// 64^2 pixels on 512^3: 0.71 ms, 0.65 in place; 768^2: 1.7, 3.6 in place).
+// The adjoint through a scatter volume, if that can be had (and its launch: an
+// 8192^2 detector with motion is beyond it).  The volume is zeroed and added
+// once per call, so the call's rays have to outweigh it (one view of 64^2
+// pixels on 512^3: 0.71 ms, 0.65 in place; 768^2: 1.7, 3.6 in place).
 bool column_adjoint(ctrex_ctx *c, int n_idx)
 {
     const Grid &G = c->grid;
-    if (c->dyr || capturing(c) || !adjoint_column_fits(G, c->has_motion && c->coef_valid, adjoint_along_z(c))) return false;
+    if (c->dyr || capturing(c)) return false;
+    if (!adjoint_column_fits(G, c->has_motion && c->coef_valid, adjoint_along_z(c))) return false;
     const double rays = ray_voxels(c, n_idx), vox = (double)grid_voxels(G);
     if (rays < 0.03 * vox) return false;
     // Turned detectors (no deformation, enough rays to fill the GPU): the rays
-    // of a warp drift apart, with fine pixels soonest, while in place they share
-    // footprints; large volumes with coarse pixels miss the L2 by way of the
-    // scatter volume.  256^3, 16 views, ms here / in place at 10, 35, 60
-    // degrees: 0.4 voxels a pixel 37.9 / 41.1, 46.3 / 42.8, 53.1 / 42.5; 2 voxels
-    // 2.25 / 2.01, 2.67 / 2.01, 2.77 / 2.00 (by the pose, whose patches keep to
-    // three CTAs per SM, fine pixels only).  Of 4872 scans (32^2 to 256^2 in x and
+    // of a warp drift apart in z, with fine pixels soonest, while in place they
+    // share footprints; large volumes with coarse pixels lose too.  256^3, 16
+    // views, ms here / in place at 10, 35, 60 degrees: 0.4 voxels a pixel 37.9 /
+    // 41.1, 46.3 / 42.8, 53.1 / 42.5; 2 voxels 2.25 / 2.01, 2.67 / 2.01, 2.77 /
+    // 2.00 (by the pose, whose patches keep to three CTAs per SM, fine pixels only).  Of 4872 scans (32^2 to 256^2 in x and
     // y, 8 to 256 slices, 1 to 60 views, 0 to 88 degrees) 157 take more than 3 %
     // longer than in place before there was a scatter volume; 330 with columns
     // throughout.
